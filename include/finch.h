@@ -14,7 +14,7 @@
  * --------------------------------
  *  - All tensor pointers are DEVICE pointers unless a parameter says "host".
  *    The caller owns every buffer, including the workspace; the library allocates
- *    only the context and one 4-byte device status word and frees only those.
+ *    only the context (with a few bytes of device memory, see finch_ctx_create) and frees only that.
  *  - Work is enqueued asynchronously on `cuda_stream` (a cudaStream_t passed as
  *    void*; NULL = the legacy default stream).  No call synchronises except
  *    finch_device_status and finch_step_host.
@@ -139,7 +139,8 @@ typedef struct {
 /* Create a context for one model shape on one device.  Fails with FINCH_ERR_UNSUPPORTED when the device is not
  * compute capability 10.x or the shape is not covered, FINCH_ERR_INVALID_ARG on inconsistent fields
  * (n_q_heads not a multiple of n_kv_heads, non-positive sizes, a rotary base below 1).  *out is set only on success.
- * Device memory the context owns, freed by finch_ctx_destroy: a 4-byte status word, a side stream with three events
+ * Device memory the context owns, freed by finch_ctx_destroy: a 4-byte status word, two 4-byte counters per layer and
+ * KV head, a side stream with three events
  * (used by finch_step_host), and, with rope_theta > 0, the cosine/sine table of the re-positioning,
  * (max_candidates + 1) x head_dim/2 pairs of fp32 (2 MiB for 4096 candidates and head_dim 128), computed in double
  * precision on the host during this call. */
@@ -171,11 +172,11 @@ finch_status finch_score(finch_ctx *ctx, const finch_tensor *prompt_q, const fin
 /* Which kernels finch_score and finch_step run for a batch (given a workspace of finch_workspace_bytes).  Host
  * arithmetic, nothing is enqueued, works on a validation-only context.  (The paper prescribes no kernel; this is how
  * its prompt x candidate block, Section "Method", is tiled here.)
- *  - FINCH_SCORE_ONE_KERNEL: bf16, head_dim 64 or 128, a single request without row_limit, at most four 128-row
- *    query tiles per KV head (queries per KV head x ceil(prompt rows / 64) <= 8), and a window length for its key
- *    tiles exists: a divisor W of the tiles per (layer, KV head) unit with W >= 4 (or the whole unit),
- *    tiles / W <= 8, the persistent grid's CTA x window slots >= 85 % full, and W x SMs x tile bytes <= 40 MiB
- *    unless no shorter window qualifies; of several the fullest, longer ones preferred.
+ *  - FINCH_SCORE_ONE_KERNEL: bf16, head_dim 64 or 128, a single request without row_limit, at most 512 query rows
+ *    per KV head (queries per KV head x prompt rows rounded up to 8), and a window length for its key tiles exists: a
+ *    divisor W of the tiles per (layer, KV head) unit with tiles / W <= 64 and either one window per SM or W >= 2,
+ *    the persistent grid's CTA x window slots >= 85 % full and W x SMs x tile bytes <= 48 MiB (unless no shorter
+ *    window qualifies); of several the one with the smallest windows x (W + 1).
  *    *window receives W (key tiles of 128 candidates).  Both sweeps of the softmax run in one persistent kernel.
  *  - FINCH_SCORE_TWO_LAUNCH: bf16, head_dim 64 or 128 otherwise (several requests, causal rows, longer prompts, no
  *    usable window): row statistics and column sums in two tensor-core launches.  *window = 0.
@@ -195,9 +196,9 @@ finch_status finch_score_plan(const finch_ctx *ctx, const finch_batch *batch, in
  *  - Limit: n_layers * n_q_heads * total_q must not exceed finch_score_static_max_rows() (2^20 rows); a larger
  *    batch is rejected with FINCH_ERR_WORKSPACE_TOO_SMALL and nothing is enqueued -- use finch_score then.
  *  - Which kernels run: the tensor-core kernels need more of the array than one entry per prompt row (in 8-byte
- *    entries, for a single request: 32 per prompt row plus 2 per layer, KV head and candidate; for a batch of
- *    requests: 5 per prompt row plus the same 2 per candidate).  A batch within the row limit whose need
- *    exceeds the array's 2^20 entries -- a whole 32-layer step of 4096 candidates does -- runs on the warp-level
+ *    entries: four per query row and key range -- rows counted with a KV head's heads padded to multiples of 8 and
+ *    their total to a multiple of 128 -- and 2 per layer, KV head and candidate).  A batch within the row limit whose
+ *    need exceeds the array's 2^20 entries -- a whole 32-layer step of 4096 candidates does -- runs on the warp-level
  *    kernels instead: the same result within the score tolerance, many times slower.  finch_score_static_path
  *    tells which it will be.  Because the kernels (or their key ranges) can differ from finch_score's, the two
  *    calls agree within the score tolerance, max(1e-3 relative, 1e-5 absolute), not bit for bit.

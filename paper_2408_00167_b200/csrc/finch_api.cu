@@ -59,8 +59,12 @@ WsLayout ws_layout(const finch_ctx *ctx, const finch_batch *b) {
     w.lse_bytes = (size_t)mv.L * mv.Hq * (size_t)b->total_q * sizeof(float2) * (kScoreMaxSplits * 4 + 1) +
                   (4 * n_kv_scores + 2) * sizeof(float) +  // row statistics, partial scores per KV head,
                   ((size_t)b->batch + 1) * 8 + 4096;       // and the item plan of a multi-request batch
-    const size_t fused = score_fused_scratch(*ctx, view_of(b)) * sizeof(float2);  // the one-kernel path's layout
-    w.lse_bytes = align_up(w.lse_bytes > fused ? w.lse_bytes : fused);
+    // what each path needs at least: the one-kernel layout, one key split of the two-launch layout
+    const size_t fused = score_fused_scratch(*ctx, view_of(b)) * sizeof(float2);
+    const size_t two = score_tc_supported(*ctx) ? score_tc_scratch_min(*ctx, view_of(b)) * sizeof(float2) : 0;
+    if (fused > w.lse_bytes) w.lse_bytes = fused;
+    if (two > w.lse_bytes) w.lse_bytes = two;
+    w.lse_bytes = align_up(w.lse_bytes);
     w.scores_off = w.lse_off + w.lse_bytes;
     w.scores_bytes = align_up((size_t)mv.L * mv.G * ((size_t)b->total_cache + b->total_chunk) * sizeof(float));
     w.total = w.scores_off + w.scores_bytes;
@@ -212,6 +216,7 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out) {
     ctx->sm_count = 0;
     ctx->copy_stream = nullptr;
     ctx->ev_entry = ctx->ev_v_ready = ctx->ev_selected = nullptr;
+    ctx->tickets = nullptr;
     ctx->launches = 0;
     if (!ctx->dry) {
         int n_dev = 0;
@@ -237,7 +242,14 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out) {
             delete ctx;
             return FINCH_ERR_OOM;
         }
+        const size_t ticket_bytes = 2 * (size_t)mv.L * mv.Hkv * sizeof(int);
+        if (cudaMalloc(&ctx->tickets, ticket_bytes) != cudaSuccess) {
+            (void)cudaGetLastError();
+            finch_ctx_destroy(ctx);
+            return FINCH_ERR_OOM;
+        }
         if (cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess ||
+            cudaMemset(ctx->tickets, 0, ticket_bytes) != cudaSuccess ||
             cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_entry, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_v_ready, cudaEventDisableTiming) != cudaSuccess ||
@@ -278,6 +290,7 @@ void finch_ctx_destroy(finch_ctx *ctx) {
     if (ctx->ev_selected) cudaEventDestroy(ctx->ev_selected);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->model.rope_table) cudaFree(const_cast<float2 *>(ctx->model.rope_table));
+    if (ctx->tickets) cudaFree(ctx->tickets);
     if (ctx->d_status) cudaFree(ctx->d_status);
     delete ctx;
 }
@@ -458,6 +471,12 @@ finch_status finch_device_status(finch_ctx *ctx, void *cuda_stream, int32_t *out
         (void)cudaGetLastError();
         return FINCH_ERR_CUDA;
     }
+    // a scoring kernel whose waits ran out leaves its counters behind: the next one needs them at zero
+    if (host && (cudaMemsetAsync(ctx->tickets, 0, 2 * (size_t)ctx->model.L * ctx->model.Hkv * sizeof(int), stream) != cudaSuccess ||
+                 cudaStreamSynchronize(stream) != cudaSuccess)) {
+        (void)cudaGetLastError();
+        return FINCH_ERR_CUDA;
+    }
     *out = host;
     return host ? FINCH_ERR_DEVICE_STATUS : FINCH_OK;
 }
@@ -477,6 +496,13 @@ namespace {
 
 constexpr size_t kStaticRows = size_t(1) << 20;  // prompt rows (layers x query heads x packed prompt tokens): 8 MiB
 static __device__ __align__(256) float2 g_static_row_stats[kStaticRows];
+
+// How much of the array the tensor-core kernels may use for a batch: two entries per layer, KV head and candidate are
+// set aside, which keeps batches of very many candidates on the warp-level kernels (their scratch is a row's entry).
+size_t static_tc_capacity(const finch_ctx *ctx, const finch_batch *b) {
+    const size_t cand = (size_t)ctx->model.L * ctx->model.Hkv * ((size_t)b->total_cache + b->total_chunk);
+    return 2 * cand < kStaticRows ? kStaticRows - 2 * cand : 0;
+}
 
 constexpr int kMaxDevices = 64;
 // device address of the array on each device, filled on first use; contexts on different host threads share it
@@ -518,7 +544,7 @@ extern "C" finch_status finch_score_static(finch_ctx *ctx, const finch_tensor *p
     float2 *row_stats = nullptr;
     if ((s = static_scratch(ctx->cfg.device, &row_stats))) return s;
     return cuda_status(run_score(*ctx, view_of(prompt_q), view_of(cache_k), view_of(chunk_k), view_of(batch), scores,
-                                 row_stats, kStaticRows, row_lse, (cudaStream_t)cuda_stream));
+                                 row_stats, static_tc_capacity(ctx, batch), row_lse, (cudaStream_t)cuda_stream));
 }
 
 extern "C" size_t finch_score_static_max_rows(void) { return kStaticRows; }
@@ -543,8 +569,8 @@ extern "C" finch_status finch_score_static_path(const finch_ctx *ctx, const finc
     finch_status s = check_batch(ctx, batch);
     if (s) return s;
     const BatchView bv = view_of(batch);
-    const size_t fused = score_fused_scratch(*ctx, bv);
+    const size_t fused = score_fused_scratch(*ctx, bv), capacity = static_tc_capacity(ctx, batch);
     *tensor_cores = score_tc_supported(*ctx) &&
-                    ((fused > 0 && fused <= kStaticRows) || score_tc_scratch_min(*ctx, bv) <= kStaticRows);
+                    ((fused > 0 && fused <= capacity) || score_tc_scratch_min(*ctx, bv) <= capacity);
     return FINCH_OK;
 }

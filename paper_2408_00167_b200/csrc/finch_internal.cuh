@@ -47,6 +47,7 @@ struct Ctx {
     int *d_status;  // device status word (nullptr for a validation-only context)
     bool dry;       // validation-only context: nothing is ever enqueued
     int sm_count;
+    int *tickets;  // [2][L * Hkv] counters of the one-kernel scoring: zero before and after every call
     mutable uint64_t launches;  // kernels enqueued through this context
     // finch_step_host only: a second stream carries the chunk's V rows to the device while the scoring kernels,
     // which do not read them, already run; events tie it to the caller's stream on both sides
@@ -129,8 +130,8 @@ cudaError_t launch_score_simt(const Ctx &ctx, const TensorView &q, const TensorV
                               const BatchView &bv, float *scores, float2 *row_stats, float *row_lse,
                               cudaStream_t stream);
 
-// tensor-core scoring (bf16, head_dim 64 or 128, either group mode).  The scratch
-// holds one float2 per prompt row and key split; up to kScoreMaxSplits splits are used when it is large enough.
+// tensor-core scoring (bf16, head_dim 64 or 128, either group mode).  The scratch holds the partial row statistics of
+// every key split; up to kScoreMaxSplits splits are used when it is large enough.
 constexpr int kScoreMaxSplits = 8;
 bool score_tc_supported(const Ctx &ctx);
 size_t score_tc_scratch_min(const Ctx &ctx, const BatchView &bv);  // least scratch (float2) of the two-launch path
@@ -138,7 +139,11 @@ cudaError_t launch_score_tc(const Ctx &ctx, const TensorView &q, const TensorVie
                             const BatchView &bv, float *scores, float2 *partial, size_t partial_capacity,
                             float *row_lse, cudaStream_t stream);
 
-// both sweeps in one persistent kernel (single-request batches without a row mask whose query tiles fit the shared
+// the column sums of the KV heads of a selection group that spans several, added in head order
+cudaError_t launch_sum_heads(const Ctx &ctx, const ModelView &mv, const BatchView &bv, const float *unit_scores, float *scores,
+                             int out_groups, int heads_per_group, cudaStream_t stream);
+
+// both sweeps in one persistent kernel (single-request batches without a row mask whose query rows fit the shared
 // memory): score_fused_scratch gives the float2 entries of scratch it needs, 0 when it does not take the batch
 size_t score_fused_scratch(const Ctx &ctx, const BatchView &bv);
 int score_fused_window(const Ctx &ctx, const BatchView &bv);  // key tiles per window; 0: the batch goes elsewhere

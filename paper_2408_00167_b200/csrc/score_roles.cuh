@@ -1,0 +1,682 @@
+// The roles of a tensor-core scoring CTA, shared by the one-kernel and the two-launch path.  A kernel walks a list of
+// segments -- (sweep, unit, key-tile range) -- and every role walks the same list with the same running counters, so
+// barrier phases stay in step without any further handshake.
+//
+//   Producer     one thread: query tiles (resident while the unit stays the same) and the ring of key tiles, by TMA.
+//   Issuer       one warp: tcgen05.mma into four accumulators of 128 tensor-memory columns in turn.
+//   Softmax      four groups of four warps (a warp per lane quarter): accumulator number A belongs to group A % 4.  A
+//                scheduler holds one warp of each group, so three of them compute while one waits for its refill.
+//   SumWriter    one warp: adds the row blocks' column sums of a key (second sweep) and writes the scores.
+//
+// What bounds it: two exponentials per logit.  On the special-function unit alone that is 1024 clocks per 128 x 128
+// logits and sweep; a quarter of the pairs goes to the FMA pipe instead.  Measured on the loops alone (accumulators
+// refilled by MMAs, no loads): 970 clocks per accumulator in the first sweep and 1060 in the second, against 1150 and
+// 1210 without the polynomial.  Bookkeeping counts: every instruction between two accumulators is paid by sixteen
+// warps, so what can be is worked out per segment, ragged ends and overflow repairs leave for a path out of line, and
+// barriers are addressed by their shared-memory address.
+#pragma once
+
+#include "score_tc_common.cuh"
+
+namespace finch {
+namespace tc {
+
+struct Cta {  // shared memory of the CTA
+    uint8_t *q_res, *ring;
+    uint64_t *q_raw;                   // queries have landed, their pad rows are still to be cleared
+    uint64_t *q_full, *q_free;         // [kQTiles] query tile has landed / its last MMAs are complete
+    uint64_t *full, *empty;            // [kMaxStages] key ring
+    uint64_t *acc_full, *acc_empty;    // [kGroups] accumulators
+    uint64_t *stats_ready;             // [2] row statistics of a second-sweep segment are staged
+    uint64_t *sum_full, *sum_empty;    // [kSumBufs] column sums handed to the writer
+    uint32_t *tmem_slot;
+    volatile int *abort_flag;
+    int *a_count;                      // softmax warps through a first-sweep segment (counts up for ever)
+    float *sums;                       // [kSumBufs][2][kRows]
+    float2 *stats;                     // [2][rows] (-ref, weight), pairs of rows interleaved
+    int *limits;                       // [2][rows] visible candidates per row (masked variant) ..
+    int2 *bounds;                      // [2][rows / 16] .. and the least and the most of every 16 rows
+    int q_slab;                        // bytes of one 64-element slab of the resident queries
+    int stages;
+    int q_tiles;                       // query tiles the shared memory holds
+    int rows_alloc;                    // rows of a statistics buffer (a multiple of 128)
+};
+
+constexpr int kBarBytes = 512;
+constexpr int kSumBytes = kSumBufs * 2 * kRows * 4;
+constexpr int cta_smem(int tile_bytes, int q_tiles, int rows_alloc, int stages, bool mask) {
+    return 1024 + (q_tiles + stages) * tile_bytes + kBarBytes + kSumBytes + 2 * rows_alloc * 8 +
+           (mask ? 2 * rows_alloc * 4 + rows_alloc : 0);
+}
+
+__device__ __forceinline__ Cta cta_layout(uint8_t *raw, int tile_bytes, int q_tiles, int rows_alloc, int stages) {
+    Cta c;
+    uint8_t *s = (uint8_t *)(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
+    c.q_res = s;
+    c.q_slab = q_tiles * kSlabBytes;
+    c.q_tiles = q_tiles;
+    c.rows_alloc = rows_alloc;
+    c.stages = stages;
+    c.ring = s + q_tiles * tile_bytes;
+    uint8_t *aux = c.ring + stages * tile_bytes;
+    uint64_t *b = (uint64_t *)aux;
+    c.q_full = b, b += kQTiles;
+    c.q_free = b, b += kQTiles;
+    c.full = b, b += kMaxStages;
+    c.empty = b, b += kMaxStages;
+    c.acc_full = b, b += kGroups;
+    c.acc_empty = b, b += kGroups;
+    c.stats_ready = b, b += 2;
+    c.sum_full = b, b += kSumBufs;
+    c.sum_empty = b, b += kSumBufs;
+    c.q_raw = b, b += 1;
+    c.tmem_slot = (uint32_t *)b;
+    c.abort_flag = (volatile int *)(c.tmem_slot + 1);
+    c.a_count = (int *)(c.tmem_slot + 2);
+    c.sums = (float *)(aux + kBarBytes);
+    c.stats = (float2 *)(aux + kBarBytes + kSumBytes);
+    c.limits = (int *)(c.stats + 2 * rows_alloc);
+    c.bounds = (int2 *)(c.limits + 2 * rows_alloc);
+    return c;
+}
+
+// Barriers and tensor memory (all 512 columns); ends with the CTA in step.  stats_arrivals: arrivals per staging.
+__device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals) {
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kQTiles; ++i) {
+            mbar_init(&c.q_full[i], 1);
+            mbar_init(&c.q_free[i], 1);
+        }
+        for (int i = 0; i < kMaxStages; ++i) {
+            mbar_init(&c.full[i], 1);
+            mbar_init(&c.empty[i], 1);
+        }
+        for (int i = 0; i < kGroups; ++i) {
+            mbar_init(&c.acc_full[i], 1);
+            mbar_init(&c.acc_empty[i], 4);
+        }
+        for (int i = 0; i < 2; ++i) mbar_init(&c.stats_ready[i], stats_arrivals);
+        for (int i = 0; i < kSumBufs; ++i) {
+            mbar_init(&c.sum_full[i], 4);
+            mbar_init(&c.sum_empty[i], 1);
+        }
+        mbar_init(c.q_raw, 1);
+        *c.abort_flag = 0;
+        *c.a_count = 0;
+        fence_barrier_init();
+    }
+    if (threadIdx.x / 32 == 1) {
+        tmem_alloc(c.tmem_slot, 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    return *c.tmem_slot;
+}
+
+// Common epilogue: everyone meets here, also after a timed-out wait.  The single-thread roles bring their warps back
+// together first: the CTA barrier must be executed by whole warps.
+__device__ __forceinline__ void cta_teardown(const Cta &c, uint32_t tmem, int *status) {
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && *c.abort_flag) atomicOr(status, FINCH_DEV_TIMEOUT);
+    if (threadIdx.x / 32 == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
+// The resident query tiles as a ring: a load of n tiles takes the next n, all behind one another, so that the queries of the
+// next unit can arrive while the MMAs still read those of the current one wherever both fit.
+struct TileRing {
+    int tiles, pos = 0;
+    __device__ int take(int n) {
+        if (pos + n > tiles) pos = 0;
+        const int base = pos;
+        pos += n;
+        return base;
+    }
+};
+
+// ------------------------------------------------------------------------------------------------ producer
+// Run by a whole warp, one elected lane issuing.
+template <int D>
+struct Producer {
+    static constexpr int kSlabs = D / 64, kTileBytes = kSlabs * kSlabBytes;
+    const Cta &c;
+    const CUtensorMap *q_big, *q_small, *cache, *chunk;
+    int heads;        // query heads per unit
+    bool clear_pads;  // pad rows may hold another request's rows: clear them
+    int st = 0, ph = 0, kcnt = 0;
+    uint32_t q_used = 0, q_ph = 0, raw_ph = 0;  // bit per query tile: loaded before / parity of its next q_free phase
+
+    __device__ __forceinline__ bool agree(bool ok) { return __all_sync(0xffffffffu, ok); }
+    __device__ bool load_key_tile(const UnitInfo &u, int t) {
+        const int stage = st, p = ph;
+        if (++st == c.stages) {
+            st = 0;
+            ph ^= 1;
+        }
+        // a producer a ring ahead of the MMAs polls rarely: its tests share a queue with the special-function unit
+        if (!agree(mbar_wait_relaxed(&c.empty[stage], p ^ 1, c.abort_flag, 500))) return false;
+        const KeyTile kt = key_tile(u, t);
+        const CUtensorMap *m = kt.is_chunk ? chunk : cache;
+        if (elect_one()) {
+            mbar_expect_tx(&c.full[stage], kTileBytes);
+            for (int s = 0; s < kSlabs; ++s)
+                tma_load_4d(c.ring + stage * kTileBytes + s * kSlabBytes, m, &c.full[stage], s * 64, kt.row0, u.G, u.l);
+        }
+        ++kcnt;
+        return true;
+    }
+    // Padded rows [r, r1) of the unit to resident rows dst ..; rows are multiples of 8, a box never leaves its head.
+    __device__ void load_rows(const UnitInfo &u, const Rows &R, int r, int r1, int dst, uint64_t *bar) {
+        while (r < r1) {
+            const int h = r / R.rp, pos = r - h * R.rp, len = min(r1 - r, R.rp - pos);
+            const bool big = len >= kBigBox;
+            for (int s = 0; s < kSlabs; ++s)
+                tma_load_4d(c.q_res + s * c.q_slab + dst * 128, big ? q_big : q_small, bar, s * 64, u.q0 + pos,
+                            u.G * heads + h, u.l);
+            r += big ? kBigBox : kRowPad;
+            dst += big ? kBigBox : kRowPad;
+        }
+    }
+    // The unit's query tiles into the ring's tiles base .., one at a time: a tile may be overwritten once the last MMAs on
+    // its old contents are complete, while the MMAs on the tiles behind it still run.
+    __device__ bool load_queries(const UnitInfo &u, const Rows &R, int base) {
+        const bool clear = clear_pads && R.rp != R.n_q;
+        const bool leader = elect_one();
+        if (clear && leader) {
+            int rows = 0;
+            for (int qb = 0; qb < R.n_qt; ++qb) rows += qb < R.n_qt - 1 ? kRows : (R.rows - qb * kRows) * (kRows / R.span);
+            mbar_expect_tx(c.q_raw, rows * 128 * kSlabs);
+        }
+        for (int qb = 0; qb < R.n_qt; ++qb) {
+            const int tile = base + qb, r = qb * kRows, n = min(kRows, R.rows - r), copies = qb < R.n_qt - 1 ? 1 : kRows / R.span;
+            if (q_used >> tile & 1u) {
+                if (!agree(mbar_wait(&c.q_free[tile], q_ph >> tile & 1u, c.abort_flag))) return false;
+                q_ph ^= 1u << tile;
+            }
+            q_used |= 1u << tile;
+            if (leader) {
+                uint64_t *bar = clear ? c.q_raw : &c.q_full[tile];
+                if (!clear) mbar_expect_tx(bar, n * copies * 128 * kSlabs);
+                for (int i = 0; i < copies; ++i) load_rows(u, R, R.r0 + r, R.r0 + r + n, tile * kRows + i * R.span, bar);
+            }
+        }
+        if (clear) {
+            // The pad rows between heads hold the next request's rows.  They weigh nothing, but a NaN among them would
+            // still reach this request's sums: zero them (the copies of a short last tile need none, lanes are skipped).
+            if (!agree(mbar_wait(c.q_raw, raw_ph, c.abort_flag))) return false;
+            raw_ph ^= 1;
+            const int pads = R.rp - R.n_q, lane = threadIdx.x & 31;  // at most seven rows of 8 pieces per head and slab
+            for (int h = R.r0 / R.rp; h * R.rp < R.r0 + R.rows; ++h)
+                for (int i = lane; i < pads * 8 * kSlabs; i += 32) {
+                    const int s = i / (pads * 8), k = i - s * pads * 8, r = h * R.rp + R.n_q + k / 8 - R.r0;
+                    if (r >= 0 && r < R.rows)
+                        *(uint4 *)(c.q_res + s * c.q_slab + (base * kRows + r) * 128 + k % 8 * 16) = uint4{0, 0, 0, 0};
+                }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (leader)
+                for (int qb = 0; qb < R.n_qt; ++qb) mbar_arrive(&c.q_full[base + qb]);
+        }
+        return true;
+    }
+    // One segment; base: the ring tiles its queries are to be loaded into, or -1: they are resident.
+    __device__ bool segment(const UnitInfo &u, const Rows &R, int t0, int t1, int base) {
+        // the segment's first key tile goes first: its ring stage is free before the query tiles are
+        if (!load_key_tile(u, t0)) return false;
+        if (base >= 0 && !load_queries(u, R, base)) return false;
+        for (int t = t0 + 1; t < t1; ++t)
+            if (!load_key_tile(u, t)) return false;
+        return true;
+    }
+    // No copy may still be in flight when the CTA retires: wait (bounded) for the last loads issued.  (A query tile's
+    // q_full phases alternate with its q_free phases: q_ph has the parity of the last load.)
+    __device__ void drain() {
+        for (int i = 0; i < kQTiles; ++i)
+            if (q_used >> i & 1u) mbar_wait(&c.q_full[i], q_ph >> i & 1u, c.abort_flag);
+        for (int i = max(0, kcnt - c.stages); i < kcnt; ++i) mbar_wait(&c.full[i % c.stages], (i / c.stages) & 1, c.abort_flag);
+    }
+};
+
+// ------------------------------------------------------------------------------------------------ MMA issuer
+// Run by a whole warp: one elected lane issues, the others keep the control flow uniform (see elect_one).
+template <int D>
+struct Issuer {
+    static constexpr int kSlabs = D / 64, kTileBytes = kSlabs * kSlabBytes;
+    const Cta &c;
+    uint32_t tmem, desc_hi, q_lo, ring_lo, q_slab;
+    uint32_t A = 0;  // accumulators issued
+    int st = 0, ph = 0;
+    uint32_t q_ph = 0;  // bit per query tile: parity of its next q_full phase
+
+    __device__ Issuer(const Cta &cta, uint32_t tm) : c(cta), tmem(tm) {
+        const uint64_t q = smem_desc_sw128(smem_u32(c.q_res)), r = smem_desc_sw128(smem_u32(c.ring));
+        desc_hi = (uint32_t)(q >> 32);
+        q_lo = (uint32_t)q;
+        ring_lo = (uint32_t)r;
+        q_slab = (uint32_t)c.q_slab >> 4;
+    }
+    // D = A B^T over head_dim; the operands differ in their descriptors' low words only (the 14-bit address field
+    // cannot carry: shared memory ends below 2^18 bytes).
+    __device__ __forceinline__ void mma(uint32_t d, uint32_t a_lo, uint32_t a_slab, uint32_t b_lo, uint32_t b_slab,
+                                        uint32_t idesc) {
+#pragma unroll
+        for (int k = 0; k < D / 16; ++k) {
+            const uint64_t a = ((uint64_t)desc_hi << 32) | (a_lo + (k / 4) * a_slab + (k % 4) * 2);
+            const uint64_t b = ((uint64_t)desc_hi << 32) | (b_lo + (k / 4) * b_slab + (k % 4) * 2);
+            if (elect_one()) {
+                if (k == 0)
+                    umma_bf16_first(d, a, b, idesc);
+                else
+                    umma_bf16_acc(d, a, b, idesc);
+            }
+        }
+    }
+    __device__ __forceinline__ void commit(uint64_t *bar) {
+        if (elect_one()) umma_commit(bar);
+    }
+    __device__ __forceinline__ bool wait(uint64_t *bar, uint32_t parity) {
+        return __all_sync(0xffffffffu, mbar_wait(bar, parity, c.abort_flag));
+    }
+    __device__ __forceinline__ bool acquire() { return wait(&c.acc_empty[A & 3], ((A >> 2) & 1) ^ 1); }
+    __device__ __forceinline__ uint32_t acc() const { return tmem + (A & 3) * kRows; }
+    __device__ __forceinline__ void publish() {
+        commit(&c.acc_full[A & 3]);
+        ++A;
+    }
+    __device__ __forceinline__ void next_key_stage() {
+        commit(&c.empty[st]);  // the stage may be refilled once these MMAs have read it
+        if (++st == c.stages) {
+            st = 0;
+            ph ^= 1;
+        }
+    }
+    __device__ __forceinline__ bool landed(int tile) {
+        const bool ok = wait(&c.q_full[tile], q_ph >> tile & 1u);
+        q_ph ^= 1u << tile;
+        return ok;
+    }
+    // First sweep: D = query tile x key tile^T, one accumulator per (key tile, query tile).  base: the queries' tiles in
+    // the ring; reload: they are being loaded; release: no later segment uses this load.
+    __device__ bool lse_segment(const Rows &R, int t0, int t1, int base, bool reload, bool release) {
+        constexpr uint32_t idesc = idesc_bf16_f32(kRows, kRows);
+        for (int t = t0; t < t1; ++t) {
+            if (!wait(&c.full[st], ph)) return false;
+            const uint32_t b_lo = ring_lo + (uint32_t)(st * (kTileBytes >> 4));
+            for (int qb = 0; qb < R.n_qt; ++qb) {
+                if (!acquire()) return false;
+                if (reload && t == t0 && !landed(base + qb)) return false;
+                tc_fence_after();
+                mma(acc(), q_lo + (uint32_t)((base + qb) * (kRows * 128 >> 4)), q_slab, b_lo, kSlabBytes >> 4, idesc);
+                publish();
+                if (release && t == t1 - 1) commit(&c.q_free[base + qb]);
+            }
+            next_key_stage();
+        }
+        return true;
+    }
+    // Second sweep: D = key tile x query rows^T.
+    __device__ bool colsum_segment(const Rows &R, int t0, int t1, int base, bool reload, bool release) {
+        const int cols = (R.rows + 15) & ~15;
+        bool side = false;  // kt = 2: this key tile takes the right half of the accumulator
+        for (int t = t0; t < t1; ++t) {
+            const bool last = t == t1 - 1;
+            if (!wait(&c.full[st], ph)) return false;
+            const uint32_t a_lo = ring_lo + (uint32_t)(st * (kTileBytes >> 4));
+            int freed = 0, seen = 0;
+            for (int s = 0; s < R.n_st; ++s) {
+                if (!side && !acquire()) return false;
+                const int row = s * R.width, n = min(R.width, cols - row), tiles = min(R.n_qt, (row + n + kRows - 1) / kRows);
+                if (reload && t == t0)
+                    for (; seen < tiles; ++seen)
+                        if (!landed(base + seen)) return false;
+                tc_fence_after();
+                mma(acc() + (side ? kRows / 2 : 0), a_lo, kSlabBytes >> 4, q_lo + (uint32_t)((base * kRows + row) * 128 >> 4),
+                    q_slab, idesc_bf16_f32(kRows, n));
+                if (R.kt == 1 || side || last) publish();
+                if (release && last) {
+                    const int done = s == R.n_st - 1 ? R.n_qt : (row + n) / kRows;
+                    for (; freed < done; ++freed) commit(&c.q_free[base + freed]);
+                }
+            }
+            next_key_stage();
+            side = R.kt == 2 && !side;
+        }
+        return true;
+    }
+};
+
+// ------------------------------------------------------------------------------------------------ softmax warps
+// The parts of the first sweep that are rarely needed, out of line so that the hot loops fit the instruction cache: n
+// columns from taddr, of which this lane's row sees nl and the warp's rows at most nv.
+template <bool MASK>
+__device__ __noinline__ float2 lse_any(uint32_t taddr, int n, int nv, int nl, bool live, float scale2, float m, float z) {
+#pragma unroll 1
+    for (int cc = 0; cc < n && cc < nv; cc += 16) {
+        uint32_t r[16];
+        __syncwarp();
+        tmem_ld_issue(taddr + cc, r);
+        tmem_ld_wait(r);
+        lse_chunk<16>(r, nl - cc, MASK ? live && nl - cc > 0 : live, scale2, m, z);
+    }
+    return make_float2(m, z);
+}
+
+template <bool MASK>
+struct Softmax {
+    const Cta &c;
+    uint32_t tmem;         // this warp's lanes of the group's accumulator
+    uint32_t full, empty;  // shared-memory addresses of its barriers
+    float scale2;
+    int lane, quarter, group, my_row;
+    uint32_t A = 0;     // accumulators of all groups before this segment
+    uint32_t mine = 0;  // accumulators this group has consumed
+    uint32_t E = 0;     // accumulators of second-sweep segments before this one
+
+    __device__ Softmax(const Cta &cta, uint32_t tm, float s2) : c(cta), scale2(s2) {
+        const int warp = threadIdx.x / 32;
+        lane = threadIdx.x & 31;
+        quarter = warp & 3;  // tcgen05.ld reaches lanes 32 * (warp % 4) ..
+        group = (warp - kCtlWarps) >> 2;
+        my_row = quarter * 32 + lane;
+        tmem = tm + ((uint32_t)(quarter * 32) << 16) + group * kRows;
+        full = smem_u32(c.acc_full + group);
+        empty = smem_u32(c.acc_empty + group);
+    }
+    // a wait's verdict is made warp-uniform so that a timeout takes the whole warp out
+    __device__ __forceinline__ bool acquire() {
+        if (!__all_sync(0xffffffffu, mbar_wait(full, mine & 1, c.abort_flag))) return false;
+        ++mine;
+        tc_fence_after();
+        return true;
+    }
+    __device__ __forceinline__ void release() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty);
+    }
+    // Row of the chunk this thread owns in query tile qb (may lie beyond R.rows).
+    __device__ __forceinline__ int row_of(const Rows &R, int qb) const {
+        return qb * kRows + (qb == R.n_qt - 1 ? my_row % R.span : my_row);
+    }
+    // First sweep over key tiles [t0, t1).  live: bit qb, this thread's row of query tile qb is a prompt row; lim (masked
+    // variant): candidates that row attends to.  Of four, two or one query tiles a group meets the same one throughout a
+    // segment; of three all, in turn: their statistics then rotate through slot 0.  On return slot k holds (m, z) of
+    // query tile (qb + k) % n_qt.
+    struct RowStats {
+        float m[3], z[3];
+        int qb;   // query tile of slot 0
+        int rel;  // position of the segment's first accumulator of this group: where its statistics are stored
+    };
+    __device__ __forceinline__ bool lse_segment(const UnitInfo &u, const Rows &R, int t0, int t1, uint32_t live,
+                                                const int (&lim)[kQTiles], RowStats &st) {
+        const int n_qt = R.n_qt, first = (group - A) & 3;  // this group's first accumulator of the segment
+        st.rel = first;
+        int qb = first % n_qt, t = t0 + first / n_qt;
+        const int step = n_qt == 1 ? 4 : (n_qt == 2 ? 2 : 1);
+        A += (t1 - t0) * n_qt;
+        const int cache_tiles = (u.c + kRows - 1) / kRows, all_tiles = n_key_tiles(u);
+        // tiles of fewer than 128 keys: the last of the cache and of the chunk
+        const int nv_cache = u.c - (cache_tiles - 1) * kRows, nv_chunk = u.m - (all_tiles - cache_tiles - 1) * kRows;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            st.m[k] = -INFINITY;
+            st.z[k] = 0.f;
+        }
+        // the copies of a short last tile share the columns
+        int n = kRows, off = 0;
+        const int short_qb = R.span < kRows ? n_qt - 1 : -1;
+        const int n_short = R.span, off_short = (quarter * 32 / R.span) * R.span;
+        bool on = false, any = false;
+        int limit = 0;
+        auto enter_tile = [&]() {
+            on = (live >> qb) & 1u;
+            any = __any_sync(0xffffffffu, on);
+            n = qb == short_qb ? n_short : kRows;
+            off = qb == short_qb ? off_short : 0;
+            if (MASK) {
+#pragma unroll
+                for (int k = 0; k < kQTiles; ++k)
+                    if (k == qb) limit = lim[k];
+            }
+        };
+        enter_tile();
+        while (t < t1) {
+            if (!acquire()) return false;
+            if (any) {
+                const uint32_t ta = tmem + off;
+                int nv = n;  // columns that hold keys
+                if (t == cache_tiles - 1) nv = nv_cache - off;
+                if (t == all_tiles - 1 && t >= cache_tiles) nv = nv_chunk - off;
+                nv = min(nv, n);
+                int nl = nv, full_cols = nv;
+                if (MASK) {
+                    nl = min(nv, limit - (t < cache_tiles ? t * kRows : u.c + (t - cache_tiles) * kRows) - off);
+                    full_cols = __reduce_min_sync(0xffffffffu, on ? nl : nv);
+                    nv = __reduce_max_sync(0xffffffffu, on ? nl : 0);
+                }
+                // a row's reference is the maximum of the first columns it meets
+                if (nv > 0) {
+                    if (__any_sync(0xffffffffu, st.m[0] == -INFINITY && on && nl > 0)) {
+                        keep_branch();
+                        uint32_t r[16];
+                        tmem_ld_issue(ta, r);
+                        tmem_ld_wait(r);
+                        mask_tail(r, nl);
+                        const float cmax = chunk_max(r);
+                        if (st.m[0] == -INFINITY) st.m[0] = cmax;
+                    }
+                    uint64_t acc0 = 0, acc1 = 0;
+                    const float negm = -(st.m[0] * scale2);
+                    int cc = 0;
+#pragma unroll 1
+                    for (; cc + 32 <= full_cols; cc += 32) {
+                        uint32_t r[32];
+                        tmem_ld_issue(ta + cc, r);
+                        tmem_ld_wait(r);
+                        lse_sum<32>(r, scale2, negm, acc0, acc1);
+                    }
+                    const float zn = st.z[0] + sum_of(acc0, acc1);
+                    if (__any_sync(0xffffffffu, !(zn <= 3.0e38f) && on && cc > 0)) {  // overflow: the whole visit, with care
+                        keep_branch();
+                        cc = 0;
+                    } else if (cc > 0) {
+                        st.z[0] = zn;
+                    }
+                    if (cc < nv) {
+                        keep_branch();
+                        const float2 s = lse_any<MASK>(ta + cc, n - cc, nv - cc, nl - cc, on, scale2, st.m[0], st.z[0]);
+                        st.m[0] = s.x;
+                        st.z[0] = s.y;
+                    }
+                }
+            }
+            release();
+            if (n_qt != 3) {
+                t += step;
+            } else {
+                keep_branch();
+                ++t;
+                if (++qb == 3) {
+                    qb = 0;
+                    ++t;
+                }
+                const float m0 = st.m[0], z0 = st.z[0];
+                st.m[0] = st.m[1];
+                st.z[0] = st.z[1];
+                st.m[1] = st.m[2];
+                st.z[1] = st.z[2];
+                st.m[2] = m0;
+                st.z[2] = z0;
+                enter_tile();
+            }
+        }
+        st.qb = qb;
+        return true;
+    }
+    // This group's part of the rows' statistics; parts: [kGroups][stride] of the segment, from the chunk's first row on.
+    __device__ __forceinline__ void store_stats(const Rows &R, const RowStats &s, uint32_t live, float2 *parts, int stride) const {
+        float2 *dst = parts + (int64_t)s.rel * stride + my_row;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            int qb = s.qb + k;
+            if (qb >= R.n_qt) qb -= R.n_qt;
+            if ((k == 0 || R.n_qt == 3) && ((live >> qb) & 1u)) dst[qb * kRows] = make_float2(s.m[k] * scale2, s.z[k]);
+        }
+    }
+    // tail: columns at or beyond nv hold no row
+    template <int NC, bool M>
+    __device__ __forceinline__ void colsum_cols(uint32_t taddr, bool tail, int nv, uint32_t sm4, float &c0, float &c1, const int *lim, int j) {
+        uint32_t r[NC];
+        tmem_ld_issue(taddr, r);
+        tmem_ld_wait(r);
+        if (tail) mask_tail(r, nv);
+        colsum_chunk<NC, M>(r, scale2, sm4, c0, c1, (const int2 *)lim, j);
+    }
+    // n columns (a multiple of 16) of one key tile against staged rows row ..: the key's column sum over nv of them.
+    __device__ __forceinline__ float colsum_visit(uint32_t ta, int n, int nv, uint32_t sm4, const int *lim, const int2 *bounds,
+                                                  int row, int j) {
+        float c0 = 0.f, c1 = 0.f;
+        int cc = 0;
+        if (!MASK) {
+#pragma unroll 1
+            for (; cc + 32 <= nv; cc += 32) colsum_cols<32, false>(ta + cc, false, 32, sm4 + cc * 8, c0, c1, nullptr, 0);
+            if (cc < n) {
+                keep_branch();
+#pragma unroll 1
+                for (; cc < n; cc += 16) colsum_cols<16, false>(ta + cc, true, nv - cc, sm4 + cc * 8, c0, c1, nullptr, 0);
+            }
+        } else {
+            const int j_lo = j - lane, j_hi = j_lo + 31;  // the warp's keys
+#pragma unroll 1
+            for (; cc < n; cc += 16) {
+                const int2 b = bounds[(row + cc) >> 4];
+                if (j_lo >= b.y) continue;  // no row of these sees any key of the warp
+                if (j_hi < b.x)
+                    colsum_cols<16, false>(ta + cc, nv - cc < 16, nv - cc, sm4 + cc * 8, c0, c1, nullptr, 0);
+                else
+                    colsum_cols<16, true>(ta + cc, nv - cc < 16, nv - cc, sm4 + cc * 8, c0, c1, lim + row + cc, j);
+            }
+        }
+        return c0 + c1;
+    }
+    // Second sweep over key tiles [t0, t1) against the staged statistics `stats` (and limits): column sums to the writer.
+    __device__ __forceinline__ bool colsum_segment(const UnitInfo &u, const Rows &R, int t0, int t1, const float2 *stats,
+                                                   const int *lim, const int2 *bounds) {
+        const int n_st = R.n_st, kt = R.kt;
+        const uint32_t first = (group - A) & 3, sm = smem_u32(stats);
+        const uint32_t sum_full = smem_u32(c.sum_full), sum_empty = smem_u32(c.sum_empty);
+        const int cols = (R.rows + 15) & ~15;
+        int s = first % n_st, t = t0 + (first / n_st) * kt;
+        const int step = n_st == 1 ? 4 * kt : (n_st == 2 ? 2 : 1);
+        const uint32_t n_acc = kt == 2 ? (t1 - t0 + 1) >> 1 : (t1 - t0) * n_st, E0 = E;
+        A += n_acc;
+        E += n_acc;
+        for (uint32_t a = E0 + first; t < t1; a += 4) {
+            if (!acquire()) return false;
+            const int row = s * R.width, n = min(R.width, cols - row), nv = min(n, R.rows - row);
+            const uint32_t sm4 = sm + row * 8;
+            const float v0 = colsum_visit(tmem, n, nv, sm4, lim, bounds, row, MASK ? key_tile(u, t).j0 + my_row : 0);
+            float v1 = 0.f;
+            if (kt == 2 && t + 1 < t1)
+                v1 = colsum_visit(tmem + kRows / 2, n, nv, sm4, lim, bounds, row, MASK ? key_tile(u, t + 1).j0 + my_row : 0);
+            release();
+            const uint32_t buf = a % kSumBufs;
+            if (!__all_sync(0xffffffffu, mbar_wait(sum_empty + buf * 8, ((a / kSumBufs) & 1) ^ 1, c.abort_flag))) return false;
+            float *out = c.sums + buf * 2 * kRows + my_row;
+            out[0] = v0;
+            if (kt == 2) out[kRows] = v1;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sum_full + buf * 8);
+            if (n_st != 3) {
+                t += step;
+            } else {
+                ++t;
+                if (++s == 3) {
+                    s = 0;
+                    ++t;
+                }
+            }
+        }
+        return true;
+    }
+};
+
+// The parts of a row's statistics, numbered: per segment, copy of the row, and group that met its query tile.  A segment
+// stores a group's part at the position of the group's first accumulator, so that with one, two or four query tiles the
+// parts of tile qb are at positions qb, qb + n_qt, ...; with three at all four.
+struct Parts {
+    int log_p, log_c, first, step, span;
+    __device__ Parts(const Rows &R, int qb) {
+        const bool last = qb == R.n_qt - 1;
+        log_c = !last || R.span == 128 ? 0 : (R.span == 64 ? 1 : 2);
+        log_p = R.n_qt == 4 ? 0 : (R.n_qt == 2 ? 1 : 2);
+        first = R.n_qt == 3 ? 0 : qb;
+        step = R.n_qt == 3 ? 1 : R.n_qt;
+        span = R.span;
+    }
+    __device__ int count(int segments) const { return segments << (log_p + log_c); }
+    // offset of part k in [segments][kGroups][stride], from the row's own slot on
+    __device__ int64_t at(int k, int stride) const {
+        const int p = k & ((1 << log_p) - 1), c = (k >> log_p) & ((1 << log_c) - 1), s = k >> (log_p + log_c);
+        return (int64_t)(s * kGroups + first + p * step) * stride + c * span;
+    }
+};
+
+// ------------------------------------------------------------------------------------------------ column-sum writer
+struct SumWriter {
+    const Cta &c;
+    int lane;
+    uint32_t A = 0;  // accumulators of the second-sweep segments so far
+    // Key tiles [t0, t1) of a second-sweep segment: the row blocks' sums of a key, added in block order, to
+    // out[candidate]; `add`: a later row chunk of the same unit adds to what the earlier ones wrote (by this same warp).
+    __device__ bool segment(const UnitInfo &u, const Rows &R, int t0, int t1, float *out, bool add) {
+        for (int t = t0; t < t1; t += R.kt) {
+            float v[2][kRows / 32];
+#pragma unroll
+            for (int i = 0; i < kRows / 32; ++i) v[0][i] = v[1][i] = 0.f;
+            for (int s = 0; s < R.n_st; ++s, ++A) {
+                const uint32_t buf = A % kSumBufs;
+                const bool ok = mbar_wait_relaxed(&c.sum_full[buf], (A / kSumBufs) & 1, c.abort_flag, 500);
+                if (!__all_sync(0xffffffffu, ok)) return false;
+                const float *src = c.sums + buf * 2 * kRows + lane;
+#pragma unroll
+                for (int i = 0; i < kRows / 32; ++i) {
+                    v[0][i] += src[i * 32];
+                    if (R.kt == 2) v[1][i] += src[kRows + i * 32];
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&c.sum_empty[buf]);
+            }
+            for (int k = 0; k < R.kt && t + k < t1; ++k) {
+                const KeyTile kt = key_tile(u, t + k);
+#pragma unroll
+                for (int i = 0; i < kRows / 32; ++i) {
+                    const int row = i * 32 + lane;
+                    if (row < kt.valid) {
+                        float *dst = out + kt.j0 + row;
+                        const float x = k ? v[1][i] : v[0][i];
+                        *dst = add ? *dst + x : x;
+                    }
+                }
+            }
+        }
+        return true;
+    }
+    // Tiles of a request without prompt rows: the empty sum.
+    __device__ void zeros(const UnitInfo &u, int t0, int t1, float *out) {
+        for (int t = t0; t < t1; ++t) {
+            const KeyTile kt = key_tile(u, t);
+            for (int row = lane; row < kt.valid; row += 32) out[kt.j0 + row] = 0.f;
+        }
+    }
+};
+
+}  // namespace tc
+}  // namespace finch

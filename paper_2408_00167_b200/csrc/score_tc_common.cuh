@@ -12,21 +12,20 @@ namespace tc {
 
 using namespace ptx;
 
-constexpr int kRows = 128;       // rows per operand tile = MMA M = MMA N
-constexpr int kSub = 64;         // prompt rows per sub-block (two per query tile)
-constexpr int kQTiles = 4;       // query tiles resident at a time
-constexpr int kGroups = 4;       // softmax groups (four warps each); accumulator number A goes to group A % 4
+constexpr int kRows = 128;       // rows per operand tile = MMA M
+constexpr int kRowPad = 8;       // a query head's prompt rows are padded to this many (the swizzle's 8-row group)
+constexpr int kMaxRows = 512;    // padded query rows resident at a time: four query tiles
+constexpr int kQTiles = kMaxRows / kRows;
+constexpr int kGroups = 4;       // softmax groups of four warps; each owns one accumulator of 128 tensor-memory columns
+constexpr int kMaxStages = 6;    // key-tile ring
+constexpr int kSumBufs = 8;      // column-sum hand-over buffers, one per accumulator in flight
+constexpr int kCtlWarps = 4;     // producer, MMA issuer, statistics warp, column-sum warp
+constexpr int kSoftmaxWarps = 16;
+constexpr int kTcThreads = (kCtlWarps + kSoftmaxWarps) * 32;
+constexpr int kBigBox = 64;      // query rows per TMA box where a head has that many; kRowPad-row boxes otherwise
 constexpr int kPlanBoundsInts = 1024;  // room for the per-CTA item bounds in the scratch (grid + 1 <= this)
-constexpr int kAccBufs = 4;      // accumulators of 128 fp32 columns in tensor memory (all 512 columns), one per group
-constexpr int kMaxStages = 4;    // key-tile ring
-constexpr int kTcThreads = 64 + kGroups * 128;
-constexpr int kSlabBytes = kRows * 128;                 // a 64-element (128-byte) wide slab of a 128-row tile
-constexpr int kStatsBytes = 2 * kQTiles * kRows * 8;  // (-ref, weight) of the resident rows, double-buffered
-constexpr int kLimitBytes = 2 * kQTiles * kRows * 4;  // visible-candidate count of the resident rows (masked variant)
-constexpr int kAuxBytes = 1024 + kStatsBytes + kLimitBytes;
-constexpr int kSmemLimit = 232448;                      // 227 KiB per CTA
-
-enum { kLse = 0, kColsum = 1 };
+constexpr int kSlabBytes = kRows * 128;  // a 64-element (128-byte) wide slab of a 128-row tile
+constexpr int kSmemLimit = 232448;       // 227 KiB per CTA
 
 struct KeyTile {
     int is_chunk;  // which tensor the rows come from
@@ -55,18 +54,39 @@ __device__ __forceinline__ KeyTile key_tile(const UnitInfo &u, int t) {
     return k;
 }
 
-// The group's prompt rows as a list of 64-row sub-blocks, head-major then position: sub-block sb covers rows
-// [p0, p0 + valid) of the group's query head hh.  Query tile t packs sub-blocks 2t and 2t + 1.
-struct SubBlock {
-    int hh, p0, valid;
+// The query rows of a scoring unit (layer, KV head, request): its query heads one after the other, each head's prompt
+// rows padded to a multiple of 8.  Row r is prompt row r % rp of head r / rp.  Units of more than kMaxRows rows are
+// worked on in chunks of kMaxRows (a row's softmax does not depend on the other rows).
+//
+// First sweep (a row per tensor-memory lane): row r of the chunk is lane r % 128 of query tile r / 128.  A warp only
+// reaches the 32 lanes of its own quarter, so a last tile of at most 64 (32) rows would leave two (three) of the four
+// schedulers idle: it is loaded twice (four times), `span` rows apart, and the copies share the columns.
+// Second sweep (a key per lane, rows along the columns): an accumulator holds one key tile against a block of at most
+// 128 rows (n_st blocks of `width`), or, for at most 64 rows, two key tiles side by side (kt = 2).
+struct Rows {
+    int n_q, rp;
+    int r0, rows;         // the chunk's first padded row, its padded rows
+    int n_qt, span;       // query tiles; rows of the last tile that are not copies (32, 64 or 128)
+    int kt, n_st, width;  // key tiles per accumulator, accumulators per key tile, columns per key tile (multiple of 16)
 };
-__device__ __forceinline__ SubBlock sub_block(int sb, int sbq, int n_sb, int n_q) {
-    SubBlock s;
-    s.hh = sb / sbq;
-    s.p0 = (sb % sbq) * kSub;
-    s.valid = sb < n_sb ? min(kSub, n_q - s.p0) : 0;
-    return s;
+__host__ __device__ inline int padded_rows(int n_q, int heads) { return heads * ((n_q + kRowPad - 1) / kRowPad * kRowPad); }
+__device__ __forceinline__ Rows make_rows(int n_q, int heads, int chunk) {
+    Rows r;
+    r.n_q = n_q;
+    r.rp = (n_q + kRowPad - 1) / kRowPad * kRowPad;
+    r.r0 = chunk * kMaxRows;
+    r.rows = max(0, min(kMaxRows, heads * r.rp - r.r0));
+    r.n_qt = (r.rows + kRows - 1) / kRows;
+    const int last = r.rows - (r.n_qt - 1) * kRows;
+    r.span = last <= 32 ? 32 : (last <= 64 ? 64 : 128);
+    const int cols = (r.rows + 15) & ~15;
+    r.kt = cols <= 64 ? 2 : 1;
+    r.n_st = (cols + kRows - 1) / kRows;
+    r.width = r.n_st > 1 ? ((cols / r.n_st + 15) & ~15) : cols;
+    return r;
 }
+// Is padded row r of the chunk a prompt row?
+__device__ __forceinline__ bool row_live(const Rows &r, int row) { return row < r.rows && (r.r0 + row) % r.rp < r.n_q; }
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -99,133 +119,153 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return r;
 }
 
-// kLse: fold 32 columns (keys) of one accumulator row into the row's running (reference, sum of exp2).
+// exp2 of a pair on the FMA pipe: x = n + f with n = round(x), |f| <= 1/2, 2^f by a polynomial, n into the exponent field.
+// The special-function unit turns out 4 results per clock and scheduler, a quarter of the FMA rate, and both sweeps
+// are bound by it: one pair in kPolyEvery goes this way and the units run side by side.  The coefficients are the
+// minimax fit in relative error of 2^f on [-1/2, 1/2] with constant term 1 (Remez exchange): error 7.9e-8 at degree 5,
+// below ex2.approx's own 2 ulp.  x is clamped to [-127, 128]: below, the result is 0 (p = 1 exactly, exponent field
+// 127 - 127); at 128 and above it is inf or NaN, which the caller's overflow test catches.
+#ifndef FINCH_POLY_EVERY
+#define FINCH_POLY_EVERY 8
+#endif
+constexpr int kPolyEvery = FINCH_POLY_EVERY;  // 0: never
+template <bool kUpper>
+__device__ __forceinline__ uint64_t exp2_poly2(uint64_t x2) {
+    float x0, x1;
+    unpack2(x2, x0, x1);
+    x0 = fmaxf(x0, -127.f);
+    x1 = fmaxf(x1, -127.f);
+    if (kUpper) {
+        x0 = fminf(x0, 128.f);
+        x1 = fminf(x1, 128.f);
+    }
+    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
+    const uint64_t x = pack2(x0, x1);
+    const uint64_t t = add2(x, pack2(kMagic, kMagic));
+    const uint64_t n = add2(t, pack2(-kMagic, -kMagic));
+    const uint64_t f = fma2(n, pack2(-1.f, -1.f), x);
+    uint64_t p = fma2(f, pack2(0x1.5a907ep-10f, 0x1.5a907ep-10f), pack2(0x1.3cf310p-7f, 0x1.3cf310p-7f));
+    p = fma2(p, f, pack2(0x1.c6bb2cp-5f, 0x1.c6bb2cp-5f));
+    p = fma2(p, f, pack2(0x1.ebf9a0p-3f, 0x1.ebf9a0p-3f));
+    p = fma2(p, f, pack2(0x1.62e424p-1f, 0x1.62e424p-1f));
+    p = fma2(p, f, pack2(1.f, 1.f));
+    float p0, p1, t0, t1;
+    unpack2(p, p0, p1);
+    unpack2(t, t0, t1);
+    return pack2(__int_as_float(__float_as_int(p0) + (__float_as_int(t0) << 23)),
+                 __int_as_float(__float_as_int(p1) + (__float_as_int(t1) << 23)));
+}
+template <bool kUpper>
+__device__ __forceinline__ uint64_t exp2_pair(uint64_t x2, int pair) {
+    if (kPolyEvery && pair % (kPolyEvery ? kPolyEvery : 1) == kPolyEvery - 1) return exp2_poly2<kUpper>(x2);
+    float x0, x1;
+    unpack2(x2, x0, x1);
+    return pack2(ex2(x0), ex2(x1));
+}
+
+// First sweep: fold NC columns (keys) of one accumulator row into the row's running (reference, sum of exp2).
 // The reference is the maximum of the row's first chunk, not the running maximum: any reference works as long as
 // the sum stays finite, and skipping the per-element maximum saves a quarter of the instructions.  If the sum
 // overflows (a later logit more than ~2^7 base-2 units above the reference, or many nearly that far) the reference
 // moves up and the chunk is redone.  Columns at or beyond nv hold no key and count nothing.
-__device__ __forceinline__ void lse_chunk(const uint32_t (&r)[32], int nv, float scale2, float &m_raw, float &z) {
-    float v[32];
+//
+// The rare parts (a tile's ragged end, a row's first chunk) sit behind warp-uniform branches with an empty asm in them:
+// without it the compiler turns them into predicated instructions, two or three more issue slots per logit.
+__device__ __forceinline__ void keep_branch() { asm volatile("" ::: "memory"); }
+template <int NC>
+__device__ __forceinline__ void mask_tail(uint32_t (&r)[NC], int nv) {
+    if (__any_sync(0xffffffffu, nv < NC)) {
+        keep_branch();
 #pragma unroll
-    for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
-    if (nv < 32) {
-#pragma unroll
-        for (int e = 1; e < 32; ++e) v[e] = e < nv ? v[e] : -INFINITY;
+        for (int e = 0; e < NC; ++e)
+            if (e >= nv) r[e] = 0xff800000u;  // -inf
     }
-    if (m_raw == -INFINITY) {
-        float cmax = v[0];
+}
+template <int NC>
+__device__ __forceinline__ float chunk_max(const uint32_t (&r)[NC]) {
+    float m = __uint_as_float(r[0]);
 #pragma unroll
-        for (int e = 1; e < 32; ++e) cmax = fmaxf(cmax, v[e]);
-        m_raw = cmax;
+    for (int e = 1; e < NC; ++e) m = fmaxf(m, __uint_as_float(r[e]));
+    return m;
+}
+// The bare sum of 32 columns against a reference (negm = -reference * scale2), in two pairs of partial sums.
+template <int NC>
+__device__ __forceinline__ void lse_sum(const uint32_t (&r)[NC], float scale2, float negm, uint64_t &acc0, uint64_t &acc1) {
+    const uint64_t s2 = pack2(scale2, scale2), n2 = pack2(negm, negm);
+#pragma unroll
+    for (int e = 0; e < NC; e += 4) {
+        acc0 = add2(acc0, exp2_pair<true>(fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), s2, n2), e / 2));
+        acc1 = add2(acc1, exp2_pair<true>(fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), s2, n2), e / 2 + 1));
     }
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        const float negm = -(m_raw * scale2);
-        const uint64_t s2 = pack2(scale2, scale2), n2 = pack2(negm, negm);
-        uint64_t acc0 = 0, acc1 = 0;  // two pairs of partial sums (+0.0f bit patterns)
-#pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-            float x0, x1, x2, x3;
-            unpack2(fma2(pack2(v[e], v[e + 1]), s2, n2), x0, x1);
-            unpack2(fma2(pack2(v[e + 2], v[e + 3]), s2, n2), x2, x3);
-            acc0 = add2(acc0, pack2(ex2(x0), ex2(x1)));
-            acc1 = add2(acc1, pack2(ex2(x2), ex2(x3)));
-        }
-        float a0, a1, a2, a3;
-        unpack2(acc0, a0, a1);
-        unpack2(acc1, a2, a3);
-        const float zn = z + ((a0 + a1) + (a2 + a3));
-        if (!(zn > 3.0e38f)) {  // finite -- or NaN, on a lane that holds no prompt row: nothing to repair
+}
+__device__ __forceinline__ float sum_of(uint64_t acc0, uint64_t acc1) {
+    float a0, a1, a2, a3;
+    unpack2(acc0, a0, a1);
+    unpack2(acc1, a2, a3);
+    return (a0 + a1) + (a2 + a3);
+}
+template <int NC>
+__device__ __forceinline__ void lse_chunk(uint32_t (&r)[NC], int nv, bool live, float scale2, float &m_raw, float &z) {
+    mask_tail(r, nv);
+    if (__any_sync(0xffffffffu, m_raw == -INFINITY && live)) {
+        keep_branch();
+        const float cmax = chunk_max(r);
+        if (m_raw == -INFINITY) m_raw = cmax;
+    }
+    auto sum = [&]() -> float {
+        uint64_t acc0 = 0, acc1 = 0;  // +0.0f bit patterns
+        lse_sum(r, scale2, -(m_raw * scale2), acc0, acc1);
+        return sum_of(acc0, acc1);
+    };
+    const float zn = z + sum();
+    if (__any_sync(0xffffffffu, !(zn <= 3.0e38f) && live)) {
+        keep_branch();
+        // Overflow (inf or NaN) on some lane: it moves its reference up and redoes the chunk.  The new reference must cover
+        // the chunk's largest logit and what has been summed so far (z = 2^e * [1, 2) against the old reference, e from
+        // z's exponent field), so that the redone sum is at most 1 + NC.  The factor between the two references (the
+        // same rounded products the chunks subtract) is applied in two halves, since z may be near 2^127 while the
+        // factor is below the smallest normal number.
+        if (!(zn <= 3.0e38f) && live) {
+            const float lift = (float)(((__float_as_int(z) >> 23) & 0xff) - 126);
+            const float m_new = fmaxf(chunk_max(r), fmaf(lift, __frcp_rn(scale2), m_raw));
+            const float half_d = 0.5f * (__fmul_rn(m_raw, scale2) - __fmul_rn(m_new, scale2));
+            z = (z * ex2(half_d)) * ex2(half_d);
+            m_raw = m_new;
+            z += sum();
+        } else if (live) {
             z = zn;
-            break;
         }
-        // overflow: move the reference up and redo the chunk
-        float cmax = v[0];
-#pragma unroll
-        for (int e = 1; e < 32; ++e) cmax = fmaxf(cmax, v[e]);
-        // The new reference must cover the chunk's largest logit and what has been summed so far (z = 2^e * [1, 2)
-        // against the old reference, e from z's exponent field), so that the redone sum is at most 1 + 32.  The
-        // factor between the two references (the same rounded products the chunks subtract) is applied in two
-        // halves, since z may be near 2^127 while the factor is below the smallest normal number.
-        const float lift = (float)(((__float_as_int(z) >> 23) & 0xff) - 126);
-        const float m_new = fmaxf(cmax, fmaf(lift, __frcp_rn(scale2), m_raw));
-        const float half_d = 0.5f * (__fmul_rn(m_raw, scale2) - __fmul_rn(m_new, scale2));
-        z = (z * ex2(half_d)) * ex2(half_d);
-        m_raw = m_new;
+    } else if (live) {
+        z = zn;
     }
 }
 
-// `live` is false on lanes whose row of the query tile holds no prompt row: they take part in the (warp-wide)
-// loads but skip the arithmetic, whose input would be whatever the shared memory held before.
-// lane_valid (masked variant): how many of the tile's columns this lane's row attends to; may be <= 0.
-template <bool MASK>
-__device__ __forceinline__ void lse_accumulate(uint32_t taddr, int valid, float scale2, bool live, float &m_raw,
-                                               float &z, int lane_valid) {
-    // one 32-column chunk at a time: with four softmax warps per scheduler the other warps cover the tensor-memory
-    // latency, and a single register buffer keeps the kernel inside its register budget
-#pragma unroll 1
-    for (int cc = 0; cc * 32 < valid; ++cc) {
-        uint32_t r[32];
-        __syncwarp();
-        tmem_ld_x32_issue(taddr + cc * 32, r);
-        tmem_ld_x32_wait(r);
-        if (MASK) {
-            const int nv = min(valid, lane_valid) - cc * 32;
-            if (live && nv > 0) lse_chunk(r, nv, scale2, m_raw, z);
-        } else {
-            if (live) lse_chunk(r, valid - cc * 32, scale2, m_raw, z);
-        }
-    }
-}
-
-// kColsum: add to (c0, c1) the weights exp2(s * scale2 - ref_r) * w_r of one accumulator row (a key) over the valid
-// prompt rows of the query tile: v0 rows in its first 64-row half, v1 in its second.  The statistics are staged
-// in pairs of rows, (-ref_a, -ref_b, w_a, w_b), so that one 128-bit load feeds two packed operations.
+// Second sweep: add to (c0, c1) the weights exp2(s * scale2 - ref_r) * w_r of NC columns (prompt rows) of one accumulator
+// row (a key).  The statistics are staged in pairs of rows, (-ref_a, -ref_b, w_a, w_b), so that one 128-bit load feeds
+// two packed operations.
 // Masked variant: lim2 holds, per pair of rows, how many candidates each row attends to; this thread's key has
 // candidate index j and counts for a row only if j is below that row's number.
-template <bool MASK>
-__device__ __forceinline__ void colsum_chunk(const uint32_t (&r)[32], int nv, float scale2, uint32_t sm4, float &c0,
-                                             float &c1, const int2 *lim2, int j) {
-    float v[32];
-#pragma unroll
-    for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
-    if (nv < 32) {
-#pragma unroll
-        for (int e = 0; e < 32; ++e) v[e] = e < nv ? v[e] : -INFINITY;  // rows past the prompt weigh nothing
-    }
+template <int NC, bool MASK>
+__device__ __forceinline__ void colsum_chunk(const uint32_t (&r)[NC], float scale2, uint32_t sm4, float &c0, float &c1,
+                                             const int2 *lim2, int j) {
     const uint64_t s2 = pack2(scale2, scale2);
     uint64_t acc = pack2(c0, c1);
 #pragma unroll
-    for (int e = 0; e < 32; e += 2) {
+    for (int e = 0; e < NC; e += 2) {
         const float4 s4 = lds128(sm4 + (e / 2) * 16);  // two prompt rows: (-ref_a, -ref_b, w_a, w_b)
-        float x0, x1;
-        unpack2(fma2(pack2(v[e], v[e + 1]), s2, pack2(s4.x, s4.y)), x0, x1);
+        uint64_t x = fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), s2, pack2(s4.x, s4.y));
         if (MASK) {
+            float x0, x1;
+            unpack2(x, x0, x1);
             const int2 l2 = lim2[e / 2];
             x0 = j < l2.x ? x0 : -INFINITY;  // exp2(-inf) = 0: the row does not see this key
             x1 = j < l2.y ? x1 : -INFINITY;
+            x = pack2(x0, x1);
         }
-        acc = fma2(pack2(ex2(x0), ex2(x1)), pack2(s4.z, s4.w), acc);
+        acc = fma2(exp2_pair<false>(x, e / 2), pack2(s4.z, s4.w), acc);
     }
     unpack2(acc, c0, c1);
 }
-
-template <bool MASK>
-__device__ __forceinline__ void colsum_accumulate(uint32_t taddr, int v0, int v1, float scale2, const float2 *sm,
-                                                  float &c0, float &c1, const int *lim, int j) {
-    const uint32_t sm4 = smem_u32(sm);  // shared-window address: the loads below are ld.shared, not generic
-    // chunks 0 and 1 cover the tile's first 64-row half (always present), chunks 2 and 3 the second half
-    const int last = v1 > 0 ? 4 : 2;
-#pragma unroll 1
-    for (int cc = 0; cc < last; ++cc) {
-        uint32_t r[32];
-        __syncwarp();
-        tmem_ld_x32_issue(taddr + cc * 32, r);
-        tmem_ld_x32_wait(r);
-        colsum_chunk<MASK>(r, (cc < 2 ? v0 : v1) - (cc & 1) * 32, scale2, sm4 + cc * 256, c0, c1,
-                           (const int2 *)lim + cc * 16, j);
-    }
-}
-
 
 // ---- merging partial row statistics.  A part is (reference, sum of exp2 against that reference), both in base-2
 // logit units; parts are folded in a fixed order into a running (M, Z), then turned into the pair the column
@@ -264,6 +304,13 @@ __device__ __forceinline__ float2 merged_pair(float M, float Z, float &lse_nat) 
     const float w = __fdividef(1.0f, __int_as_float((zbits & 0x007fffff) | 0x3f800000));
     lse_nat = (M + log2f(Z)) * kLn2;
     return make_float2(-(M + (float)k), w);
+}
+
+// rows 2k and 2k+1 share one float4: (-ref_2k, -ref_2k+1, w_2k, w_2k+1)
+__device__ __forceinline__ void stage_row(float2 *stats, int row, float2 v) {
+    float *f = (float *)stats + (row >> 1) * 4 + (row & 1);
+    f[0] = v.x;
+    f[2] = v.y;
 }
 
 // ------------------------------------------------------------------------------------------------ host side
