@@ -1,10 +1,12 @@
 // Cache compaction: gather the kept K/V rows and positions into the next cache, in kept (ascending) order.
 //
-// One CTA copies kRowsPerCta output rows of one unit (layer, selection group, request) for every KV head of the
-// group, K and V, as 16-byte pieces: consecutive threads move consecutive pieces of a row, so both the gathered
-// reads (whole rows) and the writes (contiguous rows) are fully coalesced 128-bit accesses.  A CTA takes 256 rows
-// so that the dependent chain in front of the copies (batch metadata -> kept indices -> source addresses) is paid
-// once per 128 KiB moved, and every thread has eight 16-byte loads in flight before its first store.
+// One CTA copies a block of output rows of one KV head of one request, K and V, as 16-byte pieces: consecutive threads
+// move consecutive pieces of a row, so both the gathered reads (whole rows) and the writes (contiguous rows) are fully
+// coalesced 128-bit accesses, and every thread has eight loads in flight before its first store.  The dependent chain
+// in front of the copies (batch metadata -> kept indices -> source addresses) wants large blocks, 256 rows where they
+// fill the chip twice over (c. 92 % of the copy rate); smaller problems take smaller blocks so that every SM has some.
+// KV heads are spread over the grid also where one selection group covers them all (32 heads in a CTA's loop left a
+// 32-layer step with 128 CTAs: 0.49 ms for 1 GB, re-positioned).
 #include <cuda_bf16.h>
 
 #include "finch_internal.cuh"
@@ -12,8 +14,9 @@
 namespace finch {
 namespace {
 
-constexpr int kRowsPerCta = 256;  // = kCompactThreads: one thread fetches one kept index
 constexpr int kCompactThreads = 256;
+constexpr int kMaxRowsPerCta = kCompactThreads;  // one thread fetches one kept index
+constexpr int kMinRowsPerCta = 16;
 
 // ---- rotary re-positioning (Method, "Managing the Cache"): a kept key that moves from candidate index j to output
 // slot i is rotated by delta = i - j positions; pair t of the row turns by delta * theta^(-2t/d).  Cosine and sine
@@ -90,126 +93,119 @@ __device__ __forceinline__ void rotate_interleaved(uint4 &pv, const float2 *cs, 
     }
 }
 
-// The compaction with re-positioned keys: same decomposition as compact_kernel below (a warp walks the 16-byte
-// pieces of [K | V] x KV heads of a row, four rows of loads in flight per thread), but a K piece is rotated between
-// its load and its store.  With pairs (t, t + d/2) the thread that owns a piece of the row's first half also moves
-// the partner piece of the second half.
-template <int kElems>
-__global__ void __launch_bounds__(kCompactThreads)
-compact_rope_kernel(ModelView mv, BatchView bv, const int *kept_idx, const int *out_len, TensorView cache_k,
-                    TensorView cache_v, const int *cache_pos, TensorView chunk_k, TensorView chunk_v,
-                    const int *chunk_pos, TensorView out_k, TensorView out_v, int *out_pos, int *status) {
-    __shared__ int src_idx[kRowsPerCta];
-    dependency_wait();
-    const UnitInfo u = unit_info(mv, bv, blockIdx.y, blockIdx.z);
-    if (!u.ok) {
-        if (threadIdx.x == 0) atomicOr(status, FINCH_DEV_BAD_BATCH);
-        return;
+// Rows of one tensor (K or V of a KV head): where candidate j's row starts, and output row i.
+struct RowMap {
+    const char *cache, *chunk;
+    char *out;
+    int64_t cache_step, chunk_step, out_step;
+    int c;
+    __device__ RowMap(const UnitInfo &u, int kvh, int i0, int64_t e, const TensorView &ca, const TensorView &ch,
+                      const TensorView &dst) {
+        cache = ca.ptr + ((int64_t)u.l * ca.stride_layer + (int64_t)kvh * ca.stride_head + (int64_t)u.cache0 * ca.stride_tok) * e;
+        chunk = ch.ptr + ((int64_t)u.l * ch.stride_layer + (int64_t)kvh * ch.stride_head +
+                          (int64_t)(u.chunk0 - u.c) * ch.stride_tok) * e;
+        out = const_cast<char *>(dst.ptr) + ((int64_t)u.l * dst.stride_layer + (int64_t)kvh * dst.stride_head +
+                                             (int64_t)(u.cache0 + i0) * dst.stride_tok) * e;
+        cache_step = ca.stride_tok * e;
+        chunk_step = ch.stride_tok * e;
+        out_step = dst.stride_tok * e;
+        c = u.c;
     }
-    int r = out_len[u.b];
-    if (r > u.cap) r = u.cap;
-    const int i0 = blockIdx.x * kRowsPerCta;
-    if (i0 >= r) return;
-    const int rows = min(kRowsPerCta, r - i0);
-    const int64_t unit_off = ((int64_t)u.l * mv.G + u.G) * bv.total_cache + u.cache0;
-    if (threadIdx.x < rows) {
-        int j = kept_idx[unit_off + i0 + threadIdx.x];
-        // a distance beyond the table (only possible when out_len exceeds the candidate count) is refused as well
-        if (j < 0 || j >= u.N || abs(i0 + (int)threadIdx.x - j) >= mv.rope_rows) {
-            atomicOr(status, FINCH_DEV_BAD_INDEX);
-            j = -1;
-        } else {
-            out_pos[unit_off + i0 + threadIdx.x] = j < u.c ? cache_pos[unit_off + j] : chunk_pos[u.chunk0 + j - u.c];
-        }
-        src_idx[threadIdx.x] = j;
-    }
-    __syncthreads();
+    __device__ const char *src(int j) const { return j < c ? cache + j * cache_step : chunk + j * chunk_step; }
+};
 
-    const int pieces = mv.d * mv.elem_bytes / 16;
-    const int per_row = pieces * 2 * mv.kvpg;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    constexpr int kRowsInFlight = kCompactThreads / 32;
-    constexpr int kBatch = 4;
-    const bool split_pairs = mv.rope_pairing == 0;
-    const int half = mv.d / 2;
-    for (int cs = tx; cs < per_row; cs += 32) {
-        const int piece = cs % pieces, which = cs / pieces;
-        const int kvh = u.G * mv.kvpg + which / 2;
-        const bool is_v = which & 1;
-        // with pairs (t, t + d/2) the second half of a K row is written by the owner of the first half
-        if (!is_v && split_pairs && piece >= pieces / 2) continue;
-        const bool two = !is_v && split_pairs;  // this thread moves a partner piece as well
-        const TensorView &ca = is_v ? cache_v : cache_k;
-        const TensorView &ch = is_v ? chunk_v : chunk_k;
-        const TensorView &dst = is_v ? out_v : out_k;
-        const int64_t e = mv.elem_bytes;
-        const char *ca_base = ca.ptr + ((int64_t)u.l * ca.stride_layer + (int64_t)kvh * ca.stride_head +
-                                        (int64_t)u.cache0 * ca.stride_tok) * e + piece * 16;
-        const char *ch_base = ch.ptr + ((int64_t)u.l * ch.stride_layer + (int64_t)kvh * ch.stride_head +
-                                        (int64_t)(u.chunk0 - u.c) * ch.stride_tok) * e + piece * 16;
-        char *dst_base = const_cast<char *>(dst.ptr) + ((int64_t)u.l * dst.stride_layer + (int64_t)kvh * dst.stride_head +
-                                                        (int64_t)(u.cache0 + i0) * dst.stride_tok) * e + piece * 16;
-        const int64_t ca_step = ca.stride_tok * e, ch_step = ch.stride_tok * e, dst_step = dst.stride_tok * e;
-        const int half_bytes = half * mv.elem_bytes;  // distance to the partner piece (pairs (t, t + d/2))
-        // first pair of this piece: kElems pairs per piece with split pairs, kElems / 2 with neighbouring pairs
-        const float2 *table = mv.rope_table + (split_pairs ? piece * kElems : piece * (kElems / 2));
+// Plain copies.  A thread keeps its piece of the row and walks the rows 256 / pieces apart.
+__device__ __forceinline__ void copy_rows(const RowMap &m, const int *src_idx, int rows, int pieces) {
+    constexpr int kBatch = 8;
+    const int step = kCompactThreads / pieces, r0 = threadIdx.x / pieces, off = (threadIdx.x - r0 * pieces) * 16;
+    if (r0 >= step) return;
 #pragma unroll 1
-        for (int k0 = 0; k0 * kRowsInFlight < rows; k0 += kBatch) {
-            uint4 a[kBatch], b[kBatch];
+    for (int r = r0; r < rows; r += step * kBatch) {
+        uint4 v[kBatch];
 #pragma unroll
-            for (int k = 0; k < kBatch; ++k) {  // this batch's loads first ..
-                const int row = ty + (k0 + k) * kRowsInFlight;
-                const int j = row < rows ? src_idx[row] : -1;
-                if (j >= 0) {
-                    const char *src = j < u.c ? ca_base + j * ca_step : ch_base + j * ch_step;
-                    a[k] = __ldg((const uint4 *)src);
-                    if (two) b[k] = __ldg((const uint4 *)(src + half_bytes));
-                }
-            }
+        for (int k = 0; k < kBatch; ++k) {  // all of this batch's loads first ..
+            const int row = r + k * step, j = row < rows ? src_idx[row] : -1;
+            if (j >= 0) v[k] = __ldcs((const uint4 *)(m.src(j) + off));
+        }
 #pragma unroll
-            for (int k = 0; k < kBatch; ++k) {  // .. then the rotations and the stores
-                const int row = ty + (k0 + k) * kRowsInFlight;
-                const int j = row < rows ? src_idx[row] : -1;
-                if (j < 0) continue;
-                const int delta = i0 + row - j;
-                const float2 *cs_row = table + (int64_t)abs(delta) * half;
-                const float sign = delta < 0 ? -1.f : 1.f;
-                if (two) {
-                    rotate_pieces<kElems>(a[k], b[k], cs_row, sign);
-                    *(uint4 *)(dst_base + row * dst_step + half_bytes) = b[k];
-                } else if (!is_v) {
-                    rotate_interleaved<kElems>(a[k], cs_row, sign);
-                }
-                *(uint4 *)(dst_base + row * dst_step) = a[k];
-            }
+        for (int k = 0; k < kBatch; ++k) {  // .. then its stores
+            const int row = r + k * step;
+            if (row < rows && src_idx[row] >= 0) *(uint4 *)(m.out + row * m.out_step + off) = v[k];
         }
     }
 }
 
+// Copies with rotation, four rows in flight.  kSplit: pairs (t, t + d/2), a thread moves a piece of the row's first half
+// and the partner piece of the second; else pairs (2t, 2t + 1) inside a piece.
+template <int kElems, bool kSplit>
+__device__ __forceinline__ void rotate_rows(const RowMap &m, const int *src_idx, int rows, int i0, int d, int elem_bytes,
+                                            const float2 *rope_table) {
+    constexpr int kBatch = 4;
+    const int half = d / 2, pieces = d * elem_bytes / 16 / (kSplit ? 2 : 1);
+    const int step = kCompactThreads / pieces, r0 = threadIdx.x / pieces, piece = threadIdx.x - r0 * pieces;
+    const int off = piece * 16, far = half * elem_bytes;
+    const float2 *table = rope_table + piece * (kSplit ? kElems : kElems / 2);
+    if (r0 >= step) return;
+#pragma unroll 1
+    for (int r = r0; r < rows; r += step * kBatch) {
+        uint4 a[kBatch], b[kSplit ? kBatch : 1];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            const int row = r + k * step, j = row < rows ? src_idx[row] : -1;
+            if (j >= 0) {
+                const char *src = m.src(j) + off;
+                a[k] = __ldcs((const uint4 *)src);
+                if (kSplit) b[k] = __ldcs((const uint4 *)(src + far));
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            const int row = r + k * step, j = row < rows ? src_idx[row] : -1;
+            if (j < 0) continue;
+            const int delta = i0 + row - j;
+            const float2 *cs = table + (int64_t)abs(delta) * half;
+            const float sign = delta < 0 ? -1.f : 1.f;
+            char *dst = m.out + row * m.out_step + off;
+            if (kSplit) {
+                rotate_pieces<kElems>(a[k], b[k], cs, sign);
+                *(uint4 *)(dst + far) = b[k];
+            } else {
+                rotate_interleaved<kElems>(a[k], cs, sign);
+            }
+            *(uint4 *)dst = a[k];
+        }
+    }
+}
+
+// ROPE 0: bit-for-bit copies; 1 / 2: K rows re-positioned, pairs (t, t + d/2) / (2t, 2t + 1).
+template <int ROPE, int kElems>
 __global__ void __launch_bounds__(kCompactThreads)
 compact_kernel(ModelView mv, BatchView bv, const int *kept_idx, const int *out_len, TensorView cache_k,
                TensorView cache_v, const int *cache_pos, TensorView chunk_k, TensorView chunk_v, const int *chunk_pos,
-               TensorView out_k, TensorView out_v, int *out_pos, int *status) {
-    __shared__ int src_idx[kRowsPerCta];
+               TensorView out_k, TensorView out_v, int *out_pos, int rows_per_cta, int *status) {
+    __shared__ int src_idx[kMaxRowsPerCta];
     dependency_wait();  // no early launch of the next kernel: this grid runs in many waves and needs every slot
-    const UnitInfo u = unit_info(mv, bv, blockIdx.y, blockIdx.z);
+    const int l = blockIdx.y / mv.Hkv, kvh = blockIdx.y - l * mv.Hkv, group = kvh / mv.kvpg;
+    const UnitInfo u = unit_info(mv, bv, l * mv.G + group, blockIdx.z);
     if (!u.ok) {
         if (threadIdx.x == 0) atomicOr(status, FINCH_DEV_BAD_BATCH);
         return;
     }
     int r = out_len[u.b];
     if (r > u.cap) r = u.cap;
-    const int i0 = blockIdx.x * kRowsPerCta;
+    const int i0 = blockIdx.x * rows_per_cta;
     if (i0 >= r) return;
-    const int rows = min(kRowsPerCta, r - i0);
+    const int rows = min(rows_per_cta, r - i0);
     const int64_t unit_off = ((int64_t)u.l * mv.G + u.G) * bv.total_cache + u.cache0;
+    const bool leader = kvh == group * mv.kvpg;  // the group's positions are written by its first KV head's CTA
 
     if (threadIdx.x < rows) {
         int j = kept_idx[unit_off + i0 + threadIdx.x];
-        if (j < 0 || j >= u.N) {
+        // with rotation a distance beyond the table (only possible when out_len exceeds the candidate count) is refused
+        if (j < 0 || j >= u.N || (ROPE && abs(i0 + (int)threadIdx.x - j) >= mv.rope_rows)) {
             atomicOr(status, FINCH_DEV_BAD_INDEX);
             j = -1;
-        } else {
+        } else if (leader) {
             out_pos[unit_off + i0 + threadIdx.x] = j < u.c ? cache_pos[unit_off + j] : chunk_pos[u.chunk0 + j - u.c];
         }
         src_idx[threadIdx.x] = j;
@@ -217,43 +213,12 @@ compact_kernel(ModelView mv, BatchView bv, const int *kept_idx, const int *out_l
     __syncthreads();
 
     const int pieces = mv.d * mv.elem_bytes / 16;  // 16-byte pieces per row
-    const int per_row = pieces * 2 * mv.kvpg;      // K and V, every KV head of the group
-    // A warp owns 32 consecutive pieces of an output row (fully coalesced) and walks the CTA's rows eight apart;
-    // everything that does not depend on the row is computed once per thread, outside the row loop.
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    constexpr int kRowsInFlight = kCompactThreads / 32;
-    for (int cs = tx; cs < per_row; cs += 32) {
-        const int piece = cs % pieces, which = cs / pieces;  // which = kv * 2 + {0: K, 1: V}
-        const int kvh = u.G * mv.kvpg + which / 2;
-        const bool is_v = which & 1;
-        const TensorView &ca = is_v ? cache_v : cache_k;
-        const TensorView &ch = is_v ? chunk_v : chunk_k;
-        const TensorView &dst = is_v ? out_v : out_k;
-        const int64_t e = mv.elem_bytes;
-        const char *ca_base = ca.ptr + ((int64_t)u.l * ca.stride_layer + (int64_t)kvh * ca.stride_head +
-                                        (int64_t)u.cache0 * ca.stride_tok) * e + piece * 16;
-        const char *ch_base = ch.ptr + ((int64_t)u.l * ch.stride_layer + (int64_t)kvh * ch.stride_head +
-                                        (int64_t)(u.chunk0 - u.c) * ch.stride_tok) * e + piece * 16;
-        char *dst_base = const_cast<char *>(dst.ptr) + ((int64_t)u.l * dst.stride_layer + (int64_t)kvh * dst.stride_head +
-                                                        (int64_t)(u.cache0 + i0) * dst.stride_tok) * e + piece * 16;
-        const int64_t ca_step = ca.stride_tok * e, ch_step = ch.stride_tok * e, dst_step = dst.stride_tok * e;
-        constexpr int kBatch = 8;  // rows per thread whose loads are issued before the first store
-#pragma unroll 1
-        for (int k0 = 0; k0 * kRowsInFlight < rows; k0 += kBatch) {
-            uint4 v[kBatch];
-#pragma unroll
-            for (int k = 0; k < kBatch; ++k) {  // all of this batch's loads first ..
-                const int row = ty + (k0 + k) * kRowsInFlight;
-                const int j = row < rows ? src_idx[row] : -1;
-                if (j >= 0) v[k] = __ldg((const uint4 *)(j < u.c ? ca_base + j * ca_step : ch_base + j * ch_step));
-            }
-#pragma unroll
-            for (int k = 0; k < kBatch; ++k) {  // .. then its stores
-                const int row = ty + (k0 + k) * kRowsInFlight;
-                if (row < rows && src_idx[row] >= 0) *(uint4 *)(dst_base + row * dst_step) = v[k];
-            }
-        }
-    }
+    const RowMap k_rows(u, kvh, i0, mv.elem_bytes, cache_k, chunk_k, out_k);
+    if (ROPE)
+        rotate_rows<kElems, ROPE == 1>(k_rows, src_idx, rows, i0, mv.d, mv.elem_bytes, mv.rope_table);
+    else
+        copy_rows(k_rows, src_idx, rows, pieces);
+    copy_rows(RowMap(u, kvh, i0, mv.elem_bytes, cache_v, chunk_v, out_v), src_idx, rows, pieces);
 }
 
 }  // namespace
@@ -263,18 +228,20 @@ cudaError_t launch_compact(const Ctx &ctx, const int *kept_idx, const int *out_l
                            const TensorView &chunk_v, const int *chunk_pos, const BatchView &bv, const TensorView &out_k,
                            const TensorView &out_v, int *out_pos, cudaStream_t stream) {
     const ModelView &mv = ctx.model;
-    const int units = mv.L * mv.G;
-    const int row_blocks = (bv.max_budget + kRowsPerCta - 1) / kRowsPerCta;
-    if (units == 0 || bv.batch == 0 || row_blocks == 0) return cudaSuccess;
-    dim3 grid(row_blocks, units, bv.batch);
+    const int heads = mv.L * mv.Hkv;
+    if (heads == 0 || bv.batch == 0 || bv.max_budget == 0) return cudaSuccess;
+    // the largest block that still gives every SM two CTAs
+    const int64_t sms = ctx.sm_count > 0 ? ctx.sm_count : 148;
+    int rows = kMaxRowsPerCta;
+    while (rows > kMinRowsPerCta && (int64_t)((bv.max_budget + rows - 1) / rows) * heads * bv.batch < 2 * sms) rows /= 2;
+    dim3 grid((bv.max_budget + rows - 1) / rows, heads, bv.batch);
     ctx.launches += 1;
-    if (mv.rope_theta > 0.f) {
-        auto kernel = mv.elem_bytes == 4 ? compact_rope_kernel<4> : compact_rope_kernel<8>;
-        return launch_chained(kernel, grid, dim3(kCompactThreads), 0, stream, mv, bv, kept_idx, out_len, cache_k, cache_v,
-                              cache_pos, chunk_k, chunk_v, chunk_pos, out_k, out_v, out_pos, ctx.d_status);
-    }
-    return launch_chained(compact_kernel, grid, dim3(kCompactThreads), 0, stream, mv, bv, kept_idx, out_len, cache_k, cache_v,
-                          cache_pos, chunk_k, chunk_v, chunk_pos, out_k, out_v, out_pos, ctx.d_status);
+    const bool f32 = mv.elem_bytes == 4;
+    auto kernel = compact_kernel<0, 8>;
+    if (mv.rope_theta > 0.f && mv.rope_pairing == 0) kernel = f32 ? compact_kernel<1, 4> : compact_kernel<1, 8>;
+    if (mv.rope_theta > 0.f && mv.rope_pairing == 1) kernel = f32 ? compact_kernel<2, 4> : compact_kernel<2, 8>;
+    return launch_chained(kernel, grid, dim3(kCompactThreads), 0, stream, mv, bv, kept_idx, out_len, cache_k, cache_v,
+                          cache_pos, chunk_k, chunk_v, chunk_pos, out_k, out_v, out_pos, rows, ctx.d_status);
 }
 
 }  // namespace finch
