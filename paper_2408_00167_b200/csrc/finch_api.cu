@@ -156,7 +156,7 @@ cudaError_t run_score(const Ctx &ctx, const TensorView &q, const TensorView &cac
             launch_score_tc(ctx, q, cache_k, chunk_k, bv, scores, scratch, scratch_capacity, row_lse, stream);
         if (e != cudaErrorNotSupported) return e;
     }
-    return launch_score_simt(ctx, q, cache_k, chunk_k, bv, scores, scratch, row_lse, stream);
+    return launch_score_simt(ctx, q, cache_k, chunk_k, bv, scores, scratch, scratch_capacity, row_lse, stream);
 }
 
 }  // namespace finch

@@ -124,10 +124,10 @@ cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
 
 // ---- launchers implemented in the kernel files; each returns the cudaError_t of its launches ----
 
-// warp-level dot-product scoring (any dtype, any prompt length).  row_stats [L][Hq][total_q] is scratch that holds
-// (max base-2 logit, 1 / sum of exp2) per prompt row; row_lse (nullable) is the caller-visible natural-log copy.
+// warp-level dot-product scoring (any dtype, any prompt length).  The scratch holds the partial statistics of every prompt
+// row (n_layers * n_q_heads * total_q) once per key split: at least one entry per row.
 cudaError_t launch_score_simt(const Ctx &ctx, const TensorView &q, const TensorView &cache_k, const TensorView &chunk_k,
-                              const BatchView &bv, float *scores, float2 *row_stats, float *row_lse,
+                              const BatchView &bv, float *scores, float2 *scratch, size_t capacity, float *row_lse,
                               cudaStream_t stream);
 
 // tensor-core scoring (bf16, head_dim 64 or 128, either group mode).  The scratch holds the partial row statistics of

@@ -1,120 +1,182 @@
 // Prompt-guided scoring with plain FMA dot products (fp32 inputs, head dimensions the tensor-core path does not take).
 //
-//   lse_simt     one CTA per (64 prompt rows of one query head, unit): sweeps every candidate key and keeps an
-//                online (max, sum-exp) per row -> row_stats = (max of the base-2 logits, 1 / sum), row_lse
-//   colsum_simt  one CTA per (64 candidate keys, unit): sweeps every prompt row of every head of the group and
-//                accumulates exp2(s2 - max) / sum per key -> scores
+//   lse_simt     one CTA per (row tile of one query head, unit, key split): an online (max, sum-exp) per row over the
+//                split's keys -> part (max of the base-2 logits, sum of exp2 against it)
+//   colsum_simt  one CTA per (64 candidate keys, unit): merges the parts of each prompt row, then sweeps every prompt
+//                row of every head of the group and accumulates exp2(s2 - max) / sum per key -> scores
 //
 // Keeping the row maximum and the reciprocal sum apart (instead of one log-sum-exp) keeps the exponent's argument
 // a small difference even when the logits are large; both kernels form it with the same fused multiply-add
 // (dot * scale2 - max), so the weight of a row's largest key is the same in the sum and in the column pass.
 //
-// A unit is one (layer, selection group, request).  Both kernels tile the logits 64 x 64 with a 4 x 4 register
-// micro-tile per thread and walk head_dim in slices of 32 staged through shared memory.  All sums have a fixed
-// order, so the scores are bit-identical from run to run.
-#include "finch_internal.cuh"
+// A unit is one (layer, selection group, request).  Row tiles have 16, 32 or 64 rows, the least that holds the longest
+// prompt; keys are split so that a small problem still fills the SMs (16 rows x 512 keys of 8 heads ran on 8 CTAs that
+// walked the keys one tile after another: 57 us; 6 us over 64 CTAs).  A thread owns RM x 4 logits; both operands are staged
+// as fp32 in slices of 32 dimensions, the next slice's loads in flight under the current one's arithmetic, and read as
+// 128-bit vectors into packed multiply-adds.  All sums have a fixed order, so the scores are bit-identical from run to
+// run.
+#include "score_tc_common.cuh"
 
 namespace finch {
 namespace {
 
-constexpr int kTile = 64;      // rows and keys per CTA tile
+using tc::fma2;
+using tc::unpack2;
+
+constexpr int kKeys = 64;      // keys per CTA tile
 constexpr int kSlice = 32;     // head_dim slice staged per iteration
-constexpr int kThreads = 256;  // 16 x 16 threads, 4 x 4 logits each
+constexpr int kPitch = kSlice + 4;  // floats per staged row: 128-bit reads of eight rows hit different banks
+constexpr int kThreads = 128;  // 8 row lanes x 16 key lanes
+constexpr int kMaxParts = 32;  // key splits
 
-template <typename T>
-__device__ __forceinline__ float to_f32(T v);
-template <>
-__device__ __forceinline__ float to_f32<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-// Stage a [64 rows][32 elements] slice of Q (prompt rows p0.. of head h) into shared memory as fp32.
-template <typename T>
-__device__ __forceinline__ void stage_q(float (*dst)[kSlice + 1], const TensorView &q, const UnitInfo &u, int h, int p0,
-                                        int t0) {
-    const T *base = (const T *)q.ptr + (int64_t)u.l * q.stride_layer + (int64_t)h * q.stride_head;
-    for (int e = threadIdx.x; e < kTile * kSlice; e += kThreads) {
-        const int r = e / kSlice, t = e % kSlice;
-        const int p = p0 + r;
-        dst[r][t] = p < u.n_q ? to_f32<T>(base[(int64_t)(u.q0 + p) * q.stride_tok + t0 + t]) : 0.f;
-    }
+__device__ __forceinline__ float4 load4(const float *p) { return __ldg((const float4 *)p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16 *p) {
+    const uint2 v = __ldg((const uint2 *)p);
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                       __uint_as_float(v.y & 0xffff0000u));
 }
 
-// Stage a [64 keys][32 elements] slice of the candidate keys j0.. of KV head kvh (cache rows first, then chunk rows).
+// A row-major operand tile of ROWS x d: where each of this thread's rows starts (null: no such row, zeros).
+template <typename T, int ROWS>
+struct Tile {
+    static constexpr int kPer = ROWS * (kSlice / 4) / kThreads;  // float4 per thread and slice
+    const T *row[kPer];
+    float4 next[kPer];
+    __device__ __forceinline__ static int row_of(int i) { return (threadIdx.x + i * kThreads) / (kSlice / 4); }
+    __device__ __forceinline__ void fetch(int t0) {
+        const int q = threadIdx.x % (kSlice / 4);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) next[i] = row[i] ? load4(row[i] + t0 + q * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __device__ __forceinline__ void store(float *dst) const {
+        const int q = threadIdx.x % (kSlice / 4);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) *(float4 *)(dst + row_of(i) * kPitch + q * 4) = next[i];
+    }
+};
+
+template <typename T, int ROWS>
+__device__ __forceinline__ void q_tile(Tile<T, ROWS> &t, const TensorView &q, const UnitInfo &u, int h, int p0) {
+    const T *base = (const T *)q.ptr + (int64_t)u.l * q.stride_layer + (int64_t)h * q.stride_head;
+#pragma unroll
+    for (int i = 0; i < Tile<T, ROWS>::kPer; ++i) {
+        const int p = p0 + t.row_of(i);
+        t.row[i] = p < u.n_q ? base + (int64_t)(u.q0 + p) * q.stride_tok : nullptr;
+    }
+}
+// candidate keys j0 .. of KV head kvh (cache rows first, then chunk rows)
 template <typename T>
-__device__ __forceinline__ void stage_k(float (*dst)[kSlice + 1], const TensorView &cache_k, const TensorView &chunk_k,
-                                        const UnitInfo &u, int kvh, int j0, int t0) {
+__device__ __forceinline__ void k_tile(Tile<T, kKeys> &t, const TensorView &cache_k, const TensorView &chunk_k,
+                                       const UnitInfo &u, int kvh, int j0) {
     const T *cbase = (const T *)cache_k.ptr + (int64_t)u.l * cache_k.stride_layer + (int64_t)kvh * cache_k.stride_head;
     const T *hbase = (const T *)chunk_k.ptr + (int64_t)u.l * chunk_k.stride_layer + (int64_t)kvh * chunk_k.stride_head;
-    for (int e = threadIdx.x; e < kTile * kSlice; e += kThreads) {
-        const int r = e / kSlice, t = e % kSlice;
-        const int j = j0 + r;
-        float v = 0.f;
-        if (j < u.c)
-            v = to_f32<T>(cbase[(int64_t)(u.cache0 + j) * cache_k.stride_tok + t0 + t]);
-        else if (j < u.N)
-            v = to_f32<T>(hbase[(int64_t)(u.chunk0 + j - u.c) * chunk_k.stride_tok + t0 + t]);
-        dst[r][t] = v;
+#pragma unroll
+    for (int i = 0; i < Tile<T, kKeys>::kPer; ++i) {
+        const int j = j0 + t.row_of(i);
+        t.row[i] = j < u.c ? cbase + (int64_t)(u.cache0 + j) * cache_k.stride_tok
+                           : (j < u.N ? hbase + (int64_t)(u.chunk0 + j - u.c) * chunk_k.stride_tok : nullptr);
     }
 }
 
-// acc[i][j] += sum_t Q[ty + 16 i][t] * K[tx + 16 j][t] over one staged slice.
-__device__ __forceinline__ void fma_slice(float (&acc)[4][4], const float (*qs)[kSlice + 1],
-                                          const float (*ks)[kSlice + 1], int tx, int ty) {
-#pragma unroll 8
-    for (int t = 0; t < kSlice; ++t) {
-        float a[4], b[4];
+// acc[i][j] = Q[ty + 8 i] . K[tx + 16 j] over all of head_dim; the even and the odd dimensions are summed apart.
+template <typename T, int RM>
+__device__ __forceinline__ void logits(float (&acc)[RM][4], Tile<T, RM * 8> &q, Tile<T, kKeys> &k, int d, float *qs, float *ks,
+                                       int tx, int ty) {
+    uint64_t sum[RM][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = qs[ty + 16 * i][t];
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = ks[tx + 16 * j][t];
+        for (int j = 0; j < 4; ++j) sum[i][j] = 0;
+    q.fetch(0);
+    k.fetch(0);
+    for (int t0 = 0; t0 < d; t0 += kSlice) {
+        __syncthreads();  // everyone is through with the previous slice
+        q.store(qs);
+        k.store(ks);
+        __syncthreads();
+        if (t0 + kSlice < d) {
+            q.fetch(t0 + kSlice);
+            k.fetch(t0 + kSlice);
+        }
+#pragma unroll 2
+        for (int t = 0; t < kSlice; t += 4) {
+            ulonglong2 b[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 4; ++j) b[j] = *(const ulonglong2 *)(ks + (tx + 16 * j) * kPitch + t);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+            for (int i = 0; i < RM; ++i) {
+                const ulonglong2 a = *(const ulonglong2 *)(qs + (ty + 8 * i) * kPitch + t);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sum[i][j] = fma2(a.y, b[j].y, fma2(a.x, b[j].x, sum[i][j]));
+            }
+        }
     }
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float lo, hi;
+            unpack2(sum[i][j], lo, hi);
+            acc[i][j] = lo + hi;
+        }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-lse_simt(ModelView mv, BatchView bv, TensorView q, TensorView cache_k, TensorView chunk_k, float2 *row_stats,
-         float *row_lse, int *status) {
-    __shared__ float qs[kTile][kSlice + 1];
-    __shared__ float ks[kTile][kSlice + 1];
+struct SimtParams {
+    ModelView mv;
+    BatchView bv;
+    TensorView q, cache_k, chunk_k;
+    float2 *parts;  // [splits][L][Hq][total_q] (max base-2 logit, sum of exp2 against it)
+    float *row_lse, *scores;
+    int splits;
+    int early;  // the grid is resident at once: the next kernel may be scheduled
+    int *status;
+};
+
+template <typename T, int RM>
+__global__ void __launch_bounds__(kThreads, 3)
+lse_simt(SimtParams p) {
+    __shared__ __align__(16) float qs[RM * 8 * kPitch];
+    __shared__ __align__(16) float ks[kKeys * kPitch];
+    const ModelView &mv = p.mv;
+    const BatchView &bv = p.bv;
+    dependency_wait();
+    if (p.early) dependents_may_launch();
     const UnitInfo u = unit_info(mv, bv, blockIdx.y, blockIdx.z);
     if (!u.ok) {
-        if (threadIdx.x == 0) atomicOr(status, FINCH_DEV_BAD_BATCH);
+        if (threadIdx.x == 0) atomicOr(p.status, FINCH_DEV_BAD_BATCH);
         return;
     }
     if (u.N == 0) return;
-    const int row_blocks = (bv.max_q + kTile - 1) / kTile;
-    const int hh = blockIdx.x / row_blocks, p0 = (blockIdx.x % row_blocks) * kTile;
+    constexpr int kRows = RM * 8;
+    const int row_blocks = (bv.max_q + kRows - 1) / kRows;
+    const int split = blockIdx.x % p.splits, rb = blockIdx.x / p.splits;
+    const int hh = rb / row_blocks, p0 = (rb % row_blocks) * kRows;
     if (p0 >= u.n_q) return;
     const int h = u.G * mv.hpg + hh, kvh = h / mv.g;
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
     const float scale2 = mv.scale * kLog2e;
+    const int tiles = (u.N + kKeys - 1) / kKeys, per = (tiles + p.splits - 1) / p.splits;
 
-    float run_max[4], run_sum[4];  // base-2 logits, over this thread's own key columns
-    int vis[4];                    // candidates the thread's rows attend to: all, or the row's limit (causal rows)
+    float run_max[RM], run_sum[RM];  // base-2 logits, over this thread's own key columns
+    int vis[RM];                     // candidates the thread's rows attend to: all, or the row's limit (causal rows)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < RM; ++i) {
         run_max[i] = -INFINITY;
         run_sum[i] = 0.f;
-        const int p = p0 + ty + 16 * i;
+        const int pr = p0 + ty + 8 * i;
         vis[i] = u.N;
-        if (bv.row_limit && p < u.n_q) vis[i] = max(0, min(u.N, bv.row_limit[u.q0 + p]));
+        if (bv.row_limit && pr < u.n_q) vis[i] = max(0, min(u.N, bv.row_limit[u.q0 + pr]));
     }
-    for (int j0 = 0; j0 < u.N; j0 += kTile) {
-        float acc[4][4] = {};
-        for (int t0 = 0; t0 < mv.d; t0 += kSlice) {
-            __syncthreads();
-            stage_q<T>(qs, q, u, h, p0, t0);
-            stage_k<T>(ks, cache_k, chunk_k, u, kvh, j0, t0);
-            __syncthreads();
-            fma_slice(acc, qs, ks, tx, ty);
-        }
+    Tile<T, kRows> qt;
+    Tile<T, kKeys> kt;
+    q_tile(qt, p.q, u, h, p0);
+    for (int t = split * per; t < min(tiles, (split + 1) * per); ++t) {
+        const int j0 = t * kKeys;
+        float acc[RM][4];
+        k_tile(kt, p.cache_k, p.chunk_k, u, kvh, j0);
+        logits<T, RM>(acc, qt, kt, mv.d, qs, ks, tx, ty);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < RM; ++i) {
             float tile_max = -INFINITY;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -130,8 +192,9 @@ lse_simt(ModelView mv, BatchView bv, TensorView q, TensorView cache_k, TensorVie
         }
     }
     // merge the 16 column owners of each row (the lanes tx = 0..15 of a half warp) with a butterfly
+    const int64_t rows_total = (int64_t)mv.L * mv.Hq * bv.total_q;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < RM; ++i) {
         float mx = run_max[i], sm = run_sum[i];
 #pragma unroll
         for (int off = 1; off < 16; off <<= 1) {
@@ -143,63 +206,94 @@ lse_simt(ModelView mv, BatchView bv, TensorView q, TensorView cache_k, TensorVie
             sm = a + b;  // commutative: both partners get the same bits
             mx = nmx;
         }
-        const int p = p0 + ty + 16 * i;
-        if (tx == 0 && p < u.n_q) {
-            const int64_t row = ((int64_t)u.l * mv.Hq + h) * bv.total_q + u.q0 + p;
-            if (bv.self_lse) {  // the keys the row attends to besides the candidates: one more term of the sum
-                const float ex = bv.self_lse[row] * kLog2e;
-                if (ex > -INFINITY) {
-                    const float nmx = fmaxf(mx, ex);
-                    sm = sm * exp2f(mx - nmx) + exp2f(ex - nmx);
-                    mx = nmx;
-                }
-            }
-            // (max, weight per unit of exp2): 1 / sum, times the fraction of the candidates the row sees when the
-            // per-row normalisation is on; a row that sees nothing weighs nothing
-            float w = sm > 0.f ? 1.0f / sm : 0.f;
-            if (bv.row_norm) w *= (float)vis[i] / (float)u.N;
-            row_stats[row] = make_float2(sm > 0.f ? mx : 0.f, w);
-            if (row_lse) row_lse[row] = sm > 0.f ? (mx + log2f(sm)) * kLn2 : -INFINITY;
-        }
+        const int pr = p0 + ty + 8 * i;
+        if (tx == 0 && pr < u.n_q)
+            p.parts[split * rows_total + ((int64_t)u.l * mv.Hq + h) * bv.total_q + u.q0 + pr] = make_float2(mx, sm);
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-colsum_simt(ModelView mv, BatchView bv, TensorView q, TensorView cache_k, TensorView chunk_k,
-            const float2 *row_stats, float *scores, int *status) {
-    __shared__ float qs[kTile][kSlice + 1];
-    __shared__ float ks[kTile][kSlice + 1];
-    __shared__ float red[16][kTile];
+// The parts of one row, merged in split order into (max, weight per unit of exp2): 1 / sum, times the fraction of the
+// candidates the row sees when the per-row normalisation is on; a row that sees nothing weighs nothing.
+__device__ __forceinline__ float2 merge_row_parts(const SimtParams &p, const UnitInfo &u, int64_t row, int vis, bool write_lse) {
+    const int64_t rows_total = (int64_t)p.mv.L * p.mv.Hq * p.bv.total_q;
+    float mx = -INFINITY, sm = 0.f;
+    for (int i0 = 0; i0 < p.splits; i0 += 4) {
+        float2 part[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            part[i] = i0 + i < p.splits ? p.parts[(i0 + i) * rows_total + row] : make_float2(-INFINITY, 0.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (!(part[i].y > 0.f)) continue;  // a split that holds none of the row's keys
+            const float nmx = fmaxf(mx, part[i].x);
+            sm = sm * exp2f(mx - nmx) + part[i].y * exp2f(part[i].x - nmx);
+            mx = nmx;
+        }
+    }
+    if (p.bv.self_lse) {  // the keys the row attends to besides the candidates: one more term of the sum
+        const float ex = p.bv.self_lse[row] * kLog2e;
+        if (ex > -INFINITY) {
+            const float nmx = fmaxf(mx, ex);
+            sm = sm * exp2f(mx - nmx) + exp2f(ex - nmx);
+            mx = nmx;
+        }
+    }
+    if (write_lse) p.row_lse[row] = sm > 0.f ? (mx + log2f(sm)) * kLn2 : -INFINITY;
+    float w = sm > 0.f ? 1.0f / sm : 0.f;
+    if (p.bv.row_norm && p.bv.row_limit) w *= (float)vis / (float)u.N;
+    return make_float2(sm > 0.f ? mx : 0.f, w);
+}
+
+template <typename T, int RM>
+__global__ void __launch_bounds__(kThreads, 3)
+colsum_simt(SimtParams p) {
+    constexpr int kRows = RM * 8;
+    __shared__ __align__(16) float qs[kRows * kPitch];
+    __shared__ __align__(16) float ks[kKeys * kPitch];
+    __shared__ float2 stats[kRows];
+    __shared__ int limits[kRows];
+    __shared__ float red[8][kKeys];
+    const ModelView &mv = p.mv;
+    const BatchView &bv = p.bv;
+    dependency_wait();
+    if (p.early) dependents_may_launch();
     const UnitInfo u = unit_info(mv, bv, blockIdx.y, blockIdx.z);
     if (!u.ok) {
-        if (threadIdx.x == 0) atomicOr(status, FINCH_DEV_BAD_BATCH);
+        if (threadIdx.x == 0) atomicOr(p.status, FINCH_DEV_BAD_BATCH);
         return;
     }
-    const int j0 = blockIdx.x * kTile;
+    const int j0 = blockIdx.x * kKeys;
     if (j0 >= u.N) return;
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
     const float scale2 = mv.scale * kLog2e;
 
     float col[4] = {0.f, 0.f, 0.f, 0.f};
+    Tile<T, kRows> qt;
+    Tile<T, kKeys> kt;
     for (int hh = 0; hh < mv.hpg; ++hh) {
-        const int h = u.G * mv.hpg + hh, kvh = h / mv.g;
-        const float2 *stats = row_stats + ((int64_t)u.l * mv.Hq + h) * bv.total_q + u.q0;
-        for (int p0 = 0; p0 < u.n_q; p0 += kTile) {
-            float acc[4][4] = {};
-            for (int t0 = 0; t0 < mv.d; t0 += kSlice) {
-                __syncthreads();
-                stage_q<T>(qs, q, u, h, p0, t0);
-                stage_k<T>(ks, cache_k, chunk_k, u, kvh, j0, t0);
-                __syncthreads();
-                fma_slice(acc, qs, ks, tx, ty);
+        const int h = u.G * mv.hpg + hh;
+        k_tile(kt, p.cache_k, p.chunk_k, u, h / mv.g, j0);
+        for (int p0 = 0; p0 < u.n_q; p0 += kRows) {
+            __syncthreads();  // the previous row tile's statistics have been read
+            if (threadIdx.x < kRows) {
+                const int pr = p0 + threadIdx.x;
+                float2 st = make_float2(0.f, 0.f);
+                int lim = 0;  // keys at or beyond it are masked
+                if (pr < u.n_q) {
+                    lim = bv.row_limit ? max(0, min(u.N, bv.row_limit[u.q0 + pr])) : u.N;
+                    st = merge_row_parts(p, u, ((int64_t)u.l * mv.Hq + h) * bv.total_q + u.q0 + pr, lim,
+                                         p.row_lse && blockIdx.x == 0);
+                }
+                stats[threadIdx.x] = st;
+                limits[threadIdx.x] = lim;
             }
+            float acc[RM][4];
+            q_tile(qt, p.q, u, h, p0);
+            logits<T, RM>(acc, qt, kt, mv.d, qs, ks, tx, ty);  // its barriers publish the statistics
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int p = p0 + ty + 16 * i;
-                if (p >= u.n_q) continue;
-                const float2 st = stats[p];
-                const int lim = bv.row_limit ? bv.row_limit[u.q0 + p] : u.N;  // keys at or beyond it are masked
+            for (int i = 0; i < RM; ++i) {
+                const float2 st = stats[ty + 8 * i];
+                const int lim = limits[ty + 8 * i];
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (j0 + tx + 16 * j < lim) col[j] = fmaf(exp2f(fmaf(acc[i][j], scale2, -st.x)), st.y, col[j]);
@@ -210,40 +304,55 @@ colsum_simt(ModelView mv, BatchView bv, TensorView q, TensorView cache_k, Tensor
 #pragma unroll
     for (int j = 0; j < 4; ++j) red[ty][tx + 16 * j] = col[j];
     __syncthreads();
-    if (threadIdx.x < kTile && j0 + threadIdx.x < u.N) {
+    if (threadIdx.x < kKeys && j0 + threadIdx.x < u.N) {
         float s = 0.f;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) s += red[r][threadIdx.x];
-        scores[((int64_t)u.l * mv.G + u.G) * ((int64_t)bv.total_cache + bv.total_chunk) + u.cache0 + u.chunk0 + j0 +
-               threadIdx.x] = s;
+        for (int r = 0; r < 8; ++r) s += red[r][threadIdx.x];
+        p.scores[((int64_t)u.l * mv.G + u.G) * ((int64_t)bv.total_cache + bv.total_chunk) + u.cache0 + u.chunk0 + j0 +
+                 threadIdx.x] = s;
     }
 }
 
-template <typename T>
-cudaError_t launch_t(const Ctx &ctx, const TensorView &q, const TensorView &cache_k, const TensorView &chunk_k,
-                     const BatchView &bv, float *scores, float2 *row_stats, float *row_lse,
-                     cudaStream_t stream) {
-    const ModelView &mv = ctx.model;
-    const int units = mv.L * mv.G;
-    const int row_blocks = (bv.max_q + kTile - 1) / kTile;
-    const int key_tiles = (bv.max_cache + bv.max_chunk + kTile - 1) / kTile;
+template <typename T, int RM>
+cudaError_t launch_t(const Ctx &ctx, SimtParams p, size_t capacity, cudaStream_t stream) {
+    const ModelView &mv = p.mv;
+    const BatchView &bv = p.bv;
+    const int units = mv.L * mv.G, sms = ctx.sm_count > 0 ? ctx.sm_count : 148;
+    const int row_blocks = (bv.max_q + RM * 8 - 1) / (RM * 8);
+    const int key_tiles = (bv.max_cache + bv.max_chunk + kKeys - 1) / kKeys;
     if (units == 0 || bv.batch == 0 || row_blocks == 0 || key_tiles == 0) return cudaSuccess;
-    dim3 g1(row_blocks * mv.hpg, units, bv.batch);
-    lse_simt<T><<<g1, kThreads, 0, stream>>>(mv, bv, q, cache_k, chunk_k, row_stats, row_lse, ctx.d_status);
+    // key splits: four CTAs for every SM, at least one key tile each, as far as the scratch goes
+    const int64_t ctas = (int64_t)row_blocks * mv.hpg * units * bv.batch;
+    const size_t rows = (size_t)mv.L * mv.Hq * (size_t)bv.total_q;
+    int64_t splits = (4 * (int64_t)sms + ctas - 1) / ctas;
+    splits = min(splits, (int64_t)min(key_tiles, kMaxParts));
+    if (rows) splits = min(splits, (int64_t)(capacity / rows));
+    p.splits = splits < 1 ? 1 : (int)splits;
+    p.early = ctas * p.splits <= 4 * sms;
+    dim3 g1(row_blocks * mv.hpg * p.splits, units, bv.batch);
+    cudaError_t e = launch_chained(lse_simt<T, RM>, g1, dim3(kThreads), 0, stream, p);
+    if (e != cudaSuccess) return e;
     dim3 g2(key_tiles, units, bv.batch);
-    colsum_simt<T><<<g2, kThreads, 0, stream>>>(mv, bv, q, cache_k, chunk_k, row_stats, scores, ctx.d_status);
+    p.early = (int64_t)key_tiles * units * bv.batch <= 4 * sms;
     ctx.launches += 2;
-    return cudaGetLastError();
+    return launch_chained(colsum_simt<T, RM>, g2, dim3(kThreads), 0, stream, p);
+}
+
+template <typename T>
+cudaError_t launch_rows(const Ctx &ctx, const SimtParams &p, size_t capacity, cudaStream_t stream) {
+    if (p.bv.max_q <= 16) return launch_t<T, 2>(ctx, p, capacity, stream);
+    if (p.bv.max_q <= 32) return launch_t<T, 4>(ctx, p, capacity, stream);
+    return launch_t<T, 8>(ctx, p, capacity, stream);
 }
 
 }  // namespace
 
 cudaError_t launch_score_simt(const Ctx &ctx, const TensorView &q, const TensorView &cache_k, const TensorView &chunk_k,
-                              const BatchView &bv, float *scores, float2 *row_stats, float *row_lse,
+                              const BatchView &bv, float *scores, float2 *scratch, size_t capacity, float *row_lse,
                               cudaStream_t stream) {
-    if (ctx.cfg.dtype == FINCH_F32)
-        return launch_t<float>(ctx, q, cache_k, chunk_k, bv, scores, row_stats, row_lse, stream);
-    return launch_t<__nv_bfloat16>(ctx, q, cache_k, chunk_k, bv, scores, row_stats, row_lse, stream);
+    SimtParams p{ctx.model, bv, q, cache_k, chunk_k, scratch, row_lse, scores, 1, 0, ctx.d_status};
+    return ctx.cfg.dtype == FINCH_F32 ? launch_rows<float>(ctx, p, capacity, stream)
+                                      : launch_rows<__nv_bfloat16>(ctx, p, capacity, stream);
 }
 
 }  // namespace finch
