@@ -7,6 +7,7 @@ loudly when libfinch.so is missing (build it with ``python -m paper_2408_00167_b
 from __future__ import annotations
 
 import ctypes as C
+import struct
 from dataclasses import dataclass
 from pathlib import Path
 from typing import Optional, Sequence
@@ -75,6 +76,14 @@ def load() -> C.CDLL:
         lib.finch_ctx_destroy.restype = None
         lib.finch_status_string.restype = C.c_char_p
         lib.finch_score_static_max_rows.restype = C.c_size_t
+        # the calls of a step take addresses and sizes: declared, plain Python integers go in without wrapper objects
+        p, z = C.c_void_p, C.c_size_t
+        lib.finch_score.argtypes = [p] * 8 + [z, p]
+        lib.finch_select.argtypes = [p] * 6 + [z, p]
+        lib.finch_compact.argtypes = [p] * 14
+        lib.finch_step.argtypes = [p] * 16 + [z, p]
+        lib.finch_step_host.argtypes = [p] * 21 + [z, p]
+        lib.finch_score_static.argtypes = [p] * 8
         _lib = lib
     return _lib
 
@@ -90,29 +99,58 @@ def _check(status: int, where: str) -> None:
 
 # ------------------------------------------------------------------ marshalling helpers
 
-def _tensor(t) -> finch_tensor:
-    """[L][heads][tokens][d] torch tensor (head_dim contiguous) -> finch_tensor; None -> null view."""
+def _view(t):
+    """[L][heads][tokens][d] torch tensor (head_dim contiguous) -> the four fields of a finch_tensor; None -> null view."""
     if t is None:
-        return finch_tensor(None, 0, 0, 0)
-    if t.dim() != 4 or (t.shape[3] > 1 and t.stride(3) != 1):
+        return 0, 0, 0, 0
+    s = t.stride()
+    if len(s) != 4 or (s[3] != 1 and t.shape[3] > 1):
         raise ValueError("expected a [layers][heads][tokens][head_dim] tensor with head_dim contiguous")
-    ptr = t.data_ptr() if t.numel() else None
-    return finch_tensor(ptr, t.stride(0), t.stride(1), t.stride(2))
+    return t.data_ptr(), s[0], s[1], s[2]     # data_ptr() of an empty tensor is 0
+
+
+_VIEW_BYTES = C.sizeof(finch_tensor)
+_packs = {}
+
+
+def _views(*tensors):
+    """The tensors as consecutive finch_tensor structs: (buffer to keep alive, address of the first)."""
+    n = len(tensors)
+    pack = _packs.get(n)
+    if pack is None:
+        pack = _packs[n] = (struct.Struct("=" + "Qqqq" * n), C.c_char * (n * _VIEW_BYTES))
+    buf = pack[1]()
+    fields = []
+    for t in tensors:
+        fields += _view(t)
+    pack[0].pack_into(buf, 0, *fields)
+    return buf, C.addressof(buf)
 
 
 def _ptr(t) -> Optional[int]:
-    return None if t is None or t.numel() == 0 else t.data_ptr()
+    return None if t is None else t.data_ptr() or None
 
 
 def _nbytes(t) -> int:
     return 0 if t is None else t.numel() * t.element_size()
 
 
+_current_stream = None
+
+
 def _stream(stream) -> Optional[int]:
-    if stream is None:
+    global _current_stream
+    if stream is not None:
+        return stream.cuda_stream or None
+    if _current_stream is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return stream.cuda_stream or None
+        torch.cuda.current_stream()           # initialises torch's side of CUDA
+        raw, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        if raw and device:                    # the handle itself, without a Stream object around it
+            _current_stream = lambda: raw(device())
+        else:
+            _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return _current_stream() or None
 
 
 @dataclass
@@ -180,35 +218,32 @@ def finch_workspace_bytes(ctx, batch: Batch) -> int:
 
 
 def finch_score(ctx, prompt_q, cache_k, chunk_k, batch: Batch, scores, row_lse=None, ws=None, stream=None) -> None:
-    q, ck, hk = _tensor(prompt_q), _tensor(cache_k), _tensor(chunk_k)
-    _check(load().finch_score(ctx, C.byref(q), C.byref(ck), C.byref(hk), C.byref(batch.c), C.c_void_p(_ptr(scores)),
-                              C.c_void_p(_ptr(row_lse)), C.c_void_p(_ptr(ws)), C.c_size_t(_nbytes(ws)),
-                              C.c_void_p(_stream(stream))), "finch_score")
+    keep, v = _views(prompt_q, cache_k, chunk_k)
+    _check(load().finch_score(ctx, v, v + _VIEW_BYTES, v + 2 * _VIEW_BYTES, C.addressof(batch.c), _ptr(scores), _ptr(row_lse),
+                              _ptr(ws), _nbytes(ws), _stream(stream)), "finch_score")
 
 
 def finch_select(ctx, scores, batch: Batch, kept_idx, out_len, ws=None, stream=None) -> None:
-    _check(load().finch_select(ctx, C.c_void_p(_ptr(scores)), C.byref(batch.c), C.c_void_p(_ptr(kept_idx)),
-                               C.c_void_p(_ptr(out_len)), C.c_void_p(_ptr(ws)), C.c_size_t(_nbytes(ws)),
-                               C.c_void_p(_stream(stream))), "finch_select")
+    _check(load().finch_select(ctx, _ptr(scores), C.addressof(batch.c), _ptr(kept_idx), _ptr(out_len), _ptr(ws),
+                               _nbytes(ws), _stream(stream)), "finch_select")
 
 
 def finch_compact(ctx, kept_idx, out_len, cache_k, cache_v, cache_pos, chunk_k, chunk_v, chunk_pos, batch: Batch,
                   out_k, out_v, out_pos, stream=None) -> None:
-    ts = [_tensor(t) for t in (cache_k, cache_v, chunk_k, chunk_v, out_k, out_v)]
-    _check(load().finch_compact(ctx, C.c_void_p(_ptr(kept_idx)), C.c_void_p(_ptr(out_len)), C.byref(ts[0]),
-                                C.byref(ts[1]), C.c_void_p(_ptr(cache_pos)), C.byref(ts[2]), C.byref(ts[3]),
-                                C.c_void_p(_ptr(chunk_pos)), C.byref(batch.c), C.byref(ts[4]), C.byref(ts[5]),
-                                C.c_void_p(_ptr(out_pos)), C.c_void_p(_stream(stream))), "finch_compact")
+    keep, v = _views(cache_k, cache_v, chunk_k, chunk_v, out_k, out_v)
+    z = _VIEW_BYTES
+    _check(load().finch_compact(ctx, _ptr(kept_idx), _ptr(out_len), v, v + z, _ptr(cache_pos), v + 2 * z, v + 3 * z,
+                                _ptr(chunk_pos), C.addressof(batch.c), v + 4 * z, v + 5 * z, _ptr(out_pos),
+                                _stream(stream)), "finch_compact")
 
 
 def finch_step(ctx, prompt_q, cache_k, cache_v, cache_pos, chunk_k, chunk_v, chunk_pos, batch: Batch, out_k, out_v,
                out_pos, kept_idx, out_len, scores=None, ws=None, stream=None) -> None:
-    ts = [_tensor(t) for t in (prompt_q, cache_k, cache_v, chunk_k, chunk_v, out_k, out_v)]
-    _check(load().finch_step(ctx, C.byref(ts[0]), C.byref(ts[1]), C.byref(ts[2]), C.c_void_p(_ptr(cache_pos)),
-                             C.byref(ts[3]), C.byref(ts[4]), C.c_void_p(_ptr(chunk_pos)), C.byref(batch.c),
-                             C.byref(ts[5]), C.byref(ts[6]), C.c_void_p(_ptr(out_pos)), C.c_void_p(_ptr(kept_idx)),
-                             C.c_void_p(_ptr(out_len)), C.c_void_p(_ptr(scores)), C.c_void_p(_ptr(ws)),
-                             C.c_size_t(_nbytes(ws)), C.c_void_p(_stream(stream))), "finch_step")
+    keep, v = _views(prompt_q, cache_k, cache_v, chunk_k, chunk_v, out_k, out_v)
+    z = _VIEW_BYTES
+    _check(load().finch_step(ctx, v, v + z, v + 2 * z, _ptr(cache_pos), v + 3 * z, v + 4 * z, _ptr(chunk_pos),
+                             C.addressof(batch.c), v + 5 * z, v + 6 * z, _ptr(out_pos), _ptr(kept_idx), _ptr(out_len),
+                             _ptr(scores), _ptr(ws), _nbytes(ws), _stream(stream)), "finch_step")
 
 
 def finch_device_status(ctx, stream=None) -> int:
@@ -230,10 +265,9 @@ def finch_launch_count(ctx) -> int:
 def finch_score_static(ctx, prompt_q, cache_k, chunk_k, batch: Batch, scores, row_lse=None, stream=None) -> None:
     """finch_score without a workspace: the scratch is a fixed array inside the library (see finch.h for the
     row limit and the sharing rules).  For callers that may not allocate device memory."""
-    q, ck, hk = _tensor(prompt_q), _tensor(cache_k), _tensor(chunk_k)
-    _check(load().finch_score_static(ctx, C.byref(q), C.byref(ck), C.byref(hk), C.byref(batch.c),
-                                     C.c_void_p(_ptr(scores)), C.c_void_p(_ptr(row_lse)),
-                                     C.c_void_p(_stream(stream))), "finch_score_static")
+    keep, v = _views(prompt_q, cache_k, chunk_k)
+    _check(load().finch_score_static(ctx, v, v + _VIEW_BYTES, v + 2 * _VIEW_BYTES, C.addressof(batch.c), _ptr(scores),
+                                     _ptr(row_lse), _stream(stream)), "finch_score_static")
 
 
 def finch_score_static_max_rows() -> int:
@@ -263,11 +297,10 @@ def finch_step_host(ctx, host_prompt_q, host_chunk_k, host_chunk_v, host_chunk_p
                     kept_idx, out_len, host_kept_idx, host_out_len, ws, stream=None) -> None:
     """finch_step with this step's inputs in host memory (torch CPU tensors, ideally pinned) and the kept indices
     and lengths returned to host tensors; the call returns after the stream has finished."""
-    ts = [_tensor(t) for t in (stage_q, stage_chunk_k, stage_chunk_v, cache_k, cache_v, out_k, out_v)]
+    keep, v = _views(stage_q, stage_chunk_k, stage_chunk_v, cache_k, cache_v, out_k, out_v)
+    z = _VIEW_BYTES
     _check(load().finch_step_host(
-        ctx, C.c_void_p(_ptr(host_prompt_q)), C.c_void_p(_ptr(host_chunk_k)), C.c_void_p(_ptr(host_chunk_v)),
-        C.c_void_p(_ptr(host_chunk_pos)), C.byref(ts[0]), C.byref(ts[1]), C.byref(ts[2]),
-        C.c_void_p(_ptr(stage_chunk_pos)), C.byref(ts[3]), C.byref(ts[4]), C.c_void_p(_ptr(cache_pos)),
-        C.byref(batch.c), C.byref(ts[5]), C.byref(ts[6]), C.c_void_p(_ptr(out_pos)), C.c_void_p(_ptr(kept_idx)),
-        C.c_void_p(_ptr(out_len)), C.c_void_p(_ptr(host_kept_idx)), C.c_void_p(_ptr(host_out_len)),
-        C.c_void_p(_ptr(ws)), C.c_size_t(_nbytes(ws)), C.c_void_p(_stream(stream))), "finch_step_host")
+        ctx, _ptr(host_prompt_q), _ptr(host_chunk_k), _ptr(host_chunk_v), _ptr(host_chunk_pos), v, v + z, v + 2 * z,
+        _ptr(stage_chunk_pos), v + 3 * z, v + 4 * z, _ptr(cache_pos), C.addressof(batch.c), v + 5 * z, v + 6 * z,
+        _ptr(out_pos), _ptr(kept_idx), _ptr(out_len), _ptr(host_kept_idx), _ptr(host_out_len), _ptr(ws), _nbytes(ws),
+        _stream(stream)), "finch_step_host")
