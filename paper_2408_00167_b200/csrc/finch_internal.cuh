@@ -48,12 +48,18 @@ struct Ctx {
     bool dry;       // validation-only context: nothing is ever enqueued
     int sm_count;
     int *tickets;  // [2][L * Hkv] counters of the one-kernel scoring: zero before and after every call
+    // kernels whose shared-memory limit has been raised on this context's device (a driver call: once, not per launch)
+    mutable uint32_t smem_bits;
+    bool smem_ready(int bit) const { return smem_bits >> bit & 1u; }
+    void smem_set(int bit) const { smem_bits |= 1u << bit; }
     mutable uint64_t launches;  // kernels enqueued through this context
     // finch_step_host only: a second stream carries the chunk's V rows to the device while the scoring kernels,
     // which do not read them, already run; events tie it to the caller's stream on both sides
     cudaStream_t copy_stream;
     cudaEvent_t ev_entry, ev_v_ready, ev_selected;
 };
+
+enum { kSmemSelect = 0, kSmemFused = 1, kSmemTc = 3 };  // bits of smem_bits; kSmemFused + (d == 128), kSmemTc + variant
 
 inline TensorView view_of(const finch_tensor *t) {
     return TensorView{(const char *)t->ptr, t->stride_layer, t->stride_head, t->stride_tok};

@@ -359,8 +359,12 @@ cudaError_t launch_fused_d(const Ctx &ctx, const CUtensorMap &qb, const CUtensor
     p.stages = kMaxStages;
     while (p.stages > 2 && cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) > kSmemLimit) --p.stages;
     const int smem = cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false);
-    cudaError_t e = cudaFuncSetAttribute(score_fused_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (!ctx.smem_ready(kSmemFused + (D == 128))) {
+        e = cudaFuncSetAttribute(score_fused_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e != cudaSuccess) return e;
+        ctx.smem_set(kSmemFused + (D == 128));
+    }
     dim3 grid(n_ranges < sms ? n_ranges : sms);  // persistent and resident at once: phase B waits for neighbours
     e = launch_chained(score_fused_kernel<D>, grid, dim3(kTcThreads), smem, stream, qb, qs, cm, hm, p);
     ctx.launches += 1;
@@ -388,16 +392,20 @@ int score_fused_window(const Ctx &ctx, const BatchView &bv) {
     return choose_window((long long)mv.L * mv.Hkv, tiles, ctx.sm_count > 0 ? ctx.sm_count : 148, (mv.d / 64) * kSlabBytes);
 }
 
-// Float2 entries of scratch the fused kernel needs for this batch (0: the batch is not one it takes).
-size_t score_fused_scratch(const Ctx &ctx, const BatchView &bv) {
-    const ModelView &mv = ctx.model;
-    const int W = score_fused_window(ctx, bv);
-    if (W == 0) return 0;
+namespace {
+size_t scratch_of(const ModelView &mv, const BatchView &bv, int W) {
     const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
     const size_t units = (size_t)mv.L * mv.Hkv, cand = (size_t)bv.total_cache + bv.total_chunk;
     size_t n = units * (tiles / W) * kGroups * rows_alloc_of(mv, bv);  // partial row statistics
     if (mv.G != mv.Hkv) n += (units * cand + 1) / 2;  // per-KV-head sums of a selection group that spans several
     return n;
+}
+}  // namespace
+
+// Float2 entries of scratch the fused kernel needs for this batch (0: the batch is not one it takes).
+size_t score_fused_scratch(const Ctx &ctx, const BatchView &bv) {
+    const int W = score_fused_window(ctx, bv);
+    return W ? scratch_of(ctx.model, bv, W) : 0;
 }
 
 // Returns cudaErrorNotSupported (and launches nothing) when the batch is not one the fused kernel takes, the
@@ -405,8 +413,8 @@ size_t score_fused_scratch(const Ctx &ctx, const BatchView &bv) {
 cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const TensorView &cache_k, const TensorView &chunk_k,
                                const BatchView &bv, float *scores, float2 *scratch, size_t scratch_capacity,
                                float *row_lse, cudaStream_t stream) {
-    const size_t need = score_fused_scratch(ctx, bv);
-    if (need == 0 || scratch_capacity < need) return cudaErrorNotSupported;
+    const int W = score_fused_window(ctx, bv);
+    if (W == 0 || scratch_capacity < scratch_of(ctx.model, bv, W)) return cudaErrorNotSupported;
     ModelView mv = ctx.model;  // the scoring view: a query head only ever meets its own KV head's keys
     mv.G = mv.Hkv;
     mv.hpg = mv.g;
@@ -424,8 +432,7 @@ cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const Tensor
     FusedParams p{};
     p.mv = mv;
     p.bv = bv;
-    p.W = score_fused_window(ctx, bv);
-    if (p.W == 0) return cudaErrorNotSupported;
+    p.W = W;
     p.n_seg = tiles / p.W;
     p.rows_alloc = rows_alloc_of(mv, bv);
     p.partial = scratch;

@@ -395,10 +395,15 @@ cudaError_t launch_d(const Ctx &ctx, const CUtensorMap &qb, const CUtensorMap &q
     p.stages = kMaxStages;
     while (p.stages > 2 && cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, MASK) > kSmemLimit) --p.stages;
     const int smem = cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, MASK);
-    cudaError_t e = cudaFuncSetAttribute(score_tc_kernel<kLse, D, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(score_tc_kernel<kColsum, D, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    const int bit = kSmemTc + (D == 128) * 2 + MASK;
+    if (!ctx.smem_ready(bit)) {
+        e = cudaFuncSetAttribute(score_tc_kernel<kLse, D, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(score_tc_kernel<kColsum, D, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e != cudaSuccess) return e;
+        ctx.smem_set(bit);
+    }
     p.n_items = p.splits * mv.L * mv.G * bv.batch;
     const int sms = ctx.sm_count > 0 ? ctx.sm_count : 148;
     dim3 grid(p.n_items < sms ? p.n_items : sms);  // persistent: one CTA per SM walks a contiguous range of items

@@ -1,16 +1,25 @@
-// Top-r selection per (layer, selection group, request) without a sort.
+// Top-r selection per (layer, selection group, request) without a sort, one CTA per unit.
 //
-// One CTA per unit.  Scores are mapped to order-preserving 32-bit keys; four 8-bit radix passes (most significant
-// digit first) locate the key T of the r-th largest score and how many candidates are strictly above it.  A final
-// ordered sweep keeps every candidate above T plus the lowest-indexed candidates equal to T until r are kept, and
-// writes the kept indices in increasing order (two block-wide prefix sums per 4096 candidates).
+// Scores are mapped to order-preserving 32-bit keys; the key T of the r-th largest score and the number of candidates
+// strictly above it are found by counting, then an ordered sweep keeps every candidate above T plus the lowest-indexed
+// candidates equal to T until r are kept, and writes the kept indices in increasing order.
+//
+//   select_kernel       units of at most 8192 candidates: keys in registers, a thread owns 4 or 8 consecutive candidates.
+//                       The count runs over 1024 bins between the unit's smallest and largest key, so that scores of a
+//                       narrow range still spread (8-bit digits of the whole key put most of them into one or two bins,
+//                       whose atomics serialise); the few keys of the r-th one's bin are ranked directly.  Seven
+//                       barriers in place of twenty.
+//   select_long_kernel  longer units: four 8-bit radix passes over keys in shared memory, beyond 40960 in global memory.
 #include "finch_internal.cuh"
 
 namespace finch {
 namespace {
 
-constexpr int kSelThreadsWide = 1024;  // units of more than 1024 candidates: two CTAs per SM
-constexpr int kSelThreadsSmall = 256;  // short units: eight CTAs per SM, so that many small units run in one wave
+constexpr int kLongThreads = 1024;
+constexpr int kLongKeys = 40960;  // keys in shared memory
+constexpr int kMaxShort = 8192;  // candidates per unit of select_kernel: 1024 threads x 8
+constexpr int kBins = 1024;
+constexpr int kListed = 128;  // keys of one bin that are ranked directly
 
 // Order-preserving key: larger score <=> larger key.  -0 is folded into +0; NaN gets key 0, below every number.
 __device__ __forceinline__ uint32_t order_key(float s) {
@@ -20,19 +29,14 @@ __device__ __forceinline__ uint32_t order_key(float s) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// 32 registers per thread, so 2048 threads per SM whatever the CTA size: two CTAs of 1024 threads (256 units of 4096
-// candidates run in one wave) or eight of 256 (1024 units of 1024 candidates do)
-template <int kSelThreads>
-__global__ void __launch_bounds__(kSelThreads, 2048 / kSelThreads)
-select_kernel(ModelView mv, BatchView bv, const float *scores, int *kept_idx, int *out_len, int smem_keys, int *status) {
-    constexpr int kSelWarps = kSelThreads / 32;
-    extern __shared__ uint32_t key_cache[];  // the first min(N, smem_keys) keys
-    __shared__ int hist[256];
-    __shared__ int warp_tot[2][kSelWarps];
-    __shared__ int sel_digit, sel_above;
-
-    dependency_wait();
-    dependents_may_launch();
+// What every unit starts with: its scores and output, how many to keep; false when there is nothing (more) to do.
+struct SelectUnit {
+    const float *scores;
+    int *kept;
+    int N, r;
+};
+__device__ __forceinline__ bool select_unit(const ModelView &mv, const BatchView &bv, const float *scores, int *kept_idx,
+                                            int *out_len, int *status, SelectUnit &s) {
     const int unit = blockIdx.x;
     const UnitInfo u = unit_info(mv, bv, unit, blockIdx.y);
     const int N = u.N;
@@ -44,19 +48,168 @@ select_kernel(ModelView mv, BatchView bv, const float *scores, int *kept_idx, in
             atomicOr(status, FINCH_DEV_BAD_BATCH);
             if (unit == 0) out_len[u.b] = 0;
         }
-        return;
+        return false;
     }
     if (unit == 0 && threadIdx.x == 0) out_len[u.b] = r;
-    if (r == 0) return;
+    s.scores = scores + ((int64_t)u.l * mv.G + u.G) * ((int64_t)bv.total_cache + bv.total_chunk) + u.cache0 + u.chunk0;
+    s.kept = kept_idx + ((int64_t)u.l * mv.G + u.G) * bv.total_cache + u.cache0;
+    s.N = N;
+    s.r = r;
+    if (r == N)  // a budget at or above the candidate count keeps everything, in order
+        for (int j = threadIdx.x; j < N; j += blockDim.x) s.kept[j] = j;
+    return r > 0 && r < N;
+}
 
-    const float *sc = scores + ((int64_t)u.l * mv.G + u.G) * ((int64_t)bv.total_cache + bv.total_chunk) + u.cache0 +
-                      u.chunk0;
-    int *kept = kept_idx + ((int64_t)u.l * mv.G + u.G) * bv.total_cache + u.cache0;
+// The launcher gives N <= blockDim.x * kItems for every unit.
+template <int kItems>
+__global__ void __launch_bounds__(1024)
+select_kernel(ModelView mv, BatchView bv, const float *scores, int *kept_idx, int *out_len, int *status) {
+    __shared__ __align__(16) int hist[kBins];
+    __shared__ uint32_t warp_a[32], warp_b[32], listed[kListed];
+    __shared__ int n_listed, sel_bin, sel_above, sel_count, sel_ties;
+    __shared__ uint32_t sel_key;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
 
-    if (r == N) {  // a budget at or above the candidate count keeps everything, in order
-        for (int j = threadIdx.x; j < N; j += kSelThreads) kept[j] = j;
-        return;
+    dependency_wait();
+    dependents_may_launch();
+    SelectUnit s;
+    if (!select_unit(mv, bv, scores, kept_idx, out_len, status, s)) return;
+
+    const int j0 = threadIdx.x * kItems, mine = max(0, min(kItems, s.N - j0));  // this thread's candidates
+    uint32_t key[kItems], lo = 0xffffffffu, hi = 0;
+#pragma unroll
+    for (int e = 0; e < kItems; ++e) key[e] = e < mine ? __float_as_uint(s.scores[j0 + e]) : 0u;
+#pragma unroll
+    for (int e = 0; e < kItems; ++e) {
+        key[e] = order_key(__uint_as_float(key[e]));
+        if (e < mine) {
+            lo = min(lo, key[e]);
+            hi = max(hi, key[e]);
+        }
     }
+    for (int i = threadIdx.x; i < kBins; i += blockDim.x) hist[i] = 0;
+    if (threadIdx.x == 0) n_listed = 0;
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+        warp_a[warp] = lo;
+        warp_b[warp] = hi;
+    }
+    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lane < n_warps ? warp_a[lane] : 0xffffffffu);
+    hi = __reduce_max_sync(0xffffffffu, lane < n_warps ? warp_b[lane] : 0u);
+
+    // ---- the remaining-th largest of the keys in [lo, hi]; every round shrinks the range a thousandfold
+    int remaining = s.r;
+    uint32_t T;
+    for (;;) {
+        const uint32_t range = hi - lo;
+        const int shift = max(0, 22 - __clz(range));  // range >> shift < 1024
+#pragma unroll
+        for (int e = 0; e < kItems; ++e)
+            if (e < mine && key[e] - lo <= range) atomicAdd(&hist[(key[e] - lo) >> shift], 1);
+        __syncthreads();
+        // thread i owns a run of bins, the largest keys first; find the bin in which the running count reaches `remaining`
+        const int per = (kBins + blockDim.x - 1) / blockDim.x, top = kBins - 1 - threadIdx.x * per;
+        int count = 0;
+        for (int i = 0; i < per; ++i)
+            if (top - i >= 0) count += hist[top - i];
+        int incl = count;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += v;
+        }
+        if (lane == 31) warp_a[warp] = incl;
+        __syncthreads();
+        const uint32_t before = lane < warp ? warp_a[lane] : 0u;
+        int above = (int)__reduce_add_sync(0xffffffffu, before) + incl - count;
+        if (above < remaining && remaining <= above + count) {
+            for (int i = 0; i < per; ++i) {
+                const int c = hist[top - i];
+                if (remaining <= above + c) {
+                    sel_bin = top - i;
+                    sel_above = above;
+                    sel_count = c;
+                    break;
+                }
+                above += c;
+            }
+        }
+        __syncthreads();
+        remaining -= sel_above;
+        lo += (uint32_t)sel_bin << shift;
+        hi = lo + min(hi - lo, (1u << shift) - 1u);
+        T = lo;
+        if (shift == 0) break;  // a bin is a single key
+        if (sel_count <= kListed) {
+#pragma unroll
+            for (int e = 0; e < kItems; ++e)
+                if (e < mine && key[e] - lo <= hi - lo) listed[atomicAdd(&n_listed, 1)] = key[e];
+            __syncthreads();
+            for (int i = threadIdx.x; i < sel_count; i += blockDim.x) {
+                const uint32_t k = listed[i];
+                int gt = 0, ge = 0;
+                for (int q = 0; q < sel_count; ++q) {
+                    gt += listed[q] > k;
+                    ge += listed[q] >= k;
+                }
+                if (gt < remaining && remaining <= ge) {  // equal keys write the same values
+                    sel_key = k;
+                    sel_ties = remaining - gt;
+                }
+            }
+            __syncthreads();
+            T = sel_key;
+            remaining = sel_ties;
+            break;
+        }
+        for (int i = threadIdx.x; i < kBins; i += blockDim.x) hist[i] = 0;
+        __syncthreads();
+    }
+    const int ties_to_keep = remaining;  // >= 1
+
+    // ---- ordered sweep: keep key > T, and the first `ties_to_keep` keys == T.  One block-wide scan of (above, equal).
+    uint32_t n = 0;
+#pragma unroll
+    for (int e = 0; e < kItems; ++e)
+        if (e < mine) n += key[e] > T ? 0x10000u : (key[e] == T ? 1u : 0u);
+    uint32_t incl = n;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
+    }
+    if (lane == 31) warp_b[warp] = incl;
+    __syncthreads();
+    const uint32_t at = __reduce_add_sync(0xffffffffu, lane < warp ? warp_b[lane] : 0u) + incl - n;
+    int gt = at >> 16, eq = at & 0xffffu;
+#pragma unroll
+    for (int e = 0; e < kItems; ++e) {
+        if (e >= mine) continue;
+        if (key[e] > T || (key[e] == T && eq < ties_to_keep)) s.kept[gt + min(eq, ties_to_keep)] = j0 + e;
+        gt += key[e] > T;
+        eq += key[e] == T;
+    }
+}
+
+// 32 registers per thread: two CTAs of 1024 threads per SM
+__global__ void __launch_bounds__(kLongThreads, 2)
+select_long_kernel(ModelView mv, BatchView bv, const float *scores, int *kept_idx, int *out_len, int smem_keys, int *status) {
+    constexpr int kSelThreads = kLongThreads;
+    constexpr int kSelWarps = kSelThreads / 32;
+    extern __shared__ uint32_t key_cache[];  // the first min(N, smem_keys) keys
+    __shared__ int hist[256];
+    __shared__ int warp_tot[2][kSelWarps];
+    __shared__ int sel_digit, sel_above;
+
+    dependency_wait();
+    dependents_may_launch();
+    SelectUnit s;
+    if (!select_unit(mv, bv, scores, kept_idx, out_len, status, s)) return;
+    const float *sc = s.scores;
+    int *kept = s.kept;
+    const int N = s.N, r = s.r;
 
     const int n_cached = N < smem_keys ? N : smem_keys;
     for (int j = threadIdx.x; j < n_cached; j += kSelThreads) key_cache[j] = order_key(sc[j]);
@@ -136,28 +289,6 @@ select_kernel(ModelView mv, BatchView bv, const float *scores, int *kept_idx, in
         total = buf[kSelWarps - 1];
         return (warp ? buf[warp - 1] : 0) + incl - v;
     };
-    if (N <= kSelThreads) {
-        // one candidate per thread at most: ballots and the 32 warp totals are cheaper than two scans
-        const int j = threadIdx.x;
-        const uint32_t k = j < N ? key_at(j) : 0u;
-        const bool gt = j < N && k > T;
-        const bool eq = j < N && k == T;
-        const uint32_t eq_ballot = __ballot_sync(0xffffffffu, eq);
-        if (lane == 0) warp_tot[0][warp] = __popc(eq_ballot);
-        __syncthreads();
-        int eq_before = 0;
-        for (int w = 0; w < warp; ++w) eq_before += warp_tot[0][w];
-        eq_before += __popc(eq_ballot & ((1u << lane) - 1u));
-        const bool keep = gt || (eq && eq_before < ties_to_keep);
-        const uint32_t keep_ballot = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) warp_tot[1][warp] = __popc(keep_ballot);
-        __syncthreads();
-        int keep_before = 0;
-        for (int w = 0; w < warp; ++w) keep_before += warp_tot[1][w];
-        keep_before += __popc(keep_ballot & ((1u << lane) - 1u));
-        if (keep) kept[keep_before] = j;
-        return;
-    }
     constexpr int kPerThread = 4;
     int base_eq = 0, base_keep = 0;
     for (int j0 = 0; j0 < N; j0 += kSelThreads * kPerThread) {
@@ -200,19 +331,23 @@ cudaError_t launch_select(const Ctx &ctx, const float *scores, const BatchView &
     const int units = mv.L * mv.G;
     if (units == 0 || bv.batch == 0) return cudaSuccess;
     const int max_n = bv.max_cache + bv.max_chunk;
-    int smem_keys = max_n < 40960 ? max_n : 40960;  // up to 160 KiB of keys on chip; longer inputs re-read global
-    if (smem_keys < 1) smem_keys = 1;
-    const size_t smem = (size_t)smem_keys * sizeof(uint32_t);
     dim3 grid(units, bv.batch);
     ctx.launches += 1;
-    if (max_n <= 1024)
-        return launch_chained(select_kernel<kSelThreadsSmall>, grid, dim3(kSelThreadsSmall), smem, stream, mv, bv, scores,
-                              (int *)kept_idx, out_len, smem_keys, ctx.d_status);
-    cudaError_t e =
-        cudaFuncSetAttribute(select_kernel<kSelThreadsWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_chained(select_kernel<kSelThreadsWide>, grid, dim3(kSelThreadsWide), smem, stream, mv, bv, scores,
-                          (int *)kept_idx, out_len, smem_keys, ctx.d_status);
+    if (max_n <= kMaxShort) {
+        // eight candidates per thread for long units (few barriers' worth of warps), four for short ones (latency)
+        const int items = max_n <= 2048 ? 4 : 8;
+        const int threads = max(64, ((max_n + items - 1) / items + 31) / 32 * 32);
+        return launch_chained(items == 4 ? select_kernel<4> : select_kernel<8>, grid, dim3(threads), 0, stream, mv, bv, scores,
+                              kept_idx, out_len, ctx.d_status);
+    }
+    const int smem_keys = max_n < kLongKeys ? max_n : kLongKeys;  // up to 160 KiB on chip; longer inputs re-read global
+    if (!ctx.smem_ready(kSmemSelect)) {
+        cudaError_t e = cudaFuncSetAttribute(select_long_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLongKeys * 4);
+        if (e != cudaSuccess) return e;
+        ctx.smem_set(kSmemSelect);
+    }
+    return launch_chained(select_long_kernel, grid, dim3(kLongThreads), (size_t)smem_keys * sizeof(uint32_t), stream, mv, bv,
+                          scores, kept_idx, out_len, smem_keys, ctx.d_status);
 }
 
 }  // namespace finch
