@@ -238,19 +238,14 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out) {
                 if (dev >= 0) (void)cudaSetDevice(dev);
             }
         } restore{caller_device == cfg->device ? -1 : caller_device};
-        if (cudaSetDevice(cfg->device) != cudaSuccess || cudaMalloc(&ctx->d_status, sizeof(int)) != cudaSuccess) {
+        const size_t device_bytes = (1 + 2 * (size_t)mv.L * mv.Hkv) * sizeof(int);  // status word, scoring counters
+        if (cudaSetDevice(cfg->device) != cudaSuccess || cudaMalloc(&ctx->d_status, device_bytes) != cudaSuccess) {
             (void)cudaGetLastError();
             delete ctx;
             return FINCH_ERR_OOM;
         }
-        const size_t ticket_bytes = 2 * (size_t)mv.L * mv.Hkv * sizeof(int);
-        if (cudaMalloc(&ctx->tickets, ticket_bytes) != cudaSuccess) {
-            (void)cudaGetLastError();
-            finch_ctx_destroy(ctx);
-            return FINCH_ERR_OOM;
-        }
-        if (cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess ||
-            cudaMemset(ctx->tickets, 0, ticket_bytes) != cudaSuccess ||
+        ctx->tickets = ctx->d_status + 1;
+        if (cudaMemset(ctx->d_status, 0, device_bytes) != cudaSuccess ||
             cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_entry, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_v_ready, cudaEventDisableTiming) != cudaSuccess ||
@@ -291,7 +286,6 @@ void finch_ctx_destroy(finch_ctx *ctx) {
     if (ctx->ev_selected) cudaEventDestroy(ctx->ev_selected);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->model.rope_table) cudaFree(const_cast<float2 *>(ctx->model.rope_table));
-    if (ctx->tickets) cudaFree(ctx->tickets);
     if (ctx->d_status) cudaFree(ctx->d_status);
     delete ctx;
 }

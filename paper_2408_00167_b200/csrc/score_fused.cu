@@ -5,8 +5,8 @@
 // column sum can be formed -- but here the second visit follows the first closely enough that the keys come back
 // from L2 instead of HBM, and nothing but a few bytes per prompt row leaves the SM in between:
 //
-//   * The key tiles of all units form one sequence (unit-major).  It is cut into ranges of W tiles, W a divisor of the
-//     unit's tile count; CTA i of the persistent grid takes ranges i, i + P, i + 2P, ... (one "window" each), so the
+//   * The key tiles of all units form one sequence (unit-major).  It is cut into ranges of W tiles, the last
+//     of a unit possibly shorter; CTA i of the persistent grid takes ranges i, i + P, i + 2P, ... (one "window" each), so the
 //     CTAs of a window work on neighbouring tiles and the keys in flight between the two sweeps of a window are P x W
 //     tiles (tens of MB).
 //   * Phase A of a window: D = Qtile x Ktile^T (one prompt row per TMEM lane), every softmax thread keeps the
@@ -111,29 +111,86 @@ struct Walk {
     }
 };
 
-// The statistics of one row, merged over the unit's ranges and the parts of each range, in a fixed order.
-__device__ __forceinline__ float2 merge_row(const FusedParams &p, const UnitInfo &u, const Rows &R, int n_seg, int unit, int row,
-                                            bool write_lse) {
+// (M, Z) of a row -> what the second sweep needs, and the row's log-sum-exp where it is asked for.
+__device__ __forceinline__ float2 finish_row(const FusedParams &p, const UnitInfo &u, const Rows &R, int row, float M, float Z,
+                                             bool write_lse) {
     if (!row_live(R, row)) return make_float2(0.f, 0.f);
-    const Parts parts(R, row / kRows);
-    const float2 *src = p.partial + (int64_t)unit * p.n_seg * kGroups * p.rows_alloc + row;
-    const int n = parts.count(n_seg);
-    float M = -INFINITY, Z = 0.f;
-#pragma unroll 1
-    for (int i0 = 0; i0 < n; i0 += 8) {  // eight loads in flight, folded in order
-        float2 part[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            part[i] = i0 + i < n ? __ldcg(src + parts.at(i0 + i, p.rows_alloc)) : make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) merge_part(part[i], M, Z);
-    }
     const int64_t at = ((int64_t)u.l * p.mv.Hq + u.G * p.mv.hpg + row / R.rp) * p.bv.total_q + u.q0 + row % R.rp;
     if (p.bv.self_lse) merge_self_term(p.bv.self_lse[at], M, Z);
     float lse_nat;
     const float2 out = merged_pair(M, Z, lse_nat);
     if (write_lse && p.row_lse) p.row_lse[at] = lse_nat;
     return out;
+}
+
+// The statistics of a unit, merged over its ranges and the parts of each range in a fixed order and staged, by one warp:
+// four rows and four parts of each per lane in flight.
+__device__ __forceinline__ void merge_by_warp(const FusedParams &p, const UnitInfo &u, const Rows &R, int n_seg, int unit,
+                                              bool write_lse, float2 *stats, int lane) {
+    const float2 *src = p.partial + (int64_t)unit * p.n_seg * kGroups * p.rows_alloc;
+    for (int qb = 0; qb < R.n_qt; ++qb) {
+        const Parts parts(R, qb);
+        const int n = parts.count(n_seg), row0 = qb * kRows + lane;
+        bool live[4];
+        float M[4], Z[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            live[k] = row_live(R, row0 + k * 32);
+            M[k] = -INFINITY;
+            Z[k] = 0.f;
+        }
+#pragma unroll 1
+        for (int i0 = 0; i0 < n; i0 += 4) {
+            float2 part[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 *at = src + parts.at(i0 + i, p.rows_alloc) + row0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    part[k][i] = i0 + i < n && live[k] ? __ldcg(at + k * 32) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) merge_parts(part[k], M[k], Z[k]);
+        }
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            const int row = row0 + k * 32;
+            if (row < R.rows) stage_row(stats, row, finish_row(p, u, R, row, M[0], Z[0], write_lse));
+            M[0] = M[1], M[1] = M[2], M[2] = M[3];
+            Z[0] = Z[1], Z[1] = Z[2], Z[2] = Z[3];
+        }
+    }
+}
+
+// The same by all softmax threads: a row per thread, or, for few rows, per 2 to 16 neighbouring lanes that take every
+// second to sixteenth part each (many short ranges leave hundreds of parts to a row).
+__device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInfo &u, const Rows &R, int n_seg, int unit,
+                                             bool write_lse, float2 *stats, int tid) {
+    const float2 *src = p.partial + (int64_t)unit * p.n_seg * kGroups * p.rows_alloc;
+    int log_s = 0;  // lanes per row
+    while (log_s < 4 && R.rows << (log_s + 1) <= kSoftmaxWarps * 32) ++log_s;
+    const int row = tid >> log_s, sub = tid & ((1 << log_s) - 1);
+    const bool live = row_live(R, row);
+    const Parts parts(R, live ? row / kRows : 0);
+    const int n = live ? parts.count(n_seg) : 0;
+    float M = -INFINITY, Z = 0.f;
+#pragma unroll 1
+    for (int i0 = sub; i0 < n; i0 += 8 << log_s) {
+        float2 part[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = i0 + (i << log_s);
+            part[i] = k < n ? __ldcg(src + parts.at(k, p.rows_alloc) + row) : make_float2(0.f, 0.f);
+        }
+        merge_parts(part, M, Z);
+    }
+    for (int d = 1; d < 1 << log_s; d <<= 1) {  // both partners get the same bits
+        const float om = __shfl_xor_sync(0xffffffffu, M, d), oz = __shfl_xor_sync(0xffffffffu, Z, d);
+        const float nm = fmaxf(M, om);
+        if (nm != -INFINITY) Z = Z * ex2(M - nm) + oz * ex2(om - nm);
+        M = nm;
+    }
+    if (sub == 0 && row < R.rows) stage_row(stats, row, finish_row(p, u, R, row, M, Z, write_lse));
 }
 
 template <int D>
@@ -228,8 +285,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
                     }
                 }
                 if (!__shfl_sync(0xffffffffu, good, 0)) break;
-                float2 *stats = c.stats + ((segs - 1) & 1) * p.rows_alloc;
-                for (int r = lane; r < R.rows; r += 32) stage_row(stats, r, merge_row(p, u, R, n_seg, sg.unit, r, sg.slot == 0));
+                merge_by_warp(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats + ((segs - 1) & 1) * p.rows_alloc, lane);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&c.stats_ready[(segs - 1) & 1]);
             }
@@ -276,7 +332,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
                 }
                 if (!(ok = __shfl_sync(0xffffffffu, good, 0))) break;
                 FINCH_UNIT(sg);
-                if (tid < R.rows) stage_row(c.stats, tid, merge_row(p, u, R, n_seg, sg.unit, tid, sg.slot == 0));
+                merge_by_cta(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats, tid);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&c.stats_ready[1]);
                 if (!(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[1], 0, c.abort_flag)))) break;
@@ -313,32 +369,50 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
     scores[((int64_t)l * out_groups + og) * cand + at] = s;
 }
 
-// Key tiles per range, or 0 when the one-kernel path should leave the batch to the two-launch kernels.  A range divides
-// the unit's tiles (otherwise ranges straddle units: the query tiles change inside a range and a unit's tiles are dealt
-// unevenly).  Of the divisors the one whose slowest CTA has least to do: windows x (W + 1), a window's fixed costs
-// (query loads, the exchange of the row statistics) being about one tile's work.  Several windows want at least two
-// tiles each (a window of one is all hand-over), CTA x window slots at least 85 % full (else the two-launch kernels,
-// whose key splits are chosen per launch, waste less), and keys in flight between a window's sweeps that stay in L2.
-int choose_window(long long units, int tiles_per_unit, int ctas, int tile_bytes) {
-    const long long total = units * tiles_per_unit;
-    const long long l2_budget = 48ll << 20;
+// Key tiles per range, or 0 when the one-kernel path should leave the batch to the two-launch kernels.
+//
+// One range per CTA (units x ranges fit the SMs): the range length with the smallest W x accumulators per key tile + the
+// exchange of the row statistics, which grows with the parts to be merged; any length, the unit's last range may be
+// shorter.
+// Several ranges ("windows") per CTA: a divisor of the unit's tile count of at least 4 tiles (or the whole unit) and at
+// most 8 ranges per unit -- shorter windows are all hand-over (2 tiles: 40 units x 32 tiles 0.24 ms against 0.1 on two
+// launches) --, failing that any length from 6; CTA x window slots at least 85 % full (else the two-launch kernels,
+// whose ranges are cut per CTA, waste less); keys in flight between a window's sweeps that stay in L2.  Of those the one
+// whose slowest CTA has least to do, a window's fixed costs being about one tile's work.
+int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
+    const int accs = (rows + kRows - 1) / kRows;
     int best = 0;
     long long best_cost = LLONG_MAX;
-    for (int W = 1; W <= tiles_per_unit; ++W) {
-        if (tiles_per_unit % W || tiles_per_unit / W > kMaxSegs) continue;
-        const long long ranges = total / W, windows = (ranges + ctas - 1) / ctas;
-        if (windows > 1) {
-            if (W < 2 && tiles_per_unit > 1) continue;
-            if (W > 1 && (long long)W * ctas * tile_bytes > l2_budget && best) break;
-            if ((double)ranges / (double)(windows * ctas) < 0.85) continue;
-        }
-        const long long cost = windows * (W + 1);
+    for (int n = 1; n <= T && n <= kMaxSegs && units * n <= ctas; ++n) {
+        const int W = (T + n - 1) / n, n_seg = (T + W - 1) / W;
+        const long long cost = (long long)W * accs * 4 + 12 + n_seg / 4;
         if (cost < best_cost) {
             best_cost = cost;
             best = W;
         }
     }
-    return best;
+    // a single window that leaves more than a third of the SMs idle competes with several
+    if (best && units * ((T + best - 1) / best) * 3 >= (long long)ctas * 2) return best;
+    const long long l2_budget = 48ll << 20;
+    const int single = best;
+    const long long single_cost = best ? (long long)best * 10 + 30 : LLONG_MAX;
+    best = 0;
+    best_cost = LLONG_MAX;
+    for (int pass = 0; pass < 2 && !best; ++pass)
+        for (int W = pass ? 6 : 1; W <= T; ++W) {
+            const int n_seg = (T + W - 1) / W;
+            if (pass == 0 && T % W) continue;
+            if ((W < 4 && W < T) || n_seg > 8) continue;
+            if (W > 1 && (long long)W * ctas * tile_bytes > l2_budget && (best || pass)) break;
+            const long long ranges = units * n_seg, windows = (ranges + ctas - 1) / ctas;
+            if (windows < 2 || (double)units * T / (double)(windows * W * ctas) < 0.85) continue;
+            const long long cost = windows * (W + 1);
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = W;
+            }
+        }
+    return best && best_cost * 10 < single_cost ? best : (single ? single : best);
 }
 
 int rows_alloc_of(const ModelView &mv, const BatchView &bv) {  // resident query rows: whole tiles
@@ -389,14 +463,15 @@ int score_fused_window(const Ctx &ctx, const BatchView &bv) {
         return 0;
     if (padded_rows(bv.max_q, mv.g) > kMaxRows) return 0;
     const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
-    return choose_window((long long)mv.L * mv.Hkv, tiles, ctx.sm_count > 0 ? ctx.sm_count : 148, (mv.d / 64) * kSlabBytes);
+    return choose_window((long long)mv.L * mv.Hkv, tiles, ctx.sm_count > 0 ? ctx.sm_count : 148, (mv.d / 64) * kSlabBytes,
+                         padded_rows(bv.max_q, mv.g));
 }
 
 namespace {
 size_t scratch_of(const ModelView &mv, const BatchView &bv, int W) {
     const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
     const size_t units = (size_t)mv.L * mv.Hkv, cand = (size_t)bv.total_cache + bv.total_chunk;
-    size_t n = units * (tiles / W) * kGroups * rows_alloc_of(mv, bv);  // partial row statistics
+    size_t n = units * ((tiles + W - 1) / W) * kGroups * rows_alloc_of(mv, bv);  // partial row statistics
     if (mv.G != mv.Hkv) n += (units * cand + 1) / 2;  // per-KV-head sums of a selection group that spans several
     return n;
 }
@@ -433,7 +508,7 @@ cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const Tensor
     p.mv = mv;
     p.bv = bv;
     p.W = W;
-    p.n_seg = tiles / p.W;
+    p.n_seg = (tiles + p.W - 1) / p.W;
     p.rows_alloc = rows_alloc_of(mv, bv);
     p.partial = scratch;
     p.tickets = ctx.tickets;

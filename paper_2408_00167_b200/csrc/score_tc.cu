@@ -353,8 +353,7 @@ merge_stats_kernel(TcParams p) {
         float2 part[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) part[i] = i0 + i < n ? src[parts.at(i0 + i, p.slots)] : make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) merge_part(part[i], M, Z);
+        merge_parts(part, M, Z);
     }
     if (bv.self_lse) merge_self_term(bv.self_lse[row], M, Z);  // the keys the row attends to besides the candidates
     float lse_nat;

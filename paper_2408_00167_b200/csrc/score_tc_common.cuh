@@ -271,15 +271,27 @@ __device__ __forceinline__ void colsum_chunk(const uint32_t (&r)[NC], float scal
 // logit units; parts are folded in a fixed order into a running (M, Z), then turned into the pair the column
 // sweep uses: weights are exp2(s2 - R) * w with R = M + floor(log2 Z) and w = 2^floor(log2 Z) / Z in (1/2, 1], so
 // the exponent never exceeds a few units whatever reference the parts were summed against.
-__device__ __forceinline__ void merge_part(float2 pm, float &M, float &Z) {
-    if (!(pm.y > 0.f)) return;  // a part that saw none of this row's logits
+__device__ __forceinline__ float2 normal_part(float2 pm) {
     // A part's sum can be as large as 2^127 against a reference that far below its largest logit: move the sum's
-    // exponent into the reference first, so that neither factor below leaves the fp32 range.
-    const int bits = __float_as_int(pm.y);  // pm.y >= 1: a normal number
-    const int e = ((bits >> 23) & 0xff) - 127;
-    const float px = pm.x + (float)e, py = __int_as_float((bits & 0x007fffff) | 0x3f800000);
-    const float nm = fmaxf(M, px);
-    Z = Z * ex2(M - nm) + py * ex2(px - nm);
+    // exponent into the reference, so that no factor below leaves the fp32 range.  A part that saw none of the row's
+    // logits (sum 0; any other sum is at least 1, a normal number) becomes (-inf, 0).
+    const int bits = __float_as_int(pm.y);
+    if (!(pm.y > 0.f)) return make_float2(-INFINITY, 0.f);
+    return make_float2(pm.x + (float)(((bits >> 23) & 0xff) - 127), __int_as_float((bits & 0x007fffff) | 0x3f800000));
+}
+template <int N>
+__device__ __forceinline__ void merge_parts(const float2 (&raw)[N], float &M, float &Z) {
+    float2 part[N];
+    float nm = M;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        part[i] = normal_part(raw[i]);
+        nm = fmaxf(nm, part[i].x);
+    }
+    if (nm == -INFINITY) return;
+    Z *= ex2(M - nm);
+#pragma unroll
+    for (int i = 0; i < N; ++i) Z += part[i].y * ex2(part[i].x - nm);
     M = nm;
 }
 // One more part with sum 1 whose reference is a natural-log value (the keys a row attends to besides the candidates).
