@@ -8,12 +8,11 @@
 //                scheduler holds one warp of each group, so three of them compute while one waits for its refill.
 //   SumWriter    one warp: adds the row blocks' column sums of a key (second sweep) and writes the scores.
 //
-// What bounds it: two exponentials per logit.  On the special-function unit alone that is 1024 clocks per 128 x 128
-// logits and sweep; a quarter of the pairs goes to the FMA pipe instead.  Measured on the loops alone (accumulators
-// refilled by MMAs, no loads): 970 clocks per accumulator in the first sweep and 1060 in the second, against 1150 and
-// 1210 without the polynomial.  Bookkeeping counts: every instruction between two accumulators is paid by sixteen
-// warps, so what can be is worked out per segment, ragged ends and overflow repairs leave for a path out of line, and
-// barriers are addressed by their shared-memory address.
+// What bounds it: two exponentials per logit, 1024 clocks of the special-function unit per 128 x 128 logits and sweep,
+// and the chip's power limit (large calls run at 1.70 to 1.85 GHz).  Measured on the loops alone (accumulators refilled by
+// MMAs, no loads): 1150 clocks per accumulator in the first sweep and 1210 in the second.  Bookkeeping counts: every
+// instruction between two accumulators is paid by sixteen warps, so what can be is worked out per segment, ragged ends
+// and overflow repairs leave for a path out of line, and barriers are addressed by their shared-memory address.
 #pragma once
 
 #include "score_tc_common.cuh"

@@ -119,45 +119,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     return r;
 }
 
-// exp2 of a pair on the FMA pipe: x = n + f with n = round(x), |f| <= 1/2, 2^f by a polynomial, n into the exponent field.
-// The special-function unit turns out 4 results per clock and scheduler, a quarter of the FMA rate, and both sweeps
-// are bound by it: one pair in kPolyEvery goes this way and the units run side by side.  The coefficients are the
-// minimax fit in relative error of 2^f on [-1/2, 1/2] with constant term 1 (Remez exchange): error 7.9e-8 at degree 5,
-// below ex2.approx's own 2 ulp.  x is clamped to [-127, 128]: below, the result is 0 (p = 1 exactly, exponent field
-// 127 - 127); at 128 and above it is inf or NaN, which the caller's overflow test catches.
-#ifndef FINCH_POLY_EVERY
-#define FINCH_POLY_EVERY 8
-#endif
-constexpr int kPolyEvery = FINCH_POLY_EVERY;  // 0: never
-template <bool kUpper>
-__device__ __forceinline__ uint64_t exp2_poly2(uint64_t x2) {
-    float x0, x1;
-    unpack2(x2, x0, x1);
-    x0 = fmaxf(x0, -127.f);
-    x1 = fmaxf(x1, -127.f);
-    if (kUpper) {
-        x0 = fminf(x0, 128.f);
-        x1 = fminf(x1, 128.f);
-    }
-    constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: adding it leaves round(x) in the low mantissa bits
-    const uint64_t x = pack2(x0, x1);
-    const uint64_t t = add2(x, pack2(kMagic, kMagic));
-    const uint64_t n = add2(t, pack2(-kMagic, -kMagic));
-    const uint64_t f = fma2(n, pack2(-1.f, -1.f), x);
-    uint64_t p = fma2(f, pack2(0x1.5a907ep-10f, 0x1.5a907ep-10f), pack2(0x1.3cf310p-7f, 0x1.3cf310p-7f));
-    p = fma2(p, f, pack2(0x1.c6bb2cp-5f, 0x1.c6bb2cp-5f));
-    p = fma2(p, f, pack2(0x1.ebf9a0p-3f, 0x1.ebf9a0p-3f));
-    p = fma2(p, f, pack2(0x1.62e424p-1f, 0x1.62e424p-1f));
-    p = fma2(p, f, pack2(1.f, 1.f));
-    float p0, p1, t0, t1;
-    unpack2(p, p0, p1);
-    unpack2(t, t0, t1);
-    return pack2(__int_as_float(__float_as_int(p0) + (__float_as_int(t0) << 23)),
-                 __int_as_float(__float_as_int(p1) + (__float_as_int(t1) << 23)));
-}
-template <bool kUpper>
-__device__ __forceinline__ uint64_t exp2_pair(uint64_t x2, int pair) {
-    if (kPolyEvery && pair % (kPolyEvery ? kPolyEvery : 1) == kPolyEvery - 1) return exp2_poly2<kUpper>(x2);
+// exp2 of a pair.  (A degree-5 polynomial on the FMA pipe for an eighth to a third of the pairs makes the loops alone 8
+// to 15 % shorter, but these kernels run into the chip's power limit, and at 1000 W the SM clock gives back more than
+// that: 32 layers x 8 heads x 4096 candidates x 512 rows, whole step, 0.452 ms without, 0.453 with an eighth, 0.465 with
+// a quarter.)
+__device__ __forceinline__ uint64_t exp2_pair(uint64_t x2) {
     float x0, x1;
     unpack2(x2, x0, x1);
     return pack2(ex2(x0), ex2(x1));
@@ -194,8 +160,8 @@ __device__ __forceinline__ void lse_sum(const uint32_t (&r)[NC], float scale2, f
     const uint64_t s2 = pack2(scale2, scale2), n2 = pack2(negm, negm);
 #pragma unroll
     for (int e = 0; e < NC; e += 4) {
-        acc0 = add2(acc0, exp2_pair<true>(fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), s2, n2), e / 2));
-        acc1 = add2(acc1, exp2_pair<true>(fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), s2, n2), e / 2 + 1));
+        acc0 = add2(acc0, exp2_pair(fma2(pack2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), s2, n2)));
+        acc1 = add2(acc1, exp2_pair(fma2(pack2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), s2, n2)));
     }
 }
 __device__ __forceinline__ float sum_of(uint64_t acc0, uint64_t acc1) {
@@ -262,7 +228,7 @@ __device__ __forceinline__ void colsum_chunk(const uint32_t (&r)[NC], float scal
             x1 = j < l2.y ? x1 : -INFINITY;
             x = pack2(x0, x1);
         }
-        acc = fma2(exp2_pair<false>(x, e / 2), pack2(s4.z, s4.w), acc);
+        acc = fma2(exp2_pair(x), pack2(s4.z, s4.w), acc);
     }
     unpack2(acc, c0, c1);
 }
