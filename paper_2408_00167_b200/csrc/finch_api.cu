@@ -221,14 +221,15 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out) {
     ctx->launches = 0;
     if (!ctx->dry) {
         int n_dev = 0;
-        cudaDeviceProp prop;
+        int major = 0, sms = 0;  // two attributes: the whole property struct takes milliseconds
         if (cudaGetDeviceCount(&n_dev) != cudaSuccess || cfg->device >= n_dev ||
-            cudaGetDeviceProperties(&prop, cfg->device) != cudaSuccess || prop.major != 10) {
+            cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg->device) != cudaSuccess || major != 10 ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess) {
             (void)cudaGetLastError();
             delete ctx;
             return FINCH_ERR_UNSUPPORTED;
         }
-        ctx->sm_count = prop.multiProcessorCount;
+        ctx->sm_count = sms;
         // the context's device is made current only while its resources are created; the caller's comes back after
         int caller_device = -1;
         if (cudaGetDevice(&caller_device) != cudaSuccess) caller_device = -1;
