@@ -173,10 +173,10 @@ finch_status finch_score(finch_ctx *ctx, const finch_tensor *prompt_q, const fin
  * arithmetic, nothing is enqueued, works on a validation-only context.  (The paper prescribes no kernel; this is how
  * its prompt x candidate block, Section "Method", is tiled here.)
  *  - FINCH_SCORE_ONE_KERNEL: bf16, head_dim 64 or 128, a single request without row_limit, at most 512 query rows
- *    per KV head (queries per KV head x prompt rows rounded up to 8), and a window length W for its key tiles exists:
- *    either every (layer, KV head) unit's ranges of W tiles get a CTA each, or the persistent grid takes several
- *    windows with W >= 4 (or the whole unit), at most 8 ranges per unit, the CTA x window slots >= 85 % full and
- *    W x SMs x tile bytes <= 48 MiB (unless no shorter window qualifies); divisors of the unit's tile count first.
+ *    per KV head (queries per KV head x prompt rows rounded up to 8), and a window length W for its key tiles that
+ *    is estimated to beat two launches: every (layer, KV head) unit's ranges of W tiles get a CTA each, or the
+ *    persistent grid takes several windows, W a divisor of the unit's tile count with W >= 4 (or the whole unit), at
+ *    most 8 ranges per unit and W x SMs x tile bytes <= 120 MiB.
  *    *window receives W (key tiles of 128 candidates).  Both sweeps of the softmax run in one persistent kernel.
  *  - FINCH_SCORE_TWO_LAUNCH: bf16, head_dim 64 or 128 otherwise (several requests, causal rows, longer prompts, no
  *    usable window): row statistics and column sums in two tensor-core launches.  *window = 0.

@@ -371,48 +371,41 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 
 // Key tiles per range, or 0 when the one-kernel path should leave the batch to the two-launch kernels.
 //
-// One range per CTA (units x ranges fit the SMs): the range length with the smallest W x accumulators per key tile + the
-// exchange of the row statistics, which grows with the parts to be merged; any length, the unit's last range may be
-// shorter.
-// Several ranges ("windows") per CTA: a divisor of the unit's tile count of at least 4 tiles (or the whole unit) and at
-// most 8 ranges per unit -- shorter windows are all hand-over (2 tiles: 40 units x 32 tiles 0.24 ms against 0.1 on two
-// launches) --, failing that any length from 6; CTA x window slots at least 85 % full (else the two-launch kernels,
-// whose ranges are cut per CTA, waste less); keys in flight between a window's sweeps that stay in L2.  Of those the one
-// whose slowest CTA has least to do, a window's fixed costs being about one tile's work.
+// The estimate is in units of one query tile against one key tile in both sweeps, 2500 SM clocks where the pipeline is full:
+//   one range per CTA        W x query tiles + 5 + the parts of a row to be merged: nothing hides the query load and the
+//                            exchange of the row statistics;
+//   several ("windows")      windows x (W x query tiles + 2), or + 5 where the ranges of a unit meet across CTAs and are too
+//                            short to hide it (28 x 8 units of 9 key tiles x 160 rows: whole units 55 us although a quarter
+//                            of the second window's CTAs idle, ranges of 3 tiles 82 us);
+//   two launches             the work spread evenly, + 10 for launches and merge, with 1.2 of the time per accumulator, 1.7
+//                            where a key tile has only one or two (77 us in the example).
+// With one range per CTA a unit's last range may be shorter.  Several windows: ranges that divide the unit, of at least four
+// tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
 int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
-    const int accs = (rows + kRows - 1) / kRows;
+    const int q_tiles = (rows + kRows - 1) / kRows;
+    const long long l2_budget = 120ll << 20;
+    // parts of a row's statistics per range: softmax groups that meet a query tile x copies of a short last tile
+    const int last = rows - (q_tiles - 1) * kRows;
+    const int parts = (q_tiles == 4 ? 1 : (q_tiles == 2 ? 2 : 4)) * (last <= 32 ? 4 : (last <= 64 ? 2 : 1));
     int best = 0;
-    long long best_cost = LLONG_MAX;
-    for (int n = 1; n <= T && n <= kMaxSegs && units * n <= ctas; ++n) {
-        const int W = (T + n - 1) / n, n_seg = (T + W - 1) / W;
-        const long long cost = (long long)W * accs * 4 + 12 + n_seg / 4;
+    long long best_cost = units * T * q_tiles * (q_tiles <= 2 ? 17 : 12) / ctas + 100;  // in tenths: two launches
+    for (int W = 1; W <= T; ++W) {
+        const int n_seg = (T + W - 1) / W;
+        if (n_seg > kMaxSegs || (W > 1 && n_seg == (T + W - 2) / (W - 1))) continue;  // longer, but no fewer ranges
+        const long long ranges = units * n_seg, windows = (ranges + ctas - 1) / ctas;
+        long long cost;
+        if (windows == 1) {
+            cost = (long long)W * q_tiles * 10 + 50 + n_seg * parts * 3 / 10;
+        } else {
+            if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;
+            cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20));
+        }
         if (cost < best_cost) {
             best_cost = cost;
             best = W;
         }
     }
-    // a single window that leaves more than a third of the SMs idle competes with several
-    if (best && units * ((T + best - 1) / best) * 3 >= (long long)ctas * 2) return best;
-    const long long l2_budget = 48ll << 20;
-    const int single = best;
-    const long long single_cost = best ? (long long)best * 10 + 30 : LLONG_MAX;
-    best = 0;
-    best_cost = LLONG_MAX;
-    for (int pass = 0; pass < 2 && !best; ++pass)
-        for (int W = pass ? 6 : 1; W <= T; ++W) {
-            const int n_seg = (T + W - 1) / W;
-            if (pass == 0 && T % W) continue;
-            if ((W < 4 && W < T) || n_seg > 8) continue;
-            if (W > 1 && (long long)W * ctas * tile_bytes > l2_budget && (best || pass)) break;
-            const long long ranges = units * n_seg, windows = (ranges + ctas - 1) / ctas;
-            if (windows < 2 || (double)units * T / (double)(windows * W * ctas) < 0.85) continue;
-            const long long cost = windows * (W + 1);
-            if (cost < best_cost) {
-                best_cost = cost;
-                best = W;
-            }
-        }
-    return best && best_cost * 10 < single_cost ? best : (single ? single : best);
+    return best;
 }
 
 int rows_alloc_of(const ModelView &mv, const BatchView &bv) {  // resident query rows: whole tiles
