@@ -59,9 +59,9 @@ WsLayout ws_layout(const finch_ctx *ctx, const finch_batch *b) {
     w.lse_bytes = (size_t)mv.L * mv.Hq * (size_t)b->total_q * sizeof(float2) * (kScoreMaxSplits * 4 + 1) +
                   (4 * n_kv_scores + 2) * sizeof(float) +  // row statistics, partial scores per KV head,
                   ((size_t)b->batch + 1) * 8 + 4096;       // and the item plan of a multi-request batch
-    // what each path needs at least: the one-kernel layout, one key split of the two-launch layout
+    // the one-kernel layout, the two-launch layout with the key splits it would take
     const size_t fused = score_fused_scratch(*ctx, view_of(b)) * sizeof(float2);
-    const size_t two = score_tc_supported(*ctx) ? score_tc_scratch_min(*ctx, view_of(b)) * sizeof(float2) : 0;
+    const size_t two = score_tc_supported(*ctx) ? score_tc_scratch(*ctx, view_of(b)) * sizeof(float2) : 0;
     if (fused > w.lse_bytes) w.lse_bytes = fused;
     if (two > w.lse_bytes) w.lse_bytes = two;
     w.lse_bytes = align_up(w.lse_bytes);

@@ -140,6 +140,7 @@ cudaError_t launch_score_simt(const Ctx &ctx, const TensorView &q, const TensorV
 // every key split; up to kScoreMaxSplits splits are used when it is large enough.
 constexpr int kScoreMaxSplits = 8;
 bool score_tc_supported(const Ctx &ctx);
+size_t score_tc_scratch(const Ctx &ctx, const BatchView &bv);      // what it would like
 size_t score_tc_scratch_min(const Ctx &ctx, const BatchView &bv);  // least scratch (float2) of the two-launch path
 cudaError_t launch_score_tc(const Ctx &ctx, const TensorView &q, const TensorView &cache_k, const TensorView &chunk_k,
                             const BatchView &bv, float *scores, float2 *partial, size_t partial_capacity,

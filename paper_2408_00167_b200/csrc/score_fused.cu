@@ -312,7 +312,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
             if (sg.sweep == 0) {
                 Softmax<false>::RowStats st;
                 if (!(ok = role.lse_segment(u, R, sg.t0, sg.t1, live, no_limit, st))) break;
-                role.store_stats(R, st, live, p.partial + ((int64_t)sg.unit * p.n_seg + sg.slot) * kGroups * p.rows_alloc, p.rows_alloc);
+                role.store_stats(R, st, live, p.partial + ((int64_t)sg.unit * p.n_seg + sg.slot) * kGroups * p.rows_alloc, p.rows_alloc,
+                                 false);
                 __syncwarp();
                 if (!direct) {
                     if (lane == 0) count_arrive(c.a_count);

@@ -520,13 +520,13 @@ struct Softmax {
         return true;
     }
     // This group's part of the rows' statistics; parts: [kGroups][stride] of the segment, from the chunk's first row on.
-    __device__ __forceinline__ void store_stats(const Rows &R, const RowStats &s, uint32_t live, float2 *parts, int stride) const {
+    __device__ __forceinline__ void store_stats(const Rows &R, const RowStats &s, uint32_t live, float2 *parts, int stride, bool nothing) const {
         float2 *dst = parts + (int64_t)s.rel * stride + my_row;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             int qb = s.qb + k;
             if (qb >= R.n_qt) qb -= R.n_qt;
-            if ((k == 0 || R.n_qt == 3) && ((live >> qb) & 1u)) dst[qb * kRows] = make_float2(s.m[k] * scale2, s.z[k]);
+            if ((k == 0 || R.n_qt == 3) && ((live >> qb) & 1u)) dst[qb * kRows] = nothing ? make_float2(0.f, 0.f) : make_float2(s.m[k] * scale2, s.z[k]);
         }
     }
     // tail: columns at or beyond nv hold no row

@@ -40,12 +40,13 @@ struct TcParams {
     // `mv` is the scoring view: one scoring unit per KV head
 };
 
-// One stop of a CTA's walk: a chunk of the unit's query rows against one key split.
+// One stop of a CTA's walk: a chunk of the unit's query rows against the consecutive key splits that the CTA holds of it
+// (one load of the queries for all of them).
 struct Stop {
     UnitInfo u;
     Rows R;
     int t0, t1;
-    int split, chunk;
+    int split, n_splits, chunk;
     int64_t key;    // (unit, request)
     int64_t q_key;  // equal keys share their query tiles
 };
@@ -61,9 +62,8 @@ struct Walk {
     UnitInfo req;  // metadata of request `req.b` (-1: none read yet); l and G are not kept here
     int k_tiles, tps, n_chunks;
     Rows R;
-    bool fresh;  // the item under w has not been entered
 
-    __device__ Walk(const TcParams &tp, int w0, int end) : p(tp), w(w0), w1(end), chunk(0), fresh(true) {
+    __device__ Walk(const TcParams &tp, int w0, int end) : p(tp), w(w0), w1(end), chunk(0) {
         const int units = p.mv.L * p.mv.G;
         split = w0 % p.splits;
         key = w0 / p.splits;
@@ -73,24 +73,22 @@ struct Walk {
         G = unit % p.mv.G;
         req.b = -1;
     }
-    __device__ void advance() {
-        ++w;
+    __device__ void next_unit() {  // past the splits of this unit that the CTA holds
+        w += p.splits - split;
         chunk = 0;
-        if (++split == p.splits) {
-            split = 0;
-            ++key;
-            if (++G == p.mv.G) {
-                G = 0;
-                if (++l == p.mv.L) {
-                    l = 0;
-                    ++b;
-                }
+        split = 0;
+        ++key;
+        if (++G == p.mv.G) {
+            G = 0;
+            if (++l == p.mv.L) {
+                l = 0;
+                ++b;
             }
         }
     }
-    // `empties`: also stop (with R.rows = 0) at items of requests without prompt rows.
+    // `empties`: also stop (with R.rows = 0) at units of requests without prompt rows.
     __device__ bool next(Stop &s, bool empties, bool report) {
-        for (; w < w1; advance()) {
+        for (; w < w1; next_unit()) {
             if (req.b != b) {
                 req = unit_info(p.mv, p.bv, 0, b);
                 k_tiles = n_key_tiles(req);
@@ -99,8 +97,9 @@ struct Walk {
                 R = make_rows(req.n_q, p.mv.hpg, 0);
                 if (!req.ok && report) atomicOr(p.status, FINCH_DEV_BAD_BATCH);
             }
+            s.n_splits = min(p.splits - split, w1 - w);
             s.t0 = split * tps;
-            s.t1 = min(k_tiles, s.t0 + tps);
+            s.t1 = min(k_tiles, s.t0 + s.n_splits * tps);
             if (!req.ok || s.t0 >= s.t1 || (req.n_q == 0 && !empties)) continue;
             s.u = req;
             s.u.l = l;
@@ -110,7 +109,7 @@ struct Walk {
             s.chunk = chunk;
             s.key = key;
             s.q_key = key * n_chunks + chunk + ((int64_t)b << 48);
-            if (++chunk == n_chunks) advance();
+            if (++chunk == n_chunks) next_unit();
             return true;
         }
         return false;
@@ -207,7 +206,10 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant
                 }
                 typename Softmax<MASK>::RowStats st;
                 if (!(ok = role.lse_segment(u, R, s.t0, s.t1, live, lim, st))) break;
-                role.store_stats(R, st, live, p.partial + (s.key * p.splits + s.split) * kGroups * p.slots + R.r0, p.slots);
+                // the stop's statistics stand at its first split, nothing at the others
+                float2 *parts = p.partial + (s.key * p.splits + s.split) * kGroups * p.slots + R.r0;
+                role.store_stats(R, st, live, parts, p.slots, false);
+                for (int i = 1; i < s.n_splits; ++i) role.store_stats(R, st, live, parts + (int64_t)i * kGroups * p.slots, p.slots, true);
             } else {
                 // The merged statistics of the resident rows are staged once per CTA, every softmax warp its share, into
                 // one of two buffers; a warp that has passed the barrier of epoch e has seen all warps finish epoch
@@ -366,13 +368,19 @@ merge_stats_kernel(TcParams p) {
 
 // ------------------------------------------------------------------------------------------------ host side
 
-// Key splits per unit: the smallest count (at most max_splits, at least one key tile each) whose grid fills whole
-// waves of SMs best.
-int choose_splits(int ctas_per_split, int key_tiles, int sm_count, int max_splits) {
+// Key splits per unit, at least one key tile each and at most kScoreMaxSplits: the smallest count whose grid fills whole
+// waves of SMs best, every item (unit, request, split) costing the same.  Several requests' items differ, and CTAs take
+// ranges of about equal work: where there are enough of them eight items to a CTA are fine enough (9 requests of 16 units:
+// 144 items on 148 SMs left the grid waiting for the longest prompts, 0.144 ms against 0.120); few units would only load
+// their queries on more CTAs (2 requests of 16 units: 46 us with 4 splits, 66 with 8).
+int choose_splits(int units, int batch, int key_tiles, int sm_count) {
+    const int most = min(kScoreMaxSplits, key_tiles);
+    if (batch > 1 && 2 * units * batch >= sm_count) return max(1, min(most, (8 * sm_count + units * batch - 1) / (units * batch)));
+    units *= batch;
     int best = 1;
     double best_eff = 0.0;
-    for (int s = 1; s <= max_splits && s <= key_tiles; ++s) {
-        const double waves = (double)ctas_per_split * s / sm_count;
+    for (int s = 1; s <= most; ++s) {
+        const double waves = (double)units * s / sm_count;
         const double eff = waves / (double)((long long)waves + (waves > (long long)waves ? 1 : 0));
         if (eff > best_eff * 1.05) {
             best_eff = eff;
@@ -441,10 +449,17 @@ bool score_tc_supported(const Ctx &ctx) {
     return ctx.cfg.dtype == FINCH_BF16 && (ctx.model.d == 64 || ctx.model.d == 128);
 }
 
-// The least scratch (float2 entries) the two-launch tensor-core path needs for this batch: one key split.
+// Scratch (float2 entries) of the two-launch tensor-core path: the least, with one key split, and what it would like.
 size_t score_tc_scratch_min(const Ctx &ctx, const BatchView &bv) {
     const ModelView &mv = ctx.model;
     return (size_t)bv.batch * mv.L * mv.Hkv * kGroups * slots_of(mv, bv) + scratch_rest(mv, bv);
+}
+size_t score_tc_scratch(const Ctx &ctx, const BatchView &bv) {
+    const ModelView &mv = ctx.model;
+    const int key_tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
+    if (bv.batch == 0 || key_tiles == 0) return 0;
+    const size_t splits = choose_splits(mv.L * mv.Hkv, bv.batch, key_tiles, ctx.sm_count > 0 ? ctx.sm_count : 148);
+    return splits * bv.batch * mv.L * mv.Hkv * kGroups * slots_of(mv, bv) + scratch_rest(mv, bv);
 }
 
 // `scratch` holds `capacity` float2 entries; the key-split count is limited so that everything fits.  Returns
@@ -477,14 +492,14 @@ cudaError_t launch_score_tc(const Ctx &ctx, const TensorView &q, const TensorVie
     if (!have_cache) cm = hm;  // never dereferenced: no request has cache tiles
     if (!have_chunk) hm = cm;
     const int key_tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
-    const int max_splits = (int)min((size_t)kScoreMaxSplits, (capacity - rest) / per_split);
+    const int most = (int)min((size_t)kScoreMaxSplits, (capacity - rest) / per_split);  // splits the scratch has room for
     TcParams p{};
     p.mv = mv;
     p.bv = bv;
     p.row_lse = row_lse;
     p.status = ctx.d_status;
     p.slots = slots;
-    p.splits = choose_splits(mv.L * mv.G * bv.batch, key_tiles, ctx.sm_count > 0 ? ctx.sm_count : 148, max_splits);
+    p.splits = min(most, choose_splits(mv.L * mv.G, bv.batch, key_tiles, ctx.sm_count > 0 ? ctx.sm_count : 148));
     p.work_prefix = (unsigned long long *)scratch;
     p.merged = scratch + plan;
     p.unit_scores = ctx.model.G == mv.G ? scores : (float *)(p.merged + rows);
