@@ -67,11 +67,17 @@ class DocumentCompressor:
         self._bufs = [mk(), mk()]
         self._cur = 0
         self.kept_idx = torch.full((n_layers, self.G, total_cap), -1, dtype=torch.int32, device=device)
-        self.cache_len = np.zeros(self.B, dtype=np.int32)       # host mirror of the device lengths
+        self._len = (0,) * self.B       # host mirror of the device lengths
         self._ws = None
         self._meta = {}
+        self._plans = {}
         self.steps = 0
         self._unverified = 0    # steps enqueued since the device was last compared with the host mirror
+
+    @property
+    def cache_len(self):
+        """Valid cache rows per request: the host mirror of the device lengths."""
+        return np.asarray(self._len, dtype=np.int32)
 
     # the cache the next step will read
     @property
@@ -104,7 +110,7 @@ class DocumentCompressor:
     def reset(self) -> None:
         """Start a new batch of documents in the same buffers (empty caches).  Checks the finished one first."""
         self.verify()
-        self.cache_len = np.zeros(self.B, dtype=np.int32)
+        self._len = (0,) * self.B
         self._bufs[0]["len"].zero_()
         self._cur = 0
         self.steps = 0
@@ -129,35 +135,49 @@ class DocumentCompressor:
             self._meta[key] = t
         return t
 
+    def _plan(self, q_off, chunk_off, budget):
+        """(batch, lengths after the step, workspace bytes) of one step; steps of the same shape share it."""
+        key = (q_off, chunk_off, budget, self._len, self._cur)
+        plan = self._plans.get(key)
+        if plan is not None:
+            return plan
+        B = self.B
+        budget = np.minimum(np.asarray(budget, dtype=np.int32), self.capacity).astype(np.int32)
+        qo, co = (np.asarray(a, dtype=np.int32) for a in (q_off, chunk_off))
+        assert len(qo) == len(co) == B + 1 and len(budget) == B
+        chunk_len = np.diff(co)
+        n_cand = self.cache_len + chunk_len
+        mx = lambda a: int(a.max()) if len(a) else 0
+        metadata = [self._device_i32(a) for a in (qo, co, self.cache_off, budget)]
+        c = fb.finch_batch(B, *(a.data_ptr() for a in metadata[:3]), self._bufs[self._cur]["len"].data_ptr(),
+                           metadata[3].data_ptr(), int(qo[B]), int(co[B]), int(self.cache_off[B]), mx(np.diff(qo)),
+                           mx(self.cache_len), mx(chunk_len), mx(np.minimum(budget, n_cand)), None, None, 0)
+        batch = fb.Batch(*metadata[:3], None, metadata[3], c)
+        if len(self._plans) > 256:
+            self._plans.clear()
+        plan = (batch, tuple(np.minimum(budget, n_cand).tolist()), fb.finch_workspace_bytes(self.ctx, batch))
+        self._plans[key] = plan
+        return plan
+
     def step(self, q, q_off: Sequence[int], chunk_k, chunk_v, chunk_pos, chunk_off: Sequence[int],
              budget: Sequence[int], scores=None, prompt_self_lse=None, row_limit=None, row_norm=False) -> None:
         """One finch_step: [cache ; chunk] -> the other cache.  Enqueues and returns.
 
         The lengths the previous step wrote on the device are this step's cache lengths as they are: nothing comes
         back to the host between steps, and the only host-to-device traffic is metadata that has not been seen yet."""
-        torch = self.torch
         src, dst = self._bufs[self._cur], self._bufs[self._cur ^ 1]
-        B = self.B
-        q_off = np.ascontiguousarray(q_off, dtype=np.int32)
-        chunk_off = np.ascontiguousarray(chunk_off, dtype=np.int32)
-        budget = np.minimum(np.asarray(budget, dtype=np.int32), self.capacity).astype(np.int32)
-        assert len(q_off) == len(chunk_off) == B + 1 and len(budget) == B
-        n_q, chunk_len = np.diff(q_off), np.diff(chunk_off)
-        n_cand = self.cache_len + chunk_len
-        mx = lambda a: int(a.max()) if len(a) else 0
-        c = fb.finch_batch(B, self._device_i32(q_off).data_ptr(), self._device_i32(chunk_off).data_ptr(),
-                           self._device_i32(self.cache_off).data_ptr(), src["len"].data_ptr(),
-                           self._device_i32(budget).data_ptr(), int(q_off[B]), int(chunk_off[B]), int(self.cache_off[B]),
-                           mx(n_q), mx(self.cache_len), mx(chunk_len), mx(np.minimum(budget, n_cand)),
-                           prompt_self_lse.data_ptr() if prompt_self_lse is not None else None,
-                           row_limit.data_ptr() if row_limit is not None else None, int(bool(row_norm)))
-        batch = fb.Batch(None, None, None, None, None, c, prompt_self_lse, row_limit)
-        need = fb.finch_workspace_bytes(self.ctx, batch)
+        batch, new_len, need = self._plan(*(tuple(map(int, a)) for a in (q_off, chunk_off, budget)))
+        c = batch.c
+        c.prompt_self_lse = prompt_self_lse.data_ptr() if prompt_self_lse is not None else None
+        c.row_limit = row_limit.data_ptr() if row_limit is not None else None
+        c.row_norm = int(bool(row_norm))
+        if row_limit is not None:        # another path, another workspace
+            need = fb.finch_workspace_bytes(self.ctx, batch)
         if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(need, dtype=torch.uint8, device=self.device)
+            self._ws = self.torch.empty(need, dtype=self.torch.uint8, device=self.device)
         fb.finch_step(self.ctx, q, src["k"], src["v"], src["pos"], chunk_k, chunk_v, chunk_pos, batch, dst["k"], dst["v"],
                       dst["pos"], self.kept_idx, dst["len"], scores, self._ws)
-        self.cache_len = np.minimum(budget, n_cand).astype(np.int32)   # what the step writes to dst["len"]
+        self._len = new_len              # what the step writes to dst["len"]
         self._cur ^= 1
         self.steps += 1
         self._unverified += 1
