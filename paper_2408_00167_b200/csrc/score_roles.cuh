@@ -542,8 +542,15 @@ struct Softmax {
     __device__ __forceinline__ float colsum_visit(uint32_t ta, int n, int nv, uint32_t sm4, const int *lim, const int2 *bounds,
                                                   int row, int j) {
         float c0 = 0.f, c1 = 0.f;
+        bool all = true;  // every row sees every key of the warp
+        const int j_lo = j - lane, j_hi = j_lo + 31;
+        if (MASK) {
+            const int2 lim16 = bounds[(row + min(lane & 7, (n >> 4) - 1) * 16) >> 4];
+            if (j_lo >= __reduce_max_sync(0xffffffffu, lim16.y)) return 0.f;  // no row sees any of them
+            all = j_hi < __reduce_min_sync(0xffffffffu, lim16.x);
+        }
         int cc = 0;
-        if (!MASK) {
+        if (all) {
 #pragma unroll 1
             for (; cc + 32 <= nv; cc += 32) colsum_cols<32, false>(ta + cc, false, 32, sm4 + cc * 8, c0, c1, nullptr, 0);
             if (cc < n) {
@@ -552,7 +559,7 @@ struct Softmax {
                 for (; cc < n; cc += 16) colsum_cols<16, false>(ta + cc, true, nv - cc, sm4 + cc * 8, c0, c1, nullptr, 0);
             }
         } else {
-            const int j_lo = j - lane, j_hi = j_lo + 31;  // the warp's keys
+            keep_branch();
 #pragma unroll 1
             for (; cc < n; cc += 16) {
                 const int2 b = bounds[(row + cc) >> 4];
