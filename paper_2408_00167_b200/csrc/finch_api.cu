@@ -218,6 +218,7 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out) {
     ctx->ev_entry = ctx->ev_v_ready = ctx->ev_selected = nullptr;
     ctx->tickets = nullptr;
     ctx->smem_bits = 0;
+    memset(ctx->clusters, 0, sizeof(ctx->clusters));
     ctx->launches = 0;
     if (!ctx->dry) {
         int n_dev = 0;

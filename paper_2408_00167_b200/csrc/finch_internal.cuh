@@ -52,6 +52,7 @@ struct Ctx {
     mutable uint32_t smem_bits;
     bool smem_ready(int bit) const { return smem_bits >> bit & 1u; }
     void smem_set(int bit) const { smem_bits |= 1u << bit; }
+    mutable int16_t clusters[2][17];  // answers of score_fused.cu's fits_clusters
     mutable uint64_t launches;  // kernels enqueued through this context
     // finch_step_host only: a second stream carries the chunk's V rows to the device while the scoring kernels,
     // which do not read them, already run; events tie it to the caller's stream on both sides
@@ -113,19 +114,26 @@ __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol
 __device__ __forceinline__ void dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... Params, typename... Args>
-cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                           Args &&...args) {
+cudaError_t launch_chained_cluster(void (*kernel)(Params...), int cluster, dim3 grid, dim3 block, size_t smem,
+                                   cudaStream_t stream, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args) {
+    return launch_chained_cluster(kernel, 1, grid, block, smem, stream, args...);
 }
 
 // ---- launchers implemented in the kernel files; each returns the cudaError_t of its launches ----

@@ -45,6 +45,7 @@ struct FusedParams {
     int stages;      // key-tile ring depth
     int rows_alloc;  // query rows of a unit, whole tiles
     int q_tiles;     // query tiles the shared memory holds
+    int cluster;     // CTAs of a cluster: the unit's ranges, with one window and few ranges per unit; else 1
     int delay;       // 0: a CTA has one window; 1: phase B of a window follows phase A of the next
 };
 
@@ -103,7 +104,7 @@ struct Walk {
             s.unit = rho / n_seg;
             s.slot = rho - s.unit * n_seg;
             s.t0 = s.slot * W;
-            s.t1 = min(T, s.t0 + W);
+            s.t1 = max(s.t0, min(T, s.t0 + W));
             ph ? (ph = 0, ++step) : (ph = 1);
             return true;
         }
@@ -163,9 +164,10 @@ __device__ __forceinline__ void merge_by_warp(const FusedParams &p, const UnitIn
 }
 
 // The same by all softmax threads: a row per thread, or, for few rows, per 2 to 16 neighbouring lanes that take every
-// second to sixteenth part each (many short ranges leave hundreds of parts to a row).
+// second to sixteenth part each (many short ranges leave hundreds of parts to a row).  `remote`: shared-memory address of
+// the parts, the same in every CTA of the cluster, or 0: they are in global memory.
 __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInfo &u, const Rows &R, int n_seg, int unit,
-                                             bool write_lse, float2 *stats, int tid) {
+                                             bool write_lse, float2 *stats, int tid, uint32_t remote) {
     const float2 *src = p.partial + (int64_t)unit * p.n_seg * kGroups * p.rows_alloc;
     int log_s = 0;  // lanes per row
     while (log_s < 4 && R.rows << (log_s + 1) <= kSoftmaxWarps * 32) ++log_s;
@@ -180,7 +182,14 @@ __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInf
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int k = i0 + (i << log_s);
-            part[i] = k < n ? __ldcg(src + parts.at(k, p.rows_alloc) + row) : make_float2(0.f, 0.f);
+            part[i] = make_float2(0.f, 0.f);
+            if (k >= n) continue;
+            if (remote) {
+                const int seg = parts.segment(k);
+                part[i] = ld_remote(map_to_rank(remote + ((uint32_t)parts.at(k - (seg << (parts.log_p + parts.log_c)), p.rows_alloc) + row) * 8, seg));
+            } else {
+                part[i] = __ldcg(src + parts.at(k, p.rows_alloc) + row);
+            }
         }
         merge_parts(part, M, Z);
     }
@@ -210,7 +219,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         prefetch_tensormap(&cache_map);
         prefetch_tensormap(&chunk_map);
     }
-    const uint32_t tmem = cta_setup(c, direct ? kSoftmaxWarps : 1);
+    const uint32_t tmem = cta_setup(c, direct ? kSoftmaxWarps : 1, p.cluster);
     // The inputs were written by what precedes this kernel.  The successor is NOT allowed to launch early: its CTAs
     // would take over the SMs of the CTAs that finish first and park there in their wait (measured: + 20 us on the
     // 0.5 ms step of 32 layers x 8 KV heads x 4096 candidates).
@@ -218,7 +227,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
 
     UnitInfo u = unit_info(mv, bv, 0, 0);  // l and G are set per segment
     const Rows R = make_rows(u.n_q, mv.hpg, 0);
-    const int T = n_key_tiles(u), n_seg = (T + p.W - 1) / p.W;
+    const int T = n_key_tiles(u), n_seg = p.cluster > 1 ? p.n_seg : (T + p.W - 1) / p.W;
     const bool run = u.ok && u.n_q > 0 && u.N > 0;
     const int n_ranges = mv.L * mv.G * n_seg;
     const int n_win = run && (int)blockIdx.x < n_ranges ? (n_ranges - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
@@ -239,7 +248,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
             FINCH_UNIT(sg);
             const bool reload = retain ? sg.sweep == 0 : q_unit != sg.unit;
             q_unit = sg.unit;
-            ok = role.segment(u, R, sg.t0, sg.t1, reload ? ring.take(R.n_qt) : -1);
+            if (sg.t0 < sg.t1) ok = role.segment(u, R, sg.t0, sg.t1, reload ? ring.take(R.n_qt) : -1);
         }
         role.drain();
     } else if (warp == 1) {
@@ -248,6 +257,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         Seg nx;
         for (bool more = walk.next(sg); ok && more; sg = nx) {
             more = walk.next(nx);
+            if (sg.t0 >= sg.t1) continue;  // a cluster's CTA beyond the unit's last tile
             const bool reload = retain ? sg.sweep == 0 : q_unit != sg.unit;
             const bool release = retain ? sg.sweep == 1 : more && nx.unit != sg.unit;
             q_unit = sg.unit;
@@ -312,6 +322,21 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
             if (sg.sweep == 0) {
                 Softmax<false>::RowStats st;
                 if (!(ok = role.lse_segment(u, R, sg.t0, sg.t1, live, no_limit, st))) break;
+                if (p.cluster > 1) {
+                    // the unit's ranges are the CTAs of this cluster: the parts stay in shared memory, every warp tells
+                    // every CTA that its own are written
+                    float2 *parts = c.stats + 2 * p.rows_alloc;
+                    role.store_stats(R, st, live, parts, p.rows_alloc, false);
+                    __syncwarp();
+                    if (lane < p.cluster) mbar_arrive_remote(map_to_rank(smem_u32(c.parts_ready), lane));
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_cluster(c.parts_ready, 0, c.abort_flag)))) break;
+                    FINCH_UNIT(sg);
+                    merge_by_cta(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats, threadIdx.x - kCtlWarps * 32, smem_u32(parts));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&c.stats_ready[1]);
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[1], 0, c.abort_flag)))) break;
+                    continue;
+                }
                 role.store_stats(R, st, live, p.partial + ((int64_t)sg.unit * p.n_seg + sg.slot) * kGroups * p.rows_alloc, p.rows_alloc,
                                  false);
                 __syncwarp();
@@ -333,7 +358,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
                 }
                 if (!(ok = __shfl_sync(0xffffffffu, good, 0))) break;
                 FINCH_UNIT(sg);
-                merge_by_cta(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats, tid);
+                merge_by_cta(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats, tid, 0);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&c.stats_ready[1]);
                 if (!(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[1], 0, c.abort_flag)))) break;
@@ -351,7 +376,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         }
     }
 #undef FINCH_UNIT
-    cta_teardown(c, tmem, p.status);
+    cta_teardown(c, tmem, p.status, p.cluster);
 }
 
 // scores of a selection group that spans several KV heads (one group per layer): the heads' column sums, added in
@@ -413,6 +438,34 @@ int rows_alloc_of(const ModelView &mv, const BatchView &bv) {  // resident query
     return (padded_rows(bv.max_q, mv.g) + kRows - 1) / kRows * kRows;
 }
 
+// With one window the ranges of a unit may form a cluster and exchange their row statistics through each other's shared
+// memory, where all units' clusters run at once (a cluster lies within one group of SMs, so fewer may fit than SMs would
+// allow).  The exchange through global memory and tickets costs 5.7 us of a 16 us call: stores, fence, atomic, poll, loads.
+constexpr int kMaxCluster = 16;
+template <int D>
+bool fits_clusters(const Ctx &ctx, int size, int units) {
+    int16_t &known = ctx.clusters[D == 128][size];  // clusters of this size at a time, + 1; 0: not asked yet
+    if (known == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(size);
+        cfg.blockDim = dim3(kTcThreads);
+        cfg.dynamicSmemBytes = kSmemLimit;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = size;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, score_fused_kernel<D>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            n = 0;
+        }
+        known = (int16_t)(n + 1);
+    }
+    return known > units;
+}
+
 template <int D>
 cudaError_t launch_fused_d(const Ctx &ctx, const CUtensorMap &qb, const CUtensorMap &qs, const CUtensorMap &cm,
                            const CUtensorMap &hm, FusedParams p, int n_ranges, int out_groups, int heads_per_group, float *scores,
@@ -424,17 +477,20 @@ cudaError_t launch_fused_d(const Ctx &ctx, const CUtensorMap &qb, const CUtensor
     p.delay = n_ranges > sms;
     // room for the queries of the two units that alternate, and of a third that is being loaded where they are short
     p.q_tiles = !p.delay || n_qt > 2 ? n_qt : n_qt + 2;
-    p.stages = kMaxStages;
-    while (p.stages > 2 && cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) > kSmemLimit) --p.stages;
-    const int smem = cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false);
     cudaError_t e = cudaSuccess;
     if (!ctx.smem_ready(kSmemFused + (D == 128))) {
         e = cudaFuncSetAttribute(score_fused_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_fused_kernel<D>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
         ctx.smem_set(kSmemFused + (D == 128));
     }
+    p.cluster = !p.delay && p.n_seg > 1 && p.n_seg <= kMaxCluster && fits_clusters<D>(ctx, p.n_seg, mv.L * mv.G) ? p.n_seg : 1;
+    const int parts = p.cluster > 1 ? kGroups * p.rows_alloc * 8 : 0;  // the cluster's exchange of row statistics
+    p.stages = kMaxStages;
+    while (p.stages > 2 && cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) + parts > kSmemLimit) --p.stages;
+    const int smem = cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) + parts;
     dim3 grid(n_ranges < sms ? n_ranges : sms);  // persistent and resident at once: phase B waits for neighbours
-    e = launch_chained(score_fused_kernel<D>, grid, dim3(kTcThreads), smem, stream, qb, qs, cm, hm, p);
+    e = launch_chained_cluster(score_fused_kernel<D>, p.cluster, grid, dim3(kTcThreads), smem, stream, qb, qs, cm, hm, p);
     ctx.launches += 1;
     if (e != cudaSuccess || heads_per_group == 1) return e;
     return launch_sum_heads(ctx, mv, bv, p.unit_scores, scores, out_groups, heads_per_group, stream);

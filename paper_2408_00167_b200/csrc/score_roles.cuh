@@ -28,6 +28,7 @@ struct Cta {  // shared memory of the CTA
     uint64_t *acc_full, *acc_empty;    // [kGroups] accumulators
     uint64_t *stats_ready;             // [2] row statistics of a second-sweep segment are staged
     uint64_t *sum_full, *sum_empty;    // [kSumBufs] column sums handed to the writer
+    uint64_t *parts_ready;             // the cluster's CTAs have written their partial row statistics
     uint32_t *tmem_slot;
     volatile int *abort_flag;
     int *a_count;                      // softmax warps through a first-sweep segment (counts up for ever)
@@ -69,6 +70,7 @@ __device__ __forceinline__ Cta cta_layout(uint8_t *raw, int tile_bytes, int q_ti
     c.sum_full = b, b += kSumBufs;
     c.sum_empty = b, b += kSumBufs;
     c.q_raw = b, b += 1;
+    c.parts_ready = b, b += 1;
     c.tmem_slot = (uint32_t *)b;
     c.abort_flag = (volatile int *)(c.tmem_slot + 1);
     c.a_count = (int *)(c.tmem_slot + 2);
@@ -80,7 +82,8 @@ __device__ __forceinline__ Cta cta_layout(uint8_t *raw, int tile_bytes, int q_ti
 }
 
 // Barriers and tensor memory (all 512 columns); ends with the CTA in step.  stats_arrivals: arrivals per staging.
-__device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals) {
+// cluster: CTAs that exchange row statistics through each other's shared memory (1: none).
+__device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals, int cluster = 1) {
     if (threadIdx.x == 0) {
         for (int i = 0; i < kQTiles; ++i) {
             mbar_init(&c.q_full[i], 1);
@@ -100,6 +103,7 @@ __device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals) 
             mbar_init(&c.sum_empty[i], 1);
         }
         mbar_init(c.q_raw, 1);
+        mbar_init(c.parts_ready, cluster * kSoftmaxWarps);
         *c.abort_flag = 0;
         *c.a_count = 0;
         fence_barrier_init();
@@ -110,16 +114,18 @@ __device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals) 
     }
     tc_fence_before();
     __syncthreads();
+    if (cluster > 1) cluster_sync();  // nobody arrives on a barrier that is not initialised
     tc_fence_after();
     return *c.tmem_slot;
 }
 
 // Common epilogue: everyone meets here, also after a timed-out wait.  The single-thread roles bring their warps back
 // together first: the CTA barrier must be executed by whole warps.
-__device__ __forceinline__ void cta_teardown(const Cta &c, uint32_t tmem, int *status) {
+__device__ __forceinline__ void cta_teardown(const Cta &c, uint32_t tmem, int *status, int cluster = 1) {
     __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (cluster > 1) cluster_sync();  // the neighbours have read this CTA's shared memory
     if (threadIdx.x == 0 && *c.abort_flag) atomicOr(status, FINCH_DEV_TIMEOUT);
     if (threadIdx.x / 32 == 1) {
         __syncwarp();
@@ -628,6 +634,7 @@ struct Parts {
         span = R.span;
     }
     __device__ int count(int segments) const { return segments << (log_p + log_c); }
+    __device__ int segment(int k) const { return k >> (log_p + log_c); }
     // offset of part k in [segments][kGroups][stride], from the row's own slot on
     __device__ int64_t at(int k, int stride) const {
         const int p = k & ((1 << log_p) - 1), c = (k >> log_p) & ((1 << log_c) - 1), s = k >> (log_p + log_c);
