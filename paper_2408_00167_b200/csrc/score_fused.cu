@@ -112,16 +112,15 @@ struct Walk {
     }
 };
 
-// (M, Z) of a row -> what the second sweep needs, and the row's log-sum-exp where it is asked for.
+// (M, Z) of a prompt row -> what the second sweep needs, and the row's log-sum-exp where it is asked for.
 __device__ __forceinline__ float2 finish_row(const FusedParams &p, const UnitInfo &u, const Rows &R, int row, float M, float Z,
                                              bool write_lse) {
-    if (!row_live(R, row)) return make_float2(0.f, 0.f);
-    const int64_t at = ((int64_t)u.l * p.mv.Hq + u.G * p.mv.hpg + row / R.rp) * p.bv.total_q + u.q0 + row % R.rp;
-    if (p.bv.self_lse) merge_self_term(p.bv.self_lse[at], M, Z);
-    float lse_nat;
-    const float2 out = merged_pair(M, Z, lse_nat);
-    if (write_lse && p.row_lse) p.row_lse[at] = lse_nat;
-    return out;
+    if (p.bv.self_lse || (write_lse && p.row_lse)) {
+        const int64_t at = ((int64_t)u.l * p.mv.Hq + u.G * p.mv.hpg + row / R.rp) * p.bv.total_q + u.q0 + row % R.rp;
+        if (p.bv.self_lse) merge_self_term(p.bv.self_lse[at], M, Z);
+        if (write_lse && p.row_lse) p.row_lse[at] = merged_lse(M, Z);
+    }
+    return merged_pair(M, Z);
 }
 
 // The statistics of a unit, merged over its ranges and the parts of each range in a fixed order and staged, by one warp:
@@ -153,10 +152,13 @@ __device__ __forceinline__ void merge_by_warp(const FusedParams &p, const UnitIn
 #pragma unroll
             for (int k = 0; k < 4; ++k) merge_parts(part[k], M[k], Z[k]);
         }
+        int live_k = live[0] | live[1] << 1 | live[2] << 2 | live[3] << 3;
 #pragma unroll 1
         for (int k = 0; k < 4; ++k) {
             const int row = row0 + k * 32;
-            if (row < R.rows) stage_row(stats, row, finish_row(p, u, R, row, M[0], Z[0], write_lse));
+            if (row < R.rows)
+                stage_row(stats, row, live_k & 1 ? finish_row(p, u, R, row, M[0], Z[0], write_lse) : make_float2(0.f, 0.f));
+            live_k >>= 1;
             M[0] = M[1], M[1] = M[2], M[2] = M[3];
             Z[0] = Z[1], Z[1] = Z[2], Z[2] = Z[3];
         }
@@ -199,7 +201,8 @@ __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInf
         if (nm != -INFINITY) Z = Z * ex2(M - nm) + oz * ex2(om - nm);
         M = nm;
     }
-    if (sub == 0 && row < R.rows) stage_row(stats, row, finish_row(p, u, R, row, M, Z, write_lse));
+    if (sub == 0 && row < R.rows)
+        stage_row(stats, row, live ? finish_row(p, u, R, row, M, Z, write_lse) : make_float2(0.f, 0.f));
 }
 
 template <int D>
@@ -234,7 +237,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
     if (!u.ok && threadIdx.x == 0 && blockIdx.x == 0) atomicOr(p.status, FINCH_DEV_BAD_BATCH);
     Walk walk{p.W, T, n_seg, p.delay, n_win, 0, 0};
     Seg sg;
-    bool ok = true;
+    bool ok = true, left = false;
     // With several windows the sweeps of two units alternate.  Where the ring holds both their query tiles a window loads
     // its queries once and keeps them for its second sweep (64 rows: 0.105 -> 0.09 ms for 1024 units of 8 key tiles).
     const bool retain = p.delay && 2 * R.n_qt <= p.q_tiles;
@@ -328,11 +331,18 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
                     float2 *parts = c.stats + 2 * p.rows_alloc;
                     role.store_stats(R, st, live, parts, p.rows_alloc, false);
                     __syncwarp();
+                    cluster_wait();  // everybody's barriers are initialised
                     if (lane < p.cluster) mbar_arrive_remote(map_to_rank(smem_u32(c.parts_ready), lane));
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_cluster(c.parts_ready, 0, c.abort_flag)))) break;
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_cluster(c.parts_ready, 0, c.abort_flag)))) {
+                        cluster_arrive();
+                        left = true;
+                        break;
+                    }
                     FINCH_UNIT(sg);
                     merge_by_cta(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats, threadIdx.x - kCtlWarps * 32, smem_u32(parts));
                     __syncwarp();
+                    cluster_arrive();  // through with the neighbours' shared memory
+                    left = true;
                     if (lane == 0) mbar_arrive(&c.stats_ready[1]);
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[1], 0, c.abort_flag)))) break;
                     continue;
@@ -376,7 +386,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         }
     }
 #undef FINCH_UNIT
-    cta_teardown(c, tmem, p.status, p.cluster);
+    cta_teardown(c, tmem, p.status, p.cluster, left);
 }
 
 // scores of a selection group that spans several KV heads (one group per layer): the heads' column sums, added in

@@ -114,18 +114,23 @@ __device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals, 
     }
     tc_fence_before();
     __syncthreads();
-    if (cluster > 1) cluster_sync();  // nobody arrives on a barrier that is not initialised
+    if (cluster > 1) cluster_arrive();  // the barriers are initialised: waited for ahead of the first remote arrival
     tc_fence_after();
     return *c.tmem_slot;
 }
 
 // Common epilogue: everyone meets here, also after a timed-out wait.  The single-thread roles bring their warps back
 // together first: the CTA barrier must be executed by whole warps.
-__device__ __forceinline__ void cta_teardown(const Cta &c, uint32_t tmem, int *status, int cluster = 1) {
+// left: this warp has been through both cluster barriers but the last wait.
+__device__ __forceinline__ void cta_teardown(const Cta &c, uint32_t tmem, int *status, int cluster = 1, bool left = false) {
     __syncwarp();
+    if (cluster > 1 && !left) {
+        cluster_wait();
+        cluster_arrive();
+    }
     tc_fence_before();
     __syncthreads();
-    if (cluster > 1) cluster_sync();  // the neighbours have read this CTA's shared memory
+    if (cluster > 1) cluster_wait();  // the neighbours have read this CTA's shared memory
     if (threadIdx.x == 0 && *c.abort_flag) atomicOr(status, FINCH_DEV_TIMEOUT);
     if (threadIdx.x / 32 == 1) {
         __syncwarp();

@@ -358,12 +358,11 @@ merge_stats_kernel(TcParams p) {
         merge_parts(part, M, Z);
     }
     if (bv.self_lse) merge_self_term(bv.self_lse[row], M, Z);  // the keys the row attends to besides the candidates
-    float lse_nat;
-    float2 out = merged_pair(M, Z, lse_nat);
+    float2 out = merged_pair(M, Z);
     if (bv.row_limit && bv.row_norm)  // per-row normalisation: times the fraction of the candidates the row sees
         out.y *= (float)max(0, min(u.N, bv.row_limit[u.q0 + pr])) / (float)u.N;
     p.merged[row] = out;
-    if (p.row_lse) p.row_lse[row] = lse_nat;
+    if (p.row_lse) p.row_lse[row] = merged_lse(M, Z);
 }
 
 // ------------------------------------------------------------------------------------------------ host side

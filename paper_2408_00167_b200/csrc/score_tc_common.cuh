@@ -269,18 +269,15 @@ __device__ __forceinline__ void merge_self_term(float lse_nat, float &M, float &
         M = nm;
     }
 }
-// (M, Z) -> (-R, w); lse_nat receives the row's natural-log sum-exp.  A row that attends to nothing (Z = 0) weighs
-// nothing: (0, 0) and -inf.
-__device__ __forceinline__ float2 merged_pair(float M, float Z, float &lse_nat) {
-    if (!(Z > 0.f)) {
-        lse_nat = -INFINITY;
-        return make_float2(0.f, 0.f);
-    }
+// (M, Z) -> the row's natural-log sum-exp, and (-R, w).  A row that attends to nothing (Z = 0) weighs nothing: -inf and
+// (0, 0).
+__device__ __forceinline__ float merged_lse(float M, float Z) { return Z > 0.f ? (M + log2f(Z)) * kLn2 : -INFINITY; }
+__device__ __forceinline__ float2 merged_pair(float M, float Z) {
+    if (!(Z > 0.f)) return make_float2(0.f, 0.f);
     // Z = 2^k * [1, 2) (a sum of terms in [1, 2) times factors <= 1, the largest of them 1)
     const int zbits = __float_as_int(Z);
     const int k = ((zbits >> 23) & 0xff) - 127;
     const float w = __fdividef(1.0f, __int_as_float((zbits & 0x007fffff) | 0x3f800000));
-    lse_nat = (M + log2f(Z)) * kLn2;
     return make_float2(-(M + (float)k), w);
 }
 
