@@ -123,6 +123,9 @@ __device__ __forceinline__ float2 finish_row(const FusedParams &p, const UnitInf
     return merged_pair(M, Z);
 }
 
+// The second sweep reads its rows in blocks of 16: the rows behind the last one of a unit are staged with weight 0.
+__device__ __forceinline__ int staged_rows(const Rows &R) { return (R.rows + 15) & ~15; }
+
 // The statistics of a unit, merged over its ranges and the parts of each range in a fixed order and staged, by one warp:
 // four rows and four parts of each per lane in flight.
 __device__ __forceinline__ void merge_by_warp(const FusedParams &p, const UnitInfo &u, const Rows &R, int n_seg, int unit,
@@ -156,7 +159,7 @@ __device__ __forceinline__ void merge_by_warp(const FusedParams &p, const UnitIn
 #pragma unroll 1
         for (int k = 0; k < 4; ++k) {
             const int row = row0 + k * 32;
-            if (row < R.rows)
+            if (row < staged_rows(R))
                 stage_row(stats, row, live_k & 1 ? finish_row(p, u, R, row, M[0], Z[0], write_lse) : make_float2(0.f, 0.f));
             live_k >>= 1;
             M[0] = M[1], M[1] = M[2], M[2] = M[3];
@@ -201,7 +204,7 @@ __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInf
         if (nm != -INFINITY) Z = Z * ex2(M - nm) + oz * ex2(om - nm);
         M = nm;
     }
-    if (sub == 0 && row < R.rows)
+    if (sub == 0 && row < staged_rows(R))
         stage_row(stats, row, live ? finish_row(p, u, R, row, M, Z, write_lse) : make_float2(0.f, 0.f));
 }
 

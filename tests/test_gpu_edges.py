@@ -1,0 +1,162 @@
+"""GPU parity at the sizes where the kernels' tilings and dispatch rules change: row padding, copies of a short query tile,
+query chunks, ranges of one unit exchanged through a cluster or through global memory, candidates per selection kernel,
+row blocks of the compaction, key splits of the warp-level scoring.  Against the fp64 oracle, with the harness's tolerance
+(max(1e-3 relative, 1e-5 absolute) per score, everything else exact)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2408_00167_b200 import binding as fb
+from paper_2408_00167_b200 import build as fbuild
+from paper_2408_00167_b200 import workloads as wl
+from parity_harness import GpuStep, check_parity, oracle_scores, to_device, to_host
+from test_gpu_configs import _select_only
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    fbuild.build()
+    fb.load()
+
+
+def _check(layers, Hq, Hkv, d, reqs, dtype="bf16", group_mode=0):
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, dtype=dtype,
+                    group_mode=group_mode, planted_frac=0.02, requests=tuple(wl.Request(*r) for r in reqs))
+    st = wl.steady_state(cfg, list(range(layers)), step=1)
+    g = GpuStep(cfg, st, layers)
+    try:
+        plan = fb.finch_score_plan(g.ctx, g.batch)
+        g.run_parts()
+        assert g.status() == 0
+        res = g.results()
+        for b in range(cfg.batch):      # every candidate has a number
+            lo = int(st["cache_off"][b] + st["chunk_off"][b])
+            hi = lo + int(st["cache_len"][b] + st["chunk_off"][b + 1] - st["chunk_off"][b])
+            assert np.isfinite(res["scores"][:, :, lo:hi]).all()
+        ref, ref_lse = oracle_scores(cfg, st, threads=oracle.max_threads(), want_lse=True)
+        check_parity(cfg, st, res, ref)
+        # the log of a sum of exponentials of fp32 logits: a few 2^-24 of the largest logit (below 2^6 here)
+        np.testing.assert_allclose(res["row_lse"], ref_lse, rtol=1e-5, atol=2e-5)
+    finally:
+        g.close()
+    return plan
+
+
+@pytest.mark.parametrize("heads,n_q", [(1, 1), (1, 32), (1, 33), (1, 65), (1, 128), (2, 65), (4, 37), (4, 96), (4, 128)])
+def test_query_rows_around_the_tile_sizes(heads, n_q):
+    """Padded rows per KV head from 8 to 512: one to four query tiles, a last one of 32, 64 and 128 rows."""
+    path, _ = _check(1, 2 * heads, 2, 128, [(n_q, 9999, 300, 200)])
+    assert path == fb.FINCH_SCORE_ONE_KERNEL
+
+
+@pytest.mark.parametrize("layers,Hkv,cache,chunk,window", [
+    (1, 2, 1, 127, 1),        # two tiles, one candidate in the first
+    (1, 8, 512, 512, 2),      # four ranges of two tiles: a cluster
+    (1, 8, 2048, 2048, 4),    # eight ranges
+    (5, 8, 2030, 2032, None),  # three ranges a unit, the last one shorter
+    (20, 8, 640, 256, 7),     # whole units in two windows, the second one half empty
+    (19, 16, 1024, 1024, None),   # several windows whose ranges meet across CTAs
+])
+def test_ranges_of_a_unit(layers, Hkv, cache, chunk, window):
+    path, w = _check(layers, Hkv, Hkv, 64, [(24, 99999, chunk, cache)])
+    assert path == fb.FINCH_SCORE_ONE_KERNEL and (window is None or w == window)
+
+
+@pytest.mark.parametrize("n_q,heads", [(129, 4), (145, 4), (513, 1)])
+def test_query_chunks_and_pad_rows_of_neighbouring_requests(n_q, heads):
+    """More than 512 padded rows in chunks; requests whose pad rows are the next request's rows."""
+    path, _ = _check(2, 2 * heads, 2, 128, [(n_q, 9999, 200, 150), (7, 9999, 140, 260), (n_q - 3, 9999, 100, 129)])
+    assert path == fb.FINCH_SCORE_TWO_LAUNCH
+
+
+@pytest.mark.parametrize("n", [63, 64, 65, 2047, 2048, 2049, 4095, 8191, 8192, 8193])
+@pytest.mark.parametrize("kind", ["spread", "one_value", "two_values", "outlier"])
+def test_select_at_the_limits_of_its_kernels(n, kind):
+    rng = np.random.default_rng(n)
+    L, G = 2, 2
+    s = rng.random((L, G, n), dtype=np.float32)
+    if kind == "one_value":
+        s[:] = 0.25                                   # a single key: the first round's bin holds everything
+    elif kind == "two_values":
+        s = np.where(s < 0.5, np.float32(0.5), np.nextafter(np.float32(0.5), np.float32(1))).astype(np.float32)
+    elif kind == "outlier":
+        s = (1 + s * 1e-4).astype(np.float32)         # all but one key in one bin of the first round
+        s[:, :, n // 3] = 1e30
+    for r in (1, n // 2, n - 1):
+        kept, out_len = _select_only(s, [n], [n], [0], [r], L, G)
+        assert out_len.tolist() == [r]
+        for l in range(L):
+            for g in range(G):
+                np.testing.assert_array_equal(kept[l, g, :r], oracle.select_unit(s[l, g].astype(np.float64), r))
+
+
+@pytest.mark.parametrize("Hq,Hkv,n_q,cache,chunk,d", [(8, 8, 16, 256, 256, 64), (8, 2, 17, 64, 1, 96), (8, 2, 32, 130, 65, 32),
+                                                     (8, 2, 33, 63, 64, 128), (4, 4, 65, 700, 1400, 64)])
+def test_warp_level_scoring_tiles_and_splits(Hq, Hkv, n_q, cache, chunk, d):
+    _check(1, Hq, Hkv, d, [(n_q, 9999, chunk, cache)], dtype="f32")
+
+
+def test_causal_blocks_that_see_all_none_or_part_of_their_keys():
+    """Query rows in blocks with one limit each: nothing, one key, the tile edges and their neighbours, everything."""
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=2, n_q_heads=2, n_kv_heads=1, head_dim=128, dtype="bf16", planted_frac=0.03,
+                    requests=(wl.Request(280, 9999, 300, 212),))
+    st = wl.steady_state(cfg, [0, 1], step=2)
+    N = 512
+    limit = np.repeat(np.array([0, 1, 31, 32, 33, 127, 128, 129, 211, 212, 213, 383, 384, N, N + 9], np.int32), 19)[:280]
+    limit[-40:] = np.arange(N - 40, N)                      # a ragged staircase at the end
+    g = GpuStep(cfg, st, 2, row_limit=limit)
+    try:
+        g.run_parts()
+        assert g.status() == 0
+        res = g.results()
+        ref, ref_lse = oracle_scores(cfg, st, want_lse=True, row_limit=limit)
+        check_parity(cfg, st, res, ref)
+        finite = np.isfinite(ref_lse)
+        np.testing.assert_allclose(res["row_lse"][finite], ref_lse[finite], rtol=1e-5, atol=2e-5)
+        assert np.all(np.isneginf(res["row_lse"][~finite]))
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("rope_theta", [0.0, 10000.0])
+@pytest.mark.parametrize("L,Hkv,budget", [(1, 1, 1), (1, 2, 17), (1, 4, 255), (8, 8, 257), (32, 32, 600)])
+def test_compact_row_blocks(L, Hkv, budget, rope_theta):
+    """Budgets around the row blocks of one CTA (16 to 256 rows, by how many KV heads share the chip)."""
+    import torch
+    rng = np.random.default_rng(budget)
+    d, c, m = 64, 400, 300
+    mk = lambda n: wl.to_storage(rng.standard_normal((L, Hkv, n, d)).astype(np.float32), "bf16")
+    ck, cv, hk, hv = mk(budget + c), mk(budget + c), mk(m), mk(m)
+    cache_off, chunk_off = wl.offsets([budget + c]), wl.offsets([m])
+    cpos = rng.integers(0, 1000, size=(L, Hkv, budget + c)).astype(np.int32)
+    hpos = rng.integers(1000, 2000, size=m).astype(np.int32)
+    scores = rng.random((L, Hkv, budget + c + m))
+    kept, out_len = oracle.select(scores, chunk_off=chunk_off, cache_off=cache_off, cache_len=[c], budget=[budget])
+    kw = dict(n_kv_heads=Hkv, head_dim=d, group_mode=0, chunk_off=chunk_off, cache_off=cache_off, cache_len=[c])
+    if rope_theta:
+        kw.update(rope_theta=rope_theta, rope_pairing=0)
+    want_k, want_v, want_p = oracle.compact("bf16", kept, out_len, ck, cv, cpos, hk, hv, hpos, **kw)
+    batch = fb.make_batch(wl.offsets([1]), chunk_off, cache_off, [c], [budget])
+    ctx = fb.finch_ctx_create(L, Hkv, Hkv, d, fb.FINCH_BF16, 0, max_batch=1, max_prompt=1, max_candidates=2048,
+                              rope_theta=rope_theta)
+    try:
+        dev = lambda a: to_device(a, "bf16")
+        out_k, out_v = dev(np.zeros_like(ck)), dev(np.zeros_like(cv))
+        out_pos = torch.full((L, Hkv, budget + c), -1, dtype=torch.int32, device="cuda")
+        fb.finch_compact(ctx, torch.from_numpy(kept).cuda(), torch.from_numpy(out_len).cuda(), dev(ck), dev(cv),
+                         torch.from_numpy(cpos).cuda(), dev(hk), dev(hv), torch.from_numpy(hpos).cuda(), batch,
+                         out_k, out_v, out_pos)
+        assert fb.finch_device_status(ctx) == 0
+        np.testing.assert_array_equal(to_host(out_v, "bf16"), want_v)
+        np.testing.assert_array_equal(out_pos.cpu().numpy(), want_p)
+        if not rope_theta:
+            np.testing.assert_array_equal(to_host(out_k, "bf16"), want_k)
+        else:       # fp32 rotation: one unit in the last place of a bfloat16 (2^-8 relative to its binade's top) on near-ties
+            got = wl.from_storage(to_host(out_k, "bf16"), "bf16").astype(np.float64)
+            want = wl.from_storage(want_k, "bf16").astype(np.float64)
+            row = np.sqrt((want ** 2).sum(axis=-1, keepdims=True))
+            assert np.all(np.abs(got - want) <= np.abs(want) * 2.0 ** -7 + 2e-6 * row)
+    finally:
+        fb.finch_ctx_destroy(ctx)
