@@ -9,7 +9,9 @@
 // 32-layer step with 128 CTAs: 0.49 ms for 1 GB, re-positioned).
 #include <cuda_bf16.h>
 
-#include "finch_internal.cuh"
+#include <type_traits>
+
+#include "select_core.cuh"
 
 namespace finch {
 namespace {
@@ -114,10 +116,10 @@ struct RowMap {
     __device__ const char *src(int j) const { return j < c ? cache + j * cache_step : chunk + j * chunk_step; }
 };
 
-// Plain copies.  A thread keeps its piece of the row and walks the rows 256 / pieces apart.
-__device__ __forceinline__ void copy_rows(const RowMap &m, const int *src_idx, int rows, int pieces) {
+// Plain copies.  A thread keeps its piece of the row and walks the rows threads / pieces apart.
+__device__ __forceinline__ void copy_rows(const RowMap &m, const int *src_idx, int rows, int pieces, int threads) {
     constexpr int kBatch = 8;
-    const int step = kCompactThreads / pieces, r0 = threadIdx.x / pieces, off = (threadIdx.x - r0 * pieces) * 16;
+    const int step = threads / pieces, r0 = threadIdx.x / pieces, off = (threadIdx.x - r0 * pieces) * 16;
     if (r0 >= step) return;
 #pragma unroll 1
     for (int r = r0; r < rows; r += step * kBatch) {
@@ -139,10 +141,10 @@ __device__ __forceinline__ void copy_rows(const RowMap &m, const int *src_idx, i
 // and the partner piece of the second; else pairs (2t, 2t + 1) inside a piece.
 template <int kElems, bool kSplit>
 __device__ __forceinline__ void rotate_rows(const RowMap &m, const int *src_idx, int rows, int i0, int d, int elem_bytes,
-                                            const float2 *rope_table) {
+                                            const float2 *rope_table, int threads) {
     constexpr int kBatch = 4;
     const int half = d / 2, pieces = d * elem_bytes / 16 / (kSplit ? 2 : 1);
-    const int step = kCompactThreads / pieces, r0 = threadIdx.x / pieces, piece = threadIdx.x - r0 * pieces;
+    const int step = threads / pieces, r0 = threadIdx.x / pieces, piece = threadIdx.x - r0 * pieces;
     const int off = piece * 16, far = half * elem_bytes;
     const float2 *table = rope_table + piece * (kSplit ? kElems : kElems / 2);
     if (r0 >= step) return;
@@ -177,12 +179,42 @@ __device__ __forceinline__ void rotate_rows(const RowMap &m, const int *src_idx,
     }
 }
 
+struct CompactTensors {
+    TensorView cache_k, cache_v, chunk_k, chunk_v, out_k, out_v;
+    const int *cache_pos, *chunk_pos;
+    int *out_pos;
+};
+
+// Source of output row i of a group: checks the index, and writes the row's position where `leader` (the CTA of the
+// group's first KV head).  -1: no copy.
+template <int ROPE>
+__device__ __forceinline__ int place_row(const ModelView &mv, const UnitInfo &u, const CompactTensors &t, int64_t unit_off,
+                                         bool leader, int i, int j, int *status) {
+    // with rotation a distance beyond the table (only possible when out_len exceeds the candidate count) is refused
+    if (j < 0 || j >= u.N || (ROPE && abs(i - j) >= mv.rope_rows)) {
+        atomicOr(status, FINCH_DEV_BAD_INDEX);
+        return -1;
+    }
+    if (leader) t.out_pos[unit_off + i] = j < u.c ? t.cache_pos[unit_off + j] : t.chunk_pos[u.chunk0 + j - u.c];
+    return j;
+}
+
 // ROPE 0: bit-for-bit copies; 1 / 2: K rows re-positioned, pairs (t, t + d/2) / (2t, 2t + 1).
 template <int ROPE, int kElems>
+__device__ __forceinline__ void move_rows(const ModelView &mv, const UnitInfo &u, int kvh, int i0, int rows,
+                                          const int *src_idx, const CompactTensors &t, int threads) {
+    const int pieces = mv.d * mv.elem_bytes / 16;  // 16-byte pieces per row
+    const RowMap k_rows(u, kvh, i0, mv.elem_bytes, t.cache_k, t.chunk_k, t.out_k);
+    if (ROPE)
+        rotate_rows<kElems, ROPE == 1>(k_rows, src_idx, rows, i0, mv.d, mv.elem_bytes, mv.rope_table, threads);
+    else
+        copy_rows(k_rows, src_idx, rows, pieces, threads);
+    copy_rows(RowMap(u, kvh, i0, mv.elem_bytes, t.cache_v, t.chunk_v, t.out_v), src_idx, rows, pieces, threads);
+}
+
+template <int ROPE, int kElems>
 __global__ void __launch_bounds__(kCompactThreads)
-compact_kernel(ModelView mv, BatchView bv, const int *kept_idx, const int *out_len, TensorView cache_k,
-               TensorView cache_v, const int *cache_pos, TensorView chunk_k, TensorView chunk_v, const int *chunk_pos,
-               TensorView out_k, TensorView out_v, int *out_pos, int rows_per_cta, int *status) {
+compact_kernel(ModelView mv, BatchView bv, const int *kept_idx, const int *out_len, CompactTensors t, int rows_per_cta, int *status) {
     __shared__ int src_idx[kMaxRowsPerCta];
     dependency_wait();  // no early launch of the next kernel: this grid runs in many waves and needs every slot
     const int l = blockIdx.y / mv.Hkv, kvh = blockIdx.y - l * mv.Hkv, group = kvh / mv.kvpg;
@@ -197,28 +229,62 @@ compact_kernel(ModelView mv, BatchView bv, const int *kept_idx, const int *out_l
     if (i0 >= r) return;
     const int rows = min(rows_per_cta, r - i0);
     const int64_t unit_off = ((int64_t)u.l * mv.G + u.G) * bv.total_cache + u.cache0;
-    const bool leader = kvh == group * mv.kvpg;  // the group's positions are written by its first KV head's CTA
+    if (threadIdx.x < rows)
+        src_idx[threadIdx.x] = place_row<ROPE>(mv, u, t, unit_off, kvh == group * mv.kvpg, i0 + threadIdx.x,
+                                               kept_idx[unit_off + i0 + threadIdx.x], status);
+    __syncthreads();
+    move_rows<ROPE, kElems>(mv, u, kvh, i0, rows, src_idx, t, kCompactThreads);
+}
 
-    if (threadIdx.x < rows) {
-        int j = kept_idx[unit_off + i0 + threadIdx.x];
-        // with rotation a distance beyond the table (only possible when out_len exceeds the candidate count) is refused
-        if (j < 0 || j >= u.N || (ROPE && abs(i0 + (int)threadIdx.x - j) >= mv.rope_rows)) {
-            atomicOr(status, FINCH_DEV_BAD_INDEX);
-            j = -1;
-        } else if (leader) {
-            out_pos[unit_off + i0 + threadIdx.x] = j < u.c ? cache_pos[unit_off + j] : chunk_pos[u.chunk0 + j - u.c];
-        }
-        src_idx[threadIdx.x] = j;
+// Selection and copies in one launch, for steps whose copies are a single wave of CTAs: every CTA selects for its unit
+// (the scores come from L2) and copies its own block of the kept rows, so the kept indices need not travel through
+// global memory and a launch to reach the copies.  Bound by latency: one layer of 8 KV heads, whole step, 4096 candidates
+// 39.3 -> 35.2 us, 1024 candidates 24.0 -> 21.7, 512 candidates in fp32 17.4 -> 16.0; 9 layers of 944: 50.3 -> 46.5.
+constexpr int kPickThreads = 512;
+template <int ROPE, int kElems, int kItems>
+__global__ void __launch_bounds__(kPickThreads)
+select_compact_kernel(ModelView mv, BatchView bv, const float *scores, int *kept_idx, int *out_len, CompactTensors t,
+                      int rows_per_cta, int *status) {
+    __shared__ int src_idx[kMaxRowsPerCta];
+    dependency_wait();
+    dependents_may_launch();  // the whole grid is resident
+    const int l = blockIdx.y / mv.Hkv, kvh = blockIdx.y - l * mv.Hkv, group = kvh / mv.kvpg;
+    const UnitInfo u = unit_info(mv, bv, l * mv.G + group, blockIdx.z);
+    const bool leader = kvh == group * mv.kvpg;
+    pick::SelectUnit s;
+    if (!pick::select_unit(mv, bv, u, blockIdx.x == 0 && blockIdx.y == 0, scores, kept_idx, out_len, status, s)) return;
+    const int i0 = blockIdx.x * rows_per_cta, rows = min(rows_per_cta, s.r - i0);
+    if (rows <= 0) return;
+    if (s.r == s.N) {  // everything, in order
+        for (int i = threadIdx.x; i < rows; i += blockDim.x) src_idx[i] = i0 + i;
+    } else {
+        pick::select_largest<kItems>(s, [&](int rank, int j) {
+            if ((unsigned)(rank - i0) < (unsigned)rows) src_idx[rank - i0] = j;
+        });
     }
     __syncthreads();
+    const int64_t unit_off = ((int64_t)u.l * mv.G + u.G) * bv.total_cache + u.cache0;
+    if (leader || ROPE) {
+        for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+            const int j = src_idx[i], from = place_row<ROPE>(mv, u, t, unit_off, leader, i0 + i, j, status);
+            if (leader) s.kept[i0 + i] = j;
+            if (ROPE) src_idx[i] = from;
+        }
+    }
+    if (ROPE) __syncthreads();
+    move_rows<ROPE, kElems>(mv, u, kvh, i0, rows, src_idx, t, blockDim.x);
+}
 
-    const int pieces = mv.d * mv.elem_bytes / 16;  // 16-byte pieces per row
-    const RowMap k_rows(u, kvh, i0, mv.elem_bytes, cache_k, chunk_k, out_k);
-    if (ROPE)
-        rotate_rows<kElems, ROPE == 1>(k_rows, src_idx, rows, i0, mv.d, mv.elem_bytes, mv.rope_table);
-    else
-        copy_rows(k_rows, src_idx, rows, pieces);
-    copy_rows(RowMap(u, kvh, i0, mv.elem_bytes, cache_v, chunk_v, out_v), src_idx, rows, pieces);
+// The kernel of a rotation mode: f(mode, elements per 16 bytes).
+template <typename F>
+auto by_rotation(const ModelView &mv, const F &f) {
+    const bool f32 = mv.elem_bytes == 4;
+    using Std = std::integral_constant<int, 1>;
+    if (!(mv.rope_theta > 0.f)) return f(std::integral_constant<int, 0>(), std::integral_constant<int, 8>());
+    if (mv.rope_pairing == 0)
+        return f32 ? f(Std(), std::integral_constant<int, 4>()) : f(Std(), std::integral_constant<int, 8>());
+    return f32 ? f(std::integral_constant<int, 2>(), std::integral_constant<int, 4>())
+               : f(std::integral_constant<int, 2>(), std::integral_constant<int, 8>());
 }
 
 }  // namespace
@@ -236,12 +302,42 @@ cudaError_t launch_compact(const Ctx &ctx, const int *kept_idx, const int *out_l
     while (rows > kMinRowsPerCta && (int64_t)((bv.max_budget + rows - 1) / rows) * heads * bv.batch < 2 * sms) rows /= 2;
     dim3 grid((bv.max_budget + rows - 1) / rows, heads, bv.batch);
     ctx.launches += 1;
-    const bool f32 = mv.elem_bytes == 4;
-    auto kernel = compact_kernel<0, 8>;
-    if (mv.rope_theta > 0.f && mv.rope_pairing == 0) kernel = f32 ? compact_kernel<1, 4> : compact_kernel<1, 8>;
-    if (mv.rope_theta > 0.f && mv.rope_pairing == 1) kernel = f32 ? compact_kernel<2, 4> : compact_kernel<2, 8>;
-    return launch_chained(kernel, grid, dim3(kCompactThreads), 0, stream, mv, bv, kept_idx, out_len, cache_k, cache_v,
-                          cache_pos, chunk_k, chunk_v, chunk_pos, out_k, out_v, out_pos, rows, ctx.d_status);
+    const CompactTensors t{cache_k, cache_v, chunk_k, chunk_v, out_k, out_v, cache_pos, chunk_pos, out_pos};
+    return by_rotation(mv, [&](auto rope, auto elems) {
+        return launch_chained(compact_kernel<decltype(rope)::value, decltype(elems)::value>, grid, dim3(kCompactThreads), 0, stream,
+                              mv, bv, kept_idx, out_len, t, rows, ctx.d_status);
+    });
+}
+
+cudaError_t launch_select_compact(const Ctx &ctx, const float *scores, const TensorView &cache_k, const TensorView &cache_v,
+                                  const int *cache_pos, const TensorView &chunk_k, const TensorView &chunk_v,
+                                  const int *chunk_pos, const BatchView &bv, const TensorView &out_k, const TensorView &out_v,
+                                  int *out_pos, int *kept_idx, int *out_len, cudaStream_t stream) {
+    const ModelView &mv = ctx.model;
+    const int max_n = bv.max_cache + bv.max_chunk, heads = mv.L * mv.Hkv;
+    const int64_t sms = ctx.sm_count > 0 ? ctx.sm_count : 148, units = (int64_t)heads * bv.batch;
+    // Threads for the copies even where the selection needs fewer (96 threads: 57 us for a step of 43).  One wave: one
+    // CTA per SM, two of short units, down to blocks of kMinRowsPerCta rows (two CTAs of 512 threads per SM select twice
+    // as often for blocks of half the rows: 42 us against 35); larger steps keep the two launches, where a unit is
+    // selected once.
+    const int threads = max(kCompactThreads, pick::threads_for(max_n));
+    const int64_t slots = threads > kCompactThreads ? sms : 2 * sms;
+    int rows = kMaxRowsPerCta;
+    const auto ctas = [&](int n) { return units * ((bv.max_budget + n - 1) / n); };
+    while (rows > kMinRowsPerCta && ctas(rows / 2) <= slots) rows /= 2;
+    if (units == 0 || bv.max_budget == 0 || max_n > kPickThreads * 8 || ctas(rows) > slots) {
+        const cudaError_t e = launch_select(ctx, scores, bv, kept_idx, out_len, stream);
+        return e != cudaSuccess ? e : launch_compact(ctx, kept_idx, out_len, cache_k, cache_v, cache_pos, chunk_k, chunk_v,
+                                                     chunk_pos, bv, out_k, out_v, out_pos, stream);
+    }
+    ctx.launches += 1;
+    const CompactTensors t{cache_k, cache_v, chunk_k, chunk_v, out_k, out_v, cache_pos, chunk_pos, out_pos};
+    return by_rotation(mv, [&](auto rope, auto elems) {
+        constexpr int kRope = decltype(rope)::value, kElems = decltype(elems)::value;
+        return launch_chained(pick::items_for(max_n) == 4 ? select_compact_kernel<kRope, kElems, 4> : select_compact_kernel<kRope, kElems, 8>,
+                              dim3((unsigned)(ctas(rows) / units), heads, bv.batch), dim3(threads), 0, stream,
+                              mv, bv, scores, kept_idx, out_len, t, rows, ctx.d_status);
+    });
 }
 
 }  // namespace finch

@@ -363,10 +363,10 @@ finch_status finch_step(finch_ctx *ctx, const finch_tensor *prompt_q, const finc
     const BatchView bv = view_of(batch);
     cudaError_t e = run_score(*ctx, view_of(prompt_q), view_of(cache_k), view_of(chunk_k), bv, scores, row_stats,
                               w.lse_bytes / sizeof(float2), nullptr, stream);
-    if (e == cudaSuccess) e = launch_select(*ctx, scores, bv, kept_idx, out_len, stream);
     if (e == cudaSuccess)
-        e = launch_compact(*ctx, kept_idx, out_len, view_of(cache_k), view_of(cache_v), cache_pos, view_of(chunk_k),
-                           view_of(chunk_v), chunk_pos, bv, view_of(out_k), view_of(out_v), out_pos, stream);
+        e = launch_select_compact(*ctx, scores, view_of(cache_k), view_of(cache_v), cache_pos, view_of(chunk_k),
+                                  view_of(chunk_v), chunk_pos, bv, view_of(out_k), view_of(out_v), out_pos, kept_idx, out_len,
+                                  stream);
     return cuda_status(e);
 }
 

@@ -180,4 +180,10 @@ cudaError_t launch_compact(const Ctx &ctx, const int *kept_idx, const int *out_l
                            const TensorView &chunk_v, const int *chunk_pos, const BatchView &bv, const TensorView &out_k,
                            const TensorView &out_v, int *out_pos, cudaStream_t stream);
 
+// launch_select and launch_compact, in one kernel where the step is small.
+cudaError_t launch_select_compact(const Ctx &ctx, const float *scores, const TensorView &cache_k, const TensorView &cache_v,
+                                  const int *cache_pos, const TensorView &chunk_k, const TensorView &chunk_v,
+                                  const int *chunk_pos, const BatchView &bv, const TensorView &out_k, const TensorView &out_v,
+                                  int *out_pos, int *kept_idx, int *out_len, cudaStream_t stream);
+
 }  // namespace finch

@@ -160,3 +160,43 @@ def test_compact_row_blocks(L, Hkv, budget, rope_theta):
             assert np.all(np.abs(got - want) <= np.abs(want) * 2.0 ** -7 + 2e-6 * row)
     finally:
         fb.finch_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("rope_theta", [0.0, 10000.0])
+@pytest.mark.parametrize("layers,Hkv,reqs,dtype,group_mode,keep_all", [
+    (1, 8, [(16, 9999, 256, 256)], "f32", 0, False),       # blocks of 16 rows
+    (1, 8, [(20, 9999, 2048, 2048)], "bf16", 0, False),    # the longest unit that is selected beside its copies
+    (1, 8, [(20, 9999, 2049, 2048)], "bf16", 0, False),    # one candidate more: two launches
+    (8, 37, [(8, 9999, 70, 256)], "bf16", 0, False),       # 296 blocks of 256 rows
+    (8, 37, [(8, 9999, 70, 257)], "bf16", 0, False),       # a row more: two launches
+    (2, 4, [(9, 9999, 300, 77)], "bf16", 1, False),        # one selection group per layer
+    (1, 4, [(9, 9999, 33, 15), (5, 9999, 1, 90), (3, 9999, 64, 64)], "bf16", 0, False),
+    (2, 3, [(9, 9999, 90, 200)], "f32", 1, True),          # a budget that keeps everything
+])
+def test_step_that_selects_and_copies_in_one_launch(layers, Hkv, reqs, dtype, group_mode, keep_all, rope_theta):
+    """finch_step against the oracle and, bit for bit, against the three calls it stands for."""
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=Hkv, n_kv_heads=Hkv, head_dim=64, dtype=dtype,
+                    group_mode=group_mode, planted_frac=0.05, requests=tuple(wl.Request(*r) for r in reqs))
+    st = wl.steady_state(cfg, list(range(layers)), step=1)
+    if keep_all:
+        st["cache_len"] = st["cache_len"] - np.diff(st["chunk_off"]).astype(st["cache_len"].dtype)
+    runs = []
+    for parts in (False, True):
+        g = GpuStep(cfg, st, layers)
+        try:
+            if rope_theta:
+                c = g.batch.c
+                fb.finch_ctx_destroy(g.ctx)
+                g.ctx = fb.finch_ctx_create(layers, Hkv, Hkv, 64, fb.FINCH_F32 if dtype == "f32" else fb.FINCH_BF16, group_mode,
+                                            max_batch=len(reqs), max_prompt=c.max_q, max_candidates=c.max_cache + c.max_chunk,
+                                            rope_theta=rope_theta)
+            for _ in range(1 if parts else 2):
+                g.run_parts() if parts else g.run()
+            assert g.status() == 0
+            runs.append(g.results())
+        finally:
+            g.close()
+    for name in ("kept_idx", "out_len", "out_pos", "out_k", "out_v"):
+        np.testing.assert_array_equal(runs[0][name], runs[1][name], err_msg=name)
+    if not rope_theta:
+        check_parity(cfg, st, runs[0], oracle_scores(cfg, st, threads=oracle.max_threads()))
