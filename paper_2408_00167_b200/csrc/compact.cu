@@ -240,12 +240,12 @@ compact_kernel(ModelView mv, BatchView bv, const int *kept_idx, const int *out_l
 // (the scores come from L2) and copies its own block of the kept rows, so the kept indices need not travel through
 // global memory and a launch to reach the copies.  Bound by latency: one layer of 8 KV heads, whole step, 4096 candidates
 // 39.3 -> 35.2 us, 1024 candidates 24.0 -> 21.7, 512 candidates in fp32 17.4 -> 16.0; 9 layers of 944: 50.3 -> 46.5.
-constexpr int kPickThreads = 512;
+constexpr int kPickThreads = 512, kMaxRowsPicked = 512;
 template <int ROPE, int kElems, int kItems>
 __global__ void __launch_bounds__(kPickThreads)
 select_compact_kernel(ModelView mv, BatchView bv, const float *scores, int *kept_idx, int *out_len, CompactTensors t,
                       int rows_per_cta, int *status) {
-    __shared__ int src_idx[kMaxRowsPerCta];
+    __shared__ int src_idx[kMaxRowsPicked];
     dependency_wait();
     dependents_may_launch();  // the whole grid is resident
     const int l = blockIdx.y / mv.Hkv, kvh = blockIdx.y - l * mv.Hkv, group = kvh / mv.kvpg;
@@ -316,16 +316,19 @@ cudaError_t launch_select_compact(const Ctx &ctx, const float *scores, const Ten
     const ModelView &mv = ctx.model;
     const int max_n = bv.max_cache + bv.max_chunk, heads = mv.L * mv.Hkv;
     const int64_t sms = ctx.sm_count > 0 ? ctx.sm_count : 148, units = (int64_t)heads * bv.batch;
-    // Threads for the copies even where the selection needs fewer (96 threads: 57 us for a step of 43).  One wave: one
-    // CTA per SM, two of short units, down to blocks of kMinRowsPerCta rows (two CTAs of 512 threads per SM select twice
-    // as often for blocks of half the rows: 42 us against 35); larger steps keep the two launches, where a unit is
-    // selected once.
+    // Threads for the copies even where the selection needs fewer (96 threads: 57 us for a step of 43).  A unit's rows are
+    // cut evenly into as many blocks as give every SM a CTA, two of short units (two CTAs of 512 threads per SM select
+    // twice as often for blocks of half the rows: 42 us against 35); at most a wave, three CTAs of 256 threads per SM or
+    // one of more (256 units of 800 candidates: 76.5 -> 71 us; 1024 units, several waves: 196 -> 198).  Larger steps keep
+    // the two launches, where a unit is selected once and the copies run at the copy rate; so do steps scored in two
+    // launches, whose second sweep lets its successor in early: several of these CTAs would settle on the first free SMs
+    // (64 units of 1270 candidates: 75 -> 77 us).
     const int threads = max(kCompactThreads, pick::threads_for(max_n));
-    const int64_t slots = threads > kCompactThreads ? sms : 2 * sms;
-    int rows = kMaxRowsPerCta;
-    const auto ctas = [&](int n) { return units * ((bv.max_budget + n - 1) / n); };
-    while (rows > kMinRowsPerCta && ctas(rows / 2) <= slots) rows /= 2;
-    if (units == 0 || bv.max_budget == 0 || max_n > kPickThreads * 8 || ctas(rows) > slots) {
+    const bool small = threads == kCompactThreads;
+    const int most = (bv.max_budget + kMinRowsPerCta - 1) / kMinRowsPerCta, least = (bv.max_budget + kMaxRowsPicked - 1) / kMaxRowsPicked;
+    const int blocks = units > 0 ? max(least, (int)min((int64_t)most, (small ? 2 : 1) * sms / units)) : 0;
+    const bool early_in = score_tc_supported(ctx) && score_fused_window(ctx, bv) == 0;
+    if (blocks == 0 || early_in || max_n > kPickThreads * 8 || units * blocks > (small ? 3 : 1) * sms) {
         const cudaError_t e = launch_select(ctx, scores, bv, kept_idx, out_len, stream);
         return e != cudaSuccess ? e : launch_compact(ctx, kept_idx, out_len, cache_k, cache_v, cache_pos, chunk_k, chunk_v,
                                                      chunk_pos, bv, out_k, out_v, out_pos, stream);
@@ -335,8 +338,8 @@ cudaError_t launch_select_compact(const Ctx &ctx, const float *scores, const Ten
     return by_rotation(mv, [&](auto rope, auto elems) {
         constexpr int kRope = decltype(rope)::value, kElems = decltype(elems)::value;
         return launch_chained(pick::items_for(max_n) == 4 ? select_compact_kernel<kRope, kElems, 4> : select_compact_kernel<kRope, kElems, 8>,
-                              dim3((unsigned)(ctas(rows) / units), heads, bv.batch), dim3(threads), 0, stream,
-                              mv, bv, scores, kept_idx, out_len, t, rows, ctx.d_status);
+                              dim3(blocks, heads, bv.batch), dim3(threads), 0, stream,
+                              mv, bv, scores, kept_idx, out_len, t, (bv.max_budget + blocks - 1) / blocks, ctx.d_status);
     });
 }
 

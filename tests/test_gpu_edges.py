@@ -167,8 +167,8 @@ def test_compact_row_blocks(L, Hkv, budget, rope_theta):
     (1, 8, [(16, 9999, 256, 256)], "f32", 0, False),       # blocks of 16 rows
     (1, 8, [(20, 9999, 2048, 2048)], "bf16", 0, False),    # the longest unit that is selected beside its copies
     (1, 8, [(20, 9999, 2049, 2048)], "bf16", 0, False),    # one candidate more: two launches
-    (8, 37, [(8, 9999, 70, 256)], "bf16", 0, False),       # 296 blocks of 256 rows
-    (8, 37, [(8, 9999, 70, 257)], "bf16", 0, False),       # a row more: two launches
+    (12, 37, [(8, 9999, 70, 512)], "bf16", 0, False),      # 444 blocks of 512 rows
+    (12, 37, [(8, 9999, 70, 513)], "bf16", 0, False),       # a row more: two launches
     (2, 4, [(9, 9999, 300, 77)], "bf16", 1, False),        # one selection group per layer
     (1, 4, [(9, 9999, 33, 15), (5, 9999, 1, 90), (3, 9999, 64, 64)], "bf16", 0, False),
     (2, 3, [(9, 9999, 90, 200)], "f32", 1, True),          # a budget that keeps everything
