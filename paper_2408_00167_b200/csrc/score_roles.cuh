@@ -158,8 +158,8 @@ struct Producer {
     static constexpr int kSlabs = D / 64, kTileBytes = kSlabs * kSlabBytes;
     const Cta &c;
     const CUtensorMap *q_big, *q_small, *cache, *chunk;
-    int heads;        // query heads per unit
-    bool clear_pads;  // pad rows may hold another request's rows: clear them
+    int heads;    // query heads per unit
+    int total_q;  // query rows of the packed tensor
     int st = 0, ph = 0, kcnt = 0;
     uint32_t q_used = 0, q_ph = 0, raw_ph = 0;  // bit per query tile: loaded before / parity of its next q_free phase
 
@@ -196,10 +196,16 @@ struct Producer {
     }
     // The unit's query tiles into the ring's tiles base .., one at a time: a tile may be overwritten once the last MMAs on
     // its old contents are complete, while the MMAs on the tiles behind it still run.
-    __device__ bool load_queries(const UnitInfo &u, const Rows &R, int base) {
-        const bool clear = clear_pads && R.rp != R.n_q;
+    // Pad rows inside the tensor hold whatever lies behind the request's own rows: the next request's, or rows that another
+    // call uses.  (Behind the tensor's last row the copies deliver zeros.)  They weigh nothing, but a NaN among them, or a logit
+    // whose exponential overflows, would still reach this request's sums: they are cleared.
+    __device__ __forceinline__ bool load_queries(const UnitInfo &u, const Rows &R, int base) {
+        return R.rp != R.n_q && u.q0 + R.n_q < total_q ? load_tiles<true>(u, R, base) : load_tiles<false>(u, R, base);
+    }
+    template <bool CLEAR>
+    __device__ __forceinline__ bool load_tiles(const UnitInfo &u, const Rows &R, int base) {
         const bool leader = elect_one();
-        if (clear && leader) {
+        if (CLEAR && leader) {
             int rows = 0;
             for (int qb = 0; qb < R.n_qt; ++qb) rows += qb < R.n_qt - 1 ? kRows : (R.rows - qb * kRows) * (kRows / R.span);
             mbar_expect_tx(c.q_raw, rows * 128 * kSlabs);
@@ -212,16 +218,15 @@ struct Producer {
             }
             q_used |= 1u << tile;
             if (leader) {
-                uint64_t *bar = clear ? c.q_raw : &c.q_full[tile];
-                if (!clear) mbar_expect_tx(bar, n * copies * 128 * kSlabs);
+                uint64_t *bar = CLEAR ? c.q_raw : &c.q_full[tile];
+                if (!CLEAR) mbar_expect_tx(bar, n * copies * 128 * kSlabs);
                 for (int i = 0; i < copies; ++i) load_rows(u, R, R.r0 + r, R.r0 + r + n, tile * kRows + i * R.span, bar);
             }
         }
-        if (clear) {
-            // The pad rows between heads hold the next request's rows.  They weigh nothing, but a NaN among them would
-            // still reach this request's sums: zero them (the copies of a short last tile need none, lanes are skipped).
+        if (CLEAR) {
             if (!agree(mbar_wait(c.q_raw, raw_ph, c.abort_flag))) return false;
             raw_ph ^= 1;
+            // (the copies of a short last tile need none, their lanes are skipped)
             const int pads = R.rp - R.n_q, lane = threadIdx.x & 31;  // at most seven rows of 8 pieces per head and slab
             for (int h = R.r0 / R.rp; h * R.rp < R.r0 + R.rows; ++h)
                 for (int i = lane; i < pads * 8 * kSlabs; i += 32) {

@@ -200,3 +200,32 @@ def test_step_that_selects_and_copies_in_one_launch(layers, Hkv, reqs, dtype, gr
         np.testing.assert_array_equal(runs[0][name], runs[1][name], err_msg=name)
     if not rope_theta:
         check_parity(cfg, st, runs[0], oracle_scores(cfg, st, threads=oracle.max_threads()))
+
+
+@pytest.mark.parametrize("fill", [float("nan"), 3e4])
+@pytest.mark.parametrize("layers,n_q,extra,causal", [(1, 37, 3, False), (12, 9, 40, False), (1, 150, 1, False), (2, 37, 5, True)])
+def test_rows_behind_the_requests_reach_no_score(layers, n_q, extra, causal, fill):
+    """A query tensor with rows behind the last request's: they are no prompt rows, whatever they hold.  One kernel with one
+    window and with several, more than 512 padded rows, masked rows: bit for bit the scores of the tensor without them."""
+    import torch
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=16, n_kv_heads=4, head_dim=64, planted_frac=0.02,
+                    requests=(wl.Request(n_q, 9999, 300, 500),))
+    st = wl.steady_state(cfg, list(range(layers)), step=1)
+    limit = np.linspace(1, 800, n_q).astype(np.int32) if causal else None
+    g = GpuStep(cfg, st, layers, row_limit=limit)
+    try:
+        g.run_parts()
+        want, want_lse = g.scores.clone(), g.row_lse.clone()
+        g.q = torch.cat([g.q, torch.full_like(g.q[:, :, :1], fill).expand(-1, -1, extra, -1)], dim=2)
+        g.batch.c.total_q += extra
+        if causal:
+            g.batch.row_limit = torch.cat([g.batch.row_limit, torch.full_like(g.batch.row_limit[:1], 800).expand(extra)])
+            g.batch.c.row_limit = g.batch.row_limit.data_ptr()
+        g.row_lse = torch.zeros((layers, 16, n_q + extra), device="cuda")
+        g.ws = torch.empty(fb.finch_workspace_bytes(g.ctx, g.batch), dtype=torch.uint8, device="cuda")
+        g.run_parts()
+        assert g.status() == 0 and g.guards_intact()
+        np.testing.assert_array_equal(g.scores.cpu().numpy(), want.cpu().numpy())
+        np.testing.assert_array_equal(g.row_lse[:, :, :n_q].cpu().numpy(), want_lse.cpu().numpy())
+    finally:
+        g.close()
