@@ -225,7 +225,7 @@ __device__ __forceinline__ float2 merge_row_parts(const SimtParams &p, const Uni
             part[i] = i0 + i < p.splits ? p.parts[(i0 + i) * rows_total + row] : make_float2(-INFINITY, 0.f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            if (!(part[i].y > 0.f)) continue;  // a split that holds none of the row's keys
+            if (part[i].y == 0.f) continue;  // a split that holds none of the row's keys (a NaN sum is the whole row's)
             const float nmx = fmaxf(mx, part[i].x);
             sm = sm * exp2f(mx - nmx) + part[i].y * exp2f(part[i].x - nmx);
             mx = nmx;

@@ -229,3 +229,31 @@ def test_rows_behind_the_requests_reach_no_score(layers, n_q, extra, causal, fil
         np.testing.assert_array_equal(g.row_lse[:, :, :n_q].cpu().numpy(), want_lse.cpu().numpy())
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("d,dtype", [(64, "f32"), (96, "bf16")])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_a_key_that_is_no_number_voids_its_rows_whatever_the_key_split(d, dtype, bad):
+    """Warp-level scoring: a row whose sum is NaN weighs nothing, also where the bad key lies in one of several key splits."""
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=1, n_q_heads=2, n_kv_heads=2, head_dim=d, dtype=dtype, planted_frac=0.02,
+                    requests=(wl.Request(9, 9999, 200, 300),))
+    st = wl.steady_state(cfg, [0], step=1)
+    g = GpuStep(cfg, st, 1)
+    try:
+        g.run_parts()
+        want, want_lse = g.scores.cpu().numpy().copy(), g.row_lse.cpu().numpy().copy()
+        g.cache_k[0, 0, 100, 3] = bad
+        g.run_parts()
+        got, lse = g.scores.cpu().numpy(), g.row_lse.cpu().numpy()
+        assert g.status() == 0
+        np.testing.assert_array_equal(got[0, 1], want[0, 1])            # the other head
+        np.testing.assert_array_equal(lse[0, 1], want_lse[0, 1])
+        if np.isnan(bad):
+            assert np.all(np.isneginf(lse[0, 0])) and np.isnan(got[0, 0, 100])
+            assert np.all(np.delete(got[0, 0], 100) == 0)
+        else:                                                            # a logit of -inf is a weight of 0, one of +inf voids the row
+            up = st["q"][0, 0].reshape(9, d)[:, 3]
+            up = wl.from_storage(up, dtype) > 0
+            assert np.array_equal(np.isneginf(lse[0, 0]), up)
+    finally:
+        g.close()
