@@ -468,12 +468,6 @@ finch_status finch_device_status(finch_ctx *ctx, void *cuda_stream, int32_t *out
         (void)cudaGetLastError();
         return FINCH_ERR_CUDA;
     }
-    // a scoring kernel whose waits ran out leaves its counters behind: the next one needs them at zero
-    if (host && (cudaMemsetAsync(ctx->tickets, 0, 2 * (size_t)ctx->model.L * ctx->model.Hkv * sizeof(int), stream) != cudaSuccess ||
-                 cudaStreamSynchronize(stream) != cudaSuccess)) {
-        (void)cudaGetLastError();
-        return FINCH_ERR_CUDA;
-    }
     *out = host;
     return host ? FINCH_ERR_DEVICE_STATUS : FINCH_OK;
 }

@@ -21,8 +21,9 @@
 //     complete when phase B needs them, and one warp does the merging meanwhile.  With a single window per CTA (a
 //     layer at a time: the call is latency) all softmax warps merge at once.
 //
-// Tickets live in the context, start at zero and are set back to zero by the last range that has seen them complete.
+// Tickets live in the context and are zero between calls (tickets.h).
 #include "score_roles.cuh"
+#include "tickets.h"
 
 namespace finch {
 namespace {
@@ -36,7 +37,7 @@ struct FusedParams {
     ModelView mv;  // the scoring view: one unit per KV head
     BatchView bv;
     float2 *partial;     // [units][n_seg][kGroups][rows_alloc] (reference base-2 logit, sum exp2) per row and part
-    int *tickets;        // [2][units] ranges that have published their phase A / have seen all of them published
+    int *tickets;        // [2][units] the two counters of a unit
     float *row_lse;      // nullable
     float *unit_scores;  // [L][Hkv][cand]: the column sums of one KV head's query heads
     int *status;
@@ -208,6 +209,14 @@ __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInf
         stage_row(stats, row, live ? finish_row(p, u, R, row, M, Z, write_lse) : make_float2(0.f, 0.f));
 }
 
+// One window: the first softmax thread signs off for the CTA's range when its warp gives up.
+__device__ __noinline__ void give_up(int *published, int *left, int ranges, int unit, bool publish) {
+    if (threadIdx.x != kCtlWarps * 32) return;
+    const Tickets tickets{published, left, ranges};
+    if (publish) tickets.publish(unit);
+    tickets.leave(unit);
+}
+
 template <int D>
 __global__ void __launch_bounds__(kTcThreads, 1)
 score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant__ CUtensorMap q_small,
@@ -238,6 +247,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
     const int n_ranges = mv.L * mv.G * n_seg;
     const int n_win = run && (int)blockIdx.x < n_ranges ? (n_ranges - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     if (!u.ok && threadIdx.x == 0 && blockIdx.x == 0) atomicOr(p.status, FINCH_DEV_BAD_BATCH);
+    const Tickets tickets{p.tickets, p.tickets + mv.L * mv.G, n_seg};
     Walk walk{p.W, T, n_seg, p.delay, n_win, 0, 0};
     Seg sg;
     bool ok = true, left = false;
@@ -282,25 +292,21 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         // warps reach one phase A later.  Two buffers in turn: this warp cannot be two segments ahead, it waits for
         // the softmax warps' phase A in between.
         if (!direct) {
-            int segs = 0;
-            while (ok && walk.next(sg)) {
+            int segs = 0, good = 1;
+            while (walk.next(sg)) {
                 if (sg.sweep) continue;
                 ++segs;
                 FINCH_UNIT(sg);
-                int good = 1;
-                if (lane == 0) {
-                    good = count_wait(c.a_count, kSoftmaxWarps * segs, c.abort_flag);
-                    if (good) {
-                        __threadfence();  // cumulative: covers the softmax warps' stores this thread has synchronised with
-                        atomicAdd(&p.tickets[sg.unit], 1);
-                        good = ticket_wait(&p.tickets[sg.unit], n_seg, c.abort_flag);
-                    }
-                    if (good && atomicAdd(&p.tickets[mv.L * mv.G + sg.unit], 1) == n_seg - 1) {
-                        p.tickets[sg.unit] = 0;  // everyone has seen it: back to zero for the next call
-                        p.tickets[mv.L * mv.G + sg.unit] = 0;
-                    }
-                }
-                if (!__shfl_sync(0xffffffffu, good, 0)) break;
+                if (lane == 0)  // a range that gives up still signs off, and so do those behind it
+                    good = tickets.pass(
+                        sg.unit, good,
+                        [&]() {
+                            const bool written = count_wait(c.a_count, kSoftmaxWarps * segs, c.abort_flag);
+                            __threadfence();  // cumulative: covers the softmax warps' stores this thread has synchronised with
+                            return written;
+                        },
+                        [&](const int *ticket, int n) { return ticket_wait(ticket, n, c.abort_flag); });
+                if (!__shfl_sync(0xffffffffu, good, 0)) continue;
                 merge_by_warp(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats + ((segs - 1) & 1) * p.rows_alloc, lane);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&c.stats_ready[(segs - 1) & 1]);
@@ -327,7 +333,10 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         while (ok && walk.next(sg)) {
             if (sg.sweep == 0) {
                 Softmax<false>::RowStats st;
-                if (!(ok = role.lse_segment(u, R, sg.t0, sg.t1, live, no_limit, st))) break;
+                if (!(ok = role.lse_segment(u, R, sg.t0, sg.t1, live, no_limit, st))) {
+                    if (direct && p.cluster == 1) give_up(tickets.published, tickets.left, n_seg, sg.unit, true);
+                    break;
+                }
                 if (p.cluster > 1) {
                     // the unit's ranges are the CTAs of this cluster: the parts stay in shared memory, every warp tells
                     // every CTA that its own are written
@@ -365,21 +374,21 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
                     if (tid == 0) {
                         good = mbar_wait(&c.stats_ready[0], 0, c.abort_flag);
                         __threadfence();  // cumulative, as above
-                        if (good) atomicAdd(&p.tickets[sg.unit], 1);
+                        tickets.publish(sg.unit);
                     }
                     good = good && ticket_wait(&p.tickets[sg.unit], n_seg, c.abort_flag);
                 }
-                if (!(ok = __shfl_sync(0xffffffffu, good, 0))) break;
+                if (!(ok = __shfl_sync(0xffffffffu, good, 0))) {
+                    give_up(tickets.published, tickets.left, n_seg, sg.unit, false);
+                    break;
+                }
                 FINCH_UNIT(sg);
                 merge_by_cta(p, u, R, n_seg, sg.unit, sg.slot == 0, c.stats, tid, 0);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&c.stats_ready[1]);
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[1], 0, c.abort_flag)))) break;
-                // every warp of this CTA has seen the ticket complete
-                if (tid == 0 && atomicAdd(&p.tickets[mv.L * mv.G + sg.unit], 1) == n_seg - 1) {
-                    p.tickets[sg.unit] = 0;
-                    p.tickets[mv.L * mv.G + sg.unit] = 0;
-                }
+                ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[1], 0, c.abort_flag));
+                if (tid == 0) tickets.leave(sg.unit);  // every warp of this CTA has seen the ticket complete, or gives up
+                if (!ok) break;
             } else {
                 const int b = direct ? 0 : segs_b & 1;
                 if (!direct && !(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[b], (segs_b >> 1) & 1, c.abort_flag)))) break;
