@@ -195,10 +195,9 @@ finch_status finch_score_plan(const finch_ctx *ctx, const finch_batch *batch, in
  * GPU that loads the library, held until the process exits).  The call itself allocates and frees nothing.
  *  - Limit: n_layers * n_q_heads * total_q must not exceed finch_score_static_max_rows() (2^20 rows); a larger
  *    batch is rejected with FINCH_ERR_WORKSPACE_TOO_SMALL and nothing is enqueued -- use finch_score then.
- *  - Which kernels run: the tensor-core kernels need more of the array than one entry per prompt row (in 8-byte
- *    entries: four per query row and key range -- rows counted with a KV head's heads padded to multiples of 8 and
- *    their total to a multiple of 128 -- and 2 per layer, KV head and candidate).  A batch within the row limit whose
- *    need exceeds the array's 2^20 entries -- a whole 32-layer step of 4096 candidates does -- runs on the warp-level
+ *  - Which kernels run: the tensor-core kernels take a batch (bf16, head_dim 64 or 128) whose need of 8-byte entries -- five
+ *    per prompt row and two per layer, KV head and candidate -- fits the array's 2^20.  A batch within the row limit
+ *    that needs more -- a whole 32-layer step of 4096 candidates does -- runs on the warp-level
  *    kernels instead: the same result within the score tolerance, many times slower.  finch_score_static_path
  *    tells which it will be.  Because the kernels (or their key ranges) can differ from finch_score's, the two
  *    calls agree within the score tolerance, max(1e-3 relative, 1e-5 absolute), not bit for bit.
@@ -216,8 +215,8 @@ finch_status finch_score_static(finch_ctx *ctx, const finch_tensor *prompt_q, co
 size_t finch_score_static_max_rows(void);
 
 /* Host arithmetic, nothing is enqueued: *tensor_cores = 1 when finch_score_static would run this batch on the
- * tensor-core kernels (bf16, head_dim 64 or 128, and the batch's scratch fits the built-in array), 0 when it would
- * take the warp-level kernels.  (The paper has no counterpart.)  A batch whose tensors the TMA unit cannot describe
+ * tensor-core kernels (bf16, head_dim 64 or 128, and the batch's need fits the built-in array, see above), 0 when it
+ * would take the warp-level kernels.  (The paper has no counterpart.)  A batch whose tensors the TMA unit cannot describe
  * (an outer stride of 2^40 bytes or more) takes the warp-level kernels regardless. */
 finch_status finch_score_static_path(const finch_ctx *ctx, const finch_batch *batch, int32_t *tensor_cores);
 

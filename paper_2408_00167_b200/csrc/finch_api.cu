@@ -488,11 +488,59 @@ namespace {
 constexpr size_t kStaticRows = size_t(1) << 20;  // prompt rows (layers x query heads x packed prompt tokens): 8 MiB
 static __device__ __align__(256) float2 g_static_row_stats[kStaticRows];
 
-// How much of the array the tensor-core kernels may use for a batch: two entries per layer, KV head and candidate are
-// set aside, which keeps batches of very many candidates on the warp-level kernels (their scratch is a row's entry).
-size_t static_tc_capacity(const finch_ctx *ctx, const finch_batch *b) {
-    const size_t cand = (size_t)ctx->model.L * ctx->model.Hkv * ((size_t)b->total_cache + b->total_chunk);
-    return 2 * cand < kStaticRows ? kStaticRows - 2 * cand : 0;
+// Which kernels a batch takes here.  The tensor-core kernels take it if five entries per prompt row and two per layer, KV head
+// and candidate fit the array; their scratch (whole query tiles of partial statistics) can be larger than that for short
+// prompts, and they then work on some layers, or some requests of one layer, at a time.  9 layers of 32 heads, 6 prompt rows,
+// 1671 candidates: 77 us; the warp-level kernels take 426 us.
+struct StaticPlan {
+    int layers, requests;  // of a launch; 0: the warp-level kernels
+};
+StaticPlan static_plan(const finch_ctx *ctx, const finch_batch *b) {
+    const ModelView &mv = ctx->model;
+    const size_t rows = (size_t)mv.L * mv.Hq * (size_t)b->total_q;
+    const size_t cand = (size_t)mv.L * mv.Hkv * ((size_t)b->total_cache + b->total_chunk);
+    if (!score_tc_supported(*ctx) || 5 * rows + 2 * cand + (size_t)b->batch + 513 > kStaticRows) return {0, 0};
+    Ctx part = *ctx;
+    BatchView bv = view_of(b);
+    const size_t fused = score_fused_scratch(part, bv);
+    while ((fused == 0 || fused > kStaticRows) && score_tc_scratch_min(part, bv) > kStaticRows) {
+        if (part.model.L > 1)
+            part.model.L = (part.model.L + 1) / 2;
+        else if (bv.batch > 1)
+            bv.batch = (bv.batch + 1) / 2;
+        else
+            return {0, 0};
+    }
+    return {part.model.L, bv.batch};
+}
+
+// The two-launch tensor-core kernels on `plan.layers` layers and `plan.requests` requests at a time, one after the other in the
+// same scratch.
+cudaError_t score_static_parts(const Ctx &ctx, const StaticPlan &plan, const TensorView &q, const TensorView &cache_k,
+                               const TensorView &chunk_k, const BatchView &bv, float *scores, float2 *scratch, float *row_lse,
+                               cudaStream_t stream) {
+    const ModelView &mv = ctx.model;
+    const size_t cand = (size_t)bv.total_cache + bv.total_chunk, rows = (size_t)mv.Hq * bv.total_q;
+    Ctx part = ctx;
+    cudaError_t e = cudaSuccess;
+    for (int l = 0; l < mv.L && e == cudaSuccess; l += plan.layers) {
+        part.model.L = mv.L - l < plan.layers ? mv.L - l : plan.layers;
+        auto from_layer = [&](TensorView t) {
+            if (t.ptr) t.ptr += (int64_t)l * t.stride_layer * mv.elem_bytes;
+            return t;
+        };
+        for (int b = 0; b < bv.batch && e == cudaSuccess; b += plan.requests) {
+            BatchView some = bv;
+            some.batch = bv.batch - b < plan.requests ? bv.batch - b : plan.requests;
+            some.q_off += b, some.chunk_off += b, some.cache_off += b, some.cache_len += b, some.budget += b;
+            if (some.self_lse) some.self_lse += l * rows;
+            e = launch_score_tc(part, from_layer(q), from_layer(cache_k), from_layer(chunk_k), some, scores + l * mv.G * cand,
+                                scratch, kStaticRows, row_lse ? row_lse + l * rows : nullptr, stream);
+        }
+    }
+    ctx.launches = part.launches;
+    ctx.smem_bits = part.smem_bits;
+    return e;
 }
 
 constexpr int kMaxDevices = 64;
@@ -534,15 +582,20 @@ extern "C" finch_status finch_score_static(finch_ctx *ctx, const finch_tensor *p
     if (ctx->dry) return FINCH_ERR_UNSUPPORTED;
     float2 *row_stats = nullptr;
     if ((s = static_scratch(ctx->cfg.device, &row_stats))) return s;
-    return cuda_status(run_score(*ctx, view_of(prompt_q), view_of(cache_k), view_of(chunk_k), view_of(batch), scores,
-                                 row_stats, static_tc_capacity(ctx, batch), row_lse, (cudaStream_t)cuda_stream));
+    const TensorView q = view_of(prompt_q), ck = view_of(cache_k), hk = view_of(chunk_k);
+    const BatchView bv = view_of(batch);
+    cudaStream_t stream = (cudaStream_t)cuda_stream;
+    const StaticPlan plan = static_plan(ctx, batch);
+    if (plan.layers == ctx->model.L && plan.requests == batch->batch)
+        return cuda_status(run_score(*ctx, q, ck, hk, bv, scores, row_stats, kStaticRows, row_lse, stream));
+    cudaError_t e = cudaErrorNotSupported;
+    if (plan.layers) e = score_static_parts(*ctx, plan, q, ck, hk, bv, scores, row_stats, row_lse, stream);
+    if (e == cudaErrorNotSupported) e = launch_score_simt(*ctx, q, ck, hk, bv, scores, row_stats, kStaticRows, row_lse, stream);
+    return cuda_status(e);
 }
 
 extern "C" size_t finch_score_static_max_rows(void) { return kStaticRows; }
 
-// Which kernels finch_score_static runs for a batch: the tensor-core kernels keep more than one entry per prompt row
-// in the scratch (statistics per key range and softmax group, partial column sums per candidate), so a batch can
-// fit the array's row limit and still be too large for them; it then takes the warp-level kernels.
 // Which kernels finch_score / finch_step run for a batch (workspace of finch_workspace_bytes): see the header.
 extern "C" finch_status finch_score_plan(const finch_ctx *ctx, const finch_batch *batch, int32_t *path, int32_t *window) {
     if (!path) return FINCH_ERR_INVALID_ARG;
@@ -559,9 +612,6 @@ extern "C" finch_status finch_score_static_path(const finch_ctx *ctx, const finc
     if (!tensor_cores) return FINCH_ERR_INVALID_ARG;
     finch_status s = check_batch(ctx, batch);
     if (s) return s;
-    const BatchView bv = view_of(batch);
-    const size_t fused = score_fused_scratch(*ctx, bv), capacity = static_tc_capacity(ctx, batch);
-    *tensor_cores = score_tc_supported(*ctx) &&
-                    ((fused > 0 && fused <= capacity) || score_tc_scratch_min(*ctx, bv) <= capacity);
+    *tensor_cores = static_plan(ctx, batch).layers > 0;
     return FINCH_OK;
 }

@@ -104,3 +104,59 @@ def test_static_scratch_rejects_batches_beyond_its_size():
         assert call(limit // (32 * 32) + 1) == fb.FINCH_ERR_WORKSPACE_TOO_SMALL
     finally:
         fb.finch_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("L,Hkv,g,B,p,cache,chunk,tensor_cores", [
+    (9, 32, 2, 1, 6, 590, 1081, True),          # a short prompt: whole query tiles of statistics for few rows
+    (11, 32, 1, 1, 8, 981, 426, True),
+    (64, 32, 1, 1, 8, 100, 100, True),          # more than the array holds at once: some layers at a time
+    (1, 64, 1, 40, 2, 3, 1, True),              # some requests of a layer at a time
+    (24, 4, 4, 16, 2, 28, 78, True),
+    (32, 8, 4, 1, 128, 2048, 2048, False),      # two entries per candidate do not fit
+    (32, 8, 4, 1, 205, 10, 10, False),          # 5 x 32 x 32 x 205 entries for the rows
+])
+def test_static_scratch_takes_the_tensor_cores_by_rows_and_candidates(L, Hkv, g, B, p, cache, chunk, tensor_cores):
+    """Host arithmetic: five entries per prompt row and two per layer, KV head and candidate."""
+    need = 5 * L * Hkv * g * B * p + 2 * L * Hkv * B * (cache + chunk) + B + 513
+    assert (need <= fb.finch_score_static_max_rows()) is tensor_cores
+    ctx = fb.finch_ctx_create(L, Hkv * g, Hkv, 64, fb.FINCH_BF16, max_batch=B, max_prompt=p, max_candidates=cache + chunk, device=-1)
+    try:
+        off = lambda n: [n * i for i in range(B + 1)]
+        batch = fb.make_batch(off(p), off(chunk), off(cache), [cache] * B, [cache] * B, device="cpu")
+        assert fb.finch_score_static_path(ctx, batch) is tensor_cores
+    finally:
+        fb.finch_ctx_destroy(ctx)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("L,Hkv,reqs,group_mode,self_term", [
+    (65, 32, [(8, 9999, 100, 60)], 0, True),                                    # 33 + 32 layers
+    (70, 32, [(5, 9999, 40, 70)], 1, False),
+    (1, 64, [(1 + i % 2, 9999, 1 + i % 3, 5) for i in range(40)], 0, False),   # 20 + 20 requests
+])
+def test_static_scratch_in_parts_returns_what_the_workspace_call_returns(L, Hkv, reqs, group_mode, self_term):
+    """Statistics that the array cannot hold at once: layers, or the requests of a layer, one part after the other."""
+    import torch
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=L, n_q_heads=Hkv, n_kv_heads=Hkv, head_dim=64, planted_frac=0.02,
+                    group_mode=group_mode, requests=tuple(wl.Request(*r) for r in reqs))
+    st = wl.steady_state(cfg, list(range(L)), step=1)
+    lse = None
+    if self_term:
+        lse = np.random.default_rng(0).normal(3.0, 1.0, (L, Hkv, int(st["q_off"][-1]))).astype(np.float32)
+    g = GpuStep(cfg, st, L, prompt_self_lse=lse)
+    try:
+        assert fb.finch_score_static_path(g.ctx, g.batch)
+        fb.finch_score(g.ctx, g.q, g.cache_k, g.chunk_k, g.batch, g.scores, g.row_lse, g.ws)
+        got, got_lse = torch.full_like(g.scores, float("nan")), torch.full_like(g.row_lse, float("nan"))
+        before = fb.finch_launch_count(g.ctx)
+        fb.finch_score_static(g.ctx, g.q, g.cache_k, g.chunk_k, g.batch, got, got_lse)
+        assert g.status() == 0
+        per_part = 3 + (len(reqs) > 1) + (group_mode == 1)
+        assert fb.finch_launch_count(g.ctx) - before == 2 * per_part
+        w, x = g.scores.cpu().numpy(), got.cpu().numpy()
+        valid = ~np.isnan(w)                                    # entries behind a request's candidates stay as they were
+        assert np.array_equal(valid, ~np.isnan(x))
+        assert np.all(np.abs(x[valid] - w[valid]) <= np.maximum(REL_TOL * np.abs(w[valid]), ABS_TOL))
+        np.testing.assert_allclose(got_lse.cpu().numpy(), g.row_lse.cpu().numpy(), rtol=1e-5, atol=1e-5)
+    finally:
+        g.close()
