@@ -22,7 +22,7 @@ namespace tc {
 
 struct Cta {  // shared memory of the CTA
     uint8_t *q_res, *ring;
-    uint64_t *q_raw;                   // queries have landed, their pad rows are still to be cleared
+    uint64_t *q_raw;                   // [kQTiles] a query tile has landed, its pad rows are still to be cleared
     uint64_t *q_full, *q_free;         // [kQTiles] query tile has landed / its last MMAs are complete
     uint64_t *full, *empty;            // [kMaxStages] key ring
     uint64_t *acc_full, *acc_empty;    // [kGroups] accumulators
@@ -69,7 +69,7 @@ __device__ __forceinline__ Cta cta_layout(uint8_t *raw, int tile_bytes, int q_ti
     c.stats_ready = b, b += 2;
     c.sum_full = b, b += kSumBufs;
     c.sum_empty = b, b += kSumBufs;
-    c.q_raw = b, b += 1;
+    c.q_raw = b, b += kQTiles;
     c.parts_ready = b, b += 1;
     c.tmem_slot = (uint32_t *)b;
     c.abort_flag = (volatile int *)(c.tmem_slot + 1);
@@ -86,6 +86,7 @@ __device__ __forceinline__ Cta cta_layout(uint8_t *raw, int tile_bytes, int q_ti
 __device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals, int cluster = 1) {
     if (threadIdx.x == 0) {
         for (int i = 0; i < kQTiles; ++i) {
+            mbar_init(&c.q_raw[i], 1);
             mbar_init(&c.q_full[i], 1);
             mbar_init(&c.q_free[i], 1);
         }
@@ -102,7 +103,6 @@ __device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals, 
             mbar_init(&c.sum_full[i], 4);
             mbar_init(&c.sum_empty[i], 1);
         }
-        mbar_init(c.q_raw, 1);
         mbar_init(c.parts_ready, cluster * kSoftmaxWarps);
         *c.abort_flag = 0;
         *c.a_count = 0;
@@ -152,16 +152,53 @@ struct TileRing {
 };
 
 // ------------------------------------------------------------------------------------------------ producer
-// Run by a whole warp, one elected lane issuing.
+// Pad rows that lie inside the query tensor hold whatever comes behind the request's own rows: the next request's, or rows that
+// another call uses.  (Behind the tensor's last row the copies deliver zeros.)  They weigh nothing, but a NaN among them, or a
+// logit whose exponential overflows, would still reach this request's sums: they are cleared between the copy and the MMAs.
+__device__ __forceinline__ bool pads_hold_rows(const UnitInfo &u, const Rows &R, int total_q) {
+    return R.rp != R.n_q && u.q0 + R.n_q < total_q;
+}
+
+// Run by a whole warp: clears the pad rows of query tiles as they land and hands them to the MMAs.  In the two-launch kernels
+// by a warp of its own, so that the producer runs on to the next unit's queries (31 requests of up to 3 rows and 56 candidates
+// on 29 x 8 units: 610 us with the producer waiting for every unit's rows, 412 with this).
 template <int D>
+struct PadCleaner {
+    static constexpr int kSlabs = D / 64;
+    const Cta &c;
+    uint32_t ph = 0;  // bit per query tile: parity of its next q_raw phase
+    __device__ bool clear(const Rows &R, int base) {
+        const int pads = R.rp - R.n_q, lane = threadIdx.x & 31;  // at most seven rows of 8 pieces per head and slab
+        for (int qb = 0; qb < R.n_qt; ++qb) {
+            const int tile = base + qb, r0 = R.r0 + qb * kRows, r1 = min(r0 + kRows, R.r0 + R.rows);  // padded rows of the unit
+            if (!__all_sync(0xffffffffu, mbar_wait(&c.q_raw[tile], ph >> tile & 1u, c.abort_flag))) return false;
+            ph ^= 1u << tile;
+            // (the copies of a short last tile need no clearing, their lanes are skipped)
+            for (int h = r0 / R.rp; h * R.rp < r1; ++h)
+                for (int i = lane; i < pads * 8 * kSlabs; i += 32) {
+                    const int s = i / (pads * 8), k = i - s * pads * 8, r = h * R.rp + R.n_q + k / 8;
+                    if (r >= r0 && r < r1)
+                        *(uint4 *)(c.q_res + s * c.q_slab + (tile * kRows + r - r0) * 128 + k % 8 * 16) = uint4{0, 0, 0, 0};
+                }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&c.q_full[tile]);
+        }
+        return true;
+    }
+};
+
+// Run by a whole warp, one elected lane issuing.  OWN_WARP: the PadCleaner is a warp of its own.
+template <int D, bool OWN_WARP>
 struct Producer {
     static constexpr int kSlabs = D / 64, kTileBytes = kSlabs * kSlabBytes;
     const Cta &c;
     const CUtensorMap *q_big, *q_small, *cache, *chunk;
     int heads;    // query heads per unit
     int total_q;  // query rows of the packed tensor
+    PadCleaner<D> cleaner{c};
     int st = 0, ph = 0, kcnt = 0;
-    uint32_t q_used = 0, q_ph = 0, raw_ph = 0;  // bit per query tile: loaded before / parity of its next q_free phase
+    uint32_t q_used = 0, q_ph = 0;  // bit per query tile: loaded before / parity of its next q_free phase
 
     __device__ __forceinline__ bool agree(bool ok) { return __all_sync(0xffffffffu, ok); }
     __device__ bool load_key_tile(const UnitInfo &u, int t) {
@@ -196,20 +233,13 @@ struct Producer {
     }
     // The unit's query tiles into the ring's tiles base .., one at a time: a tile may be overwritten once the last MMAs on
     // its old contents are complete, while the MMAs on the tiles behind it still run.
-    // Pad rows inside the tensor hold whatever lies behind the request's own rows: the next request's, or rows that another
-    // call uses.  (Behind the tensor's last row the copies deliver zeros.)  They weigh nothing, but a NaN among them, or a logit
-    // whose exponential overflows, would still reach this request's sums: they are cleared.
+    // RAW: a PadCleaner stands between the copies and the MMAs.
     __device__ __forceinline__ bool load_queries(const UnitInfo &u, const Rows &R, int base) {
-        return R.rp != R.n_q && u.q0 + R.n_q < total_q ? load_tiles<true>(u, R, base) : load_tiles<false>(u, R, base);
+        return pads_hold_rows(u, R, total_q) ? load_tiles<true>(u, R, base) : load_tiles<false>(u, R, base);
     }
-    template <bool CLEAR>
+    template <bool RAW>
     __device__ __forceinline__ bool load_tiles(const UnitInfo &u, const Rows &R, int base) {
         const bool leader = elect_one();
-        if (CLEAR && leader) {
-            int rows = 0;
-            for (int qb = 0; qb < R.n_qt; ++qb) rows += qb < R.n_qt - 1 ? kRows : (R.rows - qb * kRows) * (kRows / R.span);
-            mbar_expect_tx(c.q_raw, rows * 128 * kSlabs);
-        }
         for (int qb = 0; qb < R.n_qt; ++qb) {
             const int tile = base + qb, r = qb * kRows, n = min(kRows, R.rows - r), copies = qb < R.n_qt - 1 ? 1 : kRows / R.span;
             if (q_used >> tile & 1u) {
@@ -218,28 +248,12 @@ struct Producer {
             }
             q_used |= 1u << tile;
             if (leader) {
-                uint64_t *bar = CLEAR ? c.q_raw : &c.q_full[tile];
-                if (!CLEAR) mbar_expect_tx(bar, n * copies * 128 * kSlabs);
+                uint64_t *bar = RAW ? &c.q_raw[tile] : &c.q_full[tile];
+                mbar_expect_tx(bar, n * copies * 128 * kSlabs);
                 for (int i = 0; i < copies; ++i) load_rows(u, R, R.r0 + r, R.r0 + r + n, tile * kRows + i * R.span, bar);
             }
         }
-        if (CLEAR) {
-            if (!agree(mbar_wait(c.q_raw, raw_ph, c.abort_flag))) return false;
-            raw_ph ^= 1;
-            // (the copies of a short last tile need none, their lanes are skipped)
-            const int pads = R.rp - R.n_q, lane = threadIdx.x & 31;  // at most seven rows of 8 pieces per head and slab
-            for (int h = R.r0 / R.rp; h * R.rp < R.r0 + R.rows; ++h)
-                for (int i = lane; i < pads * 8 * kSlabs; i += 32) {
-                    const int s = i / (pads * 8), k = i - s * pads * 8, r = h * R.rp + R.n_q + k / 8 - R.r0;
-                    if (r >= 0 && r < R.rows)
-                        *(uint4 *)(c.q_res + s * c.q_slab + (base * kRows + r) * 128 + k % 8 * 16) = uint4{0, 0, 0, 0};
-                }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (leader)
-                for (int qb = 0; qb < R.n_qt; ++qb) mbar_arrive(&c.q_full[base + qb]);
-        }
-        return true;
+        return !RAW || OWN_WARP || cleaner.clear(R, base);
     }
     // One segment; base: the ring tiles its queries are to be loaded into, or -1: they are resident.
     __device__ bool segment(const UnitInfo &u, const Rows &R, int t0, int t1, int base) {

@@ -131,8 +131,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant
     // Barriers and tensor memory are set up; what follows reads what earlier kernels of the stream wrote.  The
     // second sweep's loads and MMAs read only the step's inputs, which were complete before the first sweep began;
     // what its immediate predecessors produce (the merged row statistics) is read by the softmax warps alone, so
-    // only they wait, and the tensor pipe already fills the accumulators while the statistics are being merged.
-    if (MODE == kLse || warp >= 2) {
+    // only they (and the writer of the scores) wait, and the tensor pipe already fills the accumulators while the
+    // statistics are being merged.
+    if (MODE == kLse || warp >= 3) {
         dependency_wait();
         dependents_may_launch();
     }
@@ -153,7 +154,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant
             prefetch_tensormap(&chunk_map);
         }
         __syncwarp();
-        Producer<D> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q};
+        Producer<D, true> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q};
         while (ok && walk.next(s, false, lane == 0)) {
             ok = role.segment(s.u, s.R, s.t0, s.t1, q_key != s.q_key ? ring.take(s.R.n_qt) : -1);
             q_key = s.q_key;
@@ -173,6 +174,14 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant
             if (reload) base = ring.take(R.n_qt);
             ok = MODE == kLse ? role.lse_segment(R, t0, t1, base, reload, release)
                               : role.colsum_segment(R, t0, t1, base, reload, release);
+        }
+    } else if (warp == 2) {
+        PadCleaner<D> role{c};
+        while (ok && walk.next(s, false, false)) {
+            if (q_key == s.q_key) continue;
+            q_key = s.q_key;
+            const int base = ring.take(s.R.n_qt);
+            if (pads_hold_rows(s.u, s.R, bv.total_q)) ok = role.clear(s.R, base);
         }
     } else if (warp == 3) {
         if (MODE == kColsum) {

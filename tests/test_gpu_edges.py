@@ -257,3 +257,31 @@ def test_a_key_that_is_no_number_voids_its_rows_whatever_the_key_split(d, dtype,
             assert np.array_equal(np.isneginf(lse[0, 0]), up)
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("heads,rows", [(1, 23), (4, 9), (2, 70)])
+def test_many_small_requests_do_not_see_their_neighbours(heads, rows):
+    """Units of one or two query tiles and a few key tiles, many to a CTA; NaN in every third request's queries."""
+    import torch
+    rng = np.random.default_rng(rows)
+    reqs = [wl.Request(int(rng.integers(1, rows + 1)), 9999, int(rng.integers(1, 140)), int(rng.integers(1, 140))) for _ in range(41)]
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=3, n_q_heads=4 * heads, n_kv_heads=4, head_dim=128, planted_frac=0.05,
+                    requests=tuple(reqs))
+    st = wl.steady_state(cfg, [0, 1, 2], step=1)
+    g = GpuStep(cfg, st, 3)
+    try:
+        g.run_parts()
+        assert g.status() == 0
+        res = g.results()
+        check_parity(cfg, st, res, oracle_scores(cfg, st, threads=oracle.max_threads()))
+        for b in range(0, 41, 3):
+            g.q[:, :, int(st["q_off"][b]):int(st["q_off"][b + 1])] = float("nan")
+        g.run_parts()
+        got = g.scores.cpu().numpy()
+        for b in range(41):
+            if b % 3:
+                lo = int(st["cache_off"][b] + st["chunk_off"][b])
+                hi = lo + int(st["cache_len"][b] + st["chunk_off"][b + 1] - st["chunk_off"][b])
+                np.testing.assert_array_equal(got[:, :, lo:hi], res["scores"][:, :, lo:hi], err_msg=f"request {b}")
+    finally:
+        g.close()
