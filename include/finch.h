@@ -150,8 +150,8 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out);
 void finch_ctx_destroy(finch_ctx *ctx);
 
 /* Bytes of device workspace that finch_score / finch_select / finch_step need for this batch (the maximum over
- * the three; finch_step includes room for the scores when the caller passes scores == NULL).  Pure host
- * arithmetic: callable without touching the device. */
+ * the three; finch_step includes room for the scores when the caller passes scores == NULL).  Enough as well for every
+ * batch whose bounds (batch, total_*, max_*) are no larger.  Pure host arithmetic: callable without touching the device. */
 finch_status finch_workspace_bytes(const finch_ctx *ctx, const finch_batch *batch, size_t *out);
 
 /* Prompt-guided scoring (Method, bullets "Sum over heads", "Extract prompt-guided submatrix", "Selection of top r

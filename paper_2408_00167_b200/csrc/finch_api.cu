@@ -296,7 +296,13 @@ finch_status finch_workspace_bytes(const finch_ctx *ctx, const finch_batch *batc
     if (!out) return FINCH_ERR_INVALID_ARG;
     finch_status s = check_batch(ctx, batch);
     if (s) return s;
-    *out = ws_layout(ctx, batch).total;
+    // A caller may size its workspace once, for the largest batch it will pass: what the calls ask for is not monotone (fewer
+    // key tiles can mean more ranges of a unit), what is reported here is.
+    WsLayout w = ws_layout(ctx, batch);
+    const BatchView bv = view_of(batch);
+    const size_t fused = score_fused_scratch_bound(*ctx, bv), two = score_tc_supported(*ctx) ? score_tc_scratch_bound(*ctx, bv) : 0;
+    const size_t bound = align_up((fused > two ? fused : two) * sizeof(float2));
+    *out = w.total + (bound > w.lse_bytes ? bound - w.lse_bytes : 0);
     return FINCH_OK;
 }
 

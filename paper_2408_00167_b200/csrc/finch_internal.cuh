@@ -149,6 +149,7 @@ cudaError_t launch_score_simt(const Ctx &ctx, const TensorView &q, const TensorV
 constexpr int kScoreMaxSplits = 8;
 bool score_tc_supported(const Ctx &ctx);
 size_t score_tc_scratch(const Ctx &ctx, const BatchView &bv);      // what it would like
+size_t score_tc_scratch_bound(const Ctx &ctx, const BatchView &bv);  // .. and would for any batch within the same bounds
 size_t score_tc_scratch_min(const Ctx &ctx, const BatchView &bv);  // least scratch (float2) of the two-launch path
 cudaError_t launch_score_tc(const Ctx &ctx, const TensorView &q, const TensorView &cache_k, const TensorView &chunk_k,
                             const BatchView &bv, float *scores, float2 *partial, size_t partial_capacity,
@@ -161,6 +162,7 @@ cudaError_t launch_sum_heads(const Ctx &ctx, const ModelView &mv, const BatchVie
 // both sweeps in one persistent kernel (single-request batches without a row mask whose query rows fit the shared
 // memory): score_fused_scratch gives the float2 entries of scratch it needs, 0 when it does not take the batch
 size_t score_fused_scratch(const Ctx &ctx, const BatchView &bv);
+size_t score_fused_scratch_bound(const Ctx &ctx, const BatchView &bv);  // the most that any batch within the same bounds needs
 int score_fused_window(const Ctx &ctx, const BatchView &bv);  // key tiles per window; 0: the batch goes elsewhere
 cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const TensorView &cache_k, const TensorView &chunk_k,
                                const BatchView &bv, float *scores, float2 *scratch, size_t scratch_capacity,

@@ -540,19 +540,31 @@ int score_fused_window(const Ctx &ctx, const BatchView &bv) {
 }
 
 namespace {
-size_t scratch_of(const ModelView &mv, const BatchView &bv, int W) {
-    const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
+size_t scratch_of(const ModelView &mv, const BatchView &bv, int n_seg) {
     const size_t units = (size_t)mv.L * mv.Hkv, cand = (size_t)bv.total_cache + bv.total_chunk;
-    size_t n = units * ((tiles + W - 1) / W) * kGroups * rows_alloc_of(mv, bv);  // partial row statistics
+    size_t n = units * n_seg * kGroups * rows_alloc_of(mv, bv);  // partial row statistics
     if (mv.G != mv.Hkv) n += (units * cand + 1) / 2;  // per-KV-head sums of a selection group that spans several
     return n;
 }
+int tiles_of(const BatchView &bv) { return (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows; }
 }  // namespace
+
+// The most that any batch within these bounds needs: a unit has at most as many ranges as give every SM one (one window),
+// or eight.
+size_t score_fused_scratch_bound(const Ctx &ctx, const BatchView &bv) {
+    if (!score_tc_supported(ctx) || bv.batch == 0 || bv.max_q == 0) return 0;
+    BatchView one = bv;
+    while (one.max_q > 0 && padded_rows(one.max_q, ctx.model.g) > kMaxRows) one.max_q -= kRowPad;  // the longest prompt it takes
+    if (one.max_q <= 0) return 0;
+    const int sms = ctx.sm_count > 0 ? ctx.sm_count : 148, per_sm = sms / (ctx.model.L * ctx.model.Hkv);
+    const int ranges = per_sm < 8 ? 8 : (per_sm < kMaxSegs ? per_sm : kMaxSegs), tiles = tiles_of(bv);
+    return scratch_of(ctx.model, one, tiles < ranges ? tiles : ranges);
+}
 
 // Float2 entries of scratch the fused kernel needs for this batch (0: the batch is not one it takes).
 size_t score_fused_scratch(const Ctx &ctx, const BatchView &bv) {
     const int W = score_fused_window(ctx, bv);
-    return W ? scratch_of(ctx.model, bv, W) : 0;
+    return W ? scratch_of(ctx.model, bv, (tiles_of(bv) + W - 1) / W) : 0;
 }
 
 // Returns cudaErrorNotSupported (and launches nothing) when the batch is not one the fused kernel takes, the
@@ -561,7 +573,7 @@ cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const Tensor
                                const BatchView &bv, float *scores, float2 *scratch, size_t scratch_capacity,
                                float *row_lse, cudaStream_t stream) {
     const int W = score_fused_window(ctx, bv);
-    if (W == 0 || scratch_capacity < scratch_of(ctx.model, bv, W)) return cudaErrorNotSupported;
+    if (W == 0 || scratch_capacity < scratch_of(ctx.model, bv, (tiles_of(bv) + W - 1) / W)) return cudaErrorNotSupported;
     ModelView mv = ctx.model;  // the scoring view: a query head only ever meets its own KV head's keys
     mv.G = mv.Hkv;
     mv.hpg = mv.g;
@@ -574,7 +586,7 @@ cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const Tensor
     if (have_chunk && !make_map(&hm, chunk_k, mv.d, bv.total_chunk, mv.Hkv, mv.L, kRows)) return cudaErrorNotSupported;
     if (!have_cache) cm = hm;  // never dereferenced: the request has no cache tiles
     if (!have_chunk) hm = cm;
-    const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
+    const int tiles = tiles_of(bv);
     const int units = mv.L * mv.G;
     FusedParams p{};
     p.mv = mv;

@@ -470,6 +470,21 @@ size_t score_tc_scratch(const Ctx &ctx, const BatchView &bv) {
     return splits * bv.batch * mv.L * mv.Hkv * kGroups * slots_of(mv, bv) + scratch_rest(mv, bv);
 }
 
+// What it would like for no batch within these bounds to want more: key splits times requests grow as bounds shrink.
+size_t score_tc_scratch_bound(const Ctx &ctx, const BatchView &bv) {
+    const ModelView &mv = ctx.model;
+    const int key_tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
+    if (bv.batch == 0 || key_tiles == 0) return 0;
+    const size_t sms = ctx.sm_count > 0 ? ctx.sm_count : 148, units = (size_t)mv.L * mv.Hkv, items = units * bv.batch;
+    const size_t most = min(kScoreMaxSplits, key_tiles);
+    size_t one = 1;  // splits of a single request
+    for (size_t t = 1; t <= most; ++t) one = max(one, (size_t)choose_splits((int)units, 1, (int)t, (int)sms));
+    // of several: choose_splits, with 8 x SMs rounded up to whole splits, or up to half the SMs' items with any number of splits
+    size_t n = units * one;
+    if (bv.batch > 1) n = max(n, min(most * items, max(8 * sms + items, most * (sms / 2 + 1))));
+    return n * kGroups * slots_of(mv, bv) + scratch_rest(mv, bv);
+}
+
 // `scratch` holds `capacity` float2 entries; the key-split count is limited so that everything fits.  Returns
 // cudaErrorNotSupported (and launches nothing) when it does not, or when the tensors cannot be described to the TMA
 // unit; the caller then uses the warp-level path for every request.

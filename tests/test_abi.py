@@ -248,3 +248,29 @@ def test_score_plan_null_arguments(lib):
     path = C.c_int32(-1)
     assert lib.finch_score_plan(ctx, C.byref(batch.c), C.byref(path), None) == fb.FINCH_OK and path.value >= 0
     fb.finch_ctx_destroy(ctx)
+
+
+def test_workspace_of_the_largest_batch_serves_every_smaller_one(lib):
+    """finch_workspace_bytes grows with every bound of the batch, and the calls accept that workspace for what lies within."""
+    import random
+    rng = random.Random(7)
+    mk = lambda B, p, c, m: _Fake.batch(B, B * p, B * m, B * c, p, c, m, c)
+    shapes = [(1, 8, 4, 128, 0), (2, 8, 1, 64, 1), (22, 8, 2, 128, 1), (32, 8, 4, 128, 0), (5, 2, 4, 64, 0), (1, 4, 4, 96, 0)]
+    for L, Hkv, g, d, group_mode in shapes:
+        ctx = fb.finch_ctx_create(L, Hkv * g, Hkv, d, fb.FINCH_BF16, group_mode, max_batch=9, max_prompt=200, max_candidates=9000,
+                                  device=-1)
+        try:
+            for _ in range(60):
+                B, p, c, m = rng.choice([1, 1, 2, 9]), rng.randint(1, 200), rng.randint(1, 4700), rng.randint(1, 2100)
+                room = fb.finch_workspace_bytes(ctx, mk(B, p, c, m))
+                for _ in range(20):
+                    near = rng.random() < 0.5       # a little smaller, or anything smaller
+                    less = lambda n: rng.randint(max(1, n - 200 if near else 1), n)
+                    b = mk(rng.randint(1, B), rng.randint(1, p), less(c), less(m))
+                    assert fb.finch_workspace_bytes(ctx, b) <= room
+                    q, ck, hk = (_Fake.tensor(i, t, d, h) for i, t, h in
+                                 ((0, b.c.total_q, Hkv * g), (1, b.c.total_cache, Hkv), (3, b.c.total_chunk, Hkv)))
+                    assert lib.finch_score(ctx, C.addressof(q), C.addressof(ck), C.addressof(hk), C.addressof(b.c), _Fake.base,
+                                           None, _Fake.base, room, None) == fb.FINCH_ERR_UNSUPPORTED
+        finally:
+            fb.finch_ctx_destroy(ctx)
