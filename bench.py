@@ -160,7 +160,8 @@ def aggregate_over_ranks(ms_local: float, tokens_local: int, world: int, backend
 def launch_replicas(n: int, argv: list, extra_env: dict = None) -> int:
     """Start n ranks of `argv` (a python command line without the interpreter) on this node, one process per GPU,
     with RANK / LOCAL_RANK / WORLD_SIZE / MASTER_ADDR / MASTER_PORT set as torchrun would; rank 0 inherits stdout.
-    Waits for all of them; if one fails the others are terminated (by their own PIDs).  Returns the worst exit code."""
+    Waits for all of them; if one fails the others are terminated (by their own PIDs).  Returns the worst exit code of the
+    ranks that ended by themselves."""
     with socket.socket() as s:
         s.bind(("127.0.0.1", 0))
         port = s.getsockname()[1]
@@ -170,17 +171,20 @@ def launch_replicas(n: int, argv: list, extra_env: dict = None) -> int:
                    MASTER_PORT=str(port), **(extra_env or {}))
         procs.append(subprocess.Popen([sys.executable, *argv], env=env,
                                       stdout=None if rank == 0 else subprocess.DEVNULL))
-    worst, pending = 0, set(range(n))
+    worst, pending, stopped = 0, set(range(n)), set()
     while pending:
         for rank in sorted(pending):
             rc = procs[rank].poll()
             if rc is None:
                 continue
             pending.discard(rank)
+            if rank in stopped:
+                continue
             worst = max(worst, abs(rc))
             if rc != 0:                      # a failed rank would leave the others waiting at a barrier
                 for other in pending:
                     procs[other].terminate()
+                stopped |= pending
         time.sleep(0.05)
     return worst
 

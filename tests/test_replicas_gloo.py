@@ -56,3 +56,11 @@ def test_launcher_reports_a_failed_rank(tmp_path):
     sys.path.insert(0, str(ROOT))
     import bench
     assert bench.launch_replicas(2, ["-c", "import os, sys; sys.exit(3 if os.environ['RANK'] == '1' else 0)"]) == 3
+
+
+def test_launcher_does_not_report_the_ranks_it_stopped(tmp_path):
+    """A rank that still runs when another fails is terminated; the exit code is the failed rank's, not the signal's."""
+    sys.path.insert(0, str(ROOT))
+    import bench
+    code = "import os, sys, time; sys.exit(3) if os.environ['RANK'] == '1' else time.sleep(60)"
+    assert bench.launch_replicas(2, ["-c", code]) == 3
