@@ -51,7 +51,14 @@ struct Ctx {
     // kernels whose shared-memory limit has been raised on this context's device (a driver call: once, not per launch)
     mutable uint32_t smem_bits;
     bool smem_ready(int bit) const { return smem_bits >> bit & 1u; }
-    void smem_set(int bit) const { smem_bits |= 1u << bit; }
+    void smem_set(int bit) const {
+        if (on_own_device()) smem_bits |= 1u << bit;
+    }
+    // What a driver call says holds for the device that is current: only this context's own may be remembered.
+    bool on_own_device() const {
+        int device = -1;
+        return cudaGetDevice(&device) == cudaSuccess && device == cfg.device;
+    }
     mutable int16_t clusters[2][17];  // answers of score_fused.cu's fits_clusters
     mutable uint64_t launches;  // kernels enqueued through this context
     // finch_step_host only: a second stream carries the chunk's V rows to the device while the scoring kernels,

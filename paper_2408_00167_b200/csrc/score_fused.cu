@@ -467,7 +467,8 @@ constexpr int kMaxCluster = 16;
 template <int D>
 bool fits_clusters(const Ctx &ctx, int size, int units) {
     int16_t &known = ctx.clusters[D == 128][size];  // clusters of this size at a time, + 1; 0: not asked yet
-    if (known == 0) {
+    int16_t now = known;
+    if (now == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(size);
         cfg.blockDim = dim3(kTcThreads);
@@ -481,11 +482,12 @@ bool fits_clusters(const Ctx &ctx, int size, int units) {
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, score_fused_kernel<D>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
-            n = 0;
+            return false;
         }
-        known = (int16_t)(n + 1);
+        now = (int16_t)(n + 1);
+        if (ctx.on_own_device()) known = now;
     }
-    return known > units;
+    return now > units;
 }
 
 template <int D>
