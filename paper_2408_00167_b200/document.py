@@ -67,17 +67,12 @@ class DocumentCompressor:
         self._bufs = [mk(), mk()]
         self._cur = 0
         self.kept_idx = torch.full((n_layers, self.G, total_cap), -1, dtype=torch.int32, device=device)
-        self._len = (0,) * self.B       # host mirror of the device lengths
+        self.cache_len = np.zeros(self.B, dtype=np.int32)       # host mirror of the device lengths: valid cache rows
         self._ws = None
         self._meta = {}
         self._plans = {}
         self.steps = 0
         self._unverified = 0    # steps enqueued since the device was last compared with the host mirror
-
-    @property
-    def cache_len(self):
-        """Valid cache rows per request: the host mirror of the device lengths."""
-        return np.asarray(self._len, dtype=np.int32)
 
     # the cache the next step will read
     @property
@@ -110,7 +105,7 @@ class DocumentCompressor:
     def reset(self) -> None:
         """Start a new batch of documents in the same buffers (empty caches).  Checks the finished one first."""
         self.verify()
-        self._len = (0,) * self.B
+        self.cache_len = np.zeros(self.B, dtype=np.int32)
         self._bufs[0]["len"].zero_()
         self._cur = 0
         self.steps = 0
@@ -137,7 +132,7 @@ class DocumentCompressor:
 
     def _plan(self, q_off, chunk_off, budget):
         """(batch, lengths after the step, workspace bytes) of one step; steps of the same shape share it."""
-        key = (q_off, chunk_off, budget, self._len, self._cur)
+        key = (*(np.asarray(a, dtype=np.int32).tobytes() for a in (q_off, chunk_off, budget, self.cache_len)), self._cur)
         plan = self._plans.get(key)
         if plan is not None:
             return plan
@@ -155,7 +150,7 @@ class DocumentCompressor:
         batch = fb.Batch(*metadata[:3], None, metadata[3], c)
         if len(self._plans) > 256:
             self._plans.clear()
-        plan = (batch, tuple(np.minimum(budget, n_cand).tolist()), fb.finch_workspace_bytes(self.ctx, batch))
+        plan = (batch, np.minimum(budget, n_cand).astype(np.int32), fb.finch_workspace_bytes(self.ctx, batch))
         self._plans[key] = plan
         return plan
 
@@ -166,7 +161,7 @@ class DocumentCompressor:
         The lengths the previous step wrote on the device are this step's cache lengths as they are: nothing comes
         back to the host between steps, and the only host-to-device traffic is metadata that has not been seen yet."""
         src, dst = self._bufs[self._cur], self._bufs[self._cur ^ 1]
-        batch, new_len, need = self._plan(*(tuple(map(int, a)) for a in (q_off, chunk_off, budget)))
+        batch, new_len, need = self._plan(q_off, chunk_off, budget)
         c = batch.c
         c.prompt_self_lse = prompt_self_lse.data_ptr() if prompt_self_lse is not None else None
         c.row_limit = row_limit.data_ptr() if row_limit is not None else None
@@ -177,7 +172,7 @@ class DocumentCompressor:
             self._ws = self.torch.empty(need, dtype=self.torch.uint8, device=self.device)
         fb.finch_step(self.ctx, q, src["k"], src["v"], src["pos"], chunk_k, chunk_v, chunk_pos, batch, dst["k"], dst["v"],
                       dst["pos"], self.kept_idx, dst["len"], scores, self._ws)
-        self._len = new_len              # what the step writes to dst["len"]
+        self.cache_len = new_len.copy()  # what the step writes to dst["len"]; the plan keeps its own
         self._cur ^= 1
         self.steps += 1
         self._unverified += 1

@@ -77,3 +77,41 @@ def test_document_driver_matches_the_oracle_step_by_step(group_mode, schedule):
                         assert planted[b] <= set(final[l, g, lo:lo + caps[b]].tolist())
     finally:
         drv.close()
+
+
+@pytest.fixture
+def host_driver(monkeypatch):
+    """A DocumentCompressor whose steps stay on the host: a validation-only context, and finch_step only noted down."""
+    from paper_2408_00167_b200 import binding as fb, build as fbuild
+    fbuild.build()
+    create, steps = fb.finch_ctx_create, []
+    monkeypatch.setattr(fb, "finch_ctx_create", lambda *a, **kw: create(*a, **dict(kw, device=-1)))
+    monkeypatch.setattr(fb, "finch_step", lambda *a, **kw: steps.append(
+        {n: getattr(a[8].c, n) for n, _ in fb.finch_batch._fields_}))
+    drv = doc.DocumentCompressor(2, 4, 2, 64, fb.FINCH_BF16, [64, 32], max_prompt=8, max_chunk=48, device="cpu")
+    drv.chunk = lambda *budget, **kw: drv.step(None, [0, 8, 12], None, None, None, [0, 40, 60], *budget, **kw)
+    yield drv, steps
+    drv._unverified = 0
+    drv.close()
+
+
+def test_document_lengths_can_be_set_by_the_caller(host_driver):
+    """A document that is taken up again: the caller restores the caches and says how long they are."""
+    drv, steps = host_driver
+    drv.cache_len = np.array([50, 30], np.int32)
+    drv.chunk([60, 32])
+    assert steps[-1]["max_cache"] == 50 and drv.cache_len.tolist() == [60, 32]
+    drv.cache_len[0] = 20                       # in place, too; the prepared steps do not see it
+    drv.chunk([60, 32])
+    assert steps[-1]["max_cache"] == 32 and drv.cache_len.tolist() == [60, 32]
+    drv.cache_len = np.array([50, 30], np.int32)
+    drv.chunk([60, 32])
+    assert steps[-1]["max_cache"] == 50 and drv.cache_len.tolist() == [60, 32]
+
+
+def test_document_budget_may_be_one_number_for_all_requests(host_driver):
+    drv, steps = host_driver
+    drv.chunk(24)
+    assert drv.cache_len.tolist() == [24, 20] and steps[-1]["max_budget"] == 24
+    drv.chunk([24])
+    assert drv.cache_len.tolist() == [24, 24]
