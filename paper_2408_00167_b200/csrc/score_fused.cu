@@ -258,7 +258,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
 #define FINCH_UNIT(s) (u.l = (s).unit / mv.G, u.G = (s).unit % mv.G)
 
     if (warp == 0) {
-        Producer<D, false> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q};
+        Producer<D, false, true> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q};
         int q_unit = -1;
         while (ok && walk.next(sg)) {
             FINCH_UNIT(sg);

@@ -188,8 +188,8 @@ struct PadCleaner {
     }
 };
 
-// Run by a whole warp, one elected lane issuing.  OWN_WARP: the PadCleaner is a warp of its own.
-template <int D, bool OWN_WARP>
+// Run by a whole warp.  OWN_WARP: the PadCleaner is a warp of its own; FIRST_SWEEP: the queries are (also) for the first sweep.
+template <int D, bool OWN_WARP, bool FIRST_SWEEP>
 struct Producer {
     static constexpr int kSlabs = D / 64, kTileBytes = kSlabs * kSlabBytes;
     const Cta &c;
@@ -219,41 +219,39 @@ struct Producer {
         ++kcnt;
         return true;
     }
-    // Padded rows [r, r1) of the unit to resident rows dst ..; rows are multiples of 8, a box never leaves its head.
-    __device__ void load_rows(const UnitInfo &u, const Rows &R, int r, int r1, int dst, uint64_t *bar) {
-        while (r < r1) {
-            const int h = r / R.rp, pos = r - h * R.rp, len = min(r1 - r, R.rp - pos);
-            const bool big = len >= kBigBox;
-            for (int s = 0; s < kSlabs; ++s)
-                tma_load_4d(c.q_res + s * c.q_slab + dst * 128, big ? q_big : q_small, bar, s * 64, u.q0 + pos,
-                            u.G * heads + h, u.l);
-            r += big ? kBigBox : kRowPad;
-            dst += big ? kBigBox : kRowPad;
-        }
+    // The n padded rows from the unit's row r on to resident query tile `tile` (and its copies, `span` rows apart).  A lane
+    // takes eight rows of one slab and copy, or issues the box of 64 rows that begins with them; no box leaves its head.  One
+    // lane that walks the boxes, up to 32 with a division each, takes a microsecond for a unit of few rows (13 requests of up
+    // to 9 rows on 19 x 8 units: 124 us, 109 with the lanes).
+    __device__ __forceinline__ void load_tile(const UnitInfo &u, const Rows &R, int r, int n, int span, int copies, int tile,
+                                              uint64_t *bar) {
+        const int lane = threadIdx.x & 31, s = lane >> 4, shift = span == 128 ? 4 : (span == 64 ? 3 : 2);
+        const int copy = (lane & 15) >> shift, i = lane & ((1 << shift) - 1);
+        const int row = r + i * kRowPad, h = row / R.rp, start = max(r, h * R.rp), end = min(r + n, (h + 1) * R.rp);
+        const int big_rows = (end - start) & ~(kBigBox - 1), at = row - start;  // boxes of 64 rows first, then of 8
+        if (elect_one()) mbar_expect_tx(bar, n * copies * 128 * kSlabs);
+        __syncwarp();
+        if (s < kSlabs && copy < copies && row < r + n && (at >= big_rows || at % kBigBox == 0))
+            tma_load_4d(c.q_res + s * c.q_slab + (tile * kRows + copy * span + i * kRowPad) * 128, at < big_rows ? q_big : q_small,
+                        bar, s * 64, u.q0 + row - h * R.rp, u.G * heads + h, u.l);
+        __syncwarp();
     }
     // The unit's query tiles into the ring's tiles base .., one at a time: a tile may be overwritten once the last MMAs on
     // its old contents are complete, while the MMAs on the tiles behind it still run.
-    // RAW: a PadCleaner stands between the copies and the MMAs.
     __device__ __forceinline__ bool load_queries(const UnitInfo &u, const Rows &R, int base) {
-        return pads_hold_rows(u, R, total_q) ? load_tiles<true>(u, R, base) : load_tiles<false>(u, R, base);
-    }
-    template <bool RAW>
-    __device__ __forceinline__ bool load_tiles(const UnitInfo &u, const Rows &R, int base) {
-        const bool leader = elect_one();
+        const bool raw = pads_hold_rows(u, R, total_q);  // a PadCleaner stands between the copies and the MMAs
+        uint64_t *const landed = raw ? c.q_raw : c.q_full;
         for (int qb = 0; qb < R.n_qt; ++qb) {
-            const int tile = base + qb, r = qb * kRows, n = min(kRows, R.rows - r), copies = qb < R.n_qt - 1 ? 1 : kRows / R.span;
+            const int tile = base + qb, r = qb * kRows, n = min(kRows, R.rows - r), span = qb < R.n_qt - 1 ? kRows : R.span;
+            const int copies = FIRST_SWEEP ? kRows / span : 1;  // the second sweep reads the rows along the columns: once
             if (q_used >> tile & 1u) {
                 if (!agree(mbar_wait(&c.q_free[tile], q_ph >> tile & 1u, c.abort_flag))) return false;
                 q_ph ^= 1u << tile;
             }
             q_used |= 1u << tile;
-            if (leader) {
-                uint64_t *bar = RAW ? &c.q_raw[tile] : &c.q_full[tile];
-                mbar_expect_tx(bar, n * copies * 128 * kSlabs);
-                for (int i = 0; i < copies; ++i) load_rows(u, R, R.r0 + r, R.r0 + r + n, tile * kRows + i * R.span, bar);
-            }
+            load_tile(u, R, R.r0 + r, n, span, copies, tile, landed + tile);
         }
-        return !RAW || OWN_WARP || cleaner.clear(R, base);
+        return !raw || OWN_WARP || cleaner.clear(R, base);
     }
     // One segment; base: the ring tiles its queries are to be loaded into, or -1: they are resident.
     __device__ bool segment(const UnitInfo &u, const Rows &R, int t0, int t1, int base) {

@@ -154,7 +154,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant
             prefetch_tensormap(&chunk_map);
         }
         __syncwarp();
-        Producer<D, true> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q};
+        Producer<D, true, MODE == kLse> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q};
         while (ok && walk.next(s, false, lane == 0)) {
             ok = role.segment(s.u, s.R, s.t0, s.t1, q_key != s.q_key ? ring.take(s.R.n_qt) : -1);
             q_key = s.q_key;
