@@ -383,7 +383,13 @@ merge_stats_kernel(TcParams p) {
 // their queries on more CTAs (2 requests of 16 units: 46 us with 4 splits, 66 with 8).
 int choose_splits(int units, int batch, int key_tiles, int sm_count) {
     const int most = min(kScoreMaxSplits, key_tiles);
-    if (batch > 1 && 2 * units * batch >= sm_count) return max(1, min(most, (8 * sm_count + units * batch - 1) / (units * batch)));
+    if (batch > 1 && 2 * units * batch >= sm_count) {
+        units *= batch;
+        // where every SM has a unit already, a split of fewer than three key tiles is mostly its queries and its statistics (23
+        // requests of 98 candidates on 4 x 8 units: 48 us with a split to each of two tiles, 44 with none)
+        const int worth = units >= sm_count ? max(1, key_tiles / 3) : key_tiles;
+        return max(1, min(min(most, worth), (8 * sm_count + units - 1) / units));
+    }
     units *= batch;
     int best = 1;
     double best_eff = 0.0;
