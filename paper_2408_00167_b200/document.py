@@ -170,8 +170,11 @@ class DocumentCompressor:
             need = fb.finch_workspace_bytes(self.ctx, batch)
         if self._ws is None or self._ws.numel() < need:
             self._ws = self.torch.empty(need, dtype=self.torch.uint8, device=self.device)
-        fb.finch_step(self.ctx, q, src["k"], src["v"], src["pos"], chunk_k, chunk_v, chunk_pos, batch, dst["k"], dst["v"],
-                      dst["pos"], self.kept_idx, dst["len"], scores, self._ws)
+        try:
+            fb.finch_step(self.ctx, q, src["k"], src["v"], src["pos"], chunk_k, chunk_v, chunk_pos, batch, dst["k"], dst["v"],
+                          dst["pos"], self.kept_idx, dst["len"], scores, self._ws)
+        finally:                         # the prepared description outlives the call, its tensors need not
+            c.prompt_self_lse = c.row_limit = None
         self.cache_len = new_len.copy()  # what the step writes to dst["len"]; the plan keeps its own
         self._cur ^= 1
         self.steps += 1

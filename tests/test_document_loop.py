@@ -115,3 +115,12 @@ def test_document_budget_may_be_one_number_for_all_requests(host_driver):
     assert drv.cache_len.tolist() == [24, 20] and steps[-1]["max_budget"] == 24
     drv.chunk([24])
     assert drv.cache_len.tolist() == [24, 24]
+
+
+def test_document_plan_keeps_no_address_of_a_calls_tensors(host_driver):
+    import torch
+    drv, steps = host_driver
+    limit, lse = torch.ones(12, dtype=torch.int32), torch.zeros(2, 4, 12)
+    drv.chunk([24, 24], row_limit=limit, prompt_self_lse=lse)
+    assert steps[-1]["row_limit"] == limit.data_ptr() and steps[-1]["prompt_self_lse"] == lse.data_ptr()
+    assert all(b.c.row_limit is None and b.c.prompt_self_lse is None for b, _, _ in drv._plans.values())
