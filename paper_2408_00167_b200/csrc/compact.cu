@@ -247,7 +247,7 @@ select_compact_kernel(ModelView mv, BatchView bv, const float *scores, int *kept
                       int rows_per_cta, int *status) {
     __shared__ int src_idx[kMaxRowsPicked];
     dependency_wait();
-    dependents_may_launch();  // the whole grid is resident
+    dependents_may_launch();  // the whole grid is resident (see launch_select_compact)
     const int l = blockIdx.y / mv.Hkv, kvh = blockIdx.y - l * mv.Hkv, group = kvh / mv.kvpg;
     const UnitInfo u = unit_info(mv, bv, l * mv.G + group, blockIdx.z);
     const bool leader = kvh == group * mv.kvpg;
@@ -287,6 +287,25 @@ auto by_rotation(const ModelView &mv, const F &f) {
                : f(std::integral_constant<int, 2>(), std::integral_constant<int, 8>());
 }
 
+// CTAs of kCompactThreads of the selecting kernel that an SM holds at a time.
+int picks_per_sm(const Ctx &ctx, const ModelView &mv, int items) {
+    return by_rotation(mv, [&](auto rope, auto elems) -> int {
+        constexpr int kRope = decltype(rope)::value, kElems = decltype(elems)::value;
+        int8_t &known = ctx.picks[kRope][kElems == 8][items == 4];
+        if (known) return known;
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &n, items == 4 ? select_compact_kernel<kRope, kElems, 4> : select_compact_kernel<kRope, kElems, 8>, kCompactThreads,
+                0) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return 1;
+        }
+        n = n > 3 ? 3 : n;  // measured with three
+        if (ctx.on_own_device()) known = (int8_t)n;
+        return n;
+    });
+}
+
 }  // namespace
 
 cudaError_t launch_compact(const Ctx &ctx, const int *kept_idx, const int *out_len, const TensorView &cache_k,
@@ -318,17 +337,17 @@ cudaError_t launch_select_compact(const Ctx &ctx, const float *scores, const Ten
     const int64_t sms = ctx.sm_count > 0 ? ctx.sm_count : 148, units = (int64_t)heads * bv.batch;
     // Threads for the copies even where the selection needs fewer (96 threads: 57 us for a step of 43).  A unit's rows are
     // cut evenly into as many blocks as give every SM a CTA, two of short units (two CTAs of 512 threads per SM select
-    // twice as often for blocks of half the rows: 42 us against 35); at most a wave, three CTAs of 256 threads per SM or
-    // one of more (256 units of 800 candidates: 76.5 -> 71 us; 1024 units, several waves: 196 -> 198).  Larger steps keep
-    // the two launches, where a unit is selected once and the copies run at the copy rate; so do steps scored in two
-    // launches, whose second sweep lets its successor in early: several of these CTAs would settle on the first free SMs
-    // (64 units of 1270 candidates: 75 -> 77 us).
+    // twice as often for blocks of half the rows: 42 us against 35); at most a wave, as many CTAs of 256 threads as an SM
+    // holds or one of more (256 units of 800 candidates: 76.5 -> 71 us; 1024 units, several waves: 196 -> 198; 384
+    // re-positioned units of 593, of whose CTAs an SM holds two: 89.6 in one launch, 78.5 in two).  Larger steps keep the two
+    // launches, where a unit is selected once and the copies run at the copy rate; so do steps scored in two launches.
     const int threads = max(kCompactThreads, pick::threads_for(max_n));
     const bool small = threads == kCompactThreads;
     const int most = (bv.max_budget + kMinRowsPerCta - 1) / kMinRowsPerCta, least = (bv.max_budget + kMaxRowsPicked - 1) / kMaxRowsPicked;
     const int blocks = units > 0 ? max(least, (int)min((int64_t)most, (small ? 2 : 1) * sms / units)) : 0;
-    const bool early_in = score_tc_supported(ctx) && score_fused_window(ctx, bv) == 0;
-    if (blocks == 0 || early_in || max_n > kPickThreads * 8 || units * blocks > (small ? 3 : 1) * sms) {
+    const bool two_launches = score_tc_supported(ctx) && score_fused_window(ctx, bv) == 0;
+    const auto wave = [&]() { return (small ? picks_per_sm(ctx, mv, pick::items_for(max_n)) : 1) * sms; };
+    if (blocks == 0 || two_launches || max_n > kPickThreads * 8 || units * blocks > wave()) {
         const cudaError_t e = launch_select(ctx, scores, bv, kept_idx, out_len, stream);
         return e != cudaSuccess ? e : launch_compact(ctx, kept_idx, out_len, cache_k, cache_v, cache_pos, chunk_k, chunk_v,
                                                      chunk_pos, bv, out_k, out_v, out_pos, stream);

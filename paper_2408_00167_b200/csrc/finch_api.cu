@@ -46,7 +46,7 @@ finch_status check_batch(const finch_ctx *ctx, const finch_batch *b) {
 }
 
 struct WsLayout {
-    size_t lse_off, lse_bytes;        // scoring scratch: row statistics per key split and group, partial scores
+    size_t lse_off, lse_bytes;        // scoring scratch: row statistics per key split and group, column sums per KV head
     size_t scores_off, scores_bytes;  // scores inside finch_step when the caller gives none
     size_t total;
 };
@@ -57,7 +57,7 @@ WsLayout ws_layout(const finch_ctx *ctx, const finch_batch *b) {
     w.lse_off = 0;
     const size_t n_kv_scores = (size_t)mv.L * mv.Hkv * ((size_t)b->total_cache + b->total_chunk);
     w.lse_bytes = (size_t)mv.L * mv.Hq * (size_t)b->total_q * sizeof(float2) * (kScoreMaxSplits * 4 + 1) +
-                  (4 * n_kv_scores + 2) * sizeof(float) +  // row statistics, partial scores per KV head,
+                  (4 * n_kv_scores + 2) * sizeof(float) +  // row statistics, room for column sums per KV head (or query head),
                   ((size_t)b->batch + 1) * 8 + 4096;       // and the item plan of a multi-request batch
     // the one-kernel layout, the two-launch layout with the key splits it would take
     const size_t fused = score_fused_scratch(*ctx, view_of(b)) * sizeof(float2);
@@ -219,6 +219,7 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out) {
     ctx->tickets = nullptr;
     ctx->smem_bits = 0;
     memset(ctx->clusters, 0, sizeof(ctx->clusters));
+    memset(ctx->picks, 0, sizeof(ctx->picks));
     ctx->launches = 0;
     if (!ctx->dry) {
         int n_dev = 0;
@@ -483,8 +484,8 @@ finch_status finch_device_status(finch_ctx *ctx, void *cuda_stream, int32_t *out
 // ---------------------------------------------------------------------------------------------------------------
 // finch_score_static: scoring for callers that cannot allocate device memory.
 //
-// finch_score keeps its intermediate results -- per-row softmax statistics, per-group partial column sums, a few
-// counters -- in a workspace the caller allocates.  Code that runs where cudaMalloc is off limits -- a plugin inside a serving process that owns
+// finch_score keeps its intermediate results -- per-row softmax statistics, column sums per KV head where a selection group
+// spans several -- in a workspace the caller allocates.  Code that runs where cudaMalloc is off limits -- a plugin inside a serving process that owns
 // all device memory and hands none out, a callback that may not block on the allocator, a latency-critical loop
 // that must not touch the driver's heap -- has no such workspace to give.  For those callers the scratch is the
 // fixed array below, which is part of the library image: every GPU that loads libfinch holds it until the process

@@ -60,6 +60,7 @@ struct Ctx {
         return cudaGetDevice(&device) == cudaSuccess && device == cfg.device;
     }
     mutable int16_t clusters[2][17];  // answers of score_fused.cu's fits_clusters
+    mutable int8_t picks[3][2][2];    // answers of compact.cu's picks_per_sm
     mutable uint64_t launches;  // kernels enqueued through this context
     // finch_step_host only: a second stream carries the chunk's V rows to the device while the scoring kernels,
     // which do not read them, already run; events tie it to the caller's stream on both sides

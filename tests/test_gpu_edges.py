@@ -163,39 +163,48 @@ def test_compact_row_blocks(L, Hkv, budget, rope_theta):
 
 
 @pytest.mark.parametrize("rope_theta", [0.0, 10000.0])
-@pytest.mark.parametrize("layers,Hkv,reqs,dtype,group_mode,keep_all", [
-    (1, 8, [(16, 9999, 256, 256)], "f32", 0, False),       # blocks of 16 rows
-    (1, 8, [(20, 9999, 2048, 2048)], "bf16", 0, False),    # the longest unit that is selected beside its copies
-    (1, 8, [(20, 9999, 2049, 2048)], "bf16", 0, False),    # one candidate more: two launches
-    (12, 37, [(8, 9999, 70, 512)], "bf16", 0, False),      # 444 blocks of 512 rows
-    (12, 37, [(8, 9999, 70, 513)], "bf16", 0, False),       # a row more: two launches
-    (2, 4, [(9, 9999, 300, 77)], "bf16", 1, False),        # one selection group per layer
-    (1, 4, [(9, 9999, 33, 15), (5, 9999, 1, 90), (3, 9999, 64, 64)], "bf16", 0, False),
-    (2, 3, [(9, 9999, 90, 200)], "f32", 1, True),          # a budget that keeps everything
+@pytest.mark.parametrize("layers,Hkv,reqs,dtype,group_mode,keep_all,d,one_launch", [
+    (1, 8, [(16, 9999, 256, 256)], "f32", 0, False, 64, True),       # blocks of 16 rows
+    (1, 8, [(20, 9999, 2048, 2048)], "bf16", 0, False, 64, True),    # the longest unit that is selected beside its copies
+    (1, 8, [(20, 9999, 2049, 2048)], "bf16", 0, False, 64, False),   # one candidate more: two launches
+    (12, 37, [(8, 9999, 70, 512)], "bf16", 0, False, 64, None),      # 444 blocks of 512 rows
+    (12, 37, [(8, 9999, 70, 513)], "bf16", 0, False, 64, False),     # a row more: two launches
+    (2, 4, [(9, 9999, 300, 77)], "bf16", 1, False, 64, True),        # one selection group per layer
+    (1, 4, [(9, 9999, 33, 15), (5, 9999, 1, 90), (3, 9999, 64, 64)], "bf16", 0, False, 64, False),   # scored in two launches
+    (1, 4, [(9, 9999, 33, 15), (5, 9999, 1, 90), (3, 9999, 64, 64)], "f32", 0, False, 64, True),     # several requests
+    (2, 3, [(9, 9999, 70, 40), (5, 9999, 20, 0), (3, 9999, 600, 300)], "bf16", 0, False, 96, True),  # one with nothing to keep
+    (2, 2, [(4, 9999, 200, 100), (7, 9999, 50, 33)], "f32", 1, False, 128, True),
+    (2, 3, [(9, 9999, 90, 200)], "f32", 1, True, 64, True),          # a budget that keeps everything
 ])
-def test_step_that_selects_and_copies_in_one_launch(layers, Hkv, reqs, dtype, group_mode, keep_all, rope_theta):
-    """finch_step against the oracle and, bit for bit, against the three calls it stands for."""
-    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=Hkv, n_kv_heads=Hkv, head_dim=64, dtype=dtype,
+def test_step_that_selects_and_copies_in_one_launch(layers, Hkv, reqs, dtype, group_mode, keep_all, d, one_launch, rope_theta):
+    """finch_step against the oracle and, bit for bit, against the three calls it stands for; by the number of its kernels it is
+    told whether the step took the one launch (None: that depends on how many of its CTAs an SM holds)."""
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=Hkv, n_kv_heads=Hkv, head_dim=d, dtype=dtype,
                     group_mode=group_mode, planted_frac=0.05, requests=tuple(wl.Request(*r) for r in reqs))
     st = wl.steady_state(cfg, list(range(layers)), step=1)
     if keep_all:
         st["cache_len"] = st["cache_len"] - np.diff(st["chunk_off"]).astype(st["cache_len"].dtype)
-    runs = []
+    runs, launches = [], []
     for parts in (False, True):
         g = GpuStep(cfg, st, layers)
         try:
             if rope_theta:
                 c = g.batch.c
                 fb.finch_ctx_destroy(g.ctx)
-                g.ctx = fb.finch_ctx_create(layers, Hkv, Hkv, 64, fb.FINCH_F32 if dtype == "f32" else fb.FINCH_BF16, group_mode,
+                g.ctx = fb.finch_ctx_create(layers, Hkv, Hkv, d, fb.FINCH_F32 if dtype == "f32" else fb.FINCH_BF16, group_mode,
                                             max_batch=len(reqs), max_prompt=c.max_q, max_candidates=c.max_cache + c.max_chunk,
                                             rope_theta=rope_theta)
             for _ in range(1 if parts else 2):
+                before = fb.finch_launch_count(g.ctx)
                 g.run_parts() if parts else g.run()
+                count = fb.finch_launch_count(g.ctx) - before
             assert g.status() == 0
             runs.append(g.results())
+            launches.append(count)
         finally:
             g.close()
+    if one_launch is not None:
+        assert launches[1] - launches[0] == int(one_launch)
     for name in ("kept_idx", "out_len", "out_pos", "out_k", "out_v"):
         np.testing.assert_array_equal(runs[0][name], runs[1][name], err_msg=name)
     if not rope_theta:
