@@ -199,7 +199,7 @@ __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInf
         }
         merge_parts(part, M, Z);
     }
-    for (int d = 1; d < 1 << log_s; d <<= 1) {  // both partners get the same bits
+    for (int d = 1; d < 1 << log_s; d <<= 1) {  // only the first lane's value is used
         const float om = __shfl_xor_sync(0xffffffffu, M, d), oz = __shfl_xor_sync(0xffffffffu, Z, d);
         const float nm = fmaxf(M, om);
         if (nm != -INFINITY) Z = Z * ex2(M - nm) + oz * ex2(om - nm);

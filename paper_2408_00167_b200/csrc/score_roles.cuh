@@ -2,7 +2,8 @@
 // segments -- (sweep, unit, key-tile range) -- and every role walks the same list with the same running counters, so
 // barrier phases stay in step without any further handshake.
 //
-//   Producer     one thread: query tiles (resident while the unit stays the same) and the ring of key tiles, by TMA.
+//   Producer     one warp: query tiles (resident while the unit stays the same) and the ring of key tiles, by TMA.
+//   PadCleaner   the producer itself or a warp of its own: zeroes pad rows of the queries that hold other rows.
 //   Issuer       one warp: tcgen05.mma into four accumulators of 128 tensor-memory columns in turn.
 //   Softmax      four groups of four warps (a warp per lane quarter): accumulator number A belongs to group A % 4.  A
 //                scheduler holds one warp of each group, so three of them compute while one waits for its refill.

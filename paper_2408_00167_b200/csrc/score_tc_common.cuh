@@ -120,8 +120,7 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 }
 
 // exp2 of a pair.  (A degree-5 polynomial on the FMA pipe for an eighth to a third of the pairs makes the loops alone 8
-// to 15 % shorter, but these kernels run into the chip's power limit, and at 1000 W the SM clock gives back more than
-// that: 32 layers x 8 heads x 4096 candidates x 512 rows, whole step, 0.452 ms without, 0.453 with an eighth, 0.465 with
+// to 15 % shorter, but not the calls, in loops of seconds under the 1000 W power limit: 32 layers x 8 heads x 4096 candidates x 512 rows, whole step, 0.452 ms without, 0.453 with an eighth, 0.465 with
 // a quarter.)
 __device__ __forceinline__ uint64_t exp2_pair(uint64_t x2) {
     float x0, x1;
@@ -135,8 +134,8 @@ __device__ __forceinline__ uint64_t exp2_pair(uint64_t x2) {
 // overflows (a later logit more than ~2^7 base-2 units above the reference, or many nearly that far) the reference
 // moves up and the chunk is redone.  Columns at or beyond nv hold no key and count nothing.
 //
-// The rare parts (a tile's ragged end, a row's first chunk) sit behind warp-uniform branches with an empty asm in them:
-// without it the compiler turns them into predicated instructions, two or three more issue slots per logit.
+// The rare parts (a tile's ragged end, a row's first chunk) sit behind warp-uniform branches with an empty asm in them, which
+// asks for a branch in place of predication: whole and ragged tiles then cost what they contain.
 __device__ __forceinline__ void keep_branch() { asm volatile("" ::: "memory"); }
 template <int NC>
 __device__ __forceinline__ void mask_tail(uint32_t (&r)[NC], int nv) {

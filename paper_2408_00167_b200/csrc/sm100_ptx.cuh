@@ -160,8 +160,7 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {  
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// True in one lane of a converged warp.  The warp's address arithmetic then stays in uniform registers, which is where
-// tcgen05.mma takes its descriptors from; a role that runs in a lane's branch moves every operand there one by one.
+// True in one lane of a converged warp: the whole warp keeps the control flow and the address arithmetic, one lane issues.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
