@@ -59,7 +59,7 @@ struct Ctx {
         int device = -1;
         return cudaGetDevice(&device) == cudaSuccess && device == cfg.device;
     }
-    mutable int16_t clusters[2][17];  // answers of score_fused.cu's fits_clusters
+    mutable int16_t clusters[4][17];  // answers of score_fused.cu's fits_clusters
     mutable int8_t picks[3][2][2];    // answers of compact.cu's picks_per_sm
     mutable uint64_t launches;  // kernels enqueued through this context
     // finch_step_host only: a second stream carries the chunk's V rows to the device while the scoring kernels,
@@ -68,7 +68,7 @@ struct Ctx {
     cudaEvent_t ev_entry, ev_v_ready, ev_selected;
 };
 
-enum { kSmemSelect = 0, kSmemFused = 1, kSmemTc = 3 };  // bits of smem_bits; kSmemFused + (d == 128), kSmemTc + variant
+enum { kSmemSelect = 0, kSmemFused = 1, kSmemTc = 5 };  // bits of smem_bits; kSmemFused + variant, kSmemTc + variant
 
 inline TensorView view_of(const finch_tensor *t) {
     return TensorView{(const char *)t->ptr, t->stride_layer, t->stride_head, t->stride_tok};

@@ -25,6 +25,8 @@
 #include "score_roles.cuh"
 #include "tickets.h"
 
+#include <type_traits>
+
 namespace finch {
 namespace {
 
@@ -217,7 +219,8 @@ __device__ __noinline__ void give_up(int *published, int *left, int ranges, int 
     tickets.leave(unit);
 }
 
-template <int D>
+// PAIR: units of one query tile, and no column sums to be added: the writer's warp is a second MMA issuer, the softmax warps write.
+template <int D, bool PAIR>
 __global__ void __launch_bounds__(kTcThreads, 1)
 score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant__ CUtensorMap q_small,
                    const __grid_constant__ CUtensorMap cache_map, const __grid_constant__ CUtensorMap chunk_map,
@@ -234,7 +237,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         prefetch_tensormap(&cache_map);
         prefetch_tensormap(&chunk_map);
     }
-    const uint32_t tmem = cta_setup(c, direct ? kSoftmaxWarps : 1, p.cluster);
+    const uint32_t tmem = cta_setup(c, direct ? kSoftmaxWarps : 1, p.cluster, PAIR ? 2 : 1);
     // The inputs were written by what precedes this kernel.  The successor is NOT allowed to launch early: its CTAs
     // would take over the SMs of the CTAs that finish first and park there in their wait (measured: + 20 us on the
     // 0.5 ms step of 32 layers x 8 KV heads x 4096 candidates).
@@ -267,8 +270,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
             if (sg.t0 < sg.t1) ok = role.segment(u, R, sg.t0, sg.t1, reload ? ring.take(R.n_qt) : -1);
         }
         role.drain();
-    } else if (warp == 1) {
-        Issuer<D> role(c, tmem);
+    } else if (warp == 1 || (PAIR && warp == 3 && u.n_q > 0)) {
+        Issuer<D, PAIR> role(c, tmem, warp >> 1);
         int q_unit = -1, odd = 0, even = 0;  // query tiles of the odd and the even windows
         Seg nx;
         for (bool more = walk.next(sg); ok && more; sg = nx) {
@@ -392,7 +395,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
             } else {
                 const int b = direct ? 0 : segs_b & 1;
                 if (!direct && !(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[b], (segs_b >> 1) & 1, c.abort_flag)))) break;
-                ok = role.colsum_segment(u, R, sg.t0, sg.t1, c.stats + b * p.rows_alloc, nullptr, nullptr);
+                ok = role.template colsum_segment<PAIR>(u, R, sg.t0, sg.t1, c.stats + b * p.rows_alloc, nullptr, nullptr,
+                                                        p.unit_scores + sg.unit * ((int64_t)bv.total_cache + bv.total_chunk) + u.cache0 + u.chunk0);
                 ++segs_b;
             }
         }
@@ -464,9 +468,9 @@ int rows_alloc_of(const ModelView &mv, const BatchView &bv) {  // resident query
 // memory, where all units' clusters run at once (a cluster lies within one group of SMs, so fewer may fit than SMs would
 // allow).  The exchange through global memory and tickets costs 5.7 us of a 16 us call: stores, fence, atomic, poll, loads.
 constexpr int kMaxCluster = 16;
-template <int D>
+template <int D, bool PAIR>
 bool fits_clusters(const Ctx &ctx, int size, int units) {
-    int16_t &known = ctx.clusters[D == 128][size];  // clusters of this size at a time, + 1; 0: not asked yet
+    int16_t &known = ctx.clusters[(D == 128) + 2 * PAIR][size];  // clusters of this size at a time, + 1; 0: not asked yet
     int16_t now = known;
     if (now == 0) {
         cudaLaunchConfig_t cfg = {};
@@ -480,7 +484,7 @@ bool fits_clusters(const Ctx &ctx, int size, int units) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, score_fused_kernel<D>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&n, score_fused_kernel<D, PAIR>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
             return false;
         }
@@ -490,7 +494,7 @@ bool fits_clusters(const Ctx &ctx, int size, int units) {
     return now > units;
 }
 
-template <int D>
+template <int D, bool PAIR>
 cudaError_t launch_fused_d(const Ctx &ctx, const CUtensorMap &qb, const CUtensorMap &qs, const CUtensorMap &cm,
                            const CUtensorMap &hm, FusedParams p, int n_ranges, int out_groups, int heads_per_group, float *scores,
                            cudaStream_t stream) {
@@ -502,19 +506,19 @@ cudaError_t launch_fused_d(const Ctx &ctx, const CUtensorMap &qb, const CUtensor
     // room for the queries of the two units that alternate, and of a third that is being loaded where they are short
     p.q_tiles = !p.delay || n_qt > 2 ? n_qt : n_qt + 2;
     cudaError_t e = cudaSuccess;
-    if (!ctx.smem_ready(kSmemFused + (D == 128))) {
-        e = cudaFuncSetAttribute(score_fused_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_fused_kernel<D>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (!ctx.smem_ready(kSmemFused + (D == 128) + 2 * PAIR)) {
+        e = cudaFuncSetAttribute(score_fused_kernel<D, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_fused_kernel<D, PAIR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
-        ctx.smem_set(kSmemFused + (D == 128));
+        ctx.smem_set(kSmemFused + (D == 128) + 2 * PAIR);
     }
-    p.cluster = !p.delay && p.n_seg > 1 && p.n_seg <= kMaxCluster && fits_clusters<D>(ctx, p.n_seg, mv.L * mv.G) ? p.n_seg : 1;
+    p.cluster = !p.delay && p.n_seg > 1 && p.n_seg <= kMaxCluster && fits_clusters<D, PAIR>(ctx, p.n_seg, mv.L * mv.G) ? p.n_seg : 1;
     const int parts = p.cluster > 1 ? kGroups * p.rows_alloc * 8 : 0;  // the cluster's exchange of row statistics
     p.stages = kMaxStages;
     while (p.stages > 2 && cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) + parts > kSmemLimit) --p.stages;
     const int smem = cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) + parts;
     dim3 grid(n_ranges < sms ? n_ranges : sms);  // persistent and resident at once: phase B waits for neighbours
-    e = launch_chained_cluster(score_fused_kernel<D>, p.cluster, grid, dim3(kTcThreads), smem, stream, qb, qs, cm, hm, p);
+    e = launch_chained_cluster(score_fused_kernel<D, PAIR>, p.cluster, grid, dim3(kTcThreads), smem, stream, qb, qs, cm, hm, p);
     ctx.launches += 1;
     if (e != cudaSuccess || heads_per_group == 1) return e;
     return launch_sum_heads(ctx, mv, bv, p.unit_scores, scores, out_groups, heads_per_group, stream);
@@ -602,8 +606,14 @@ cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const Tensor
     p.row_lse = row_lse;
     p.status = ctx.d_status;
     const int n_ranges = units * p.n_seg;
-    return mv.d == 64 ? launch_fused_d<64>(ctx, qb, qs, cm, hm, p, n_ranges, ctx.model.G, ctx.model.kvpg, scores, stream)
-                      : launch_fused_d<128>(ctx, qb, qs, cm, hm, p, n_ranges, ctx.model.G, ctx.model.kvpg, scores, stream);
+    const auto launch = [&](auto d, auto pair) {
+        return launch_fused_d<decltype(d)::value, decltype(pair)::value>(ctx, qb, qs, cm, hm, p, n_ranges, ctx.model.G, ctx.model.kvpg,
+                                                                         scores, stream);
+    };
+    const auto by_dim = [&](auto pair) {
+        return mv.d == 64 ? launch(std::integral_constant<int, 64>(), pair) : launch(std::integral_constant<int, 128>(), pair);
+    };
+    return p.rows_alloc == kRows ? by_dim(std::true_type()) : by_dim(std::false_type());
 }
 
 }  // namespace finch

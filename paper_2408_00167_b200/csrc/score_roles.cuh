@@ -84,16 +84,17 @@ __device__ __forceinline__ Cta cta_layout(uint8_t *raw, int tile_bytes, int q_ti
 
 // Barriers and tensor memory (all 512 columns); ends with the CTA in step.  stats_arrivals: arrivals per staging.
 // cluster: CTAs that exchange row statistics through each other's shared memory (1: none).
-__device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals, int cluster = 1) {
+// issuers: MMA issuers that share the key and query tiles.
+__device__ __forceinline__ uint32_t cta_setup(const Cta &c, int stats_arrivals, int cluster = 1, int issuers = 1) {
     if (threadIdx.x == 0) {
         for (int i = 0; i < kQTiles; ++i) {
             mbar_init(&c.q_raw[i], 1);
             mbar_init(&c.q_full[i], 1);
-            mbar_init(&c.q_free[i], 1);
+            mbar_init(&c.q_free[i], issuers);
         }
         for (int i = 0; i < kMaxStages; ++i) {
             mbar_init(&c.full[i], 1);
-            mbar_init(&c.empty[i], 1);
+            mbar_init(&c.empty[i], issuers);
         }
         for (int i = 0; i < kGroups; ++i) {
             mbar_init(&c.acc_full[i], 1);
@@ -274,7 +275,14 @@ struct Producer {
 
 // ------------------------------------------------------------------------------------------------ MMA issuer
 // Run by a whole warp: one elected lane issues, the others keep the control flow uniform (see elect_one).
-template <int D>
+//
+// PAIR: two warps issue, for units of one query tile, every second accumulator (and its key tiles) each.  One warp needs 1300 clocks for
+// the accumulator of a key tile even where nothing is late -- two barrier tests of 150 to 200 beside warps whose exponentials fill the
+// queue that barriers share with them, 390 for the eight MMAs, 220 for the commits -- against 500 of MMAs and, for 64 rows, as
+// many of exponentials.  (32 x 32 units of 8 key tiles x 64 rows 101 -> 98 us, of 11 x 80 rows 141 -> 131; 23 x 8 units of 16 tiles x 24
+// rows, head_dim 64, 38.5 -> 31.3.)  With more query tiles the softmax warps are the slower side.  Both pass every key tile, and a stage is
+// refilled when both have: a barrier's parity tells a phase from its neighbours only, so neither may fall two loads behind or ahead.
+template <int D, bool PAIR = false>
 struct Issuer {
     static constexpr int kSlabs = D / 64, kTileBytes = kSlabs * kSlabBytes;
     const Cta &c;
@@ -282,8 +290,9 @@ struct Issuer {
     uint32_t A = 0;  // accumulators issued
     int st = 0, ph = 0;
     uint32_t q_ph = 0;  // bit per query tile: parity of its next q_full phase
+    uint32_t half;      // PAIR: the accumulators this warp issues, odd or even
 
-    __device__ Issuer(const Cta &cta, uint32_t tm) : c(cta), tmem(tm) {
+    __device__ Issuer(const Cta &cta, uint32_t tm, uint32_t h = 0) : c(cta), tmem(tm), half(h) {
         const uint64_t q = smem_desc_sw128(smem_u32(c.q_res)), r = smem_desc_sw128(smem_u32(c.ring));
         desc_hi = (uint32_t)(q >> 32);
         q_lo = (uint32_t)q;
@@ -318,8 +327,11 @@ struct Issuer {
         commit(&c.acc_full[A & 3]);
         ++A;
     }
-    __device__ __forceinline__ void next_key_stage() {
-        commit(&c.empty[st]);  // the stage may be refilled once these MMAs have read it
+    __device__ __forceinline__ void next_key_stage(bool read = true) {
+        if (read)
+            commit(&c.empty[st]);  // the stage may be refilled once these MMAs have read it
+        else if (elect_one())
+            mbar_arrive(&c.empty[st]);
         if (++st == c.stages) {
             st = 0;
             ph ^= 1;
@@ -334,41 +346,55 @@ struct Issuer {
     // the ring; reload: they are being loaded; release: no later segment uses this load.
     __device__ bool lse_segment(const Rows &R, int t0, int t1, int base, bool reload, bool release) {
         constexpr uint32_t idesc = idesc_bf16_f32(kRows, kRows);
+        if (PAIR && reload && !landed(base)) return false;
         for (int t = t0; t < t1; ++t) {
             if (!wait(&c.full[st], ph)) return false;
+            if (PAIR && (A & 1) != half) {  // the other issuer's
+                ++A;
+                next_key_stage(false);
+                continue;
+            }
             const uint32_t b_lo = ring_lo + (uint32_t)(st * (kTileBytes >> 4));
             for (int qb = 0; qb < R.n_qt; ++qb) {
                 if (!acquire()) return false;
-                if (reload && t == t0 && !landed(base + qb)) return false;
+                if (!PAIR && reload && t == t0 && !landed(base + qb)) return false;
                 tc_fence_after();
                 mma(acc(), q_lo + (uint32_t)((base + qb) * (kRows * 128 >> 4)), q_slab, b_lo, kSlabBytes >> 4, idesc);
                 publish();
-                if (release && t == t1 - 1) commit(&c.q_free[base + qb]);
+                if (!PAIR && release && t == t1 - 1) commit(&c.q_free[base + qb]);
             }
             next_key_stage();
         }
+        if (PAIR && release) commit(&c.q_free[base]);  // also where none of the segment's accumulators was this warp's
         return true;
     }
     // Second sweep: D = key tile x query rows^T.
     __device__ bool colsum_segment(const Rows &R, int t0, int t1, int base, bool reload, bool release) {
         const int cols = (R.rows + 15) & ~15;
         bool side = false;  // kt = 2: this key tile takes the right half of the accumulator
+        if (PAIR && reload && !landed(base)) return false;
         for (int t = t0; t < t1; ++t) {
             const bool last = t == t1 - 1;
             if (!wait(&c.full[st], ph)) return false;
+            if (PAIR && (A & 1) != half) {  // the other issuer's
+                next_key_stage(false);
+                if (R.kt == 1 || side || last) ++A;
+                side = R.kt == 2 && !side;
+                continue;
+            }
             const uint32_t a_lo = ring_lo + (uint32_t)(st * (kTileBytes >> 4));
             int freed = 0, seen = 0;
             for (int s = 0; s < R.n_st; ++s) {
                 if (!side && !acquire()) return false;
                 const int row = s * R.width, n = min(R.width, cols - row), tiles = min(R.n_qt, (row + n + kRows - 1) / kRows);
-                if (reload && t == t0)
+                if (!PAIR && reload && t == t0)
                     for (; seen < tiles; ++seen)
                         if (!landed(base + seen)) return false;
                 tc_fence_after();
                 mma(acc() + (side ? kRows / 2 : 0), a_lo, kSlabBytes >> 4, q_lo + (uint32_t)((base * kRows + row) * 128 >> 4),
                     q_slab, idesc_bf16_f32(kRows, n));
                 if (R.kt == 1 || side || last) publish();
-                if (release && last) {
+                if (!PAIR && release && last) {
                     const int done = s == R.n_st - 1 ? R.n_qt : (row + n) / kRows;
                     for (; freed < done; ++freed) commit(&c.q_free[base + freed]);
                 }
@@ -376,6 +402,7 @@ struct Issuer {
             next_key_stage();
             side = R.kt == 2 && !side;
         }
+        if (PAIR && release) commit(&c.q_free[base]);
         return true;
     }
 };
@@ -601,9 +628,11 @@ struct Softmax {
         }
         return c0 + c1;
     }
-    // Second sweep over key tiles [t0, t1) against the staged statistics `stats` (and limits): column sums to the writer.
+    // Second sweep over key tiles [t0, t1) against the staged statistics `stats` (and limits): column sums to the writer, or,
+    // DIRECT, for units of one query tile, whose keys have no other rows, to the scores `out`.
+    template <bool DIRECT = false>
     __device__ __forceinline__ bool colsum_segment(const UnitInfo &u, const Rows &R, int t0, int t1, const float2 *stats,
-                                                   const int *lim, const int2 *bounds) {
+                                                   const int *lim, const int2 *bounds, float *scores = nullptr) {
         const int n_st = R.n_st, kt = R.kt;
         const uint32_t first = (group - A) & 3, sm = smem_u32(stats);
         const uint32_t sum_full = smem_u32(c.sum_full), sum_empty = smem_u32(c.sum_empty);
@@ -622,6 +651,16 @@ struct Softmax {
             if (kt == 2 && t + 1 < t1)
                 v1 = colsum_visit(tmem + kRows / 2, n, nv, sm4, lim, bounds, row, MASK ? key_tile(u, t + 1).j0 + my_row : 0);
             release();
+            if (DIRECT) {
+                const KeyTile k0 = key_tile(u, t);
+                if (my_row < k0.valid) scores[k0.j0 + my_row] = v0;
+                if (kt == 2 && t + 1 < t1) {
+                    const KeyTile k1 = key_tile(u, t + 1);
+                    if (my_row < k1.valid) scores[k1.j0 + my_row] = v1;
+                }
+                t += step;
+                continue;
+            }
             const uint32_t buf = a % kSumBufs;
             if (!__all_sync(0xffffffffu, mbar_wait(sum_empty + buf * 8, ((a / kSumBufs) & 1) ^ 1, c.abort_flag))) return false;
             float *out = c.sums + buf * 2 * kRows + my_row;

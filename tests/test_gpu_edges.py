@@ -294,3 +294,17 @@ def test_many_small_requests_do_not_see_their_neighbours(heads, rows):
                 np.testing.assert_array_equal(got[:, :, lo:hi], res["scores"][:, :, lo:hi], err_msg=f"request {b}")
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("layers,Hkv,heads,d,n_q,cache,chunk", [
+    (1, 2, 1, 128, 1, 1, 127),        # one window of one and of two key tiles: an issuer without a tile of its own
+    (1, 2, 1, 64, 64, 300, 200),      # two key tiles to an accumulator, an odd number of tiles
+    (1, 2, 1, 64, 65, 300, 200),      # the same with one
+    (20, 8, 1, 128, 128, 640, 256),   # several windows of an odd number of tiles: the issuers swap tiles from window to window
+    (20, 8, 4, 64, 16, 1000, 129),    # .. and of an odd number of accumulators
+    (5, 32, 1, 64, 40, 128, 384),     # ranges that fit no ring of key tiles twice
+])
+def test_units_of_one_query_tile(layers, Hkv, heads, d, n_q, cache, chunk):
+    """Up to 128 padded rows per KV head: two MMA issuers, scores written by the softmax warps."""
+    path, _ = _check(layers, Hkv * heads, Hkv, d, [(n_q, 9999, chunk, cache)])
+    assert path == fb.FINCH_SCORE_ONE_KERNEL
