@@ -433,6 +433,12 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 //                            where a key tile has only one or two (77 us in the example).
 // With one range per CTA a unit's last range may be shorter.  Several windows: ranges that divide the unit, of at least four
 // tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
+// The ranges of a unit exchange their statistics faster as a cluster, where all units' clusters run at once: 30 tenths (36 units of 8
+// key tiles x 96 rows: 17.2 us in ranges of 2 tiles, whose 36 clusters of 4 do not fit, 13.4 in ranges of 3; 16 units of 15 tiles x 128
+// rows 17.2, 13.7).
+constexpr int kMaxCluster = 16;
+// Clusters of so many CTAs, one to an SM, that a device of this kind says it holds.  An estimate here: a launch asks (fits_clusters).
+constexpr int kClusters[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
 int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
     const int q_tiles = (rows + kRows - 1) / kRows;
     const long long l2_budget = 120ll << 20;
@@ -448,6 +454,7 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
         long long cost;
         if (windows == 1) {
             cost = (long long)W * q_tiles * 10 + 50 + n_seg * parts * 3 / 10;
+            if (n_seg > 1 && (n_seg > kMaxCluster || units > kClusters[n_seg])) cost += 30;
         } else {
             if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;
             cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20));
@@ -467,7 +474,6 @@ int rows_alloc_of(const ModelView &mv, const BatchView &bv) {  // resident query
 // With one window the ranges of a unit may form a cluster and exchange their row statistics through each other's shared
 // memory, where all units' clusters run at once (a cluster lies within one group of SMs, so fewer may fit than SMs would
 // allow).  The exchange through global memory and tickets costs 5.7 us of a 16 us call: stores, fence, atomic, poll, loads.
-constexpr int kMaxCluster = 16;
 template <int D, bool PAIR>
 bool fits_clusters(const Ctx &ctx, int size, int units) {
     int16_t &known = ctx.clusters[(D == 128) + 2 * PAIR][size];  // clusters of this size at a time, + 1; 0: not asked yet
