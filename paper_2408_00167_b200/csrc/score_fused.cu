@@ -181,7 +181,7 @@ __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInf
     while (log_s < 4 && R.rows << (log_s + 1) <= kSoftmaxWarps * 32) ++log_s;
     const int row = tid >> log_s, sub = tid & ((1 << log_s) - 1);
     const bool live = row_live(R, row);
-    const Parts parts(R, live ? row / kRows : 0);
+    const Parts parts(R, live ? row / kRows : 0, p.W);
     const int n = live ? parts.count(n_seg) : 0;
     float M = -INFINITY, Z = 0.f;
 #pragma unroll 1
@@ -453,7 +453,8 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
         const long long ranges = units * n_seg, windows = (ranges + ctas - 1) / ctas;
         long long cost;
         if (windows == 1) {
-            cost = (long long)W * q_tiles * 10 + 50 + n_seg * parts * 3 / 10;
+            // (of three query tiles a range of one or two key tiles has a quarter or half of the parts, see Parts)
+            cost = (long long)W * q_tiles * 10 + 50 + n_seg * (q_tiles == 3 && W < 3 ? parts / 4 * W : parts) * 3 / 10;
             if (n_seg > 1 && (n_seg > kMaxCluster || units > kClusters[n_seg])) cost += 30;
         } else {
             if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;

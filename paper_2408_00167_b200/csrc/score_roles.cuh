@@ -684,15 +684,19 @@ struct Softmax {
 
 // The parts of a row's statistics, numbered: per segment, copy of the row, and group that met its query tile.  A segment
 // stores a group's part at the position of the group's first accumulator, so that with one, two or four query tiles the
-// parts of tile qb are at positions qb, qb + n_qt, ...; with three at all four.
+// parts of tile qb are at positions qb, qb + n_qt, ...; with three at all four.  Accumulator a of a segment is query tile a % n_qt, so
+// segments of one or two key tiles (`tiles`, at most) hold no more parts of a tile than that, at positions qb, qb + n_qt, ... modulo
+// four: of three query tiles in ranges of one key tile one in four places is written (reading all of them from the cluster's
+// shared memory took 11 us of a call of 28).
 struct Parts {
     int log_p, log_c, first, step, span;
-    __device__ Parts(const Rows &R, int qb) {
+    __device__ Parts(const Rows &R, int qb, int tiles = kGroups) {
         const bool last = qb == R.n_qt - 1;
         log_c = !last || R.span == 128 ? 0 : (R.span == 64 ? 1 : 2);
-        log_p = R.n_qt == 4 ? 0 : (R.n_qt == 2 ? 1 : 2);
-        first = R.n_qt == 3 ? 0 : qb;
-        step = R.n_qt == 3 ? 1 : R.n_qt;
+        log_p = min(R.n_qt == 4 ? 0 : (R.n_qt == 2 ? 1 : 2), tiles == 1 ? 0 : (tiles == 2 ? 1 : 2));
+        const bool all = R.n_qt == 3 && log_p == 2;
+        first = all ? 0 : qb;
+        step = all ? 1 : R.n_qt;
         span = R.span;
     }
     __device__ int count(int segments) const { return segments << (log_p + log_c); }
@@ -700,7 +704,7 @@ struct Parts {
     // offset of part k in [segments][kGroups][stride], from the row's own slot on
     __device__ int64_t at(int k, int stride) const {
         const int p = k & ((1 << log_p) - 1), c = (k >> log_p) & ((1 << log_c) - 1), s = k >> (log_p + log_c);
-        return (int64_t)(s * kGroups + first + p * step) * stride + c * span;
+        return (int64_t)(s * kGroups + ((first + p * step) & (kGroups - 1))) * stride + c * span;
     }
 };
 

@@ -274,3 +274,12 @@ def test_workspace_of_the_largest_batch_serves_every_smaller_one(lib):
                                            None, _Fake.base, room, None) == fb.FINCH_ERR_UNSUPPORTED
         finally:
             fb.finch_ctx_destroy(ctx)
+
+
+def test_score_plan_takes_ranges_whose_clusters_fit(lib):
+    """One window: the shortest ranges only if a device holds a cluster of them for every unit at once."""
+    one = fb.FINCH_SCORE_ONE_KERNEL
+    assert _plan(9, 16, 4, 64, 17, 692, 230) == (one, 3)       # 36 units: 45 clusters of 3 fit, 33 of 4 do not
+    assert _plan(8, 16, 4, 64, 17, 692, 230) == (one, 2)       # 32 units
+    assert _plan(2, 8, 8, 64, 123, 699, 1069)[1] > 2           # 16 units of 15 tiles: 15 clusters of 8
+    assert _plan(1, 32, 8, 128, 128, 2048, 2048) == (one, 2)   # no length with clusters makes up for longer ranges

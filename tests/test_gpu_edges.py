@@ -308,3 +308,15 @@ def test_units_of_one_query_tile(layers, Hkv, heads, d, n_q, cache, chunk):
     """Up to 128 padded rows per KV head: two MMA issuers, scores written by the softmax warps."""
     path, _ = _check(layers, Hkv * heads, Hkv, d, [(n_q, 9999, chunk, cache)])
     assert path == fb.FINCH_SCORE_ONE_KERNEL
+
+
+@pytest.mark.parametrize("layers,heads,n_q,cache,chunk,window", [
+    (3, 4, 72, 300, 66, 1),      # three query tiles, ranges of one key tile: one part of a row's statistics to a range
+    (12, 4, 72, 300, 500, 2),    # .. of two
+    (20, 4, 73, 500, 900, 4),    # .. of four, the last one shorter
+    (3, 4, 24, 900, 200, 1),     # copies of a row, one query tile
+    (3, 4, 40, 2000, 1000, 2),   # two query tiles
+])
+def test_parts_of_a_rows_statistics_in_short_ranges(layers, heads, n_q, cache, chunk, window):
+    path, w = _check(layers, 2 * heads, 2, 128, [(n_q, 99999, chunk, cache)])
+    assert (path, w) == (fb.FINCH_SCORE_ONE_KERNEL, window)
