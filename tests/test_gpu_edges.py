@@ -211,6 +211,29 @@ def test_step_that_selects_and_copies_in_one_launch(layers, Hkv, reqs, dtype, gr
         check_parity(cfg, st, runs[0], oracle_scores(cfg, st, threads=oracle.max_threads()))
 
 
+@pytest.mark.parametrize("layers,Hkv,n_q,cache,chunk", [(1, 2, 520, 100, 70), (3, 4, 513, 700, 129), (1, 1, 600, 2048, 2048)])
+def test_single_request_scored_in_two_launches_selects_and_copies_in_one(layers, Hkv, n_q, cache, chunk):
+    """More than 512 prompt rows per KV head: the step has one kernel less than its three calls, and their results."""
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=Hkv, n_kv_heads=Hkv, head_dim=64, planted_frac=0.05,
+                    requests=(wl.Request(n_q, 9999, chunk, cache),))
+    st = wl.steady_state(cfg, list(range(layers)), step=1)
+    runs, launches = [], []
+    for parts in (False, True):
+        g = GpuStep(cfg, st, layers)
+        try:
+            assert fb.finch_score_plan(g.ctx, g.batch)[0] == fb.FINCH_SCORE_TWO_LAUNCH
+            before = fb.finch_launch_count(g.ctx)
+            g.run_parts() if parts else g.run()
+            launches.append(fb.finch_launch_count(g.ctx) - before)
+            assert g.status() == 0
+            runs.append(g.results())
+        finally:
+            g.close()
+    assert launches[1] - launches[0] == 1
+    for name in ("kept_idx", "out_len", "out_pos", "out_k", "out_v"):
+        np.testing.assert_array_equal(runs[0][name], runs[1][name], err_msg=name)
+
+
 @pytest.mark.parametrize("fill", [float("nan"), 3e4])
 @pytest.mark.parametrize("layers,n_q,extra,causal", [(1, 37, 3, False), (12, 9, 40, False), (1, 150, 1, False), (2, 37, 5, True)])
 def test_rows_behind_the_requests_reach_no_score(layers, n_q, extra, causal, fill):
