@@ -139,7 +139,7 @@ typedef struct {
 /* Create a context for one model shape on one device.  Fails with FINCH_ERR_UNSUPPORTED when the device is not
  * compute capability 10.x or the shape is not covered, FINCH_ERR_INVALID_ARG on inconsistent fields
  * (n_q_heads not a multiple of n_kv_heads, non-positive sizes, a rotary base below 1).  *out is set only on success.
- * Device memory the context owns, freed by finch_ctx_destroy: a 4-byte status word, two 4-byte counters per layer and
+ * Device memory the context owns, freed by finch_ctx_destroy: a 4-byte status word, four 4-byte counters per layer and
  * KV head, a side stream with three events
  * (used by finch_step_host), and, with rope_theta > 0, the cosine/sine table of the re-positioning,
  * (max_candidates + 1) x head_dim/2 pairs of fp32 (2 MiB for 4096 candidates and head_dim 128), computed in double
@@ -173,7 +173,8 @@ finch_status finch_score(finch_ctx *ctx, const finch_tensor *prompt_q, const fin
  * arithmetic, nothing is enqueued, works on a validation-only context.  (The paper prescribes no kernel; this is how
  * its prompt x candidate block, Section "Method", is tiled here.)
  *  - FINCH_SCORE_ONE_KERNEL: bf16, head_dim 64 or 128, a single request without row_limit, at most 512 query rows
- *    per KV head (queries per KV head x prompt rows rounded up to 8), and a window length W for its key tiles that
+ *    per KV head (queries per KV head x prompt rows rounded up to 8; at most 1024 where half the query heads of a KV head
+ *    can be worked on at a time and every range has a CTA), and a window length W for its key tiles that
  *    is estimated to beat two launches: every (layer, KV head) unit's ranges of W tiles get a CTA each, or the
  *    persistent grid takes several windows, W a divisor of the unit's tile count with W >= 4 (or the whole unit), at
  *    most 8 ranges per unit and W x SMs x tile bytes <= 120 MiB.

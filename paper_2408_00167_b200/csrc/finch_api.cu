@@ -241,7 +241,7 @@ finch_status finch_ctx_create(const finch_config *cfg, finch_ctx **out) {
                 if (dev >= 0) (void)cudaSetDevice(dev);
             }
         } restore{caller_device == cfg->device ? -1 : caller_device};
-        const size_t device_bytes = (1 + 2 * (size_t)mv.L * mv.Hkv) * sizeof(int);  // status word, scoring counters
+        const size_t device_bytes = (1 + 4 * (size_t)mv.L * mv.Hkv) * sizeof(int);  // status word, scoring counters
         if (cudaSetDevice(cfg->device) != cudaSuccess || cudaMalloc(&ctx->d_status, device_bytes) != cudaSuccess) {
             (void)cudaGetLastError();
             delete ctx;

@@ -47,7 +47,7 @@ struct Ctx {
     int *d_status;  // device status word (nullptr for a validation-only context)
     bool dry;       // validation-only context: nothing is ever enqueued
     int sm_count;
-    int *tickets;  // [2][L * Hkv] counters of the one-kernel scoring: zero before and after every call
+    int *tickets;  // [2][units] counters, at most two units to a layer and KV head, of the one-kernel scoring: zero before and after every call
     // kernels whose shared-memory limit has been raised on this context's device (a driver call: once, not per launch)
     mutable uint32_t smem_bits;
     bool smem_ready(int bit) const { return smem_bits >> bit & 1u; }

@@ -1,5 +1,5 @@
 // Prompt-guided scoring with both sweeps in ONE persistent kernel (single-request batches, bf16, head_dim 64/128,
-// at most 512 padded query rows per KV head, no per-row mask).
+// at most 512 padded query rows per KV head, or, in small calls, per half of its query heads; no per-row mask).
 //
 // The logits S = Q K^T of a unit (layer, KV head) are visited twice -- the row log-sum-exp must be known before any
 // column sum can be formed -- but here the second visit follows the first closely enough that the keys come back
@@ -49,6 +49,7 @@ struct FusedParams {
     int rows_alloc;  // query rows of a unit, whole tiles
     int q_tiles;     // query tiles the shared memory holds
     int cluster;     // CTAs of a cluster: the unit's ranges, with one window and few ranges per unit; else 1
+    int key_shift;   // units that share a KV head, as a power of two (scoring_view)
     int delay;       // 0: a CTA has one window; 1: phase B of a window follows phase A of the next
 };
 
@@ -261,7 +262,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
 #define FINCH_UNIT(s) (u.l = (s).unit / mv.G, u.G = (s).unit % mv.G)
 
     if (warp == 0) {
-        Producer<D, false, true> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q};
+        Producer<D, false, true> role{c, &q_big, &q_small, &cache_map, &chunk_map, mv.hpg, bv.total_q, p.key_shift};
         int q_unit = -1;
         while (ok && walk.next(sg)) {
             FINCH_UNIT(sg);
@@ -468,8 +469,19 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
     return best;
 }
 
-int rows_alloc_of(const ModelView &mv, const BatchView &bv) {  // resident query rows: whole tiles
-    return (padded_rows(bv.max_q, mv.g) + kRows - 1) / kRows * kRows;
+// The scoring view: a query head only ever meets its own KV head's keys, so a unit is a KV head.  One of more query rows than stay
+// resident is two units of half its query heads each, where that suffices; their column sums are added afterwards, as those of
+// a selection group's KV heads are.
+ModelView scoring_view(const ModelView &model, const BatchView &bv) {
+    ModelView mv = model;
+    const int halves = padded_rows(bv.max_q, model.g) > kMaxRows && model.g % 2 == 0 ? 2 : 1;
+    mv.G = mv.Hkv * halves;
+    mv.hpg = mv.g / halves;
+    mv.kvpg = 1;
+    return mv;
+}
+int rows_alloc_of(const ModelView &mv, const BatchView &bv) {  // resident query rows: whole tiles (mv: the scoring view)
+    return (padded_rows(bv.max_q, mv.hpg) + kRows - 1) / kRows * kRows;
 }
 
 // With one window the ranges of a unit may form a cluster and exchange their row statistics through each other's shared
@@ -543,20 +555,26 @@ cudaError_t launch_sum_heads(const Ctx &ctx, const ModelView &mv, const BatchVie
 // Key tiles per window the fused kernel would use for this batch; 0: the batch is not one it takes (several
 // requests, causal rows, more query rows per KV head than stay resident, no window length that fits: see choose_window).
 int score_fused_window(const Ctx &ctx, const BatchView &bv) {
-    const ModelView &mv = ctx.model;
     if (!score_tc_supported(ctx) || bv.batch != 1 || bv.row_limit || bv.max_q == 0 || bv.max_cache + bv.max_chunk == 0)
         return 0;
-    if (padded_rows(bv.max_q, mv.g) > kMaxRows) return 0;
+    const ModelView mv = scoring_view(ctx.model, bv);
+    const int rows = padded_rows(bv.max_q, mv.hpg), sms = ctx.sm_count > 0 ? ctx.sm_count : 148;
+    if (rows > kMaxRows) return 0;
     const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
-    return choose_window((long long)mv.L * mv.Hkv, tiles, ctx.sm_count > 0 ? ctx.sm_count : 148, (mv.d / 64) * kSlabBytes,
-                         padded_rows(bv.max_q, mv.g));
+    const int W = choose_window((long long)mv.L * mv.G, tiles, sms, (mv.d / 64) * kSlabBytes, rows);
+    // Halves of a KV head's queries: with one window only, where the calls are latency and two launches of two chunks of rows each take
+    // longer (scoring of 27 single requests of 1 to 12 layers, 129 to 256 prompt rows x 4 heads: 1.45 times as fast, 6 x 2 units of 9
+    // key tiles x 992 rows 41.2 -> 25.0 us, 3 x 8 of 19 x 752 56.4 -> 46.5; none slower).  Both halves fetch the keys.
+    if (mv.G != mv.Hkv && W && (long long)mv.L * mv.G * ((tiles + W - 1) / W) > sms) return 0;
+    return W;
 }
 
 namespace {
-size_t scratch_of(const ModelView &mv, const BatchView &bv, int n_seg) {
-    const size_t units = (size_t)mv.L * mv.Hkv, cand = (size_t)bv.total_cache + bv.total_chunk;
+size_t scratch_of(const ModelView &model, const BatchView &bv, int n_seg) {
+    const ModelView mv = scoring_view(model, bv);
+    const size_t units = (size_t)mv.L * mv.G, cand = (size_t)bv.total_cache + bv.total_chunk;
     size_t n = units * n_seg * kGroups * rows_alloc_of(mv, bv);  // partial row statistics
-    if (mv.G != mv.Hkv) n += (units * cand + 1) / 2;  // per-KV-head sums of a selection group that spans several
+    if (mv.G != model.G) n += (units * cand + 1) / 2;  // sums of the units of a selection group that spans several
     return n;
 }
 int tiles_of(const BatchView &bv) { return (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows; }
@@ -571,7 +589,12 @@ size_t score_fused_scratch_bound(const Ctx &ctx, const BatchView &bv) {
     if (one.max_q <= 0) return 0;
     const int sms = ctx.sm_count > 0 ? ctx.sm_count : 148, per_sm = sms / (ctx.model.L * ctx.model.Hkv);
     const int ranges = per_sm < 8 ? 8 : (per_sm < kMaxSegs ? per_sm : kMaxSegs), tiles = tiles_of(bv);
-    return scratch_of(ctx.model, one, tiles < ranges ? tiles : ranges);
+    const size_t whole = scratch_of(ctx.model, one, tiles < ranges ? tiles : ranges);
+    // halves of a KV head's queries: one range to an SM, as many rows as stay resident, sums of every unit
+    const size_t units = 2 * (size_t)ctx.model.L * ctx.model.Hkv;
+    if (ctx.model.g % 2 || padded_rows(bv.max_q, ctx.model.g) <= kMaxRows || units > (size_t)sms) return whole;
+    const size_t half = (size_t)sms * kGroups * kMaxRows + (units * ((size_t)bv.total_cache + bv.total_chunk) + 1) / 2;
+    return half > whole ? half : whole;
 }
 
 // Float2 entries of scratch the fused kernel needs for this batch (0: the batch is not one it takes).
@@ -587,10 +610,7 @@ cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const Tensor
                                float *row_lse, cudaStream_t stream) {
     const int W = score_fused_window(ctx, bv);
     if (W == 0 || scratch_capacity < scratch_of(ctx.model, bv, (tiles_of(bv) + W - 1) / W)) return cudaErrorNotSupported;
-    ModelView mv = ctx.model;  // the scoring view: a query head only ever meets its own KV head's keys
-    mv.G = mv.Hkv;
-    mv.hpg = mv.g;
-    mv.kvpg = 1;
+    const ModelView mv = scoring_view(ctx.model, bv);
     CUtensorMap qb, qs, cm, hm;
     if (!make_map(&qb, q, mv.d, bv.total_q, mv.Hq, mv.L, kBigBox)) return cudaErrorNotSupported;
     if (!make_map(&qs, q, mv.d, bv.total_q, mv.Hq, mv.L, kRowPad)) return cudaErrorNotSupported;
@@ -609,12 +629,13 @@ cudaError_t launch_score_fused(const Ctx &ctx, const TensorView &q, const Tensor
     p.rows_alloc = rows_alloc_of(mv, bv);
     p.partial = scratch;
     p.tickets = ctx.tickets;
-    p.unit_scores = ctx.model.G == mv.Hkv ? scores : (float *)(scratch + (size_t)units * p.n_seg * kGroups * p.rows_alloc);
+    p.key_shift = mv.G == mv.Hkv ? 0 : 1;
+    p.unit_scores = ctx.model.G == mv.G ? scores : (float *)(scratch + (size_t)units * p.n_seg * kGroups * p.rows_alloc);
     p.row_lse = row_lse;
     p.status = ctx.d_status;
     const int n_ranges = units * p.n_seg;
     const auto launch = [&](auto d, auto pair) {
-        return launch_fused_d<decltype(d)::value, decltype(pair)::value>(ctx, qb, qs, cm, hm, p, n_ranges, ctx.model.G, ctx.model.kvpg,
+        return launch_fused_d<decltype(d)::value, decltype(pair)::value>(ctx, qb, qs, cm, hm, p, n_ranges, ctx.model.G, mv.G / ctx.model.G,
                                                                          scores, stream);
     };
     const auto by_dim = [&](auto pair) {

@@ -198,6 +198,7 @@ struct Producer {
     const CUtensorMap *q_big, *q_small, *cache, *chunk;
     int heads;    // query heads per unit
     int total_q;  // query rows of the packed tensor
+    int key_shift = 0;  // units that share a KV head, as a power of two
     PadCleaner<D> cleaner{c};
     int st = 0, ph = 0, kcnt = 0;
     uint32_t q_used = 0, q_ph = 0;  // bit per query tile: loaded before / parity of its next q_free phase
@@ -216,7 +217,7 @@ struct Producer {
         if (elect_one()) {
             mbar_expect_tx(&c.full[stage], kTileBytes);
             for (int s = 0; s < kSlabs; ++s)
-                tma_load_4d(c.ring + stage * kTileBytes + s * kSlabBytes, m, &c.full[stage], s * 64, kt.row0, u.G, u.l);
+                tma_load_4d(c.ring + stage * kTileBytes + s * kSlabBytes, m, &c.full[stage], s * 64, kt.row0, u.G >> key_shift, u.l);
         }
         ++kcnt;
         return true;

@@ -333,6 +333,20 @@ def test_units_of_one_query_tile(layers, Hkv, heads, d, n_q, cache, chunk):
     assert path == fb.FINCH_SCORE_ONE_KERNEL
 
 
+@pytest.mark.parametrize("layers,Hkv,heads,n_q,cache,chunk,group_mode,one", [
+    (1, 2, 4, 129, 100, 70, 0, True),      # 544 rows: two halves of 272, three query tiles each
+    (2, 2, 2, 255, 300, 300, 1, True),     # a query head each, sums over four units to a group
+    (3, 2, 8, 128, 1000, 500, 0, True),    # 512 rows each
+    (3, 2, 8, 129, 300, 200, 0, False),    # 544: two launches
+    (1, 2, 3, 200, 300, 200, 0, False),    # an odd number of query heads
+    (40, 2, 4, 160, 300, 200, 0, False),   # more halves than SMs
+])
+def test_halves_of_a_kv_heads_queries(layers, Hkv, heads, n_q, cache, chunk, group_mode, one):
+    """513 to 1024 padded rows per KV head: two units that share its keys, their column sums added."""
+    path, _ = _check(layers, Hkv * heads, Hkv, 128, [(n_q, 9999, chunk, cache)], group_mode=group_mode)
+    assert path == (fb.FINCH_SCORE_ONE_KERNEL if one else fb.FINCH_SCORE_TWO_LAUNCH)
+
+
 @pytest.mark.parametrize("layers,heads,n_q,cache,chunk,window", [
     (3, 4, 72, 300, 66, 1),      # three query tiles, ranges of one key tile: one part of a row's statistics to a range
     (12, 4, 72, 300, 500, 2),    # .. of two
