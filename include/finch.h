@@ -174,7 +174,7 @@ finch_status finch_score(finch_ctx *ctx, const finch_tensor *prompt_q, const fin
  * its prompt x candidate block, Section "Method", is tiled here.)
  *  - FINCH_SCORE_ONE_KERNEL: bf16, head_dim 64 or 128, a single request without row_limit, at most 512 query rows
  *    per KV head (queries per KV head x prompt rows rounded up to 8; at most 1024 where half the query heads of a KV head
- *    can be worked on at a time and every range has a CTA), and a window length W for its key tiles that
+ *    can be worked on at a time and every range has a CTA or is a whole unit), and a window length W for its key tiles that
  *    is estimated to beat two launches: every (layer, KV head) unit's ranges of W tiles get a CTA each, or the
  *    persistent grid takes several windows, W a divisor of the unit's tile count with W >= 4 (or the whole unit), at
  *    most 8 ranges per unit and W x SMs x tile bytes <= 120 MiB.

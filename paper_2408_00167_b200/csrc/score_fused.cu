@@ -432,6 +432,7 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 //                            of the second window's CTAs idle, ranges of 3 tiles 82 us);
 //   two launches             the work spread evenly, + 10 for launches and merge, with 1.2 of the time per accumulator, 1.7
 //                            where a key tile has only one or two (77 us in the example).
+// margin: by how many per cent several windows have to be better.
 // With one range per CTA a unit's last range may be shorter.  Several windows: ranges that divide the unit, of at least four
 // tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
 // The ranges of a unit exchange their statistics faster as a cluster, where all units' clusters run at once: 30 tenths (36 units of 8
@@ -440,7 +441,7 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 constexpr int kMaxCluster = 16;
 // Clusters of so many CTAs, one to an SM, that a device of this kind says it holds.  An estimate here: a launch asks (fits_clusters).
 constexpr int kClusters[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
-int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
+int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, int margin) {
     const int q_tiles = (rows + kRows - 1) / kRows;
     const long long l2_budget = 120ll << 20;
     // parts of a row's statistics per range: softmax groups that meet a query tile x copies of a short last tile
@@ -459,7 +460,7 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows) {
             if (n_seg > 1 && (n_seg > kMaxCluster || units > kClusters[n_seg])) cost += 30;
         } else {
             if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;
-            cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20));
+            cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20)) * (100 + margin) / 100;
         }
         if (cost < best_cost) {
             best_cost = cost;
@@ -561,11 +562,14 @@ int score_fused_window(const Ctx &ctx, const BatchView &bv) {
     const int rows = padded_rows(bv.max_q, mv.hpg), sms = ctx.sm_count > 0 ? ctx.sm_count : 148;
     if (rows > kMaxRows) return 0;
     const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
-    const int W = choose_window((long long)mv.L * mv.G, tiles, sms, (mv.d / 64) * kSlabBytes, rows);
-    // Halves of a KV head's queries: with one window only, where the calls are latency and two launches of two chunks of rows each take
-    // longer (scoring of 27 single requests of 1 to 12 layers, 129 to 256 prompt rows x 4 heads: 1.45 times as fast, 6 x 2 units of 9
-    // key tiles x 992 rows 41.2 -> 25.0 us, 3 x 8 of 19 x 752 56.4 -> 46.5; none slower).  Both halves fetch the keys.
-    if (mv.G != mv.Hkv && W && (long long)mv.L * mv.G * ((tiles + W - 1) / W) > sms) return 0;
+    const int W = choose_window((long long)mv.L * mv.G, tiles, sms, (mv.d / 64) * kSlabBytes, rows, mv.G == mv.Hkv ? 0 : 10);
+    // Halves of a KV head's queries: with one window, where the calls are latency and two launches of two chunks of rows each take longer
+    // (scoring of 27 single requests of 1 to 12 layers, 129 to 256 prompt rows x 4 heads: 1.45 times as fast, 6 x 2 units of 9 key tiles
+    // x 992 rows 41.2 -> 25.0 us, 3 x 8 of 19 x 752 56.4 -> 46.5; none slower), and as whole units in several (14 x 8 units of 8 x 896
+    // 100.6 -> 89.4, 32 x 4 of 20 x 712 177 -> 163, 23 x 8 of 11 x 544 130 -> 126).  In shorter ranges of several windows, whose
+    // statistics meet across CTAs, 11 x 8 units of 20 x 800 took 166 us instead of 146.  Both halves fetch the keys: where the estimates
+    // are within 10 %, two launches (31 x 8 units of 17 x 832 325 us, 334 in halves; 24 x 8 of 12 x 576 136, 140).
+    if (mv.G != mv.Hkv && W < tiles && (long long)mv.L * mv.G * ((tiles + (W ? W : 1) - 1) / (W ? W : 1)) > sms) return 0;
     return W;
 }
 
@@ -590,10 +594,10 @@ size_t score_fused_scratch_bound(const Ctx &ctx, const BatchView &bv) {
     const int sms = ctx.sm_count > 0 ? ctx.sm_count : 148, per_sm = sms / (ctx.model.L * ctx.model.Hkv);
     const int ranges = per_sm < 8 ? 8 : (per_sm < kMaxSegs ? per_sm : kMaxSegs), tiles = tiles_of(bv);
     const size_t whole = scratch_of(ctx.model, one, tiles < ranges ? tiles : ranges);
-    // halves of a KV head's queries: one range to an SM, as many rows as stay resident, sums of every unit
+    // halves of a KV head's queries: one range to an SM, or to a unit, as many rows as stay resident, sums of every unit
     const size_t units = 2 * (size_t)ctx.model.L * ctx.model.Hkv;
-    if (ctx.model.g % 2 || padded_rows(bv.max_q, ctx.model.g) <= kMaxRows || units > (size_t)sms) return whole;
-    const size_t half = (size_t)sms * kGroups * kMaxRows + (units * ((size_t)bv.total_cache + bv.total_chunk) + 1) / 2;
+    if (ctx.model.g % 2 || padded_rows(bv.max_q, ctx.model.g) <= kMaxRows) return whole;
+    const size_t half = (units > (size_t)sms ? units : sms) * kGroups * kMaxRows + (units * ((size_t)bv.total_cache + bv.total_chunk) + 1) / 2;
     return half > whole ? half : whole;
 }
 

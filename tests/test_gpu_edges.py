@@ -339,7 +339,8 @@ def test_units_of_one_query_tile(layers, Hkv, heads, d, n_q, cache, chunk):
     (3, 2, 8, 128, 1000, 500, 0, True),    # 512 rows each
     (3, 2, 8, 129, 300, 200, 0, False),    # 544: two launches
     (1, 2, 3, 200, 300, 200, 0, False),    # an odd number of query heads
-    (40, 2, 4, 160, 300, 200, 0, False),   # more halves than SMs
+    (70, 2, 4, 160, 300, 200, 0, True),    # more halves than SMs: whole units in two windows
+    (11, 8, 4, 195, 634, 1817, 0, False),  # .. whose ranges would meet across CTAs
 ])
 def test_halves_of_a_kv_heads_queries(layers, Hkv, heads, n_q, cache, chunk, group_mode, one):
     """513 to 1024 padded rows per KV head: two units that share its keys, their column sums added."""
