@@ -4,12 +4,14 @@
 //
 //   Producer     one warp: query tiles (resident while the unit stays the same) and the ring of key tiles, by TMA.
 //   PadCleaner   the producer itself or a warp of its own: zeroes pad rows of the queries that hold other rows.
-//   Issuer       one warp: tcgen05.mma into four accumulators of 128 tensor-memory columns in turn.
+//   Issuer       one warp: tcgen05.mma into four accumulators of 128 tensor-memory columns in turn; in the one-kernel path two
+//                warps, every second accumulator each, for units of one query tile.
 //   Softmax      four groups of four warps (a warp per lane quarter): accumulator number A belongs to group A % 4.  A
 //                scheduler holds one warp of each group, so three of them compute while one waits for its refill.
-//   SumWriter    one warp: adds the row blocks' column sums of a key (second sweep) and writes the scores.
+//   SumWriter    one warp: adds the row blocks' column sums of a key (second sweep) and writes the scores.  Where two warps
+//                issue there is one block, and the softmax warps write.
 //
-// What bounds it: two exponentials per logit, 1024 clocks of the special-function unit per 128 x 128 logits and sweep,
+// What bounds it, for units of several query tiles: two exponentials per logit, 1024 clocks of the special-function unit per 128 x 128 logits and sweep,
 // and the chip's power limit (large calls run at 1.70 to 1.85 GHz).  Measured on the loops alone (accumulators refilled by
 // MMAs, no loads): 1150 clocks per accumulator in the first sweep and 1210 in the second.  Bookkeeping counts: every
 // instruction between two accumulators is paid by sixteen warps, so what can be is worked out per segment, ragged ends
