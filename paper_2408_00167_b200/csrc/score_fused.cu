@@ -590,13 +590,13 @@ size_t score_fused_scratch_bound(const Ctx &ctx, const BatchView &bv) {
     if (!score_tc_supported(ctx) || bv.batch == 0 || bv.max_q == 0) return 0;
     BatchView one = bv;
     while (one.max_q > 0 && padded_rows(one.max_q, ctx.model.g) > kMaxRows) one.max_q -= kRowPad;  // the longest prompt it takes
-    if (one.max_q <= 0) return 0;
     const int sms = ctx.sm_count > 0 ? ctx.sm_count : 148, per_sm = sms / (ctx.model.L * ctx.model.Hkv);
     const int ranges = per_sm < 8 ? 8 : (per_sm < kMaxSegs ? per_sm : kMaxSegs), tiles = tiles_of(bv);
-    const size_t whole = scratch_of(ctx.model, one, tiles < ranges ? tiles : ranges);
-    // halves of a KV head's queries: one range to an SM, or to a unit, as many rows as stay resident, sums of every unit
+    const size_t whole = one.max_q > 0 ? scratch_of(ctx.model, one, tiles < ranges ? tiles : ranges) : 0;
+    // halves of a KV head's queries, also where all its heads are too many for the shortest prompt: one range to an SM, or to a
+    // unit, as many rows as stay resident, sums of every unit
+    if (ctx.model.g % 2 || padded_rows(bv.max_q, ctx.model.g) <= kMaxRows || padded_rows(1, ctx.model.g / 2) > kMaxRows) return whole;
     const size_t units = 2 * (size_t)ctx.model.L * ctx.model.Hkv;
-    if (ctx.model.g % 2 || padded_rows(bv.max_q, ctx.model.g) <= kMaxRows) return whole;
     const size_t half = (units > (size_t)sms ? units : sms) * kGroups * kMaxRows + (units * ((size_t)bv.total_cache + bv.total_chunk) + 1) / 2;
     return half > whole ? half : whole;
 }

@@ -255,13 +255,16 @@ def test_workspace_of_the_largest_batch_serves_every_smaller_one(lib):
     import random
     rng = random.Random(7)
     mk = lambda B, p, c, m: _Fake.batch(B, B * p, B * m, B * c, p, c, m, c)
-    shapes = [(1, 8, 4, 128, 0), (2, 8, 1, 64, 1), (22, 8, 2, 128, 1), (32, 8, 4, 128, 0), (5, 2, 4, 64, 0), (1, 4, 4, 96, 0)]
-    for L, Hkv, g, d, group_mode in shapes:
+    shapes = [(1, 8, 4, 128, 0, 200), (2, 8, 1, 64, 1, 200), (22, 8, 2, 128, 1, 200), (32, 8, 4, 128, 0, 200), (5, 2, 4, 64, 0, 200),
+              (1, 4, 4, 96, 0, 200), (2, 2, 16, 128, 0, 80), (1, 1, 64, 128, 0, 24), (2, 1, 63, 64, 1, 24),
+              # eight rows of all query heads of a KV head are more than stay resident, eight of half of them are not
+              (1, 1, 66, 128, 0, 24), (1, 1, 72, 128, 0, 24), (1, 1, 128, 128, 0, 24), (2, 1, 96, 64, 1, 24), (1, 1, 130, 64, 0, 24)]
+    for L, Hkv, g, d, group_mode, longest in shapes:
         ctx = fb.finch_ctx_create(L, Hkv * g, Hkv, d, fb.FINCH_BF16, group_mode, max_batch=9, max_prompt=200, max_candidates=9000,
                                   device=-1)
         try:
             for _ in range(60):
-                B, p, c, m = rng.choice([1, 1, 2, 9]), rng.randint(1, 200), rng.randint(1, 4700), rng.randint(1, 2100)
+                B, p, c, m = rng.choice([1, 1, 2, 9]), rng.randint(1, longest), rng.randint(1, 4700), rng.randint(1, 2100)
                 room = fb.finch_workspace_bytes(ctx, mk(B, p, c, m))
                 for _ in range(20):
                     near = rng.random() < 0.5       # a little smaller, or anything smaller
