@@ -25,6 +25,7 @@
 #include "score_roles.cuh"
 #include "tickets.h"
 
+#include <climits>
 #include <type_traits>
 
 namespace finch {
@@ -437,7 +438,9 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 // tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
 // The ranges of a unit exchange their statistics faster as a cluster, where all units' clusters run at once: 30 tenths (36 units of 8
 // key tiles x 96 rows: 17.2 us in ranges of 2 tiles, whose 36 clusters of 4 do not fit, 13.4 in ranges of 3; 16 units of 15 tiles x 128
-// rows 17.2, 13.7).
+// rows 17.2, 13.7).  They weigh between two window lengths only: against two launches one window is far from its limit, with an
+// exchange through tickets too (2 units of 25 tiles x 512 rows 19.2 us, 36 in two launches; 8 of 13 x 416, head_dim 64, 19.6 and 24.9;
+// 60 such calls 0.91 to 0.53 of the time).
 constexpr int kMaxCluster = 16;
 // Clusters of so many CTAs, one to an SM, that a device of this kind says it holds.  An estimate here: a launch asks (fits_clusters).
 constexpr int kClusters[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
@@ -448,22 +451,23 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, in
     const int last = rows - (q_tiles - 1) * kRows;
     const int parts = (q_tiles == 4 ? 1 : (q_tiles == 2 ? 2 : 4)) * (last <= 32 ? 4 : (last <= 64 ? 2 : 1));
     int best = 0;
-    long long best_cost = units * T * q_tiles * (q_tiles <= 2 ? 17 : 12) / ctas + 100;  // in tenths: two launches
+    const long long two_launches = units * T * q_tiles * (q_tiles <= 2 ? 17 : 12) / ctas + 100;  // in tenths
+    long long best_cost = LLONG_MAX;
     for (int W = 1; W <= T; ++W) {
         const int n_seg = (T + W - 1) / W;
         if (n_seg > kMaxSegs || (W > 1 && n_seg == (T + W - 2) / (W - 1))) continue;  // longer, but no fewer ranges
         const long long ranges = units * n_seg, windows = (ranges + ctas - 1) / ctas;
-        long long cost;
+        long long cost, apart = 0;  // apart: what the exchange through tickets adds
         if (windows == 1) {
             // (of three query tiles a range of one or two key tiles has a quarter or half of the parts, see Parts)
             cost = (long long)W * q_tiles * 10 + 50 + n_seg * (q_tiles == 3 && W < 3 ? parts / 4 * W : parts) * 3 / 10;
-            if (n_seg > 1 && (n_seg > kMaxCluster || units > kClusters[n_seg])) cost += 30;
+            if (n_seg > 1 && (n_seg > kMaxCluster || units > kClusters[n_seg])) apart = 30;
         } else {
             if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;
             cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20)) * (100 + margin) / 100;
         }
-        if (cost < best_cost) {
-            best_cost = cost;
+        if (cost < two_launches && cost + apart < best_cost) {
+            best_cost = cost + apart;
             best = W;
         }
     }

@@ -286,3 +286,17 @@ def test_score_plan_takes_ranges_whose_clusters_fit(lib):
     assert _plan(8, 16, 4, 64, 17, 692, 230) == (one, 2)       # 32 units
     assert _plan(2, 8, 8, 64, 123, 699, 1069)[1] > 2           # 16 units of 15 tiles: 15 clusters of 8
     assert _plan(1, 32, 8, 128, 128, 2048, 2048) == (one, 2)   # no length with clusters makes up for longer ranges
+
+
+@pytest.mark.parametrize("layers,q_heads,kv_heads,n_q,cache,chunk", [
+    (1, 16, 8, 203, 140, 1320),     # 8 units of 13 key tiles: 7 clusters of 13
+    (1, 16, 2, 64, 1664, 1536),     # more ranges than a cluster has CTAs
+    (4, 8, 4, 208, 1408, 1280),
+    (3, 32, 8, 72, 2048, 1920),     # three query tiles
+    (2, 16, 2, 72, 768, 768),       # halves of a KV head's query heads
+])
+def test_score_plan_keeps_one_window_where_no_clusters_fit(lib, layers, q_heads, kv_heads, n_q, cache, chunk):
+    """Ranges that exchange through tickets are still shorter than two launches."""
+    path, window = _plan(layers, q_heads, kv_heads, 128, n_q, cache, chunk)
+    tiles = -(-cache // 128) + -(-chunk // 128)
+    assert path == fb.FINCH_SCORE_ONE_KERNEL and 0 < window < tiles
