@@ -175,7 +175,9 @@ __device__ __forceinline__ void merge_by_warp(const FusedParams &p, const UnitIn
 
 // The same by all softmax threads: a row per thread, or, for few rows, per 2 to 16 neighbouring lanes that take every
 // second to sixteenth part each (many short ranges leave hundreds of parts to a row).  `remote`: shared-memory address of
-// the parts, the same in every CTA of the cluster, or 0: they are in global memory.
+// the parts, the same in every CTA of the cluster, or 0: they are in global memory.  What a part's address costs counts: a row of a
+// short last tile has four parts to a range (4 units of 31 ranges x 400 rows 30.2 us with a condition on each load and the
+// positions taken modulo four in it, 26.0 so).
 __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInfo &u, const Rows &R, int n_seg, int unit,
                                              bool write_lse, float2 *stats, int tid, uint32_t remote) {
     const float2 *src = p.partial + (int64_t)unit * p.n_seg * kGroups * p.rows_alloc;
@@ -189,17 +191,20 @@ __device__ __forceinline__ void merge_by_cta(const FusedParams &p, const UnitInf
 #pragma unroll 1
     for (int i0 = sub; i0 < n; i0 += 8 << log_s) {
         float2 part[8];
+        if (remote) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int k = i0 + (i << log_s);
-            part[i] = make_float2(0.f, 0.f);
-            if (k >= n) continue;
-            if (remote) {
-                const int seg = parts.segment(k);
-                part[i] = ld_remote(map_to_rank(remote + ((uint32_t)parts.at(k - (seg << (parts.log_p + parts.log_c)), p.rows_alloc) + row) * 8, seg));
-            } else {
-                part[i] = __ldcg(src + parts.at(k, p.rows_alloc) + row);
+            for (int i = 0; i < 8; ++i) {
+                const int k = i0 + (i << log_s), seg = parts.segment(k);
+                const uint32_t at = (uint32_t)parts.at(k - (seg << (parts.log_p + parts.log_c)), p.rows_alloc) + row;
+                part[i] = k < n ? ld_remote(map_to_rank(remote + at * 8, seg)) : make_float2(0.f, 0.f);
             }
+        } else {
+            // (loads without a condition: eight in flight; a lane with fewer parts left reads its last one again)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) part[i] = __ldcg(src + parts.at(min(i0 + (i << log_s), n - 1), p.rows_alloc) + row);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i0 + (i << log_s) >= n) part[i] = make_float2(0.f, 0.f);
         }
         merge_parts(part, M, Z);
     }
@@ -439,8 +444,7 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 // The ranges of a unit exchange their statistics faster as a cluster, where all units' clusters run at once: 30 tenths (36 units of 8
 // key tiles x 96 rows: 17.2 us in ranges of 2 tiles, whose 36 clusters of 4 do not fit, 13.4 in ranges of 3; 16 units of 15 tiles x 128
 // rows 17.2, 13.7).  They weigh between two window lengths only: against two launches one window is far from its limit, with an
-// exchange through tickets too (2 units of 25 tiles x 512 rows 19.2 us, 36 in two launches; 8 of 13 x 416, head_dim 64, 19.6 and 24.9;
-// 60 such calls 0.91 to 0.53 of the time).
+// exchange through tickets too (2 units of 25 tiles x 512 rows 19.2 us, 36 in two launches; 8 of 13 x 416, head_dim 64, 19.6 and 24.9).
 constexpr int kMaxCluster = 16;
 // Clusters of so many CTAs, one to an SM, that a device of this kind says it holds.  An estimate here: a launch asks (fits_clusters).
 constexpr int kClusters[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};

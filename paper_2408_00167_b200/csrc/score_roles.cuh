@@ -699,7 +699,7 @@ struct Parts {
         log_p = min(R.n_qt == 4 ? 0 : (R.n_qt == 2 ? 1 : 2), tiles == 1 ? 0 : (tiles == 2 ? 1 : 2));
         const bool all = R.n_qt == 3 && log_p == 2;
         first = all ? 0 : qb;
-        step = all ? 1 : R.n_qt;
+        step = all ? 1 : (R.n_qt < 3 ? R.n_qt : (qb == 0 ? 3 : -1));  // of three: qb and the position three on, modulo four
         span = R.span;
     }
     __device__ int count(int segments) const { return segments << (log_p + log_c); }
@@ -707,7 +707,7 @@ struct Parts {
     // offset of part k in [segments][kGroups][stride], from the row's own slot on
     __device__ int64_t at(int k, int stride) const {
         const int p = k & ((1 << log_p) - 1), c = (k >> log_p) & ((1 << log_c) - 1), s = k >> (log_p + log_c);
-        return (int64_t)(s * kGroups + ((first + p * step) & (kGroups - 1))) * stride + c * span;
+        return (int64_t)(s * kGroups + first + p * step) * stride + c * span;
     }
 };
 
