@@ -438,7 +438,9 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 //                            of the second window's CTAs idle, ranges of 3 tiles 82 us);
 //   two launches             the work spread evenly, + 10 for launches and merge, with 1.2 of the time per accumulator, 1.7
 //                            where a key tile has only one or two (77 us in the example).
-// margin: by how many per cent several windows have to be better.
+// halves: a unit is half the query heads of a KV head.  Both halves fetch the keys: several windows have to be better by a tenth, and
+// are whole units, unless a divisor would be estimated better still: there two launches are shorter (24 x 32 units of 14 key tiles x
+// 288 rows 564 us, 601 in whole units).
 // With one range per CTA a unit's last range may be shorter.  Several windows: ranges that divide the unit, of at least four
 // tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
 // The ranges of a unit exchange their statistics faster as a cluster, where all units' clusters run at once: 30 tenths (36 units of 8
@@ -448,7 +450,7 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 constexpr int kMaxCluster = 16;
 // Clusters of so many CTAs, one to an SM, that a device of this kind says it holds.  An estimate here: a launch asks (fits_clusters).
 constexpr int kClusters[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
-int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, int margin) {
+int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, bool halves) {
     const int q_tiles = (rows + kRows - 1) / kRows;
     const long long l2_budget = 120ll << 20;
     // parts of a row's statistics per range: softmax groups that meet a query tile x copies of a short last tile
@@ -456,7 +458,8 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, in
     const int parts = (q_tiles == 4 ? 1 : (q_tiles == 2 ? 2 : 4)) * (last <= 32 ? 4 : (last <= 64 ? 2 : 1));
     int best = 0;
     const long long two_launches = units * T * q_tiles * (q_tiles <= 2 ? 17 : 12) / ctas + 100;  // in tenths
-    long long best_cost = LLONG_MAX;
+    long long best_cost = LLONG_MAX, barred = LLONG_MAX;
+    bool several = false;
     for (int W = 1; W <= T; ++W) {
         const int n_seg = (T + W - 1) / W;
         if (n_seg > kMaxSegs || (W > 1 && n_seg == (T + W - 2) / (W - 1))) continue;  // longer, but no fewer ranges
@@ -468,14 +471,19 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, in
             if (n_seg > 1 && (n_seg > kMaxCluster || units > kClusters[n_seg])) apart = 30;
         } else {
             if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;
-            cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20)) * (100 + margin) / 100;
+            cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20)) * (halves ? 11 : 10) / 10;
+            if (halves && W < T) {
+                barred = min(barred, cost);
+                continue;
+            }
         }
         if (cost < two_launches && cost + apart < best_cost) {
             best_cost = cost + apart;
             best = W;
+            several = windows > 1;
         }
     }
-    return best;
+    return several && barred <= best_cost ? 0 : best;
 }
 
 // The scoring view: a query head only ever meets its own KV head's keys, so a unit is a KV head.  One of more query rows than stay
@@ -570,15 +578,13 @@ int score_fused_window(const Ctx &ctx, const BatchView &bv) {
     const int rows = padded_rows(bv.max_q, mv.hpg), sms = ctx.sm_count > 0 ? ctx.sm_count : 148;
     if (rows > kMaxRows) return 0;
     const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
-    const int W = choose_window((long long)mv.L * mv.G, tiles, sms, (mv.d / 64) * kSlabBytes, rows, mv.G == mv.Hkv ? 0 : 10);
     // Halves of a KV head's queries: with one window, where the calls are latency and two launches of two chunks of rows each take longer
     // (scoring of 27 single requests of 1 to 12 layers, 129 to 256 prompt rows x 4 heads: 1.45 times as fast, 6 x 2 units of 9 key tiles
     // x 992 rows 41.2 -> 25.0 us, 3 x 8 of 19 x 752 56.4 -> 46.5; none slower), and as whole units in several (14 x 8 units of 8 x 896
     // 100.6 -> 89.4, 32 x 4 of 20 x 712 177 -> 163, 23 x 8 of 11 x 544 130 -> 126).  In shorter ranges of several windows, whose
-    // statistics meet across CTAs, 11 x 8 units of 20 x 800 took 166 us instead of 146.  Both halves fetch the keys: where the estimates
-    // are within 10 %, two launches (31 x 8 units of 17 x 832 325 us, 334 in halves; 24 x 8 of 12 x 576 136, 140).
-    if (mv.G != mv.Hkv && W < tiles && (long long)mv.L * mv.G * ((tiles + (W ? W : 1) - 1) / (W ? W : 1)) > sms) return 0;
-    return W;
+    // statistics meet across CTAs, 11 x 8 units of 20 x 800 took 166 us instead of 146.  Where the estimates are within 10 %, two
+    // launches (31 x 8 units of 17 x 832 325 us, 334 in halves; 24 x 8 of 12 x 576 136, 140).
+    return choose_window((long long)mv.L * mv.G, tiles, sms, (mv.d / 64) * kSlabBytes, rows, mv.G != mv.Hkv);
 }
 
 namespace {

@@ -300,3 +300,13 @@ def test_score_plan_keeps_one_window_where_no_clusters_fit(lib, layers, q_heads,
     path, window = _plan(layers, q_heads, kv_heads, 128, n_q, cache, chunk)
     tiles = -(-cache // 128) + -(-chunk // 128)
     assert path == fb.FINCH_SCORE_ONE_KERNEL and 0 < window < tiles
+
+
+def test_score_plan_of_halves_keeps_a_window_that_is_allowed(lib):
+    """512 rows in each half of a KV head's queries: a shorter window that halves do not take hides no longer one that they do."""
+    one, two = fb.FINCH_SCORE_ONE_KERNEL, fb.FINCH_SCORE_TWO_LAUNCH
+    assert _plan(3, 64, 8, 128, 128, 1024, 1920) == (one, 8)
+    assert _plan(3, 64, 8, 128, 128, 1024, 2048) == (one, 8)      # 24 key tiles, divisible by the four of a shorter window
+    assert _plan(3, 64, 8, 128, 128, 1024, 2176) == (one, 9)
+    assert _plan(24, 256, 32, 128, 72, 896, 896) == (two, 0)      # several windows: a divisor would be the better range
+    assert _plan(70, 8, 2, 128, 160, 300, 200)[0] == one          # .. or the whole unit is
