@@ -431,54 +431,63 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 // Key tiles per range, or 0 when the one-kernel path should leave the batch to the two-launch kernels.
 //
 // The estimate is in units of one query tile against one key tile in both sweeps, 2500 SM clocks where the pipeline is full:
-//   one range per CTA        W x query tiles + 5 + the parts of a row to be merged: nothing hides the query load and the
-//                            exchange of the row statistics;
+//   one range per CTA        W x query tiles (0.7 W for at most 64 rows) + 4, + 0.3 for every eight parts of a row that a lane of
+//                            the merge reads (merge_rounds): nothing hides the query load and the exchange of the row statistics.
+//                            As a cluster, where all units' clusters run at once, the ranges of a unit exchange for 1 at 16 of
+//                            them; else for 1.5 and, as the CTAs that poll, up to 1 more; + 0.5 for single tiles (36 units of 8 key tiles x 96 rows:
+//                            17.2 us in ranges of 2 tiles, whose 36 clusters of 4 do not fit, 13.4 in ranges of 3; 2 units of
+//                            27 x 256 14.5 us in 27 ranges without a cluster, 18.5 in clusters of 14);
 //   several ("windows")      windows x (W x query tiles + 2), or + 5 where the ranges of a unit meet across CTAs and are too
 //                            short to hide it (28 x 8 units of 9 key tiles x 160 rows: whole units 55 us although a quarter
 //                            of the second window's CTAs idle, ranges of 3 tiles 82 us);
-//   two launches             the work spread evenly, + 10 for launches and merge, with 1.2 of the time per accumulator, 1.7
-//                            where a key tile has only one or two (77 us in the example).
+//   two launches             the work spread evenly with 1.2 of the time per accumulator, + 14 for launches and merge; against several
+//                            windows + 10 and 1.7 per accumulator where a key tile has only one or two (77 us in the example).
+// The constants are fits to 1450 calls of 1 to 1300 units, 2 to 32 key tiles and 8 to 512 rows, where the chosen way takes 1.009 times
+// as long as the best one in the geometric mean (1.022 with 5, 0.03 a part, 3 for any missing cluster and 10 for two launches, which
+// sent few units with many short ranges to two launches: 2 units of 23 tiles x 24 rows 25.6 us, 12.8 in ranges of 2).
 // halves: a unit is half the query heads of a KV head.  Both halves fetch the keys: several windows have to be better by a tenth, and
 // are whole units, unless a divisor would be estimated better still: there two launches are shorter (24 x 32 units of 14 key tiles x
-// 288 rows 564 us, 601 in whole units).
+// 288 rows 564 us, 601 in whole units), as they are for units of fewer than eight accumulators (176 of 2 x 320 rows 31.3 us, 35.7).
 // With one range per CTA a unit's last range may be shorter.  Several windows: ranges that divide the unit, of at least four
 // tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
-// The ranges of a unit exchange their statistics faster as a cluster, where all units' clusters run at once: 30 tenths (36 units of 8
-// key tiles x 96 rows: 17.2 us in ranges of 2 tiles, whose 36 clusters of 4 do not fit, 13.4 in ranges of 3; 16 units of 15 tiles x 128
-// rows 17.2, 13.7).  They weigh between two window lengths only: against two launches one window is far from its limit, with an
-// exchange through tickets too (2 units of 25 tiles x 512 rows 19.2 us, 36 in two launches; 8 of 13 x 416, head_dim 64, 19.6 and 24.9).
 constexpr int kMaxCluster = 16;
-// Clusters of so many CTAs, one to an SM, that a device of this kind says it holds.  An estimate here: a launch asks (fits_clusters).
+// Clusters of so many CTAs, one to an SM, that a device of this kind says it holds.  An estimate, so that a plan needs no device: a
+// launch asks (fits_clusters), and on a device that holds others the rule only loses time.
 constexpr int kClusters[kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7};
+// Rounds of eight loads that a lane of merge_by_cta makes for a row of the last query tile, the one with copies, as Parts counts them.
+int merge_rounds(int rows, int n_seg, int W) {
+    const int q_tiles = (rows + kRows - 1) / kRows, last = rows - (q_tiles - 1) * kRows;
+    const int met = W < 3 ? W : kGroups, groups = q_tiles == 4 ? 1 : (q_tiles == 2 ? min(2, met) : met);
+    int lanes = 1;
+    while (lanes < 16 && rows * lanes * 2 <= kSoftmaxWarps * 32) lanes *= 2;
+    return (n_seg * groups * (last <= 32 ? 4 : (last <= 64 ? 2 : 1)) + 8 * lanes - 1) / (8 * lanes);
+}
 int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, bool halves) {
     const int q_tiles = (rows + kRows - 1) / kRows;
     const long long l2_budget = 120ll << 20;
-    // parts of a row's statistics per range: softmax groups that meet a query tile x copies of a short last tile
-    const int last = rows - (q_tiles - 1) * kRows;
-    const int parts = (q_tiles == 4 ? 1 : (q_tiles == 2 ? 2 : 4)) * (last <= 32 ? 4 : (last <= 64 ? 2 : 1));
     int best = 0;
-    const long long two_launches = units * T * q_tiles * (q_tiles <= 2 ? 17 : 12) / ctas + 100;  // in tenths
+    // in tenths: two launches as the limit of several windows and of one, a key tile of units of at most 64 rows
+    const long long all = units * T * q_tiles, two_launches = all * (q_tiles <= 2 ? 17 : 12) / ctas + 100, two_small = all * 12 / ctas + 140;
+    const int tile = rows <= kRows / 2 ? 7 : q_tiles * 10;
     long long best_cost = LLONG_MAX, barred = LLONG_MAX;
     bool several = false;
     for (int W = 1; W <= T; ++W) {
         const int n_seg = (T + W - 1) / W;
         if (n_seg > kMaxSegs || (W > 1 && n_seg == (T + W - 2) / (W - 1))) continue;  // longer, but no fewer ranges
         const long long ranges = units * n_seg, windows = (ranges + ctas - 1) / ctas;
-        long long cost, apart = 0;  // apart: what the exchange through tickets adds
+        long long cost;
         if (windows == 1) {
-            // (of three query tiles a range of one or two key tiles has a quarter or half of the parts, see Parts)
-            cost = (long long)W * q_tiles * 10 + 50 + n_seg * (q_tiles == 3 && W < 3 ? parts / 4 * W : parts) * 3 / 10;
-            if (n_seg > 1 && (n_seg > kMaxCluster || units > kClusters[n_seg])) apart = 30;
+            const bool clusters = n_seg <= kMaxCluster && units <= kClusters[n_seg];
+            cost = (long long)W * tile + 40 + 3 * merge_rounds(rows, n_seg, W);
+            if (n_seg > 1) cost += (clusters ? n_seg * 10 / 16 : 15 + ranges * 10 / ctas) + (W == 1 ? 5 : 0);
         } else {
             if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;
             cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20)) * (halves ? 11 : 10) / 10;
-            if (halves && W < T) {
-                barred = min(barred, cost);
-                continue;
-            }
+            if (halves && W < T) barred = min(barred, cost);
+            if (halves && (W < T || W * q_tiles < 8)) continue;
         }
-        if (cost < two_launches && cost + apart < best_cost) {
-            best_cost = cost + apart;
+        if (cost < (windows == 1 ? two_small : two_launches) && cost < best_cost) {
+            best_cost = cost;
             best = W;
             several = windows > 1;
         }

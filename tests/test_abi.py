@@ -310,3 +310,12 @@ def test_score_plan_of_halves_keeps_a_window_that_is_allowed(lib):
     assert _plan(3, 64, 8, 128, 128, 1024, 2176) == (one, 9)
     assert _plan(24, 256, 32, 128, 72, 896, 896) == (two, 0)      # several windows: a divisor would be the better range
     assert _plan(70, 8, 2, 128, 160, 300, 200)[0] == one          # .. or the whole unit is
+
+
+def test_score_plan_of_small_calls(lib):
+    """Few units: long ranges do not pay for a cluster, nor two launches for the parts of short ones; short halves are no whole units."""
+    one, two = fb.FINCH_SCORE_ONE_KERNEL, fb.FINCH_SCORE_TWO_LAUNCH
+    assert _plan(1, 4, 2, 128, 128, 1792, 1664) == (one, 1)       # 2 units of 27 key tiles x 256 rows
+    assert _plan(1, 6, 2, 128, 8, 1536, 1408)[0] == one           # .. of 23 x 24
+    assert _plan(24, 32, 4, 128, 96, 128, 128) == (two, 0)        # 192 halves of 2 key tiles x 384 rows
+    assert _plan(70, 8, 2, 128, 160, 300, 200)[0] == one          # .. 280 of 5 x 320
