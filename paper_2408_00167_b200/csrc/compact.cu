@@ -340,16 +340,17 @@ cudaError_t launch_select_compact(const Ctx &ctx, const float *scores, const Ten
     // twice as often for blocks of half the rows: 42 us against 35); at most a wave, as many CTAs of 256 threads as an SM
     // holds or one of more (256 units of 800 candidates: 76.5 -> 71 us; 1024 units, several waves: 196 -> 198; 384
     // re-positioned units of 593, of whose CTAs an SM holds two: 89.6 in one launch, 78.5 in two).  Larger steps keep the two
-    // launches, where a unit is selected once and the copies run at the copy rate.  So do batches of several requests that
-    // are scored in two launches: measured while their second sweep let its successor in early (64 units of 1270 candidates 75 us,
-    // 77 in one launch); it no longer does, and in one launch small ones would be up to 12 % shorter (4 requests on 3 x 8 units
-    // 38.9 us, 36.0).  A single request takes the one launch however it was scored (prompts of more than 512 rows per KV head,
-    // 16 steps of 1 to 8 layers: 2 to 12 % shorter, 7 x 4 units of 751 candidates 47.9 -> 42.9 us).
+    // launches, where a unit is selected once and the copies run at the copy rate.  So do batches of several requests on the tensor
+    // cores: in one launch most small ones would be shorter (140 steps of 2 to 8 requests on 1 to 12 layers: 1.03 times as fast, up to
+    // 1.12; 4 requests on 3 x 8 units 38.9 us, 36.0), but not those of few long units, each selected again by several CTAs of 512
+    // threads (5 requests on 8 units of 2239 candidates 47.1 us, 50.5), and no line between them has been drawn.  A single request
+    // takes the one launch however it was scored (prompts of more than 512 rows per KV head, 16 steps of 1 to 8 layers: 2 to 12 %
+    // shorter, 7 x 4 units of 751 candidates 47.9 -> 42.9 us; 40 causal ones of 8 to 1500 rows 1 to 14 %).
     const int threads = max(kCompactThreads, pick::threads_for(max_n));
     const bool small = threads == kCompactThreads;
     const int most = (bv.max_budget + kMinRowsPerCta - 1) / kMinRowsPerCta, least = (bv.max_budget + kMaxRowsPicked - 1) / kMaxRowsPicked;
     const int blocks = units > 0 ? max(least, (int)min((int64_t)most, (small ? 2 : 1) * sms / units)) : 0;
-    const bool two_launches = bv.batch > 1 && score_tc_supported(ctx) && score_fused_window(ctx, bv) == 0;
+    const bool two_launches = bv.batch > 1 && score_tc_supported(ctx);
     const auto wave = [&]() { return (small ? picks_per_sm(ctx, mv, pick::items_for(max_n)) : 1) * sms; };
     if (blocks == 0 || two_launches || max_n > kPickThreads * 8 || units * blocks > wave()) {
         const cudaError_t e = launch_select(ctx, scores, bv, kept_idx, out_len, stream);
