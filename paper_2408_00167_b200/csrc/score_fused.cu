@@ -37,12 +37,12 @@ using namespace tc;
 constexpr int kMaxSegs = 64;  // ranges per unit (each prompt row merges a few statistics of every range)
 
 struct FusedParams {
-    ModelView mv;  // the scoring view: one unit per KV head
+    ModelView mv;  // the scoring view: one unit per KV head, or two of half its query heads
     BatchView bv;
     float2 *partial;     // [units][n_seg][kGroups][rows_alloc] (reference base-2 logit, sum exp2) per row and part
     int *tickets;        // [2][units] the two counters of a unit
     float *row_lse;      // nullable
-    float *unit_scores;  // [L][Hkv][cand]: the column sums of one KV head's query heads
+    float *unit_scores;  // [units][cand]: the column sums of a unit's query heads
     int *status;
     int W;           // key tiles per range
     int n_seg;       // ranges per unit, from the host bounds (the device's lengths may need fewer)
@@ -434,9 +434,9 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 //   one range per CTA        W x query tiles (0.7 W for at most 64 rows) + 4, + 0.3 for every eight parts of a row that a lane of
 //                            the merge reads (merge_rounds): nothing hides the query load and the exchange of the row statistics.
 //                            As a cluster, where all units' clusters run at once, the ranges of a unit exchange for 1 at 16 of
-//                            them; else for 1.5 and, as the CTAs that poll, up to 1 more; + 0.5 for single tiles (36 units of 8 key tiles x 96 rows:
-//                            17.2 us in ranges of 2 tiles, whose 36 clusters of 4 do not fit, 13.4 in ranges of 3; 2 units of
-//                            27 x 256 14.5 us in 27 ranges without a cluster, 18.5 in clusters of 14);
+//                            them; else for 1.5 and, as the CTAs that poll, up to 1 more; + 0.5 for single tiles (36 units of
+//                            8 key tiles x 96 rows: 17.2 us in ranges of 2 tiles, whose 36 clusters of 4 do not fit, 13.4 in
+//                            ranges of 3; 2 units of 27 x 256 14.5 us in 27 ranges without a cluster, 18.5 in clusters of 14);
 //   several ("windows")      windows x (W x query tiles + 2), or + 5 where the ranges of a unit meet across CTAs and are too
 //                            short to hide it (28 x 8 units of 9 key tiles x 160 rows: whole units 55 us although a quarter
 //                            of the second window's CTAs idle, ranges of 3 tiles 82 us);

@@ -632,7 +632,7 @@ struct Softmax {
         return c0 + c1;
     }
     // Second sweep over key tiles [t0, t1) against the staged statistics `stats` (and limits): column sums to the writer, or,
-    // DIRECT, for units of one query tile, whose keys have no other rows, to the scores `out`.
+    // DIRECT, for units of one query tile, whose keys have no other rows, to `scores`.
     template <bool DIRECT = false>
     __device__ __forceinline__ bool colsum_segment(const UnitInfo &u, const Rows &R, int t0, int t1, const float2 *stats,
                                                    const int *lim, const int2 *bounds, float *scores = nullptr) {

@@ -19,7 +19,7 @@ constexpr int kQTiles = kMaxRows / kRows;
 constexpr int kGroups = 4;       // softmax groups of four warps; each owns one accumulator of 128 tensor-memory columns
 constexpr int kMaxStages = 6;    // key-tile ring
 constexpr int kSumBufs = 8;      // column-sum hand-over buffers, one per accumulator in flight
-constexpr int kCtlWarps = 4;     // producer, MMA issuer, statistics warp, column-sum warp
+constexpr int kCtlWarps = 4;     // producer, MMA issuer, statistics warp, column-sum warp or second MMA issuer
 constexpr int kSoftmaxWarps = 16;
 constexpr int kTcThreads = (kCtlWarps + kSoftmaxWarps) * 32;
 constexpr int kBigBox = 64;      // query rows per TMA box where a head has that many; kRowPad-row boxes otherwise

@@ -237,7 +237,7 @@ def test_score_plan_of_the_benchmark_configurations(lib):
     assert _plan(32, 32, 8, 128, 128, 2048, 2048, requests=2) == (two, 0)
     assert _plan(32, 32, 8, 128, 128, 2048, 2048, dtype=fb.FINCH_F32) == (warp, 0)
     assert _plan(2, 8, 8, 96, 64, 512, 512) == (warp, 0)
-    assert _plan(32, 32, 8, 128, 192, 2048, 2048) == (two, 0)     # 4 heads x 3 sub-blocks = 12 > 8
+    assert _plan(32, 32, 8, 128, 192, 2048, 2048) == (two, 0)     # 768 rows: halves, which two launches beat by the estimate
     assert _plan(32, 32, 8, 128, 128, 2048, 2048)[1] * 128 * 4 == 4096  # four windows per unit
 
 

@@ -234,11 +234,47 @@ def test_single_request_scored_in_two_launches_selects_and_copies_in_one(layers,
         np.testing.assert_array_equal(runs[0][name], runs[1][name], err_msg=name)
 
 
+@pytest.mark.parametrize("layers,Hq,Hkv,n_q,cache,chunk,rope_theta", [
+    (1, 2, 2, 40, 100, 40, 0.0),           # few rows
+    (3, 8, 4, 300, 700, 129, 10000.0),     # 608 rows per KV head, kept keys rotated
+    (2, 4, 1, 520, 300, 900, 0.0),         # five chunks of rows
+])
+def test_causal_request_selects_and_copies_in_one_launch(layers, Hq, Hkv, n_q, cache, chunk, rope_theta):
+    """A single request with limits: finch_step has one kernel less than its three calls, their results, and the oracle's scores."""
+    cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=64, planted_frac=0.05,
+                    requests=(wl.Request(n_q, 9999, chunk, cache),))
+    st = wl.steady_state(cfg, list(range(layers)), step=1)
+    limit = np.minimum(cache + 1 + np.arange(n_q), cache + chunk).astype(np.int32)
+    runs, launches = [], []
+    for parts in (False, True):
+        g = GpuStep(cfg, st, layers, row_limit=limit)
+        try:
+            if rope_theta:
+                fb.finch_ctx_destroy(g.ctx)
+                g.ctx = fb.finch_ctx_create(layers, Hq, Hkv, 64, fb.FINCH_BF16, 0, max_batch=1, max_prompt=n_q,
+                                            max_candidates=g.batch.c.max_cache + g.batch.c.max_chunk, rope_theta=rope_theta)
+            assert fb.finch_score_plan(g.ctx, g.batch)[0] == fb.FINCH_SCORE_TWO_LAUNCH
+            before = fb.finch_launch_count(g.ctx)
+            g.run_parts() if parts else g.run()
+            launches.append(fb.finch_launch_count(g.ctx) - before)
+            assert g.status() == 0
+            runs.append(g.results())
+        finally:
+            g.close()
+    assert launches[1] - launches[0] == 1
+    for name in ("kept_idx", "out_len", "out_pos", "out_k", "out_v"):
+        np.testing.assert_array_equal(runs[0][name], runs[1][name], err_msg=name)
+    if not rope_theta:
+        check_parity(cfg, st, runs[0], oracle_scores(cfg, st, threads=oracle.max_threads(), row_limit=limit))
+
+
 @pytest.mark.parametrize("fill", [float("nan"), 3e4])
-@pytest.mark.parametrize("layers,n_q,extra,causal", [(1, 37, 3, False), (12, 9, 40, False), (1, 150, 1, False), (2, 37, 5, True)])
+@pytest.mark.parametrize("layers,n_q,extra,causal", [(1, 37, 3, False), (12, 9, 40, False), (1, 150, 1, False), (1, 257, 3, False),
+                                                     (2, 37, 5, True)])
 def test_rows_behind_the_requests_reach_no_score(layers, n_q, extra, causal, fill):
     """A query tensor with rows behind the last request's: they are no prompt rows, whatever they hold.  One kernel with one
-    window and with several, more than 512 padded rows, masked rows: bit for bit the scores of the tensor without them."""
+    window and with several, halves of a KV head's queries, chunks of 512 rows in two launches (1056 padded rows), masked
+    rows: bit for bit the scores of the tensor without them."""
     import torch
     cfg = wl.scaled(wl.CONFIGS["c3"], n_layers=layers, n_q_heads=16, n_kv_heads=4, head_dim=64, planted_frac=0.02,
                     requests=(wl.Request(n_q, 9999, 300, 500),))
@@ -337,6 +373,8 @@ def test_units_of_one_query_tile(layers, Hkv, heads, d, n_q, cache, chunk):
     (1, 2, 4, 129, 100, 70, 0, True),      # 544 rows: two halves of 272, three query tiles each
     (2, 2, 2, 255, 300, 300, 1, True),     # a query head each, sums over four units to a group
     (3, 2, 8, 128, 1000, 500, 0, True),    # 512 rows each
+    (2, 1, 72, 8, 300, 200, 0, True),      # so many query heads that no prompt's rows are resident whole
+    (1, 2, 128, 5, 100, 300, 1, True),     # .. nor more than eight of half of them
     (3, 2, 8, 129, 300, 200, 0, False),    # 544: two launches
     (1, 2, 3, 200, 300, 200, 0, False),    # an odd number of query heads
     (70, 2, 4, 160, 300, 200, 0, True),    # more halves than SMs: whole units in two windows

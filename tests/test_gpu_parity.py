@@ -99,6 +99,9 @@ def test_wide_logit_range_on_the_tensor_core_path(scale):
     ("f32", 4, 2, 64, [(70, 999, 130, 65), (3, 999, 20, 10)], 0),            # warp-level path
     ("f32", 4, 2, 32, [(33, 999, 50, 40)], 1),                               # warp-level path, per-layer groups
     ("bf16", 4, 2, 64, [(40, 9999, 90, 70)], 1),                             # per-layer groups (tensor-core path, heads summed)
+    ("bf16", 8, 2, 128, [(150, 9999, 300, 333)], 0),                         # one request of 608 rows: halves of a KV head's queries
+    ("bf16", 8, 2, 64, [(256, 9999, 200, 170)], 1),                          # .. of 512 rows each, summed per layer
+    ("bf16", 6, 2, 64, [(180, 9999, 90, 170)], 0),                           # 552 rows of three heads: no halves, two launches
 ])
 def test_prompt_self_term_in_the_softmax_denominator(dtype, Hq, Hkv, d, reqs, group_mode):
     # the full attention row of a prompt token also covers the prompt's own keys (Method, "N = m + n^que + c"):
