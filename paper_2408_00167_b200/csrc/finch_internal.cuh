@@ -68,7 +68,7 @@ struct Ctx {
     cudaEvent_t ev_entry, ev_v_ready, ev_selected;
 };
 
-enum { kSmemSelect = 0, kSmemFused = 1, kSmemTc = 5 };  // bits of smem_bits; kSmemFused + variant, kSmemTc + variant
+enum { kSmemSelect = 0, kSmemFused = 1, kSmemTc = 9 };  // bits of smem_bits; kSmemFused + variant, kSmemTc + variant
 
 inline TensorView view_of(const finch_tensor *t) {
     return TensorView{(const char *)t->ptr, t->stride_layer, t->stride_head, t->stride_tok};

@@ -51,7 +51,6 @@ struct FusedParams {
     int q_tiles;     // query tiles the shared memory holds
     int cluster;     // CTAs of a cluster: the unit's ranges, with one window and few ranges per unit; else 1
     int key_shift;   // units that share a KV head, as a power of two (scoring_view)
-    int delay;       // 0: a CTA has one window; 1: phase B of a window follows phase A of the next
 };
 
 __device__ __forceinline__ int ld_acquire_gpu(const int *p) {
@@ -96,7 +95,7 @@ struct Seg {
     int sweep, unit, t0, t1, slot, win;
 };
 
-// The segments of one CTA, in order: phase A of window k, then phase B of window k - delay.
+// The segments of one CTA, in order: phase A of window k, then phase B of window k - delay (0 with one window, 1 with several).
 struct Walk {
     int W, T, n_seg, delay, n_win, step, ph;
     __device__ bool next(Seg &s) {
@@ -227,7 +226,10 @@ __device__ __noinline__ void give_up(int *published, int *left, int ranges, int 
 }
 
 // PAIR: units of one query tile, and no column sums to be added: the writer's warp is a second MMA issuer, the softmax warps write.
-template <int D, bool PAIR>
+// ONE: a CTA has one window at most, and the softmax warps merge the statistics themselves.  (Kernels of their own: with either merge
+// in the other's kernel its loops came out by up to 2 % slower or faster as the other's code changed.  32 x 32 units of 8 key tiles x
+// 64 rows 89.3 -> 87.6 us, 32 x 8 of 27 x 256 165.0 -> 160.6, 28 x 8 of 9 x 160 52.6 -> 51.4, 192 of 8 x 64, head_dim 64, 24.2 -> 23.1.)
+template <int D, bool PAIR, bool ONE>
 __global__ void __launch_bounds__(kTcThreads, 1)
 score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_constant__ CUtensorMap q_small,
                    const __grid_constant__ CUtensorMap cache_map, const __grid_constant__ CUtensorMap chunk_map,
@@ -237,14 +239,14 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
     const ModelView &mv = p.mv;
     const BatchView &bv = p.bv;
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp-uniform for the compiler
-    const bool direct = p.delay == 0;  // the softmax warps merge the statistics themselves
+    const int cluster = ONE ? p.cluster : 1;
     if (threadIdx.x == 0) {
         prefetch_tensormap(&q_big);
         prefetch_tensormap(&q_small);
         prefetch_tensormap(&cache_map);
         prefetch_tensormap(&chunk_map);
     }
-    const uint32_t tmem = cta_setup(c, direct ? kSoftmaxWarps : 1, p.cluster, PAIR ? 2 : 1);
+    const uint32_t tmem = cta_setup(c, ONE ? kSoftmaxWarps : 1, cluster, PAIR ? 2 : 1);
     // The inputs were written by what precedes this kernel.  The successor is NOT allowed to launch early: its CTAs
     // would take over the SMs of the CTAs that finish first and park there in their wait (measured: + 20 us on the
     // 0.5 ms step of 32 layers x 8 KV heads x 4096 candidates).
@@ -252,18 +254,18 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
 
     UnitInfo u = unit_info(mv, bv, 0, 0);  // l and G are set per segment
     const Rows R = make_rows(u.n_q, mv.hpg, 0);
-    const int T = n_key_tiles(u), n_seg = p.cluster > 1 ? p.n_seg : (T + p.W - 1) / p.W;
+    const int T = n_key_tiles(u), n_seg = cluster > 1 ? p.n_seg : (T + p.W - 1) / p.W;
     const bool run = u.ok && u.n_q > 0 && u.N > 0;
     const int n_ranges = mv.L * mv.G * n_seg;
     const int n_win = run && (int)blockIdx.x < n_ranges ? (n_ranges - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     if (!u.ok && threadIdx.x == 0 && blockIdx.x == 0) atomicOr(p.status, FINCH_DEV_BAD_BATCH);
     const Tickets tickets{p.tickets, p.tickets + mv.L * mv.G, n_seg};
-    Walk walk{p.W, T, n_seg, p.delay, n_win, 0, 0};
+    Walk walk{p.W, T, n_seg, ONE ? 0 : 1, n_win, 0, 0};
     Seg sg;
     bool ok = true, left = false;
     // With several windows the sweeps of two units alternate.  Where the ring holds both their query tiles a window loads
     // its queries once and keeps them for its second sweep (64 rows: 0.105 -> 0.09 ms for 1024 units of 8 key tiles).
-    const bool retain = p.delay && 2 * R.n_qt <= p.q_tiles;
+    const bool retain = !ONE && 2 * R.n_qt <= p.q_tiles;
     TileRing ring{p.q_tiles};
 #define FINCH_UNIT(s) (u.l = (s).unit / mv.G, u.G = (s).unit % mv.G)
 
@@ -301,7 +303,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         // every range of the unit has published and stages the merged rows for the segment's phase B, which the softmax
         // warps reach one phase A later.  Two buffers in turn: this warp cannot be two segments ahead, it waits for
         // the softmax warps' phase A in between.
-        if (!direct) {
+        if (!ONE) {
             int segs = 0, good = 1;
             while (walk.next(sg)) {
                 if (sg.sweep) continue;
@@ -344,17 +346,17 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
             if (sg.sweep == 0) {
                 Softmax<false>::RowStats st;
                 if (!(ok = role.lse_segment(u, R, sg.t0, sg.t1, live, no_limit, st))) {
-                    if (direct && p.cluster == 1) give_up(tickets.published, tickets.left, n_seg, sg.unit, true);
+                    if (ONE && cluster == 1) give_up(tickets.published, tickets.left, n_seg, sg.unit, true);
                     break;
                 }
-                if (p.cluster > 1) {
+                if (cluster > 1) {
                     // the unit's ranges are the CTAs of this cluster: the parts stay in shared memory, every warp tells
                     // every CTA that its own are written
                     float2 *parts = c.stats + 2 * p.rows_alloc;
                     role.store_stats(R, st, live, parts, p.rows_alloc, false);
                     __syncwarp();
                     cluster_wait();  // everybody's barriers are initialised
-                    if (lane < p.cluster) mbar_arrive_remote(map_to_rank(smem_u32(c.parts_ready), lane));
+                    if (lane < cluster) mbar_arrive_remote(map_to_rank(smem_u32(c.parts_ready), lane));
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait_cluster(c.parts_ready, 0, c.abort_flag)))) {
                         cluster_arrive();
                         left = true;
@@ -372,7 +374,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
                 role.store_stats(R, st, live, p.partial + ((int64_t)sg.unit * p.n_seg + sg.slot) * kGroups * p.rows_alloc, p.rows_alloc,
                                  false);
                 __syncwarp();
-                if (!direct) {
+                if (!ONE) {
                     if (lane == 0) count_arrive(c.a_count);
                     continue;
                 }
@@ -400,8 +402,8 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
                 if (tid == 0) tickets.leave(sg.unit);  // every warp of this CTA has seen the ticket complete, or gives up
                 if (!ok) break;
             } else {
-                const int b = direct ? 0 : segs_b & 1;
-                if (!direct && !(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[b], (segs_b >> 1) & 1, c.abort_flag)))) break;
+                const int b = ONE ? 0 : segs_b & 1;
+                if (!ONE && !(ok = __all_sync(0xffffffffu, mbar_wait(&c.stats_ready[b], (segs_b >> 1) & 1, c.abort_flag)))) break;
                 ok = role.template colsum_segment<PAIR>(u, R, sg.t0, sg.t1, c.stats + b * p.rows_alloc, nullptr, nullptr,
                                                         p.unit_scores + sg.unit * ((int64_t)bv.total_cache + bv.total_chunk) + u.cache0 + u.chunk0);
                 ++segs_b;
@@ -409,7 +411,7 @@ score_fused_kernel(const __grid_constant__ CUtensorMap q_big, const __grid_const
         }
     }
 #undef FINCH_UNIT
-    cta_teardown(c, tmem, p.status, p.cluster, left);
+    cta_teardown(c, tmem, p.status, cluster, left);
 }
 
 // scores of a selection group that spans several KV heads (one group per layer): the heads' column sums, added in
@@ -529,7 +531,7 @@ bool fits_clusters(const Ctx &ctx, int size, int units) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, score_fused_kernel<D, PAIR>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&n, score_fused_kernel<D, PAIR, true>, &cfg) != cudaSuccess) {
             (void)cudaGetLastError();
             return false;
         }
@@ -547,23 +549,25 @@ cudaError_t launch_fused_d(const Ctx &ctx, const CUtensorMap &qb, const CUtensor
     const ModelView &mv = p.mv;
     const BatchView &bv = p.bv;
     const int sms = ctx.sm_count > 0 ? ctx.sm_count : 148, n_qt = p.rows_alloc / kRows;
-    p.delay = n_ranges > sms;
+    const bool one = n_ranges <= sms;
     // room for the queries of the two units that alternate, and of a third that is being loaded where they are short
-    p.q_tiles = !p.delay || n_qt > 2 ? n_qt : n_qt + 2;
+    p.q_tiles = one || n_qt > 2 ? n_qt : n_qt + 2;
+    const auto kernel = one ? score_fused_kernel<D, PAIR, true> : score_fused_kernel<D, PAIR, false>;
+    const int bit = kSmemFused + (D == 128) + 2 * PAIR + 4 * one;
     cudaError_t e = cudaSuccess;
-    if (!ctx.smem_ready(kSmemFused + (D == 128) + 2 * PAIR)) {
-        e = cudaFuncSetAttribute(score_fused_kernel<D, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(score_fused_kernel<D, PAIR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (!ctx.smem_ready(bit)) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+        if (e == cudaSuccess && one) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
-        ctx.smem_set(kSmemFused + (D == 128) + 2 * PAIR);
+        ctx.smem_set(bit);
     }
-    p.cluster = !p.delay && p.n_seg > 1 && p.n_seg <= kMaxCluster && fits_clusters<D, PAIR>(ctx, p.n_seg, mv.L * mv.G) ? p.n_seg : 1;
+    p.cluster = one && p.n_seg > 1 && p.n_seg <= kMaxCluster && fits_clusters<D, PAIR>(ctx, p.n_seg, mv.L * mv.G) ? p.n_seg : 1;
     const int parts = p.cluster > 1 ? kGroups * p.rows_alloc * 8 : 0;  // the cluster's exchange of row statistics
     p.stages = kMaxStages;
     while (p.stages > 2 && cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) + parts > kSmemLimit) --p.stages;
     const int smem = cta_smem(kTileBytes, p.q_tiles, p.rows_alloc, p.stages, false) + parts;
     dim3 grid(n_ranges < sms ? n_ranges : sms);  // persistent and resident at once: phase B waits for neighbours
-    e = launch_chained_cluster(score_fused_kernel<D, PAIR>, p.cluster, grid, dim3(kTcThreads), smem, stream, qb, qs, cm, hm, p);
+    e = launch_chained_cluster(kernel, p.cluster, grid, dim3(kTcThreads), smem, stream, qb, qs, cm, hm, p);
     ctx.launches += 1;
     if (e != cudaSuccess || heads_per_group == 1) return e;
     return launch_sum_heads(ctx, mv, bv, p.unit_scores, scores, out_groups, heads_per_group, stream);
