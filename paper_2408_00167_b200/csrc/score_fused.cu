@@ -449,7 +449,7 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 // sent few units with many short ranges to two launches: 2 units of 23 tiles x 24 rows 25.6 us, 12.8 in ranges of 2).
 // halves: a unit is half the query heads of a KV head.  Both halves fetch the keys: several windows have to be better by a tenth, and
 // are whole units, unless a divisor would be estimated better still: there two launches are shorter (24 x 32 units of 14 key tiles x
-// 288 rows 564 us, 601 in whole units), as they are for units of fewer than eight accumulators (176 of 2 x 320 rows 31.3 us, 35.7).
+// 288 rows 564 us, 601 in whole units), as they are for units of fewer than twelve accumulators (176 of 2 x 320 rows 31.3 us, 35.7; 192 of 2 x 464 41.8, 44.5).
 // With one range per CTA a unit's last range may be shorter.  Several windows: ranges that divide the unit, of at least four
 // tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
 constexpr int kMaxCluster = 16;
@@ -486,7 +486,7 @@ int choose_window(long long units, int T, int ctas, int tile_bytes, int rows, bo
             if ((W < 4 && W < T) || n_seg > 8 || T % W || (long long)W * ctas * tile_bytes > l2_budget) continue;
             cost = windows * (W * q_tiles * 10 + (n_seg > 1 && W * q_tiles < 16 ? 50 : 20)) * (halves ? 11 : 10) / 10;
             if (halves && W < T) barred = min(barred, cost);
-            if (halves && (W < T || W * q_tiles < 8)) continue;
+            if (halves && (W < T || W * q_tiles < 12)) continue;
         }
         if (cost < (windows == 1 ? two_small : two_launches) && cost < best_cost) {
             best_cost = cost;

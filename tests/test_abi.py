@@ -318,4 +318,5 @@ def test_score_plan_of_small_calls(lib):
     assert _plan(1, 4, 2, 128, 128, 1792, 1664) == (one, 1)       # 2 units of 27 key tiles x 256 rows
     assert _plan(1, 6, 2, 128, 8, 1536, 1408)[0] == one           # .. of 23 x 24
     assert _plan(24, 32, 4, 128, 96, 128, 128) == (two, 0)        # 192 halves of 2 key tiles x 384 rows
-    assert _plan(70, 8, 2, 128, 160, 300, 200)[0] == one          # .. 280 of 5 x 320
+    assert _plan(12, 32, 8, 128, 227, 33, 27) == (two, 0)         # .. of 2 x 464
+    assert _plan(70, 8, 2, 128, 160, 300, 200)[0] == one          # 280 of 5 x 320
