@@ -449,7 +449,8 @@ sum_heads_kernel(ModelView mv, BatchView bv, const float *unit_scores, float *sc
 // sent few units with many short ranges to two launches: 2 units of 23 tiles x 24 rows 25.6 us, 12.8 in ranges of 2).
 // halves: a unit is half the query heads of a KV head.  Both halves fetch the keys: several windows have to be better by a tenth, and
 // are whole units, unless a divisor would be estimated better still: there two launches are shorter (24 x 32 units of 14 key tiles x
-// 288 rows 564 us, 601 in whole units), as they are for units of fewer than twelve accumulators (176 of 2 x 320 rows 31.3 us, 35.7; 192 of 2 x 464 41.8, 44.5).
+// 288 rows 564 us, 601 in whole units), as they are for units of fewer than twelve accumulators (176 of 2 x 320 rows 31.3 us, 35.7;
+// 192 of 2 x 464 41.8, 44.5).
 // With one range per CTA a unit's last range may be shorter.  Several windows: ranges that divide the unit, of at least four
 // tiles (or the unit), at most 8 to a unit, and keys in flight between a window's sweeps that mostly stay in L2.
 constexpr int kMaxCluster = 16;
@@ -592,11 +593,12 @@ int score_fused_window(const Ctx &ctx, const BatchView &bv) {
     if (rows > kMaxRows) return 0;
     const int tiles = (bv.max_cache + kRows - 1) / kRows + (bv.max_chunk + kRows - 1) / kRows;
     // Halves of a KV head's queries: with one window, where the calls are latency and two launches of two chunks of rows each take longer
-    // (scoring of 27 single requests of 1 to 12 layers, 129 to 256 prompt rows x 4 heads: 1.45 times as fast, 6 x 2 units of 9 key tiles
-    // x 992 rows 41.2 -> 25.0 us, 3 x 8 of 19 x 752 56.4 -> 46.5; none slower), and as whole units in several (14 x 8 units of 8 x 896
-    // 100.6 -> 89.4, 32 x 4 of 20 x 712 177 -> 163, 23 x 8 of 11 x 544 130 -> 126).  In shorter ranges of several windows, whose
-    // statistics meet across CTAs, 11 x 8 units of 20 x 800 took 166 us instead of 146.  Where the estimates are within 10 %, two
-    // launches (31 x 8 units of 17 x 832 325 us, 334 in halves; 24 x 8 of 12 x 576 136, 140).
+    // (36 single requests of 1 to 12 layers, 129 to 256 prompt rows x 4 heads: scoring 1.3 times as fast, 1.45 the 27 that the rule
+    // takes; 6 x 2 units of 9 key tiles x 992 rows 41.2 -> 25.0 us, 3 x 8 of 19 x 752 56.4 -> 46.5), and as whole units in several
+    // (224 halves of 4 x 320 rows 51.4 -> 47.2, 256 of 10 x 384 105 -> 91, 1280 of 11 x 368 453 -> 408).  In shorter ranges of several
+    // windows, whose statistics meet across CTAs, 11 x 8 units of 20 x 800 took 166 us instead of 146.  Where the estimates are within
+    // 10 %, two launches (31 x 8 units of 17 x 832 325 us, 334 in halves; 24 x 8 of 12 x 576 136, 140), although some would be shorter
+    // (14 x 8 of 8 x 896 100.6, 89.4).
     return choose_window((long long)mv.L * mv.G, tiles, sms, (mv.d / 64) * kSlabBytes, rows, mv.G != mv.Hkv);
 }
 
